@@ -8,6 +8,7 @@
 // DevState block (bound, mark counts, new sizes) between phases.
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -166,6 +167,7 @@ struct mincut_graph {
   // row-wise contraction (allocated at the first contraction that uses it)
   RowScratch rows{};
   long long acc_zeroed = 0;  // dense accumulator slots known to be zero
+  long long m_bound = 0;     // while m_pending: an upper bound of M
   bool m_pending = false;    // M of the current graph is in st->m_rows (not yet read)
   int64_t* rpG = nullptr;
   int* colG = nullptr;
@@ -189,6 +191,12 @@ struct mincut_graph {
   unsigned long long* seq_multi_tree = nullptr;
   int* seq_multi_order = nullptr;
   int* seq_multi_mark = nullptr;
+  // certificate forests (allocated at first use)
+  long long fo_qsoft = 1;  // a quarter of the input's mean entry weight
+  uint8_t* fo_tag = nullptr;
+  int* fo_r = nullptr;
+  int2* fo_items = nullptr;
+  unsigned char* fo_ctl = nullptr;
   // sort
   SortScratch sort{};
   // state
@@ -470,6 +478,15 @@ int ensure_seq_multi(mincut_graph* g, int want) {
   return k;
 }
 
+int ensure_forest(mincut_graph* g) {
+  if (g->fo_ctl) return MINCUT_OK;
+  if (!galloc(g, &g->fo_tag, g->n0) || !galloc(g, &g->fo_r, g->n0) ||
+      !galloc(g, &g->fo_items, forest_item_cap(g->n0, g->M0)) ||
+      !galloc(g, &g->fo_ctl, (long long)forest_ctl_bytes()))
+    return fail(MINCUT_ERR_OOM, "forest buffers");
+  return MINCUT_OK;
+}
+
 int ensure_lp(mincut_graph* g) {
   if (g->lab[0]) return MINCUT_OK;
   const size_t wsz = g->wt64 ? 8 : 4;
@@ -619,6 +636,7 @@ int contract_current(mincut_graph* g, int* n2_out, long long* m2_out, bool compo
   g->cur = nxt;
   g->n = n2;
   g->M = m2;
+  g->m_bound = M;
   g->m_pending = m2 < 0;
   *n2_out = n2;
   *m2_out = m2;
@@ -628,6 +646,12 @@ int contract_current(mincut_graph* g, int* n2_out, long long* m2_out, bool compo
 // Graphs of at most this many vertices skip the concurrent passes in the
 // rounds after one where they marked almost nothing.
 constexpr int kSkipConcurrentMaxN = 8192;
+
+// Forests that join fewer than 1 / kForestWeakDiv of the vertices leave the
+// round to the other marks as well.  Where they work they join a fifth to all
+// of the vertices (planted cuts 0.20-0.25 in the first round, R-MAT cores
+// 0.998); where they do not (two interleaved heavy cycles) none at all.
+constexpr int kForestWeakDiv = 8;
 
 struct RoundCfg {
   int lp_iters, lp_min_n;
@@ -640,6 +664,7 @@ struct RoundCfg {
   int cf_private = 0;  // concurrent passes with private visit sets
   int seq_passes = 1;  // sequential passes when the concurrent ones mark nothing (0: auto)
   int seq_kernel = 0;  // 0: warp-driven passes; 1: block passes (smaller-id ties)
+  bool forest = false;  // certificate forests first; the other marks only if they join little
   bool coarsen = false;  // heuristic round: also join every label-propagation cluster
   bool skip_concurrent = false;  // capforest 1: go straight to the whole-graph passes
   // capforest 1, >= 0: the concurrent passes stand down (decided on the
@@ -664,6 +689,7 @@ struct RoundOut {
   long long lambda = kInf;
   long long marks_pr = 0, marks_cf = 0;
   long long marks_cc = 0;  // of marks_cf, those of the concurrent passes
+  bool forest_weak = false;  // the forests joined too little: the other marks ran too
   bool cc_ran = false;     // the concurrent passes ran (were not skipped)
   long long cf_nscanned = 0, cf_nmarks = 0;
   int src = 0;  // which bound source set lambda this round
@@ -686,18 +712,42 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     ProfScope ps(P_DEGREE, n, s);
     CK(degrees_min<WT>(deg, n, g->blk, g->st, s, &g->launches));
   }
-  int rc = sync_state(g);
+  int rc;
+  const bool forest = c.forest && n > 2;
+  if (forest) {
+    // the sort keys are free during the marking: they hold the union-finds
+    rc = ensure_forest(g);
+    if (rc) return rc;
+    ProfScope ps(P_FOREST, g->m_pending ? 0 : g->M, s);
+    CK(forest_marks<WT>(n, g->m_pending ? g->m_bound : g->M, rp, col, w, deg,
+                        reinterpret_cast<int*>(g->keys[0]), 2 * std::max<long long>(g->Mraw, 1),
+                        g->fo_tag, g->fo_r, g->fo_items, g->fo_ctl, g->parent, g->fo_qsoft, g->sms,
+                        g->spin_limit, g->st, s, &g->launches));
+  }
+  rc = sync_state(g);
   if (rc) return rc;
   if (g->m_pending) {  // the previous contraction's entry count came with this sync
     g->M = g->hst->m_rows;
     g->m_pending = false;
   }
   const long long M = g->M;
-  long long lam = (long long)g->hst->lambda;
+  // the degree bound, then what the forests' prefix cuts add to it
+  const bool cf_first = forest && g->hst->cf_val == g->hst->lambda &&
+                        g->hst->cf_pass == kForestPass;
+  long long lam = cf_first ? std::min(lambda_before, (long long)g->hst->deg_val)
+                           : (long long)g->hst->lambda;
   if (lam < lambda_before) {
     ProfScope ps(P_WITNESS, g->n0, s);
     CK(side_from_vertex(g->side0, g->map0, g->n0, g->hst->deg_arg, s, &g->launches));
     o->src = 1;
+    lambda_before = lam;
+  }
+  if (cf_first) {
+    lam = (long long)g->hst->lambda;
+    ProfScope ps(P_WITNESS, g->n0, s);
+    CK(side_from_batches(g->side0, g->map0, g->n0, g->fo_tag, g->hst->cf_len, g->sms, s,
+                         &g->launches));
+    o->src = 3;
     lambda_before = lam;
   }
   o->lambda = lam;
@@ -707,6 +757,14 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   }
   { ProfScope ps(P_TILES, n, s);
     CK(tile_rows(rp, n, M, g->tile_row, s, &g->launches)); }
+  if (forest) {
+    o->marks_cf = (long long)g->hst->marks_cf;
+    if (o->marks_cf * kForestWeakDiv >= n) {  // enough: the forests are the round's marks
+      o->lambda = lam;
+      return MINCUT_OK;
+    }
+    o->forest_weak = true;
+  }
   const int* lab_final = nullptr;
   if (c.lp_now && c.lp_iters > 0 && n >= c.lp_min_n) {
     rc = ensure_lp(g);
@@ -737,7 +795,7 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
                          cudaMemcpyDeviceToHost, s));
   }
   { ProfScope ps(P_UF, n, s);
-    CK(uf_init(g->parent, n, s, &g->launches));
+    if (!forest) CK(uf_init(g->parent, n, s, &g->launches));  // (else the forests' components)
     if (c.coarsen && lab_final)
       CK(uf_from_groups(g->parent, lab_final, g->gmin, n, g->st, s, &g->launches)); }
   uint8_t* flags_dev = c.pr_flags_host ? reinterpret_cast<uint8_t*>(g->vals[1]) : nullptr;
@@ -951,6 +1009,12 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
   // ran: they stand down in rounds whose PR tests hook at least n / 64
   bool cc_low = false;
   bool barely = false;  // the last contraction kept at least half the vertices
+  // certificate forests lead every round of a solve left to its defaults; once
+  // they joined too little, they wait until the graph has halved
+  const bool forests = !op.deterministic && op.seq_kernel == 0 && op.seq_passes == 0 &&
+                       op.cf_visit == 0 && op.max_rounds == 0 && !op.lp_every_round;
+  int forest_below = INT_MAX;
+  bool lp_done = !lp_allowed;
   for (;; ++*round_io) {
     const int round = *round_io;
     if (op.max_rounds > 0 && round >= op.max_rounds) break;
@@ -963,7 +1027,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     c.skip_concurrent = skip_cc && g->n <= kSkipConcurrentMaxN;
     c.eager_seq = c.skip_concurrent && barely;
     c.cc_skip_pr = cc_low && c.capforest == 1 && op.cf_visit != 2 ? (g->n + 63) / 64 : -1;
-    c.lp_now = lp_allowed && (op.lp_every_round || round == 0);
+    c.forest = forests && g->n < forest_below;
+    c.lp_now = lp_allowed && (op.lp_every_round || !lp_done);
     c.passes = op.passes > 0 ? op.passes : std::max(32, std::min(g->max_passes, g->n / 4));
     c.seed = op.seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(round + 1);
     const auto t0 = std::chrono::steady_clock::now();
@@ -972,6 +1037,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     int rc = mark_round<WT>(g, c, lambda, &o);
     if (rc) return rc;
     if (o.src) stl->lambda_source = o.src;
+    if (o.forest_weak) forest_below = n_before / 2;
+    if (!c.forest || o.forest_weak) lp_done = true;
     // concurrent passes that marked almost nothing before the whole-graph
     // passes had to run: small graphs skip them in the next round
     // (and keep skipping them while those passes keep running)
@@ -1368,6 +1435,7 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
   const size_t wsz = g->wt64 ? 8 : 4;
   g->n0 = n;
   g->Mraw = Mraw;
+  g->fo_qsoft = Mraw > 0 ? std::max<long long>(1, (long long)(hws[0] / (4ull * (unsigned long long)Mraw))) : 1;
   const long long Mb = std::max<long long>(Mraw, 1);
   // buffers
   bool ok = true;

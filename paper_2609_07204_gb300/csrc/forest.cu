@@ -1,0 +1,568 @@
+// forest.cu -- certificate forests: the marking step of a round as one
+// edge-parallel pass over the whole graph (one cooperative kernel).
+//
+// Certificate.  Let lam be the round's bound, q a quantum and k = ceil(lam/q).
+// An edge of weight c has floor(c/q) units.  Every edge puts its units into
+// k edge sets F_0 .. F_{k-1}: into the lowest levels whose components do not
+// yet join its ends, at most one unit per level, level i only once its ends
+// are joined in F_{i-1}.  Components of F_i therefore refine those of F_{i-1}
+// (the forest decomposition of Nagamochi and Ibaraki, with forests that need
+// not come from a maximum-adjacency order), so two vertices joined in F_{k-1}
+// are joined in each of the k edge-disjoint sets: their connectivity is at
+// least k q >= lam and they may be contracted.  This holds for every order of
+// the edges and every interleaving of threads: a level's union-find only ever
+// merges, and "joined in F_{i-1}" once read stays true.
+//
+// Order.  How much F_{k-1} joins does depend on the order.  A maximum-
+// adjacency order is the best known and strictly sequential; here the vertices
+// are scanned in a few batches, each the unscanned vertices of highest r (the
+// units inserted at them), at least 1 / kFoFrac of the vertices left where so
+// many are queued.  Counted on the CPU on the planted cut (2 x 2^13 vertices,
+// the entries of a batch in random order), the vertices F_{k-1} leaves: exact
+// order 0.80 n, batches of 1/50 0.80 n, 1/20 0.81 n, 1/10 0.83 n, 1/4 0.93 n:
+// ~50 grid-wide steps replace one dependent step per vertex.
+//
+// The prefix cuts of the batches (alpha, as in a CAPFOREST pass) are cuts of
+// the graph: the smallest lowers the bound, the scanned batches up to it its
+// witness.
+//
+// Cost.  An entry is read once, with its vertex: a stream read of (col, w) and
+// the far end's tag byte (scanned before: done).  The rest queue per warp, so
+// that the divergent part runs with full warps: the far end's r (the level to
+// try first), usually two adjacent levels of each end's row of parent words
+// (vertex-major: one 32-byte sector) and one CAS per unit, all random accesses
+// to L1 and L2 in a dependent chain of ~2 us.  Bound by that latency, hence:
+// cached reads everywhere (a root's word read through L2 by all SMs is one hot
+// line: 2.4x on the 2 x 2^19 cut together with the queues), halved paths, up
+// to four levels' CAS in flight, items fetched by whichever warp is free.
+//
+// Measured against the whole-graph CAPFOREST passes that such rounds needed
+// before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
+// 1,260 ms -> 17.0 ms, 2 x 2^15 82.8 -> 7.6 ms, G(2000, 16000) 2.03 -> 1.28 ms;
+// against PR tests, label propagation and concurrent passes: R-MAT scale 20
+// 10-core 3.69 -> 2.27 ms (1.0 ms of it here), scale 16
+// 1.12 -> 0.96 ms.
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace mc {
+
+namespace {
+
+constexpr int kFoThreads = 256;
+constexpr int kFoChunk = 256;     // entries of a row handled by one warp at a time
+constexpr int kFoMaxK = 254;      // levels (histogram bins: k + 1)
+constexpr int kFoBatches = 100;   // from this batch on, everything left is one batch
+constexpr int kFoFrac = 16;       // a batch takes at least 1 / kFoFrac of the vertices left
+constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
+
+struct FoCtl {
+  unsigned bar;        // grid barrier arrivals
+  unsigned abort_;     // a barrier wait ran out
+  unsigned items;      // work items listed so far
+  unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
+  long long alpha;     // cut of the scanned set
+  unsigned next[2];    // items fetched in a batch beyond the first deal (by its parity)
+  int hist[256];       // unscanned vertices by min(r, k)
+};
+
+struct FoArgs {
+  int n;
+  const int64_t* rp;
+  const int* col;
+  const void* w;
+  const void* deg;
+  int* F;              // n * k parent words, vertex-major; -1: root
+  long long fcap;      // ints in F
+  uint8_t* tag;        // per vertex: the batch it was scanned in (0: not yet), kFoMain
+  int* r;              // per vertex: units inserted at it while unscanned
+  int2* items;         // (vertex, chunk of its row)
+  int* parent;
+  FoCtl* ctl;
+  DevState* st;
+  long long spin;
+  long long qsoft;     // quantum that loses little of the weights
+};
+
+// Grid barrier number `gen` (1, 2, ...): false when the wait ran out (here or
+// in another block), after which every block leaves.
+__device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spin, int* s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned want = gen * gridDim.x;
+    unsigned v = atomicAdd(&c->bar, 1u) + 1u;
+    bool ok = true;
+    long long it = 0;
+    while (v < want) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->bar) : "memory");
+      if (++it > spin || *(volatile unsigned*)&c->abort_) {
+        atomicExch(&c->abort_, 1u);
+        ok = false;
+        break;
+      }
+    }
+    __threadfence();
+    *s_ok = ok ? 1 : 0;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// Top of x's tree at a level, halving the path, through cached loads: a stale
+// word names an ancestor all the same, so the result is an ancestor and, but
+// for merges this SM has not seen yet, the root.  Only words that are no
+// root's are written, with an ancestor.  F points at vertex 0's word.
+__device__ __forceinline__ int fo_root(int* F, int k, int x) {
+  for (;;) {
+    int* px = F + (long long)x * k;
+    const int p = *px;
+    if (p < 0) return x;
+    const int g = F[(long long)p * k];
+    if (g < 0) return p;
+    *px = g;
+    x = g;
+  }
+}
+
+// The same through L2, current at the time of each read.
+__device__ __forceinline__ int fo_root_l2(const int* F, int k, int x) {
+  for (;;) {
+    const int p = __ldcg(F + (long long)x * k);
+    if (p < 0) return x;
+    x = p;
+  }
+}
+
+// Whether x and y are known to be joined at the level (false may be stale).
+__device__ __forceinline__ bool fo_joined(int* F, int k, int x, int y) {
+  const int a = F[(long long)x * k], b = F[(long long)y * k];
+  const int a1 = a < 0 ? x : a, b1 = b < 0 ? y : b;
+  if (a1 == b1) return true;
+  if (a < 0 && b < 0) return false;
+  return fo_root(F, k, x) == fo_root(F, k, y);
+}
+
+// Join x and y at the level: true when they were separate.  The larger of the
+// two tops goes under the smaller one, whether that is still a root or not:
+// parents are smaller than their children, so it is not in the larger top's
+// own tree.  All reads are cached (a root's word is read by every thread: in
+// L2 its one line would serve them in turn); only the CAS has to see the
+// present, and where it fails it returns the way up.
+__device__ __forceinline__ bool fo_join(int* F, int k, int x, int y) {
+  for (;;) {
+    x = fo_root(F, k, x);
+    y = fo_root(F, k, y);
+    if (x == y) return false;
+    const int hi = max(x, y), lo = min(x, y);
+    const int p = atomicCAS(F + (long long)hi * k, -1, lo);
+    if (p < 0) return true;
+    x = p;  // p < hi: every turn moves up
+    y = lo;
+  }
+}
+
+// Insert `units` units of the edge {x, y}, level `guess` tried first; returns
+// the units inserted, or -1 if the last level joins x and y already.
+__device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units, int guess) {
+  int lo = 0, hi = guess;  // first level that does not join x and y, in [lo, hi]
+  if (fo_joined(F + guess, k, x, y)) {
+    if (guess == k - 1) return -1;
+    lo = guess + 1;
+    hi = k;
+    for (int st = 1; lo < hi; st *= 2) {
+      const int m = min(hi - 1, lo + st - 1);
+      if (!fo_joined(F + m, k, x, y)) {
+        hi = m;
+        break;
+      }
+      lo = m + 1;
+    }
+    if (lo >= k) return -1;
+  } else {
+    for (int st = 1; lo < hi; st *= 2) {
+      const int m = max(lo, hi - st);
+      if (fo_joined(F + m, k, x, y)) {
+        lo = m + 1;
+        break;
+      }
+      hi = m;
+    }
+  }
+  while (lo < hi) {
+    const int m = (lo + hi) >> 1;
+    if (fo_joined(F + m, k, x, y)) lo = m + 1;
+    else hi = m;
+  }
+  // up to four levels at a time: where one end is a root and the other's
+  // parent (or it) is smaller, which is most, the CAS goes out at once, the
+  // levels' round trips side by side
+  const int asked = units;
+  int* px = F + (long long)x * k;
+  int* py = F + (long long)y * k;
+  while (lo < k && units > 0) {
+    const int cnt = min(min(units, k - lo), 4);
+    int p[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      p[j] = 0;  // >= 0: this level is left to fo_join
+      if (j < cnt) {
+        const int a = px[lo + j], b = py[lo + j];
+        const int a1 = a < 0 ? x : a, b1 = b < 0 ? y : b;
+        if (b < 0 && a1 < y) p[j] = atomicCAS(&py[lo + j], -1, a1);
+        else if (a < 0 && b1 < x) p[j] = atomicCAS(&px[lo + j], -1, b1);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < cnt && (p[j] < 0 || fo_join(F + lo + j, k, x, y))) --units;
+    lo += cnt;
+  }
+  return asked - units;
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
+  __shared__ int s_hist[256];   // this block's changes since the last flush
+  __shared__ int s_all[256];
+  __shared__ unsigned s_scan[kFoThreads / 32];
+  __shared__ unsigned s_base;
+  __shared__ int s_ok, s_t, s_left, s_main;
+  __shared__ int2 s_q[kFoThreads / 32][64];      // queued edges of each warp
+  __shared__ uint8_t s_qu[kFoThreads / 32][64];  // and their units
+  __shared__ long long s_alpha[kFoThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int n = a.n;
+  const long long lam = (long long)*(volatile unsigned long long*)&a.st->lambda;
+  if (n <= 2 || lam <= 0 || lam >= kInf) return;  // (the round stops or has no bound)
+  const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
+  if (kcap < 1) return;
+  const long long q = max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + 7) / 8));
+  const int k = (int)((lam + q - 1) / q);
+  const WT* __restrict__ w = reinterpret_cast<const WT*>(a.w);
+  const WT* __restrict__ deg = reinterpret_cast<const WT*>(a.deg);
+  int* F = a.F;
+  uint8_t* tag = a.tag;
+  int* ru = a.r;
+  FoCtl* ctl = a.ctl;
+  const int gtid = blockIdx.x * kFoThreads + tid, gsize = gridDim.x * kFoThreads;
+  // ---- every vertex a root at every level, nothing scanned; the first batch
+  // is vertex 0
+  {
+    const long long words = (long long)n * k, quads = words / 4;
+    const int4 r4 = make_int4(-1, -1, -1, -1);
+    for (long long i = gtid; i < quads; i += gsize) reinterpret_cast<int4*>(F)[i] = r4;
+    for (long long i = quads * 4 + gtid; i < words; i += gsize) F[i] = -1;
+    for (int v = gtid; v < n; v += gsize) {
+      tag[v] = v == 0 ? 1 : 0;
+      ru[v] = 0;
+    }
+    for (int i = tid; i < 256; i += kFoThreads) s_hist[i] = 0;
+    if (blockIdx.x == 0) {
+      const int chunks = max(1, (int)((a.rp[1] - a.rp[0] + kFoChunk - 1) / kFoChunk));
+      for (int c = tid; c < chunks; c += kFoThreads) __stcg(&a.items[c], make_int2(0, c));
+      if (tid == 0) {
+        atomicExch(&ctl->items, (unsigned)chunks);
+        ctl->hist[0] = n - 1;
+      }
+    }
+  }
+  unsigned gen = 0;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+  unsigned start = 0;
+  long long best = kInf;
+  int best_batch = 0;
+  for (int b = 1;; ++b) {
+    if (b > 1) {
+      // ---- the batch: the highest r until 1 / kFoFrac of the vertices left
+      // are taken; the whole queue if it is smaller; everything left when
+      // nothing is queued (another component) or after kFoBatches batches
+      for (int i = tid; i < 256; i += kFoThreads) s_all[i] = i <= k ? __ldcg(&ctl->hist[i]) : 0;
+      __syncthreads();
+      if (wp == 0) {
+        int left = 0;
+        for (int i = lane; i <= k; i += 32) left += s_all[i];
+        left = warp_sum(left);
+        if (lane == 0) {
+          const int need = max(1, left / kFoFrac);
+          int t = k, acc = s_all[k];
+          while (t > 1 && acc < need) acc += s_all[--t];
+          if (acc == 0 || b >= kFoBatches) t = 0;
+          s_t = t;
+          s_left = left;
+        }
+      }
+      __syncthreads();
+      const int left = s_left, t = s_t;
+      // the batches before this one are a proper subset while anything is left
+      const long long al = *(volatile long long*)&ctl->alpha;
+      if (left > 0 && al < best) {
+        best = al;
+        best_batch = b - 1;
+      }
+      if (left <= 0) break;
+      for (long long v0 = (long long)blockIdx.x * kFoThreads; v0 < n;
+           v0 += (long long)gridDim.x * kFoThreads) {
+        const int v = (int)v0 + tid;
+        int chunks = 0;
+        if (v < n) {
+          const unsigned tg = tag[v];
+          if ((tg & 127u) == 0) {
+            const int key = min(ru[v], k);
+            if (key >= t) {
+              tag[v] = (uint8_t)(tg | (unsigned)b);
+              atomicSub(&s_hist[key], 1);
+              chunks = max(1, (int)((a.rp[v + 1] - a.rp[v] + kFoChunk - 1) / kFoChunk));
+            }
+          }
+        }
+        int incl = chunks;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(FULL, incl, o);
+          if (lane >= o) incl += u;
+        }
+        if (lane == 31) s_scan[wp] = incl;
+        __syncthreads();
+        unsigned before = 0, total = 0;
+#pragma unroll
+        for (int i = 0; i < kFoThreads / 32; ++i) {
+          if (i < wp) before += s_scan[i];
+          total += s_scan[i];
+        }
+        if (tid == 0 && total) s_base = atomicAdd(&ctl->items, total);
+        __syncthreads();
+        const unsigned at = s_base + before + (unsigned)(incl - chunks);
+        for (int c = 0; c < chunks; ++c) __stcg(&a.items[at + c], make_int2(v, c));
+        __syncthreads();
+      }
+      if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+    }
+    // ---- scan the batch: warps fetch items as they get free and walk their
+    // entries as one list; the entries that may change a forest queue up in
+    // shared memory until a full warp of them can be inserted together
+    const unsigned end = *(volatile unsigned*)&ctl->items;
+    const unsigned nitems = end - start;
+    const unsigned warps = gridDim.x * (kFoThreads / 32);
+    unsigned per = 1;
+    while (per < 32 && per * 8 * warps <= nitems) per *= 2;
+    const int rep = (int)*(volatile unsigned*)&ctl->main - 1;
+    const int main_root = rep >= 0 ? fo_root(F + (k - 1), k, rep) : -1;
+    if (tid == 0) s_main = rep >= 0;
+    long long alpha = 0;
+    int qn = 0;  // queued edges of this warp
+    __syncthreads();
+    unsigned i0 = (unsigned)(blockIdx.x * (kFoThreads / 32) + wp) * per;  // the first is dealt
+    while (i0 < nitems || qn > 0) {
+      int x = -1, len = 0;
+      unsigned eb = 0;
+      if (lane < (int)per && i0 + lane < nitems) {
+        const int2 it = __ldcg(&a.items[start + i0 + lane]);
+        x = it.x;
+        const unsigned rb = (unsigned)a.rp[x], re = (unsigned)a.rp[x + 1];
+        eb = rb + (unsigned)it.y * kFoChunk;
+        len = (int)min((unsigned)kFoChunk, re - eb);
+        if (it.y == 0) alpha += (long long)deg[x];
+      }
+      const bool last = i0 >= nitems;
+      if (!last && lane == 0) i0 = warps * per + atomicAdd(&ctl->next[b & 1], per);
+      i0 = __shfl_sync(FULL, i0, 0);
+      int incl = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += u;
+      }
+      const int total = __shfl_sync(FULL, incl, 31);
+      const unsigned e_first = eb - (unsigned)(incl - len);  // position 0, as if it were x's
+      for (int p0 = 0; p0 < total || last; p0 += 32) {
+        if (!last) {
+          const int p = p0 + lane;
+          int o = 0;  // the item of position p: the first whose inclusive end is above p
+#pragma unroll
+          for (int stp = 16; stp > 0; stp >>= 1) {
+            const int v = __shfl_sync(FULL, incl, o + stp - 1);
+            if (v <= p) o += stp;
+          }
+          const int xx = __shfl_sync(FULL, x, o);
+          const unsigned e = __shfl_sync(FULL, e_first, o) + (unsigned)p;
+          bool keep = false;
+          int y = 0, u = 0;
+          if (p < total) {
+            y = a.col[e];
+            const long long c = (long long)w[e];
+            const unsigned ty = tag[y], tx = tag[xx];
+            const int by = (int)(ty & 127u);
+            u = (int)min((long long)k, q == 1 ? c : c / q);
+            if (by != 0 && by < b) {  // inserted when y was scanned
+              alpha -= 2 * c;
+            } else {
+              // both ends in this batch: the smaller id inserts
+              if (by == b) alpha -= c;
+              keep = u > 0 && !(by == b && xx > y) && !(ty & tx & kFoMain);
+            }
+          }
+          const unsigned bal = __ballot_sync(FULL, keep);
+          if (keep) {
+            const int at = qn + __popc(bal & lanemask_lt());
+            s_q[wp][at] = make_int2(xx, y);
+            s_qu[wp][at] = (uint8_t)u;
+          }
+          qn += __popc(bal);
+          __syncwarp();
+          if (qn < 32) continue;
+        }
+        // insert up to 32 queued edges (the last ones of the queue)
+        const int take = min(qn, 32);
+        qn -= take;
+        if (lane < take) {
+          const int2 xy = s_q[wp][qn + lane];
+          const int u = s_qu[wp][qn + lane];
+          const int y = xy.y;
+          const unsigned ty = tag[y];
+          const bool out = (ty & 127u) == 0;
+          const int got = fo_insert(F, k, xy.x, y, u, min(ru[y], k - 1));
+          if (got < 0) {
+            if (main_root >= 0 && fo_root(F + (k - 1), k, y) == main_root) {
+              tag[y] = (uint8_t)(ty | kFoMain);
+              tag[xy.x] = (uint8_t)(tag[xy.x] | kFoMain);
+            }
+            if (out && ru[y] < k) {
+              const int old = atomicMax(&ru[y], k);
+              if (old < k) {
+                atomicSub(&s_hist[old], 1);
+                atomicAdd(&s_hist[k], 1);
+              }
+            }
+          } else if (got > 0 && out) {
+            const int old = atomicAdd(&ru[y], got);
+            if (old < k) {
+              atomicSub(&s_hist[old], 1);
+              atomicAdd(&s_hist[min(k, old + got)], 1);
+              if (old + got >= k && !*(volatile int*)&s_main) {
+                *(volatile int*)&s_main = 1;
+                atomicCAS(&ctl->main, 0u, (unsigned)y + 1u);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (last && qn == 0) break;
+      }
+    }
+    if (blockIdx.x == 0 && tid == 0) ctl->next[(b + 1) & 1] = 0;
+    alpha = warp_sum(alpha);
+    if (lane == 0) s_alpha[wp] = alpha;
+    __syncthreads();
+    if (tid == 0) {
+      long long sum = 0;
+      for (int i = 0; i < kFoThreads / 32; ++i) sum += s_alpha[i];
+      if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->alpha), (unsigned long long)sum);
+    }
+    for (int i = tid; i <= k; i += kFoThreads) {
+      const int d = s_hist[i];
+      if (d) {
+        atomicAdd(&ctl->hist[i], d);
+        s_hist[i] = 0;
+      }
+    }
+    start = end;
+    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+  }
+  // ---- the round's marks: the components of the last level
+  unsigned joined = 0;
+  for (int v = gtid; v < n; v += gsize) {
+    const int r = fo_root_l2(F + (k - 1), k, v);
+    a.parent[v] = r;
+    joined += r != v;
+  }
+  joined = warp_sum(joined);
+  if (lane == 0 && joined) atomicAdd(&a.st->marks_cf, (unsigned long long)joined);
+  if (blockIdx.x == 0 && tid == 0) {
+    if (best < lam) {
+      atomicMin(&a.st->lambda, (unsigned long long)best);
+      a.st->cf_val = (unsigned long long)best;
+      a.st->cf_pass = kForestPass;
+      a.st->cf_len = best_batch;
+    }
+  }
+}
+
+__global__ void fo_timeout_kernel(const FoCtl* c, DevState* st) {
+  if (c->abort_) set_error(st, ERR_TIMEOUT);
+}
+
+__global__ void side_batch_kernel(uint8_t* side0, const int* __restrict__ map0, int n0,
+                                  const uint8_t* __restrict__ tag, int last) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n0; i += gridDim.x * blockDim.x) {
+    const int b = (int)(tag[map0[i]] & 127u);
+    side0[i] = b >= 1 && b <= last ? 1 : 0;
+  }
+}
+
+}  // namespace
+
+long long forest_item_cap(long long n, long long M) { return n + M / kFoChunk + 1; }
+size_t forest_ctl_bytes() { return sizeof(FoCtl); }
+
+template <typename WT>
+cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, const WT* w,
+                         const WT* deg, int* F, long long fcap, uint8_t* tag, int* r,
+                         int2* items, void* ctl, int* parent, long long qsoft, int sms, long long spin, DevState* st,
+                         cudaStream_t s, int* launches) {
+  static int per_sm[2] = {0, 0};
+  const int wi = sizeof(WT) == 8 ? 1 : 0;
+  if (!per_sm[wi]) {
+    int p = 0;
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, forest_kernel<WT>, kFoThreads, 0);
+    if (e != cudaSuccess) return e;
+    per_sm[wi] = std::max(1, p);
+  }
+  cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(FoCtl), s);
+  if (e != cudaSuccess) return e;
+  FoArgs a{};
+  a.n = n;
+  a.rp = rp;
+  a.col = col;
+  a.w = w;
+  a.deg = deg;
+  a.F = F;
+  a.fcap = fcap;
+  a.tag = tag;
+  a.r = r;
+  a.qsoft = qsoft;
+  a.items = items;
+  a.parent = parent;
+  a.ctl = static_cast<FoCtl*>(ctl);
+  a.st = st;
+  a.spin = spin;
+  const long long want = (std::max<long long>(M, n) + 4 * kFoThreads - 1) / (4 * kFoThreads);
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(want, (long long)sms * per_sm[wi]));
+  void* params[] = {&a};
+  e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
+                                  params, 0, s);
+  if (e != cudaSuccess) return e;
+  fo_timeout_kernel<<<1, 1, 0, s>>>(a.ctl, st);
+  *launches += 2;
+  return cudaGetLastError();
+}
+
+cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uint8_t* tag, int last,
+                              int sms, cudaStream_t s, int* launches) {
+  side_batch_kernel<<<std::max(1, std::min((n0 + 255) / 256, sms * 8)), 256, 0, s>>>(
+      side0, map0, n0, tag, last);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+#define MC_FO_INST(WT)                                                                           \
+  template cudaError_t forest_marks<WT>(int, long long, const int64_t*, const int*, const WT*,   \
+                                        const WT*, int*, long long, uint8_t*, int*, int2*,       \
+                                        void*, int*, long long, int, long long, DevState*, cudaStream_t, int*);
+MC_FO_INST(int32_t)
+MC_FO_INST(int64_t)
+
+}  // namespace mc

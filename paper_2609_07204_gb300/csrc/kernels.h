@@ -92,7 +92,8 @@ void set_last_error(const char* msg);
 // stream (category, units processed).  Resolved after the stream synchronises.
 enum ProfCat {
   P_DEGREE, P_LP_SWEEP, P_LP_BOUND, P_PR, P_CF_PASSES, P_CF_SEQ, P_UF, P_EMIT,
-  P_SORT_HIST, P_SORT_PASS, P_BUILD, P_TILES, P_WITNESS, P_OTHER, P_ROWS, P_BATCH_WARP, P_NCAT
+  P_SORT_HIST, P_SORT_PASS, P_BUILD, P_TILES, P_WITNESS, P_OTHER, P_ROWS, P_BATCH_WARP,
+  P_FOREST, P_NCAT
 };
 const char* prof_name(int cat);
 struct Profiler;
@@ -344,6 +345,27 @@ cudaError_t capforest_warp_passes(int n, long long M, const int64_t* rp, const i
                                   int* order_pool, int* mark_pool, unsigned long long* pass_best,
                                   int* pass_len, int stop_low, DevState* st, cudaStream_t s,
                                   int* launches);
+
+// --------------------------------------------------------------- forest.cu
+// Certificate forests of the current graph: parent[v] = the smallest vertex
+// of v's component of the last forest (vertices of one component have
+// connectivity at least st->lambda at launch), the number of joined vertices
+// added to st->marks_cf; prefix cuts below the bound lower st->lambda and
+// name their witness in cf_val, cf_pass = kForestPass, cf_len = last batch
+// (side_from_batches over `state`).  Does nothing when n <= 2 or the bound is
+// 0.  F: fcap ints of scratch, at least 2 per vertex; state: n; items:
+// forest_item_cap(n, M); ctl: forest_ctl_bytes().  One cooperative kernel;
+// its grid barriers wait at most `spin` reads (ERR_TIMEOUT).
+constexpr int kForestPass = -0x7fffffff;
+long long forest_item_cap(long long n, long long M);
+size_t forest_ctl_bytes();
+template <typename WT>
+cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, const WT* w,
+                         const WT* deg, int* F, long long fcap, uint8_t* tag, int* r,
+                         int2* items, void* ctl, int* parent, long long qsoft, int sms, long long spin, DevState* st,
+                         cudaStream_t s, int* launches);
+cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uint8_t* tag, int last,
+                              int sms, cudaStream_t s, int* launches);
 
 // ------------------------------------------------------------- contract.cu
 // Row-wise contraction when most groups are single vertices: singleton rows

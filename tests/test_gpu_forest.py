@@ -1,0 +1,66 @@
+"""Certificate forests (the marking step that leads a default solve's rounds)
+at the sizes where they can go wrong: fewer vertices than a warp, rows beyond
+one chunk, weights beyond the levels, several components, 64-bit weights, long
+paths, cliques.  Every value against the oracle or a closed form, every side
+against the cut weight."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests import graphs as G
+from tests.test_gpu_parity import _check_solve, canon, mc
+
+pytestmark = pytest.mark.gpu
+
+def _hub_and_cycle(n, hub_w):
+    """A hub joined to every vertex of a random cycle (rows of n - 1 entries)."""
+    rng = np.random.default_rng(n)
+    e = [(0, i) for i in range(1, n)] + [(i, i % (n - 1) + 1) for i in range(1, n)]
+    w = [int(x) for x in rng.integers(1, hub_w + 1, n - 1)] + \
+        [int(x) for x in rng.integers(1, 8, n - 1)]
+    return G.from_edges(n, e, w)
+
+@pytest.mark.parametrize("n", [3, 4, 5, 31, 32, 33, 255, 257, 700])
+def test_small_random(n):
+    rng = np.random.default_rng(n)
+    for hi in (1, 10, 1000, 2_000_000):
+        g = G.random_graph(n, min(1.0, 8.0 / n), rng, 1, hi, connected=True)
+        _check_solve(n, canon(n, *g))
+
+@pytest.mark.parametrize("n,hub_w", [(258, 1), (513, 40), (1025, 400), (2050, 3)])
+def test_long_rows(n, hub_w):
+    c = canon(n, *_hub_and_cycle(n, hub_w))
+    _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+
+@pytest.mark.parametrize("n", [600, 5000, 70_001])
+def test_long_cycles(n):
+    """Θ(n) diameter: the last batch takes what the others left."""
+    rng = np.random.default_rng(n)
+    w = rng.integers(3, 50, n)
+    two = np.sort(w)[:2].sum()
+    _check_solve(n, canon(n, *G.cycle(n, [int(x) for x in w])), expect=int(two))
+
+def test_components_and_cliques():
+    a = G.complete(60, 7)
+    _check_solve(60, canon(60, *a), expect=59 * 7)
+    # two components: cut 0
+    rp, col, w = a
+    both = (np.concatenate([rp, rp[1:] + rp[-1]]), np.concatenate([col, col + 60]).astype(np.int32),
+            np.concatenate([w, w]))
+    _check_solve(120, canon(120, *both), expect=0)
+
+def test_planted_cut_64bit_weights():
+    """Unit weights scaled past a total of 2^31: the same rounds in 64 bits."""
+    s = synth.planted(1 << 10, 21 << 10, 30, 9, 1, 11)
+    c = (s.row_ptr, s.col, s.w.astype(np.int64))
+    lam = oracle.noi(s.n, *c)[0]
+    assert _check_solve(s.n, c, expect=lam)["seq_passes"] == 0
+    big = (s.row_ptr, s.col, s.w.astype(np.int64) * 60_000)
+    _check_solve(s.n, big, expect=lam * 60_000)
+
+@pytest.mark.parametrize("seed", range(3))
+def test_random_sparse_20000(seed):
+    g = synth.er_connected(20_000, 100_000, 1, 30, 50 + seed)
+    c = (g.row_ptr, g.col, g.w.astype(np.int64))
+    _check_solve(g.n, c, expect=oracle.noi(g.n, *c)[0])
