@@ -192,7 +192,7 @@ struct mincut_graph {
   int* seq_multi_order = nullptr;
   int* seq_multi_mark = nullptr;
   // certificate forests (allocated at first use)
-  long long fo_qsoft = 1;  // a quarter of the input's mean entry weight
+  long long fo_qsoft = 1;  // half the input's mean entry weight
   uint8_t* fo_tag = nullptr;
   int* fo_r = nullptr;
   int2* fo_items = nullptr;
@@ -1435,7 +1435,8 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
   const size_t wsz = g->wt64 ? 8 : 4;
   g->n0 = n;
   g->Mraw = Mraw;
-  g->fo_qsoft = Mraw > 0 ? std::max<long long>(1, (long long)(hws[0] / (4ull * (unsigned long long)Mraw))) : 1;
+  if (Mraw > 0)
+    g->fo_qsoft = std::max<long long>(1, (long long)((hws[0] / (unsigned long long)Mraw + 1) / 2));
   const long long Mb = std::max<long long>(Mraw, 1);
   // buffers
   bool ok = true;

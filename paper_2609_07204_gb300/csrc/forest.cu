@@ -16,11 +16,13 @@
 // Order.  How much F_{k-1} joins does depend on the order.  A maximum-
 // adjacency order is the best known and strictly sequential; here the vertices
 // are scanned in a few batches, each the unscanned vertices of highest r (the
-// units inserted at them), at least 1 / kFoFrac of the vertices left where so
-// many are queued.  Counted on the CPU on the planted cut (2 x 2^13 vertices,
+// units that met them), at least 1 / kFoFrac of the vertices left and 1 / kFoTail
+// of all where so many are queued.  Counted on the CPU on the planted cut (2 x 2^13 vertices,
 // the entries of a batch in random order), the vertices F_{k-1} leaves: exact
 // order 0.80 n, batches of 1/50 0.80 n, 1/20 0.81 n, 1/10 0.83 n, 1/4 0.93 n:
-// ~50 grid-wide steps replace one dependent step per vertex.
+// ~30 grid-wide steps replace one dependent step per vertex (1/16 without the
+// 1/64 of all, ~50 steps: 6% slower on both planted cuts; 1/8 as fast, but now
+// and then a round too weak).
 //
 // The prefix cuts of the batches (alpha, as in a CAPFOREST pass) are cuts of
 // the graph: the smallest lowers the bound, the scanned batches up to it its
@@ -31,18 +33,22 @@
 // that the divergent part runs with full warps: the far end's r (the level to
 // try first), usually two adjacent levels of each end's row of parent words
 // (vertex-major: one 32-byte sector) and one CAS per unit, all random accesses
-// to L1 and L2 in a dependent chain of ~2 us.  Bound by that latency, hence:
-// cached reads everywhere (a root's word read through L2 by all SMs is one hot
-// line: 2.4x on the 2 x 2^19 cut together with the queues), halved paths, up
-// to four levels' CAS in flight, items fetched by whichever warp is free.
+// to L1 and L2 in a dependent chain of ~2 us.  Bound by that latency and by
+// what makes the chain longer, hence (each measured on whole solves): cached
+// reads everywhere and queues (2.4x), links by rank instead of by id and the
+// far end's count raised before the insertion (together 1.2x on the planted
+// cuts, 1.3x on R-MAT), up to four levels' CAS in flight, long rows in pieces
+// of 64 (against 256: 1.2x on the 2 x 2^19 cut, whose merged regions become
+// rows of 10^5 entries), pieces fetched by whichever warp is free.
 //
 // Measured against the whole-graph CAPFOREST passes that such rounds needed
 // before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
-// 1,260 ms -> 17.0 ms, 2 x 2^15 82.8 -> 7.6 ms, G(2000, 16000) 2.03 -> 1.28 ms;
-// against PR tests, label propagation and concurrent passes: R-MAT scale 20
-// 10-core 3.69 -> 2.27 ms (1.0 ms of it here), scale 16
-// 1.12 -> 0.96 ms.
+// 1,310 ms -> 16.3 ms, 2 x 2^15 81 -> 6.3 ms; against PR tests, label
+// propagation and concurrent passes: R-MAT scale 20 10-core 3.65 -> 1.73 ms,
+// scale 16 1.15 -> 0.66 ms, random weighted n = 150,001 (with its creation)
+// 2.63 -> 1.07 ms.
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -51,16 +57,23 @@ namespace mc {
 
 namespace {
 
-constexpr int kFoThreads = 256;
-constexpr int kFoChunk = 256;     // entries of a row handled by one warp at a time
+constexpr int kFoThreads = 512;
+constexpr int kFoChunk = 64;      // entries of a row handled by one warp at a time
 constexpr int kFoMaxK = 254;      // levels (histogram bins: k + 1)
+constexpr int kFoLevels = 8;      // levels wanted where the weights allow it (qsoft): fewer
+                                  // unions, and on random weights 1..100 all of the joins
 constexpr int kFoBatches = 100;   // from this batch on, everything left is one batch
-constexpr int kFoFrac = 16;       // a batch takes at least 1 / kFoFrac of the vertices left
+constexpr int kFoFrac = 12;       // a batch takes at least 1 / kFoFrac of the vertices left,
+constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
+constexpr unsigned kFoAbort = ~0u;
+
 struct FoCtl {
-  unsigned bar;        // grid barrier arrivals
-  unsigned abort_;     // a barrier wait ran out
+  unsigned bar;        // grid barrier: arrivals
+  unsigned pad[31];
+  unsigned release;    // grid barrier: the last one complete, or kFoAbort
+  unsigned pad2[31];
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
   long long alpha;     // cut of the scanned set
@@ -77,7 +90,7 @@ struct FoArgs {
   int* F;              // n * k parent words, vertex-major; -1: root
   long long fcap;      // ints in F
   uint8_t* tag;        // per vertex: the batch it was scanned in (0: not yet), kFoMain
-  int* r;              // per vertex: units inserted at it while unscanned
+  int* r;              // per vertex: units that met it while unscanned
   int2* items;         // (vertex, chunk of its row)
   int* parent;
   FoCtl* ctl;
@@ -87,22 +100,32 @@ struct FoArgs {
 };
 
 // Grid barrier number `gen` (1, 2, ...): false when the wait ran out (here or
-// in another block), after which every block leaves.
+// in another block), after which every block leaves.  The last block to arrive
+// releases the others through a word of its own line: the arrivals, atomics on
+// one word, do not queue up behind the polls (with both on one word a barrier
+// of 608 blocks took ~10 us).
 __device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spin, int* s_ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned want = gen * gridDim.x;
-    unsigned v = atomicAdd(&c->bar, 1u) + 1u;
     bool ok = true;
-    long long it = 0;
-    while (v < want) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->bar) : "memory");
-      if (++it > spin || *(volatile unsigned*)&c->abort_) {
-        atomicExch(&c->abort_, 1u);
-        ok = false;
-        break;
+    if (atomicAdd(&c->bar, 1u) + 1u == gen * gridDim.x) {
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->release), "r"(gen) : "memory");
+    } else {
+      unsigned v = 0;
+      long long it = 0;
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->release) : "memory");
+        if (v >= gen) break;
+        if (++it > spin) {  // (the value ends the wait of the others, too)
+          asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->release), "r"(kFoAbort)
+                       : "memory");
+          v = kFoAbort;
+          break;
+        }
+        __nanosleep(20);
       }
+      ok = v != kFoAbort;
     }
     __threadfence();
     *s_ok = ok ? 1 : 0;
@@ -111,29 +134,38 @@ __device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spi
   return *s_ok != 0;
 }
 
-// Top of x's tree at a level, halving the path, through cached loads: a stale
-// word names an ancestor all the same, so the result is an ancestor and, but
-// for merges this SM has not seen yet, the root.  Only words that are no
-// root's are written, with an ancestor.  F points at vertex 0's word.
-__device__ __forceinline__ int fo_root(int* F, int k, int x) {
+// A level's union-find, linked by rank: a root's word is -1 - rank, another's
+// its parent, and (rank, id) grows from child to parent, so concurrent links
+// close no cycle.  (Linked by id instead, the links of one batch build random
+// recursive trees, ~ln n deep, and every walk pays their depth.)  All reads
+// are cached: a stale word names an ancestor all the same, or an older rank of
+// a root; a root's word is read by every thread, and in L2 its one line would
+// serve them in turn.  Only the CAS has to see the present.
+
+// Top of x's tree, halving the path: an ancestor and, but for merges this SM
+// has not seen yet, the root; val: its word.  Only words that are no root's
+// are written, with an ancestor.  F points at vertex 0's word of the level.
+__device__ __forceinline__ int fo_root(int* F, int k, int x, int& val) {
   for (;;) {
     int* px = F + (long long)x * k;
     const int p = *px;
-    if (p < 0) return x;
+    if (p < 0) {
+      val = p;
+      return x;
+    }
     const int g = F[(long long)p * k];
-    if (g < 0) return p;
+    if (g < 0) {
+      val = g;
+      return p;
+    }
     *px = g;
     x = g;
   }
 }
 
-// The same through L2, current at the time of each read.
-__device__ __forceinline__ int fo_root_l2(const int* F, int k, int x) {
-  for (;;) {
-    const int p = __ldcg(F + (long long)x * k);
-    if (p < 0) return x;
-    x = p;
-  }
+__device__ __forceinline__ int fo_root(int* F, int k, int x) {
+  int val;
+  return fo_root(F, k, x, val);
 }
 
 // Whether x and y are known to be joined at the level (false may be stale).
@@ -145,22 +177,58 @@ __device__ __forceinline__ bool fo_joined(int* F, int k, int x, int y) {
   return fo_root(F, k, x) == fo_root(F, k, y);
 }
 
-// Join x and y at the level: true when they were separate.  The larger of the
-// two tops goes under the smaller one, whether that is still a root or not:
-// parents are smaller than their children, so it is not in the larger top's
-// own tree.  All reads are cached (a root's word is read by every thread: in
-// L2 its one line would serve them in turn); only the CAS has to see the
-// present, and where it fails it returns the way up.
-__device__ __forceinline__ bool fo_join(int* F, int k, int x, int y) {
+// Join the trees whose tops x and y (words vx, vy) are, or were when read:
+// true when they were separate.
+__device__ __forceinline__ bool fo_link(int* F, int k, int x, int vx, int y, int vy) {
   for (;;) {
-    x = fo_root(F, k, x);
-    y = fo_root(F, k, y);
     if (x == y) return false;
-    const int hi = max(x, y), lo = min(x, y);
-    const int p = atomicCAS(F + (long long)hi * k, -1, lo);
-    if (p < 0) return true;
-    x = p;  // p < hi: every turn moves up
-    y = lo;
+    if (vx < vy || (vx == vy && x > y)) {  // x: the lesser of the two
+      int t = x;
+      x = y;
+      y = t;
+      t = vx;
+      vx = vy;
+      vy = t;
+    }
+    const int p = atomicCAS(F + (long long)x * k, vx, y);
+    if (p == vx) {
+      if (vx == vy) atomicCAS(F + (long long)y * k, vy, vy - 1);
+      return true;
+    }
+    if (p < 0) {  // still a root, of a higher rank
+      vx = p;
+    } else {
+      // this SM held an old word: the store brings the new one into its cache
+      // (else every thread that meets it sends its own failing CAS)
+      F[(long long)x * k] = p;
+      x = fo_root(F, k, p, vx);
+    }
+  }
+}
+
+__device__ __forceinline__ bool fo_join(int* F, int k, int x, int y) {
+  int vx, vy;
+  x = fo_root(F, k, x, vx);
+  y = fo_root(F, k, y, vy);
+  return fo_link(F, k, x, vx, y, vy);
+}
+
+// A vertex about to be scanned takes rank 1 where it is still alone.  Of an
+// edge's two trees the scanned end's has a top of rank 1 and more then, and an
+// unscanned vertex alone is the lesser: it goes under the scanned end's parent
+// (or the end itself) without a look at its rank, which a first link need not
+// raise either -- all neighbours' links would do that, on one word.  For the
+// same reason a long row starts higher, by its length.
+__device__ __forceinline__ void fo_scanned(int* F, int k, int v, long long len) {
+  int* f = F + (long long)v * k;
+  const int word = len > 64 ? -2 - (58 - __clzll(len)) : -2;  // rank 1, + log2(len) - 5
+  for (int i0 = 0; i0 < k; i0 += 8) {
+    int w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = i0 + j < k ? f[i0 + j] : 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (w[j] == -1) f[i0 + j] = word;
   }
 }
 
@@ -196,9 +264,8 @@ __device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units,
     if (fo_joined(F + m, k, x, y)) lo = m + 1;
     else hi = m;
   }
-  // up to four levels at a time: where one end is a root and the other's
-  // parent (or it) is smaller, which is most, the CAS goes out at once, the
-  // levels' round trips side by side
+  // up to four levels at a time: where y is alone (fo_scanned), which is most,
+  // the levels' round trips go side by side
   const int asked = units;
   int* px = F + (long long)x * k;
   int* py = F + (long long)y * k;
@@ -207,17 +274,15 @@ __device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units,
     int p[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      p[j] = 0;  // >= 0: this level is left to fo_join
+      p[j] = 0;  // not -1: this level is left to fo_join
       if (j < cnt) {
         const int a = px[lo + j], b = py[lo + j];
-        const int a1 = a < 0 ? x : a, b1 = b < 0 ? y : b;
-        if (b < 0 && a1 < y) p[j] = atomicCAS(&py[lo + j], -1, a1);
-        else if (a < 0 && b1 < x) p[j] = atomicCAS(&px[lo + j], -1, b1);
+        if (b == -1) p[j] = atomicCAS(&py[lo + j], -1, a < 0 ? x : a);
       }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (j < cnt && (p[j] < 0 || fo_join(F + lo + j, k, x, y))) --units;
+      if (j < cnt && (p[j] == -1 || fo_join(F + lo + j, k, x, y))) --units;
     lo += cnt;
   }
   return asked - units;
@@ -239,7 +304,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   if (n <= 2 || lam <= 0 || lam >= kInf) return;  // (the round stops or has no bound)
   const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
   if (kcap < 1) return;
-  const long long q = max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + 7) / 8));
+  const long long q = max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + kFoLevels - 1) / kFoLevels));
   const int k = (int)((lam + q - 1) / q);
   const WT* __restrict__ w = reinterpret_cast<const WT*>(a.w);
   const WT* __restrict__ deg = reinterpret_cast<const WT*>(a.deg);
@@ -253,15 +318,18 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   {
     const long long words = (long long)n * k, quads = words / 4;
     const int4 r4 = make_int4(-1, -1, -1, -1);
-    for (long long i = gtid; i < quads; i += gsize) reinterpret_cast<int4*>(F)[i] = r4;
-    for (long long i = quads * 4 + gtid; i < words; i += gsize) F[i] = -1;
+    const long long own = (k + 3) / 4;  // (vertex 0's words are set below)
+    for (long long i = own + gtid; i < quads; i += gsize) reinterpret_cast<int4*>(F)[i] = r4;
+    for (long long i = max(quads, own) * 4 + gtid; i < words; i += gsize) F[i] = -1;
+    for (int i = gtid; i < min(own * 4, words); i += gsize) F[i] = i < k ? -2 : -1;
     for (int v = gtid; v < n; v += gsize) {
       tag[v] = v == 0 ? 1 : 0;
       ru[v] = 0;
     }
     for (int i = tid; i < 256; i += kFoThreads) s_hist[i] = 0;
     if (blockIdx.x == 0) {
-      const int chunks = max(1, (int)((a.rp[1] - a.rp[0] + kFoChunk - 1) / kFoChunk));
+      const long long len = a.rp[1] - a.rp[0];
+      const int chunks = max(1, (int)((len + kFoChunk - 1) / kFoChunk));
       for (int c = tid; c < chunks; c += kFoThreads) __stcg(&a.items[c], make_int2(0, c));
       if (tid == 0) {
         atomicExch(&ctl->items, (unsigned)chunks);
@@ -286,7 +354,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
         for (int i = lane; i <= k; i += 32) left += s_all[i];
         left = warp_sum(left);
         if (lane == 0) {
-          const int need = max(1, left / kFoFrac);
+          const int need = max(left / kFoFrac, max(n / kFoTail, 32));
           int t = k, acc = s_all[k];
           while (t > 1 && acc < need) acc += s_all[--t];
           if (acc == 0 || b >= kFoBatches) t = 0;
@@ -314,7 +382,9 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
             if (key >= t) {
               tag[v] = (uint8_t)(tg | (unsigned)b);
               atomicSub(&s_hist[key], 1);
-              chunks = max(1, (int)((a.rp[v + 1] - a.rp[v] + kFoChunk - 1) / kFoChunk));
+              const long long len = a.rp[v + 1] - a.rp[v];
+              chunks = max(1, (int)((len + kFoChunk - 1) / kFoChunk));
+              fo_scanned(F, k, v, len);
             }
           }
         }
@@ -340,8 +410,9 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
       if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
     }
-    // ---- scan the batch: warps fetch items as they get free and walk their
-    // entries as one list; the entries that may change a forest queue up in
+    // ---- scan the batch: a warp walks the entries of a few items (short rows,
+    // pieces of long ones) as one list, fetched as warps get free (dealt in
+    // turn: 1.15-1.4x the time); the entries that may change a forest queue up in
     // shared memory until a full warp of them can be inserted together
     const unsigned end = *(volatile unsigned*)&ctl->items;
     const unsigned nitems = end - start;
@@ -354,7 +425,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     long long alpha = 0;
     int qn = 0;  // queued edges of this warp
     __syncthreads();
-    unsigned i0 = (unsigned)(blockIdx.x * (kFoThreads / 32) + wp) * per;  // the first is dealt
+    unsigned i0 = (unsigned)(blockIdx.x * (kFoThreads / 32) + wp) * per;
     while (i0 < nitems || qn > 0) {
       int x = -1, len = 0;
       unsigned eb = 0;
@@ -417,36 +488,41 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
         // insert up to 32 queued edges (the last ones of the queue)
         const int take = min(qn, 32);
         qn -= take;
+        int from = 0, to = 0;  // y's key before and after, if it changed
         if (lane < take) {
           const int2 xy = s_q[wp][qn + lane];
           const int u = s_qu[wp][qn + lane];
           const int y = xy.y;
           const unsigned ty = tag[y];
           const bool out = (ty & 127u) == 0;
-          const int got = fo_insert(F, k, xy.x, y, u, min(ru[y], k - 1));
-          if (got < 0) {
-            if (main_root >= 0 && fo_root(F + (k - 1), k, y) == main_root) {
-              tag[y] = (uint8_t)(ty | kFoMain);
-              tag[xy.x] = (uint8_t)(tag[xy.x] | kFoMain);
-            }
-            if (out && ru[y] < k) {
-              const int old = atomicMax(&ru[y], k);
-              if (old < k) {
-                atomicSub(&s_hist[old], 1);
-                atomicAdd(&s_hist[k], 1);
-              }
-            }
-          } else if (got > 0 && out) {
-            const int old = atomicAdd(&ru[y], got);
-            if (old < k) {
-              atomicSub(&s_hist[old], 1);
-              atomicAdd(&s_hist[min(k, old + got)], 1);
-              if (old + got >= k && !*(volatile int*)&s_main) {
+          // y's count goes up first: the edges that meet at y get levels of
+          // their own to try (from a count raised after the insertion each
+          // would climb past all those in flight: 60 us a batch)
+          int g = ru[y];
+          if (g < k) {
+            g = atomicAdd(&ru[y], u);
+            if (out && g < k) {
+              from = g;
+              to = min(k, g + u);
+              if (to == k && !*(volatile int*)&s_main) {
                 *(volatile int*)&s_main = 1;
                 atomicCAS(&ctl->main, 0u, (unsigned)y + 1u);
               }
             }
+            if (g >= k) ru[y] = k;  // (this SM's old copy would bring every edge here)
           }
+          if (fo_insert(F, k, xy.x, y, u, min(g, k - 1)) < 0 && main_root >= 0 &&
+              fo_root(F + (k - 1), k, y) == main_root) {
+            tag[y] = (uint8_t)(ty | kFoMain);
+            tag[xy.x] = (uint8_t)(tag[xy.x] | kFoMain);
+          }
+        }
+        // one shared atomic per distinct change, not per lane
+        const unsigned change = from < to ? ((unsigned)from << 8) | (unsigned)to : 0u;
+        const unsigned same = __match_any_sync(FULL, change);
+        if (change && (same & lanemask_lt()) == 0) {
+          atomicSub(&s_hist[from], __popc(same));
+          atomicAdd(&s_hist[to], __popc(same));
         }
         __syncwarp();
         if (last && qn == 0) break;
@@ -471,13 +547,21 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     start = end;
     if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
   }
-  // ---- the round's marks: the components of the last level
+  // ---- the round's marks: the components of the last level, each under its
+  // smallest member (r, done with, holds it per root; a warp's vertices of one
+  // root send one atomic)
+  for (int v = gtid; v < n; v += gsize) ru[v] = INT_MAX;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
   unsigned joined = 0;
-  for (int v = gtid; v < n; v += gsize) {
-    const int r = fo_root_l2(F + (k - 1), k, v);
-    a.parent[v] = r;
-    joined += r != v;
+  for (int v0 = gtid - lane; v0 < n; v0 += gsize) {
+    const int v = v0 + lane;
+    const int r = v < n ? fo_root(F + (k - 1), k, v) : -1;
+    const unsigned same = __match_any_sync(FULL, r);
+    if (r >= 0 && (same & lanemask_lt()) == 0) atomicMin(&ru[r], v);
+    joined += r >= 0 && r != v;
   }
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+  for (int v = gtid; v < n; v += gsize) a.parent[v] = ru[fo_root(F + (k - 1), k, v)];
   joined = warp_sum(joined);
   if (lane == 0 && joined) atomicAdd(&a.st->marks_cf, (unsigned long long)joined);
   if (blockIdx.x == 0 && tid == 0) {
@@ -491,7 +575,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
 }
 
 __global__ void fo_timeout_kernel(const FoCtl* c, DevState* st) {
-  if (c->abort_) set_error(st, ERR_TIMEOUT);
+  if (c->release == kFoAbort) set_error(st, ERR_TIMEOUT);
 }
 
 __global__ void side_batch_kernel(uint8_t* side0, const int* __restrict__ map0, int n0,
@@ -539,7 +623,7 @@ cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, 
   a.ctl = static_cast<FoCtl*>(ctl);
   a.st = st;
   a.spin = spin;
-  const long long want = (std::max<long long>(M, n) + 4 * kFoThreads - 1) / (4 * kFoThreads);
+  const long long want = (std::max<long long>(M, n) + 2 * kFoThreads - 1) / (2 * kFoThreads);
   const int blocks = (int)std::max<long long>(1, std::min<long long>(want, (long long)sms * per_sm[wi]));
   void* params[] = {&a};
   e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
