@@ -79,7 +79,8 @@ __device__ BwSlot bw_slot(int* base, long long slot_words, int slot, int nmax, i
 }
 
 __global__ void __launch_bounds__(kBwWarps * 32)
-    batch_warp_kernel(const int* __restrict__ list, int nlist, int* cursor,
+    batch_warp_kernel(const int* __restrict__ list, int nlist_max,
+                      const int* __restrict__ nlist_dev, int* cursor,
                       const int* __restrict__ voff0, const int64_t* __restrict__ rp0,
                       const int* __restrict__ col0, const int* __restrict__ w0, int* scratch,
                       long long slot_words, int nmax, int mmax, uint32_t pr_mask,
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(kBwWarps * 32)
   unsigned* l2 = l1 + kBwMaxN / 32;                            // kBwMaxN / 1024
   int* tl = reinterpret_cast<int*>(l2 + kBwMaxN / 1024);       // 32
   int* tcount = tl + 32;                                       // 1
+  const int nlist = nlist_dev ? min(*nlist_dev, nlist_max) : nlist_max;
   int fail = 0;  // the first failed check: 1 rounds, 2 union-find, 3 / 4 tree descent
   for (;;) {
     int item = 0;
@@ -403,7 +405,8 @@ cudaError_t batch_warp_mark(const int* list, int nlist, int* done_g, DevState* s
   return cudaGetLastError();
 }
 
-cudaError_t batch_warp_solve(const int* list, int nlist, int* cursor, const int* voff0,
+cudaError_t batch_warp_solve(const int* list, int nlist, const int* nlist_dev, int* cursor,
+                             const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
                              unsigned long long* lam_g, uint8_t* side0, DevState* st,
@@ -415,7 +418,7 @@ cudaError_t batch_warp_solve(const int* list, int nlist, int* cursor, const int*
   const int blocks = slots / kBwWarps;
   if (!bw_set_smem()) return cudaErrorInvalidValue;
   batch_warp_kernel<<<blocks, kBwWarps * 32, kBwSmemBytes, s>>>(
-      list, nlist, cursor, voff0, rp0, col0, w0, scratch, batch_warp_slot_words(nmax, mmax), nmax,
+      list, nlist, nlist_dev, cursor, voff0, rp0, col0, w0, scratch, batch_warp_slot_words(nmax, mmax), nmax,
       mmax, pr_mask, lam_g, side0, st);
   ++*launches;
   return cudaGetLastError();

@@ -215,7 +215,9 @@ struct mincut_graph {
   int bw_auto = -1;           // threshold chosen by timing (batch_small_n = 0), -1: not yet
   int* bw_list = nullptr;     // graph ids, most entries first
   int bw_count = 0, bw_nmax = 0, bw_mmax = 0;
-  int* bw_cursor = nullptr;
+  int* bw_cursor = nullptr;    // work queues of the block and the warp solver, then the
+                               // number of graphs the block solver left
+  int* bw_left = nullptr;      // and their ids
   int* bw_scratch = nullptr;
   long long bw_scratch_words = 0;
   int bw_slots = 0;
@@ -229,8 +231,10 @@ struct mincut_graph {
     const int* scratch = nullptr;
     const int* voff = nullptr;  // the offsets buffer in use (round solves swap it)
     unsigned pr = 0;
+    bool blocks = false;
     bool operator==(const BwKey& o) const {
-      return threshold == o.threshold && scratch == o.scratch && voff == o.voff && pr == o.pr;
+      return threshold == o.threshold && scratch == o.scratch && voff == o.voff && pr == o.pr &&
+             blocks == o.blocks;
     }
   } bw_key, bw_exec_key;
   int bw_key_runs = 0;
@@ -1013,11 +1017,31 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
   // they joined too little, they wait until the graph has halved
   const bool forests = !op.deterministic && op.seq_kernel == 0 && op.seq_passes == 0 &&
                        op.cf_visit == 0 && op.max_rounds == 0 && !op.lp_every_round;
-  int forest_below = INT_MAX;
+  int forest_below = INT_MAX, small_below = INT_MAX;
   bool lp_done = !lp_allowed;
   for (;; ++*round_io) {
     const int round = *round_io;
     if (op.max_rounds > 0 && round >= op.max_rounds) break;
+    if (forests && sizeof(WT) == 4 && g->n <= kSmMaxN && g->n < small_below) {
+      {
+        ProfScope ps(P_SMALL, g->n, g->stream);
+        CK(small_solve(g->n, g->crp(), g->ccol(), (const int*)g->cw(), g->keys[0], g->keys[1],
+                       std::min(kSmMaxM, std::max<long long>(g->Mraw, 1)), op.pr_mask & 3u, g->cur_side, g->map0,
+                       g->n0, g->side0, g->sms, g->st, g->stream, &g->launches));
+      }
+      const int rcs = sync_state(g);
+      if (rcs) return rcs;
+      if ((long long)g->hst->lambda < lambda) {
+        lambda = (long long)g->hst->lambda;
+        stl->lambda_source = g->hst->small_improved;
+      }
+      if (g->hst->small_status == 1) {
+        stl->rounds += g->hst->small_rounds;
+        stl->entries_processed += g->m_pending ? g->hst->m_rows : g->M;
+        break;
+      }
+      small_below = g->n / 2;
+    }
     if (op.cf_visit == 2) {
       if (rate[0] < 0) mode = 0;
       else if (rate[1] < 0) mode = 1;
@@ -1541,7 +1565,8 @@ int bw_prepare(mincut_graph* g, int threshold) {
   g->bw_mmax = std::max(mmax, 1);
   if (ids.empty()) return MINCUT_OK;
   if (!g->bw_list) {
-    if (!galloc(g, &g->bw_list, G) || !galloc(g, &g->bw_cursor, 1))
+    if (!galloc(g, &g->bw_list, G) || !galloc(g, &g->bw_cursor, 4) ||
+        !galloc(g, &g->bw_left, G))
       return fail(MINCUT_ERR_OOM, "batch warp list");
   }
   CK(cudaMemcpyAsync(g->bw_list, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice,
@@ -1565,11 +1590,34 @@ int bw_prepare(mincut_graph* g, int threshold) {
   return MINCUT_OK;
 }
 
-// A solve whose graphs all take the one-warp solver: state reset, then the
+// The listed small graphs: a block per graph (small.cu), then one warp for
+// each of those it left; in the deterministic mode all of them one warp each.
+cudaError_t bw_solve_list(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s,
+                          int* launches) {
+  BatchState& b = g->batch;
+  if (!blocks)
+    return batch_warp_solve(g->bw_list, g->bw_count, nullptr, g->bw_cursor, b.voff0, g->rp0,
+                            g->col0, (const int*)g->w0, g->bw_scratch, g->bw_slots, g->bw_nmax,
+                            g->bw_mmax, pr, b.lam_g, g->side0, g->st, s, launches);
+  cudaError_t e = small_batch(g->bw_list, g->bw_count, g->bw_cursor, b.voff0, g->rp0, g->col0,
+                              (const int*)g->w0, g->bw_scratch,
+                              batch_warp_slot_words(g->bw_nmax, g->bw_mmax), g->bw_slots,
+                              g->bw_nmax, g->bw_mmax, pr, b.lam_g, g->side0, g->bw_left,
+                              g->bw_cursor + 2, g->sms, s, launches);
+  if (e == cudaSuccess)
+    e = batch_warp_solve(g->bw_left, g->bw_count, g->bw_cursor + 2, g->bw_cursor + 1, b.voff0,
+                         g->rp0, g->col0, (const int*)g->w0, g->bw_scratch,
+                         std::min(g->bw_slots, g->sms), g->bw_nmax, g->bw_mmax, pr, b.lam_g,
+                         g->side0, g->st, s, launches);
+  return e;
+}
+
+// A solve whose graphs all take the small solvers: state reset, then the
 // warp solver over the whole list (no round kernels, no host decisions
 // before the completion check).  Only stream-ordered calls, so that it can
 // be captured.
-cudaError_t bw_enqueue(mincut_graph* g, uint32_t pr, cudaStream_t s, int* launches) {
+cudaError_t bw_enqueue(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s,
+                       int* launches) {
   BatchState& b = g->batch;
   const int G = b.G;
   cudaError_t e = cudaMemsetAsync(g->st, 0, sizeof(DevState), s);
@@ -1586,10 +1634,7 @@ cudaError_t bw_enqueue(mincut_graph* g, uint32_t pr, cudaStream_t s, int* launch
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(g->side0, 0, (size_t)g->n0, s);
   if (e == cudaSuccess) e = batch_warp_mark(g->bw_list, g->bw_count, b.done_g, g->st, s, launches);
-  if (e == cudaSuccess)
-    e = batch_warp_solve(g->bw_list, g->bw_count, g->bw_cursor, b.voff0, g->rp0, g->col0,
-                         (const int*)g->w0, g->bw_scratch, g->bw_slots, g->bw_nmax, g->bw_mmax,
-                         pr, b.lam_g, g->side0, g->st, s, launches);
+  if (e == cudaSuccess) e = bw_solve_list(g, pr, blocks, s, launches);
   return e;
 }
 
@@ -1626,6 +1671,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
     key.scratch = g->bw_scratch;
     key.voff = b.voff;
     key.pr = op.pr_mask & 3u;
+    key.blocks = !op.deterministic;
     g->bw_key_runs = key == g->bw_key ? g->bw_key_runs + 1 : 1;
     g->bw_key = key;
     if (g->bw_exec && !(g->bw_exec_key == key)) {
@@ -1637,7 +1683,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
       if (!g->bw_capture) CK(cudaStreamCreateWithFlags(&g->bw_capture, cudaStreamNonBlocking));
       int nl = 0;
       CK(cudaStreamBeginCapture(g->bw_capture, cudaStreamCaptureModeThreadLocal));
-      cudaError_t e = bw_enqueue(g, key.pr, g->bw_capture, &nl);
+      cudaError_t e = bw_enqueue(g, key.pr, key.blocks, g->bw_capture, &nl);
       cudaGraph_t graph = nullptr;
       const cudaError_t e2 = cudaStreamEndCapture(g->bw_capture, &graph);
       if (e == cudaSuccess) e = e2;
@@ -1654,7 +1700,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
       CK(cudaGraphLaunch(g->bw_exec, s));
       g->launches += g->bw_exec_launches;
     } else {
-      CK(bw_enqueue(g, key.pr, s, &g->launches));
+      CK(bw_enqueue(g, key.pr, key.blocks, s, &g->launches));
     }
   } else {
     CK(cudaMemsetAsync(g->st, 0, sizeof(DevState), s));
@@ -1726,9 +1772,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
       ProfScope ps(P_BATCH_WARP, g->bw_count, s);
       // PR1 / PR2 only: on one warp the PR3 / PR4 intersections cost several
       // times the rest of a graph's solve (the pass of each round marks anyway)
-      CK(batch_warp_solve(g->bw_list, g->bw_count, g->bw_cursor, b.voff0, g->rp0, g->col0,
-                          (const int*)g->w0, g->bw_scratch, g->bw_slots, g->bw_nmax, g->bw_mmax,
-                          op.pr_mask & 3u, b.lam_g, g->side0, g->st, s, &g->launches));
+      CK(bw_solve_list(g, op.pr_mask & 3u, !op.deterministic, s, &g->launches));
     }
   }
   int rc = sync_state(g);

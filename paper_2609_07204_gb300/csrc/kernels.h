@@ -70,8 +70,10 @@ cudaError_t batch_warp_mark(const int* list, int nlist, int* done_g, DevState* s
 // weights, total below 2^31) into lam_g and side0.  scratch: slots slots (a
 // multiple of batch_warp_block_warps()) of
 // batch_warp_slot_words(nmax, mmax) ints; every listed graph has at most nmax
-// vertices and mmax entries.  cursor: one int of work-queue state.
-cudaError_t batch_warp_solve(const int* list, int nlist, int* cursor, const int* voff0,
+// vertices and mmax entries.  cursor: one int of work-queue state.  nlist_dev
+// (nullable): the number of listed graphs, at most nlist, on the device.
+cudaError_t batch_warp_solve(const int* list, int nlist, const int* nlist_dev, int* cursor,
+                             const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
                              unsigned long long* lam_g, uint8_t* side0, DevState* st,
@@ -93,7 +95,7 @@ void set_last_error(const char* msg);
 enum ProfCat {
   P_DEGREE, P_LP_SWEEP, P_LP_BOUND, P_PR, P_CF_PASSES, P_CF_SEQ, P_UF, P_EMIT,
   P_SORT_HIST, P_SORT_PASS, P_BUILD, P_TILES, P_WITNESS, P_OTHER, P_ROWS, P_BATCH_WARP,
-  P_FOREST, P_NCAT
+  P_FOREST, P_SMALL, P_NCAT
 };
 const char* prof_name(int cat);
 struct Profiler;
@@ -366,6 +368,29 @@ cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, 
                          cudaStream_t s, int* launches);
 cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uint8_t* tag, int last,
                               int sms, cudaStream_t s, int* launches);
+
+// ---------------------------------------------------------------- small.cu
+// All rounds on a current graph of at most kSmMaxN vertices (32-bit weights,
+// total below 2^31) in one block, from the bound st->lambda: lowers
+// st->lambda, side0 (through map0) gets the witness when it did, and
+// st->small_status says 1 = solved, 2 = left to the other rounds (more than
+// mcap entries, or a round that joined nothing).  ed0, ed1: mcap words
+// and 2 more each; cur_side: n bytes.
+constexpr int kSmMaxN = 2048;
+constexpr long long kSmMaxM = 1ll << 17;
+cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,
+                        void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side, const int* map0, int n0,
+                        uint8_t* side0, int sms, DevState* st, cudaStream_t s, int* launches);
+
+// A batch's graphs (at most kSmMaxN vertices each), a block per graph at a
+// time from a work queue: values and sides of those solved, the others'
+// ids in left[0 .. *nleft) for batch_warp_solve.  scratch: `slots` slots of
+// slot_words >= 2 mmax + 8 words.
+cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff0,
+                        const int64_t* rp0, const int* col0, const int* w0, int* scratch,
+                        long long slot_words, int slots, int nmax, int mmax, uint32_t pr_mask,
+                        unsigned long long* lam_g, uint8_t* side0, int* left, int* nleft, int sms,
+                        cudaStream_t s, int* launches);
 
 // ------------------------------------------------------------- contract.cu
 // Row-wise contraction when most groups are single vertices: singleton rows

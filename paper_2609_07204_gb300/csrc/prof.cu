@@ -25,7 +25,7 @@ static const char* kNames[P_NCAT] = {"degree", "lp_sweep", "lp_bound", "pr_marks
                                      "capforest_passes", "capforest_seq", "union_find", "emit",
                                      "sort_hist", "sort_pass", "build_csr", "tile_rows",
                                      "witness", "other", "contract_rows", "batch_warp",
-                                     "forest"};
+                                     "forest", "small_solve"};
 
 const char* prof_name(int cat) { return (cat >= 0 && cat < P_NCAT) ? kNames[cat] : "?"; }
 
