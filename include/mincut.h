@@ -95,11 +95,11 @@ typedef struct mincut_options {
                                 start vertex with private arrays: 1 = the single pass of
                                 Algorithm 2; 0 = auto (one per SM, device memory permitting) */
     int32_t batch_small_n;   /* mincut_batch_solve: graphs of at most this many vertices (and at
-                                most 2048) are solved one per warp, each running all its rounds
-                                alone (one CAPFOREST pass per round; of pr_mask only PR1/PR2);
-                                the others share the batch's round kernels.  0 = auto (chosen
-                                by timing candidate thresholds on the first solve of the batch,
-                                then kept); < 0 = every graph in the round kernels */
+                                most 2048) are solved each on its own, a thread block per graph
+                                (deterministic = 1: a warp, one CAPFOREST pass per round; of
+                                pr_mask only PR1/PR2 either way); the others share the batch's
+                                round kernels.  0 = auto (2048); < 0 = every graph in the round
+                                kernels */
     int32_t seq_kernel;      /* kernel of the whole-graph CAPFOREST passes: 0 (default) one
                                 warp per pass, the next vertex among those of highest priority
                                 taken from the last scanned row when it holds one (else the
@@ -230,12 +230,12 @@ int mincut_batch_from_csr(int64_t num_graphs, const int64_t* vertex_offsets,
 
 /* Exact minimum cut of every graph of a batch (Algorithm 2 per graph; label
  * propagation is not used).  Graphs of at most opts->batch_small_n vertices
- * are solved one per warp in one persistent launch (a work queue, largest
- * first); the others share one set of round kernels, each graph with its own
+ * are solved one per thread block in one persistent launch (a work queue,
+ * largest first); the others share one set of round kernels, each graph with its own
  * bound, stop test and witness.  cut_values: host int64[num_graphs].  side_bitmap (nullable, host or device, ceil(n/64)
  * words): bit v = 1 iff vertex v is on the side of its graph's minimum cut
  * that does not hold the graph's first vertex.  When every graph takes the
- * one-warp solver and profiling is off, the second solve of the batch with
+ * small-graph solver and profiling is off, the second solve of the batch with
  * the same split captures that solve's launches as a CUDA graph (on a stream
  * the library creates) and later solves replay it on the batch's stream;
  * both are released by mincut_graph_destroy. */
@@ -243,8 +243,7 @@ int mincut_batch_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut
                        uint64_t* side_bitmap, mincut_stats* stats);
 
 /* How the last mincut_batch_solve split the batch: *small_n = the vertex
- * threshold of the one-warp-per-graph solver it used (the timed choice when
- * opts->batch_small_n was 0; -1 before any solve), *small_graphs = the graphs
+ * threshold of the small-graph solver it used (-1 before any solve), *small_graphs = the graphs
  * it solved that way.  MINCUT_ERR_INVALID if g is not a batch. */
 int mincut_batch_info(const mincut_graph* g, int32_t* small_n, int64_t* small_graphs);
 
@@ -316,8 +315,8 @@ int mincut_release_cached(int device);
  * admitted requests stay under hbm_cap_bytes (a request alone is always
  * admitted).  A worker that takes a request with n <= pack_max_n also takes
  * the small requests queued right behind it (up to pack_max_requests and
- * pack_max_vertices) and solves them as one packed batch; larger requests
- * are solved alone.  Values are exact, so a request's value does not depend
+ * pack_max_vertices; of at most 2,048 vertices, whatever pack_max_n says) and
+ * solves them as one packed batch; larger requests are solved alone.  Values are exact, so a request's value does not depend
  * on what it was solved with. */
 typedef struct mincut_server mincut_server;
 typedef struct mincut_server_options {

@@ -14,7 +14,6 @@
 // mix.
 #include <algorithm>
 #include <chrono>
-#include <atomic>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
@@ -27,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/mincut.h"
+#include "kernels.h"
 
 namespace {
 
@@ -68,9 +68,6 @@ struct mincut_server {
   bool stopping = false;
   std::vector<std::thread> workers;
   mincut_server_stats st{};
-  // warp-solver threshold of packed solves when solve.batch_small_n = 0: timed
-  // on the first packed solve, then reused (0: not yet, -1: none)
-  std::atomic<int> bw_small_n{0};
 };
 
 namespace {
@@ -100,8 +97,7 @@ void solve_alone(const mincut_server_options& o, cudaStream_t s, const ReqPtr& r
   mincut_graph_destroy(g);
 }
 
-void solve_packed(mincut_server* S, const mincut_server_options& o, cudaStream_t s,
-                  std::vector<ReqPtr>& reqs) {
+void solve_packed(const mincut_server_options& o, cudaStream_t s, std::vector<ReqPtr>& reqs) {
   const size_t G = reqs.size();
   std::vector<int64_t> voff(G + 1, 0);
   int64_t entries = 0;
@@ -130,15 +126,8 @@ void solve_packed(mincut_server* S, const mincut_server_options& o, cudaStream_t
   std::vector<uint64_t> bm;
   if (rc == MINCUT_OK) {
     if (o.want_bitmap) bm.assign((size_t)((voff[G] + 63) / 64), 0);
-    mincut_options so = o.solve;
-    const int tuned = S->bw_small_n.load();
-    if (so.batch_small_n == 0 && tuned != 0) so.batch_small_n = tuned;
-    rc = mincut_batch_solve(g, &so, vals.data(), o.want_bitmap ? bm.data() : nullptr, nullptr);
-    if (rc == MINCUT_OK && so.batch_small_n == 0) {
-      int32_t t = 0;
-      int64_t k = 0;
-      if (mincut_batch_info(g, &t, &k) == MINCUT_OK) S->bw_small_n.store(t > 0 ? t : -1);
-    }
+    rc = mincut_batch_solve(g, &o.solve, vals.data(), o.want_bitmap ? bm.data() : nullptr,
+                            nullptr);
     mincut_graph_destroy(g);
   }
   if (rc != MINCUT_OK) {  // isolate the failing request(s)
@@ -186,11 +175,15 @@ void worker_loop(mincut_server* S, int wid) {
       take.push_back(h);
       S->inflight_bytes += h->footprint;
       S->inflight += 1;
-      if (h->n <= o.pack_max_n && o.pack_max_requests > 1) {
+      // packed together: what a batch solves a block per graph; beyond that a
+      // request alone (0.3 ms) is faster than its share of the round kernels
+      // (10 ms and more a batch)
+      const int64_t pack_n = std::min<int64_t>(o.pack_max_n, mc::kBwMaxN);
+      if (h->n <= pack_n && o.pack_max_requests > 1) {
         int64_t verts = h->n;
         while (!S->queue.empty() && (int)take.size() < o.pack_max_requests) {
           const ReqPtr& q = S->queue.front();
-          if (q->n > o.pack_max_n || verts + q->n > o.pack_max_vertices ||
+          if (q->n > pack_n || verts + q->n > o.pack_max_vertices ||
               S->inflight_bytes + q->footprint > o.hbm_cap_bytes)
             break;
           verts += q->n;
@@ -212,7 +205,7 @@ void worker_loop(mincut_server* S, int wid) {
     const double t = now_ms();
     for (auto& r : take) r->t_start = t;
     if (take.size() == 1) solve_alone(o, s, take[0]);
-    else solve_packed(S, o, s, take);
+    else solve_packed(o, s, take);
     finish(S, take);
   }
   cudaStreamDestroy(s);
