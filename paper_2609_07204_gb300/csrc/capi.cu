@@ -53,6 +53,12 @@ int bits_for(long long x) {  // bits to hold values in [0, x)
 __global__ void iota_kernel(int* a, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = i;
 }
+// The identity map and no bound yet.
+__global__ void solve_start_kernel(int* map0, int n, DevState* st) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    map0[i] = i;
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->lambda = (unsigned long long)kInf;
+}
 __global__ void widen32_kernel(const int32_t* __restrict__ in, int64_t* __restrict__ out, long long M) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < M;
        i += (long long)gridDim.x * blockDim.x)
@@ -128,6 +134,11 @@ struct mincut_graph {
   mincut_allocator alloc{};
   bool user_alloc = false;
   std::vector<Alloc> allocs;
+  // in_slab(): sizes are summed, then buffers are cut from one allocation
+  bool counting = false;
+  size_t counted = 0;
+  unsigned char* slab = nullptr;
+  size_t slab_left = 0;
   bool wt64 = false;
   int sms = kDefaultSms;
   // canonical input
@@ -338,6 +349,16 @@ void pinned_state_put(DevState* p) {
 void* dev_alloc(mincut_graph* g, size_t bytes) {
   bytes = std::max<size_t>(bytes, 16);
   bytes = (bytes + 255) / 256 * 256;
+  if (g->counting) {
+    g->counted += bytes;
+    return g;  // (never used: the cutting pass follows)
+  }
+  if (bytes <= g->slab_left) {
+    void* cut = g->slab;
+    g->slab += bytes;
+    g->slab_left -= bytes;
+    return cut;
+  }
   void* p = nullptr;
   if (g->user_alloc) {
     p = g->alloc.alloc(bytes, (void*)g->stream, g->alloc.ctx);
@@ -372,6 +393,27 @@ template <typename T>
 bool galloc(mincut_graph* g, T** out, long long count) {
   *out = static_cast<T*>(dev_alloc(g, (size_t)std::max<long long>(count, 1) * sizeof(T)));
   return *out != nullptr;
+}
+
+// The buffers that `allocate` asks for (galloc / dev_alloc calls, the same on
+// every run) as one allocation: a stream-ordered allocation and its release
+// cost ~2 us, and a graph has some 80 buffers.  dev_free does nothing for a
+// buffer of a slab but its first, which is the slab.
+template <typename F>
+bool in_slab(mincut_graph* g, F allocate) {
+  g->counting = true;
+  g->counted = 0;
+  allocate();
+  g->counting = false;
+  const size_t total = g->counted;
+  void* p = dev_alloc(g, total);
+  if (!p) return false;
+  g->slab = static_cast<unsigned char*>(p);
+  g->slab_left = total;
+  const bool ok = allocate();
+  g->slab = nullptr;
+  g->slab_left = 0;
+  return ok;
 }
 
 void free_all(mincut_graph* g) {
@@ -423,21 +465,23 @@ int ensure_rows(mincut_graph* g) {
   const size_t wsz = g->wt64 ? 8 : 4;
   const long long n = g->n0, M = std::max<long long>(g->M0, 1);
   RowScratch& r = g->rows;
-  if (!galloc(g, &r.cnt, n + 1) || !galloc(g, &r.gen, n + 1) || !galloc(g, &r.len, n + 1) ||
-      !galloc(g, &r.kcnt, n + 1) || !galloc(g, &r.off, n + 1) ||
-      !galloc(g, &r.part, (n + 1) / 4096 + 3) ||
-      !galloc(g, &r.side_v, M) || !galloc(g, &r.vinfo, n + 1) || !galloc(g, &g->rpG, n + 1) ||
-      !galloc(g, &r.dsum, n + 1) || !galloc(g, &r.did, n + 1) ||
-      !galloc(g, &r.chunk, 4 * M / kDenseChunk + n + 64) ||
-      !galloc(g, &r.dense_group, n + 1) ||
-      !(r.acc = dev_alloc(g, (size_t)4 * M * wsz)) ||
-      !galloc(g, &g->colG, M) ||
-      !(g->wG = dev_alloc(g, (size_t)M * wsz)) || !(g->side_w = dev_alloc(g, (size_t)M * wsz)) ||
-      !galloc(g, &r.rep, n + 1) || !galloc(g, &r.fcl, n + 1) || !galloc(g, &r.kpc, n + 1) ||
-      !galloc(g, &r.side_c, M) || !(r.rec = dev_alloc(g, (size_t)(n + 1) * 16)) ||
-      !galloc(g, &r.tile_ht, M / kEntryTile + 2) || !galloc(g, &r.tile_rowG, M / kEntryTile + 2) ||
-      !galloc(g, &r.list, n + 1) || !galloc(g, &r.list_len, 2) ||
-      !galloc(g, &r.vmap, n / 32 + 2) || !galloc(g, &r.mvbits, n / 32 + 2)) {
+  const bool ok = in_slab(g, [&] {
+    return galloc(g, &r.cnt, n + 1) && galloc(g, &r.gen, n + 1) && galloc(g, &r.len, n + 1) &&
+           galloc(g, &r.kcnt, n + 1) && galloc(g, &r.off, n + 1) &&
+           galloc(g, &r.part, (n + 1) / 4096 + 3) && galloc(g, &r.side_v, M) &&
+           galloc(g, &r.vinfo, n + 1) && galloc(g, &g->rpG, n + 1) && galloc(g, &r.dsum, n + 1) &&
+           galloc(g, &r.did, n + 1) && galloc(g, &r.chunk, 4 * M / kDenseChunk + n + 64) &&
+           galloc(g, &r.dense_group, n + 1) && (r.acc = dev_alloc(g, (size_t)4 * M * wsz)) &&
+           galloc(g, &g->colG, M) && (g->wG = dev_alloc(g, (size_t)M * wsz)) &&
+           (g->side_w = dev_alloc(g, (size_t)M * wsz)) && galloc(g, &r.rep, n + 1) &&
+           galloc(g, &r.fcl, n + 1) && galloc(g, &r.kpc, n + 1) && galloc(g, &r.side_c, M) &&
+           (r.rec = dev_alloc(g, (size_t)(n + 1) * 16)) &&
+           galloc(g, &r.tile_ht, M / kEntryTile + 2) &&
+           galloc(g, &r.tile_rowG, M / kEntryTile + 2) && galloc(g, &r.list, n + 1) &&
+           galloc(g, &r.list_len, 2) && galloc(g, &r.vmap, n / 32 + 2) &&
+           galloc(g, &r.mvbits, n / 32 + 2);
+  });
+  if (!ok) {
     r.cnt = nullptr;
     return fail(MINCUT_ERR_OOM, "row-wise contraction buffers");
   }
@@ -483,10 +527,14 @@ int ensure_seq_multi(mincut_graph* g, int want) {
 
 int ensure_forest(mincut_graph* g) {
   if (g->fo_ctl) return MINCUT_OK;
-  if (!galloc(g, &g->fo_tag, g->n0) || !galloc(g, &g->fo_r, g->n0) ||
-      !galloc(g, &g->fo_items, forest_item_cap(g->n0, g->M0)) ||
-      !galloc(g, &g->fo_ctl, (long long)forest_ctl_bytes()))
+  if (!in_slab(g, [&] {
+        return galloc(g, &g->fo_tag, g->n0) && galloc(g, &g->fo_r, g->n0) &&
+               galloc(g, &g->fo_items, forest_item_cap(g->n0, g->M0)) &&
+               galloc(g, &g->fo_ctl, (long long)forest_ctl_bytes());
+      })) {
+    g->fo_ctl = nullptr;
     return fail(MINCUT_ERR_OOM, "forest buffers");
+  }
   return MINCUT_OK;
 }
 
@@ -1175,9 +1223,9 @@ int solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_value,
   g->m_pending = false;
   if (op.spin_limit > 0) g->spin_limit = op.spin_limit;
   CK(cudaMemsetAsync(g->st, 0, sizeof(DevState), s));
-  int rc = set_lambda(g, kInf);
-  if (rc) return rc;
-  iota_kernel<<<std::min((g->n0 + 255) / 256, g->sms * 8), 256, 0, s>>>(g->map0, g->n0);
+  int rc = MINCUT_OK;
+  solve_start_kernel<<<std::min((g->n0 + 255) / 256, g->sms * 8), 256, 0, s>>>(g->map0, g->n0,
+                                                                                g->st);
   ++g->launches;
   long long lambda = kInf;
   mincut_stats stl{};
@@ -1400,32 +1448,31 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
     return rc;
   };
   if (!(g->hst = pinned_state_get())) return bail(fail(MINCUT_ERR_OOM, "pinned state"));
-  if (!galloc(g, &g->st, 1) || !galloc(g, &g->m2_dev, 1)) return bail(fail(MINCUT_ERR_OOM, "state"));
+  // row_ptr first, checked on the device before any entry is read through it
+  // (a bad one leaves the input pass without work), then one pass over the
+  // entries: copy, weight statistics, canonical test and symmetry fingerprint
+  // together; both checks come back with one synchronisation
+  const long long ntiles = (std::max<long long>(Mraw, 1) + kEntryTile - 1) / kEntryTile + 2;
+  unsigned long long* wst = nullptr;
+  if (!in_slab(g, [&] {
+        return galloc(g, &g->st, 1) && galloc(g, &g->m2_dev, 1) && galloc(g, &wst, 10) &&
+               galloc(g, &g->tile_row, ntiles);
+      }))
+    return bail(fail(MINCUT_ERR_OOM, "state"));
   if (cudaMemsetAsync(g->st, 0, sizeof(DevState), s) != cudaSuccess)
     return bail(fail(MINCUT_ERR_CUDA, "memset state"));
-  // row_ptr first (checked before any entry is read through it), then one
-  // ingestion pass over the entries: copy, weight statistics, canonical
-  // test and symmetry fingerprint together
   int64_t* rp_raw = nullptr;
   int32_t* w_raw = nullptr;
   int* col_raw = nullptr;
-  if (!galloc(g, &rp_raw, n + 1) || !galloc(g, &w_raw, Mraw) || !galloc(g, &col_raw, Mraw))
+  if (!in_slab(g, [&] { return galloc(g, &rp_raw, n + 1) && galloc(g, &col_raw, Mraw); }) ||
+      !galloc(g, &w_raw, Mraw))
     return bail(fail(MINCUT_ERR_OOM, "raw input"));
   const cudaMemcpyKind kind = dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (cudaMemcpyAsync(rp_raw, row_ptr, (size_t)(n + 1) * sizeof(int64_t), kind, s) != cudaSuccess)
     return bail(fail(MINCUT_ERR_CUDA, "copy row_ptr: %s", cudaGetErrorString(cudaGetLastError())));
-  unsigned long long* wst = nullptr;
-  if (!galloc(g, &wst, 10)) return bail(fail(MINCUT_ERR_OOM, "stats"));
   cudaMemsetAsync(wst, 0, 10 * sizeof(unsigned long long), s);
   input_stats_kernel<<<std::max(1, std::min(g->sms * 8, (n + 255) / 256)), 256, 0, s>>>(
       rp_raw, n, w_raw, 0, wst);
-  unsigned long long hws[6] = {0, 0, 0, 0, 0, 0};
-  cudaMemcpyAsync(hws, wst, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess)
-    return bail(fail(MINCUT_ERR_CUDA, "row_ptr check: %s", cudaGetErrorString(cudaGetLastError())));
-  if (hws[2]) return bail(fail(MINCUT_ERR_INVALID, "row_ptr is not non-decreasing"));
-  const long long ntiles = (std::max<long long>(Mraw, 1) + kEntryTile - 1) / kEntryTile + 2;
-  if (!galloc(g, &g->tile_row, ntiles)) return bail(fail(MINCUT_ERR_OOM, "tile rows"));
   unsigned long long* ist = wst + 4;
   if (Mraw > 0) {
     // entries the device can address are read in place (device input, or
@@ -1440,14 +1487,19 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
       col_src = col_raw;
       w_src = w_raw;
     }
-    if (tile_rows(rp_raw, n, Mraw, g->tile_row, s, &g->launches) != cudaSuccess ||
-        ingest_csr(n, Mraw, rp_raw, col_src, w_src, col_raw, w_raw, g->tile_row, ist, s,
-                   &g->launches) != cudaSuccess ||
-        cudaMemcpyAsync(hws, ist, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
+    if (ingest_csr(n, Mraw, rp_raw, col_src, w_src, col_raw, w_raw, g->tile_row, wst + 2, ist, s,
+                   &g->launches) != cudaSuccess)
       return bail(fail(MINCUT_ERR_CUDA, "input pass: %s", cudaGetErrorString(cudaGetLastError())));
   }
+  // (the pinned mirror of the state serves as the landing place)
+  static_assert(sizeof(DevState) >= 10 * sizeof(unsigned long long), "landing place");
+  if (cudaMemcpyAsync(g->hst, wst, 10 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return bail(fail(MINCUT_ERR_CUDA, "input pass: %s", cudaGetErrorString(cudaGetLastError())));
+  unsigned long long hall[10], *hws = hall + 4;
+  memcpy(hall, g->hst, sizeof(hall));
+  if (hall[2]) return bail(fail(MINCUT_ERR_INVALID, "row_ptr is not non-decreasing"));
   if (hws[1]) return bail(fail(MINCUT_ERR_INVALID, "negative weight"));
   g->wt64 = hws[0] > 0x7fffffffull;
   // An input already in canonical form (the form every contraction writes)
@@ -1462,29 +1514,32 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
     g->fo_qsoft = std::max<long long>(1, (long long)((hws[0] / (unsigned long long)Mraw + 1) / 2));
   const long long Mb = std::max<long long>(Mraw, 1);
   // buffers
-  bool ok = true;
-  for (int i = 0; i < 2; ++i) {
-    ok = ok && galloc(g, &g->rp[i], n + 1) && galloc(g, &g->col[i], Mb) &&
-         (g->w[i] = dev_alloc(g, (size_t)Mb * wsz)) && galloc(g, &g->keys[i], Mb) &&
-         (g->vals[i] = dev_alloc(g, (size_t)Mb * wsz));
-  }
   const long long scan_parts = (std::max<long long>(Mb, n) + 4095) / 4096 + 2;
   g->max_table = 1024;
   g->max_passes = graph_max_passes(n, g->sms);
-  ok = ok && (g->deg0 = dev_alloc(g, (size_t)n * wsz)) &&
-       (g->degb[0] = dev_alloc(g, (size_t)n * wsz)) && (g->degb[1] = dev_alloc(g, (size_t)n * wsz)) &&
-       galloc(g, &g->blk, 2 * 1024) && galloc(g, &g->parent, n) && galloc(g, &g->L, n) &&
-       galloc(g, &g->flags, n) && galloc(g, &g->rank, n) && galloc(g, &g->part, scan_parts) &&
-       galloc(g, &g->uid, Mb) && galloc(g, &g->owner, n) && galloc(g, &g->gmin, n) &&
-       galloc(g, &g->map0, n) && galloc(g, &g->side0, n) && galloc(g, &g->cur_side, n) &&
-       galloc(g, &g->bitmap_dev, (n + 63) / 64) && galloc(g, &g->short_bits, n / 32 + 2) &&
-       galloc(g, &g->visit_log, (long long)g->max_passes * g->max_table) &&
-       galloc(g, &g->pass_best, g->max_passes) && galloc(g, &g->pass_len, g->max_passes) &&
-       galloc(g, &g->pass_counter, 1) && (g->seq_r = dev_alloc(g, (size_t)n * wsz)) &&
-       galloc(g, &g->seq_mark, n) && galloc(g, &g->seq_tree, seq_tree_words(n)) &&
-       galloc(g, &g->seq_order, n) && galloc(g, &g->sort.hist, 8 * 256) &&
-       galloc(g, &g->sort.goff, 8 * 256) &&
-       galloc(g, &g->sort.lookback, sort_lookback_words(Mb));
+  const bool ok = in_slab(g, [&] {
+    bool a = true;
+    for (int i = 0; i < 2; ++i) {
+      a = a && galloc(g, &g->rp[i], n + 1) && galloc(g, &g->col[i], Mb) &&
+          (g->w[i] = dev_alloc(g, (size_t)Mb * wsz)) && galloc(g, &g->keys[i], Mb) &&
+          (g->vals[i] = dev_alloc(g, (size_t)Mb * wsz));
+    }
+    return a && (g->deg0 = dev_alloc(g, (size_t)n * wsz)) &&
+           (g->degb[0] = dev_alloc(g, (size_t)n * wsz)) &&
+           (g->degb[1] = dev_alloc(g, (size_t)n * wsz)) && galloc(g, &g->blk, 2 * 1024) &&
+           galloc(g, &g->parent, n) && galloc(g, &g->L, n) && galloc(g, &g->flags, n) &&
+           galloc(g, &g->rank, n) && galloc(g, &g->part, scan_parts) && galloc(g, &g->uid, Mb) &&
+           galloc(g, &g->owner, n) && galloc(g, &g->gmin, n) && galloc(g, &g->map0, n) &&
+           galloc(g, &g->side0, n) && galloc(g, &g->cur_side, n) &&
+           galloc(g, &g->bitmap_dev, (n + 63) / 64) && galloc(g, &g->short_bits, n / 32 + 2) &&
+           galloc(g, &g->visit_log, (long long)g->max_passes * g->max_table) &&
+           galloc(g, &g->pass_best, g->max_passes) && galloc(g, &g->pass_len, g->max_passes) &&
+           galloc(g, &g->pass_counter, 1) && (g->seq_r = dev_alloc(g, (size_t)n * wsz)) &&
+           galloc(g, &g->seq_mark, n) && galloc(g, &g->seq_tree, seq_tree_words(n)) &&
+           galloc(g, &g->seq_order, n) && galloc(g, &g->sort.hist, 8 * 256) &&
+           galloc(g, &g->sort.goff, 8 * 256) &&
+           galloc(g, &g->sort.lookback, sort_lookback_words(Mb));
+  });
   if (!ok) return bail(fail(MINCUT_ERR_OOM, "device buffers for n=%d M=%lld", n, Mraw));
   g->sort.lookback_words = sort_lookback_words(Mb);
   const bool validate = (flags & MINCUT_SKIP_VALIDATE) == 0;
@@ -1499,7 +1554,6 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
     } else {
       g->w0 = w_raw;
     }
-    dev_free(g, wst);
     g->M0 = Mraw;
     if (validate && !sym_fingerprint_ok)
       return bail(fail(MINCUT_ERR_INVALID, "input CSR is not symmetric"));
@@ -1525,10 +1579,8 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
     }
   }
   cudaStreamSynchronize(s);
-  dev_free(g, rp_raw);
+  dev_free(g, rp_raw);  // (and col_raw with it)
   dev_free(g, w_raw);
-  dev_free(g, col_raw);
-  dev_free(g, wst);
   int rc = g->wt64 ? canonicalize_input<int64_t>(g, n, Mraw, validate)
                    : canonicalize_input<int32_t>(g, n, Mraw, validate);
   if (rc) return bail(rc);
@@ -1987,12 +2039,15 @@ int mincut_batch_from_csr(int64_t num_graphs, const int64_t* vertex_offsets,
     words += seq_tree_words((int)(vertex_offsets[i + 1] - vertex_offsets[i]));
   }
   v32[G] = (int)n;
-  if (!galloc(g, &b.voff0, G + 1) || !galloc(g, &b.gid0, n) || !galloc(g, &b.voff, G + 1) ||
-      !galloc(g, &b.voff_next, G + 1) || !galloc(g, &b.gid, n) || !galloc(g, &b.lam_g, G) ||
-      !galloc(g, &b.lam_before, G) || !galloc(g, &b.deg_best, G) || !galloc(g, &b.cf_best, G) ||
-      !galloc(g, &b.cf_len, G) || !galloc(g, &b.marks_g, G) || !galloc(g, &b.done_g, G) ||
-      !galloc(g, &b.wit_kind, G) || !galloc(g, &b.wit_x, G) || !galloc(g, &b.level_off, G) ||
-      !galloc(g, &g->batch_levels, words) || !galloc(g, &g->batch_vals, G))
+  if (!in_slab(g, [&] {
+        return galloc(g, &b.voff0, G + 1) && galloc(g, &b.gid0, n) && galloc(g, &b.voff, G + 1) &&
+               galloc(g, &b.voff_next, G + 1) && galloc(g, &b.gid, n) && galloc(g, &b.lam_g, G) &&
+               galloc(g, &b.lam_before, G) && galloc(g, &b.deg_best, G) &&
+               galloc(g, &b.cf_best, G) && galloc(g, &b.cf_len, G) && galloc(g, &b.marks_g, G) &&
+               galloc(g, &b.done_g, G) && galloc(g, &b.wit_kind, G) && galloc(g, &b.wit_x, G) &&
+               galloc(g, &b.level_off, G) && galloc(g, &g->batch_levels, words) &&
+               galloc(g, &g->batch_vals, G);
+      }))
     return bail(fail(MINCUT_ERR_OOM, "batch arrays"));
   if (cudaMemcpyAsync(b.voff0, v32.data(), (size_t)(G + 1) * sizeof(int), cudaMemcpyHostToDevice, s) ||
       cudaMemcpyAsync(b.level_off, loff.data(), (size_t)G * sizeof(long long), cudaMemcpyHostToDevice, s))
@@ -2047,7 +2102,7 @@ int mincut_batch_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut
   int rc;
   {
     ProfGuard pg(g, op.profile != 0);
-    rc = batch_solve_impl<int32_t>(g, op, cut_values, side_bitmap, stats, small_n, true);
+    rc = batch_solve_impl<int32_t>(g, op, cut_values, side_bitmap, stats, small_n);
   }
   g->cur = -1;
   g->n = g->n0;

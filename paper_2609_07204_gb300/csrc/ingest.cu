@@ -54,7 +54,9 @@ __global__ void __launch_bounds__(kETThreads)
                   const int* __restrict__ col_src, const int* __restrict__ w_src,
                   int* __restrict__ col_dst, int* __restrict__ w_dst,
                   const int* __restrict__ tile_row, int ntiles,
+                  const unsigned long long* __restrict__ bad_rp,
                   unsigned long long* __restrict__ stats) {
+  if (*bad_rp) return;  // row_ptr is not to be read through
   __shared__ TileRowsSmem tr;
   __shared__ int s_col[kETThreads];
   __shared__ unsigned long long s_red[4][kETThreads / 32];
@@ -129,19 +131,36 @@ __global__ void __launch_bounds__(kETThreads)
   }
 }
 
+// The row of each entry tile's first entry (tile_rows_kernel), unless row_ptr
+// is not to be trusted.
+__global__ void input_tiles_kernel(const int64_t* __restrict__ rp, int n,
+                                   int* __restrict__ tile_row,
+                                   const unsigned long long* __restrict__ bad_rp) {
+  if (*bad_rp) return;
+  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+    const long long b = rp[u], e = rp[u + 1];
+    if (e <= b) continue;
+    const long long t1 = (e + kET - 1) / kET;
+    for (long long t = (b + kET - 1) / kET; t < t1; ++t) tile_row[t] = u;
+  }
+}
+
 }  // namespace
 
 cudaError_t ingest_csr(int n, long long M, const int64_t* rp, const int* col_src,
-                       const int* w_src, int* col_dst, int* w_dst, const int* tile_row,
-                       unsigned long long* stats, cudaStream_t s, int* launches) {
+                       const int* w_src, int* col_dst, int* w_dst, int* tile_row,
+                       const unsigned long long* bad_rp, unsigned long long* stats, cudaStream_t s, int* launches) {
   if (M <= 0) return cudaGetLastError();
   const int ntiles = (int)((M + kET - 1) / kET);
+  input_tiles_kernel<<<grid_blocks(n, 256, 8), 256, 0, s>>>(
+      rp, n, tile_row, bad_rp);
+  ++*launches;
   if (col_dst != col_src)
     ingest_kernel<true><<<ntiles, kETThreads, 0, s>>>(n, M, rp, col_src, w_src, col_dst, w_dst,
-                                                      tile_row, ntiles, stats);
+                                                      tile_row, ntiles, bad_rp, stats);
   else
     ingest_kernel<false><<<ntiles, kETThreads, 0, s>>>(n, M, rp, col_src, w_src, col_dst,
-                                                       w_dst, tile_row, ntiles, stats);
+                                                       w_dst, tile_row, ntiles, bad_rp, stats);
   ++*launches;
   return cudaGetLastError();
 }

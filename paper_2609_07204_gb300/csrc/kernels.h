@@ -167,10 +167,12 @@ cudaError_t build_csr(const u64* keys, const WT* vals, int N, int vbits, int n2,
 // zeroed by the caller): [0] sum of the non-negative weights, [1] any
 // negative weight, [2] any entry outside the canonical form, [3], [4] the
 // signed symmetry fingerprints and [5] the (u < v) - (u > v) balance, all
-// zero for a symmetric canonical graph.  tile_row: tile_rows() of rp.
+// zero for a symmetric canonical graph.  tile_row is set to tile_rows() of
+// rp.  Nothing is read through rp when *bad_rp (on the device) is not 0.
 cudaError_t ingest_csr(int n, long long M, const int64_t* rp, const int* col_src,
-                       const int* w_src, int* col_dst, int* w_dst, const int* tile_row,
-                       unsigned long long* stats, cudaStream_t s, int* launches);
+                       const int* w_src, int* col_dst, int* w_dst, int* tile_row,
+                       const unsigned long long* bad_rp, unsigned long long* stats,
+                       cudaStream_t s, int* launches);
 
 template <typename WT>
 cudaError_t check_symmetric(int n, long long M, const int64_t* rp, const int* col, const WT* w,
