@@ -26,7 +26,10 @@
 //
 // The prefix cuts of the batches (alpha, as in a CAPFOREST pass) are cuts of
 // the graph: the smallest lowers the bound, the scanned batches up to it its
-// witness.
+// witness, and the marks are taken from the level that the lowered bound asks
+// for.  A batch does not reach below half the highest r, so one ends where a
+// region ends (planted cut 2 x 2^19: the cut of 25 is found in the first round,
+// which joins 0.43 n instead of 0.22 n; 16.0 -> 9.1 ms, 2 x 2^15 6.3 -> 3.9).
 //
 // Cost.  An entry is read once, with its vertex: a stream read of (col, w) and
 // the far end's tag byte (scanned before: done).  The rest queue per warp, so
@@ -43,10 +46,10 @@
 //
 // Measured against the whole-graph CAPFOREST passes that such rounds needed
 // before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
-// 1,310 ms -> 16.3 ms, 2 x 2^15 81 -> 6.3 ms; against PR tests, label
-// propagation and concurrent passes: R-MAT scale 20 10-core 3.65 -> 1.73 ms,
+// 1,310 ms -> 9.1 ms, 2 x 2^15 81 -> 3.9 ms; against PR tests, label
+// propagation and concurrent passes: R-MAT scale 20 10-core 3.65 -> 1.5 ms,
 // scale 16 1.15 -> 0.66 ms, random weighted n = 150,001 (with its creation)
-// 2.63 -> 1.07 ms.
+// 2.63 -> 1.0 ms.
 #include <algorithm>
 #include <climits>
 
@@ -355,8 +358,14 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
         left = warp_sum(left);
         if (lane == 0) {
           const int need = max(left / kFoFrac, max(n / kFoTail, 32));
-          int t = k, acc = s_all[k];
-          while (t > 1 && acc < need) acc += s_all[--t];
+          // (not below half the highest r: a batch that ends where a
+          // region ends has that region's cut as its alpha)
+          int t = k, acc = s_all[k], low = max(1, k / 2);
+          while (t > 1 && acc < need && (acc == 0 || t > low)) {
+            const int c = s_all[--t];
+            if (acc == 0 && c > 0) low = max(1, t / 2);
+            acc += c;
+          }
           if (acc == 0 || b >= kFoBatches) t = 0;
           s_t = t;
           s_left = left;
@@ -547,21 +556,24 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     start = end;
     if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
   }
-  // ---- the round's marks: the components of the last level, each under its
+  // ---- the round's marks: the components of the last level (the last that
+  // the bound still asks for: a prefix cut may have lowered it), each under its
   // smallest member (r, done with, holds it per root; a warp's vertices of one
   // root send one atomic)
+  const long long lam_end = min(lam, best);
+  int* Fe = F + (lam_end > 0 ? (int)((lam_end + q - 1) / q) - 1 : 0);
   for (int v = gtid; v < n; v += gsize) ru[v] = INT_MAX;
   if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
   unsigned joined = 0;
   for (int v0 = gtid - lane; v0 < n; v0 += gsize) {
     const int v = v0 + lane;
-    const int r = v < n ? fo_root(F + (k - 1), k, v) : -1;
+    const int r = v < n ? fo_root(Fe, k, v) : -1;
     const unsigned same = __match_any_sync(FULL, r);
     if (r >= 0 && (same & lanemask_lt()) == 0) atomicMin(&ru[r], v);
     joined += r >= 0 && r != v;
   }
   if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
-  for (int v = gtid; v < n; v += gsize) a.parent[v] = ru[fo_root(F + (k - 1), k, v)];
+  for (int v = gtid; v < n; v += gsize) a.parent[v] = ru[fo_root(Fe, k, v)];
   joined = warp_sum(joined);
   if (lane == 0 && joined) atomicAdd(&a.st->marks_cf, (unsigned long long)joined);
   if (blockIdx.x == 0 && tid == 0) {

@@ -505,8 +505,10 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
         break;
       }
     }
-    // ---- PR1 / PR2 (Sec. 2.1) join in the last level too: of parallel edges
-    // each alone, which is a weaker test of the same edge
+    // the last level that the bound still asks for
+    int* top = sm.F + (int)((lam + q - 1) / q) - 1;
+    // ---- PR1 / PR2 (Sec. 2.1) join in it too: of parallel edges each alone,
+    // which is a weaker test of the same edge
     if (pr_mask) {
       for (int e = tid; e < m; e += T) {
         const unsigned d = ed.ends[e];
@@ -514,12 +516,11 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
         const int u = d & 0xffff, v = d >> 16;
         if (((pr_mask & 1u) && c >= lam) ||
             ((pr_mask & 2u) && (sm.deg[u] < 2 * c || sm.deg[v] < 2 * c)))
-          sm_join(sm.F + (k - 1), k, u, v);
+          sm_join(top, k, u, v);
       }
       __syncthreads();
     }
     // ---- labels: the rank of the root
-    const int* top = sm.F + (k - 1);
     int n2 = 0;
     for (int v0 = 0; v0 < n; v0 += T) {
       const int v = v0 + tid;
