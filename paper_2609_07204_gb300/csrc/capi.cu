@@ -614,12 +614,14 @@ int contract_rows(mincut_graph* g, int n2, int nxt, long long* m2_out, bool defe
 // the caller's next synchronisation (g->m_pending) instead of waiting here.
 template <typename WT>
 int contract_current(mincut_graph* g, int* n2_out, long long* m2_out, bool compose,
-                     bool defer_m = false) {
+                     bool defer_m = false, bool labelled = false) {
   cudaStream_t s = g->stream;
   const int n = g->n;
   const long long M = g->M;
-  { ProfScope ps(P_UF, n, s);
-    CK(uf_relabel(g->parent, g->L, g->flags, g->rank, g->part, n, g->st, s, &g->launches)); }
+  if (!labelled) {
+    ProfScope ps(P_UF, n, s);
+    CK(uf_relabel(g->parent, g->L, g->flags, g->rank, g->part, n, g->st, s, &g->launches));
+  }
   // the row classification runs before the vertex count n2 is known on the
   // host (n bounds it): one synchronisation serves both
   const bool try_rows = g->rowwise && M > 0 && n > 2;
@@ -716,6 +718,7 @@ struct RoundCfg {
   int seq_passes = 1;  // sequential passes when the concurrent ones mark nothing (0: auto)
   int seq_kernel = 0;  // 0: warp-driven passes; 1: block passes (smaller-id ties)
   bool forest = false;  // certificate forests first; the other marks only if they join little
+  bool small_rest = false;  // then the one-block solver, if they leave few vertices
   bool coarsen = false;  // heuristic round: also join every label-propagation cluster
   bool skip_concurrent = false;  // capforest 1: go straight to the whole-graph passes
   // capforest 1, >= 0: the concurrent passes stand down (decided on the
@@ -740,6 +743,9 @@ struct RoundOut {
   long long lambda = kInf;
   long long marks_pr = 0, marks_cf = 0;
   long long marks_cc = 0;  // of marks_cf, those of the concurrent passes
+  bool labelled = false;   // L, flags, rank and st->n_next are those of the marks
+  bool solved = false;     // the rest of the solve ran behind the round's forests
+  int rest_rounds = 0;     // and its rounds
   bool forest_weak = false;  // the forests joined too little: the other marks ran too
   bool cc_ran = false;     // the concurrent passes ran (were not skipped)
   long long cf_nscanned = 0, cf_nmarks = 0;
@@ -757,6 +763,7 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   const int* col = g->ccol();
   const WT* w = (const WT*)g->cw();
   const WT* deg = (const WT*)g->cdeg();
+  const void* cw32 = g->cw();  // (the 32-bit weights where WT is int32_t)
   reset_round_kernel<<<1, 1, 0, s>>>(g->st);
   ++g->launches;
   if (n >= 2) {
@@ -769,11 +776,23 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     // the sort keys are free during the marking: they hold the union-finds
     rc = ensure_forest(g);
     if (rc) return rc;
-    ProfScope ps(P_FOREST, g->m_pending ? 0 : g->M, s);
-    CK(forest_marks<WT>(n, g->m_pending ? g->m_bound : g->M, rp, col, w, deg,
-                        reinterpret_cast<int*>(g->keys[0]), 2 * std::max<long long>(g->Mraw, 1),
-                        g->fo_tag, g->fo_r, g->fo_items, g->fo_ctl, g->parent, g->fo_qsoft, g->sms,
-                        g->spin_limit, g->st, s, &g->launches));
+    { ProfScope ps(P_FOREST, g->m_pending ? 0 : g->M, s);
+      CK(forest_marks<WT>(n, g->m_pending ? g->m_bound : g->M, rp, col, w, deg,
+                          reinterpret_cast<int*>(g->keys[0]), 2 * std::max<long long>(g->Mraw, 1),
+                          g->fo_tag, g->fo_r, g->fo_items, g->fo_ctl, g->parent, g->fo_qsoft,
+                          g->sms, g->spin_limit, g->st, s, &g->launches)); }
+    if (sizeof(WT) == 4 && c.small_rest) {
+      // the labels, and when few are left the rest of the solve, before the
+      // host has seen anything of the round
+      { ProfScope ps(P_UF, n, s);
+        CK(uf_relabel(g->parent, g->L, g->flags, g->rank, g->part, n, g->st, s, &g->launches)); }
+      ProfScope ps(P_SMALL, n, s);
+      CK(small_rest<int32_t>(n, rp, col, (const int32_t*)cw32, g->L, g->keys[0], g->keys[1],
+                             std::min(kSmMaxM, std::max<long long>(g->Mraw, 1)), c.pr_mask & 3u,
+                             g->cur_side, (int*)g->fo_ctl, (int*)g->vals[0],
+                             std::max<long long>(g->Mraw, 1), g->fo_items, g->sms, g->st, s,
+                             &g->launches));
+    }
   }
   rc = sync_state(g);
   if (rc) return rc;
@@ -783,23 +802,37 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   }
   const long long M = g->M;
   // the degree bound, then what the forests' prefix cuts add to it
-  const bool cf_first = forest && g->hst->cf_val == g->hst->lambda &&
-                        g->hst->cf_pass == kForestPass;
-  long long lam = cf_first ? std::min(lambda_before, (long long)g->hst->deg_val)
-                           : (long long)g->hst->lambda;
+  // (and what the one-block solve of the rest lowered it to)
+  const bool rest = forest && sizeof(WT) == 4 && c.small_rest;
+  const bool cf_first = forest && g->hst->cf_pass == kForestPass;
+  const bool rest_first = rest && g->hst->small_improved != 0;
+  long long lam = cf_first || rest_first ? std::min(lambda_before, (long long)g->hst->deg_val)
+                                         : (long long)g->hst->lambda;
   if (lam < lambda_before) {
     ProfScope ps(P_WITNESS, g->n0, s);
     CK(side_from_vertex(g->side0, g->map0, g->n0, g->hst->deg_arg, s, &g->launches));
     o->src = 1;
     lambda_before = lam;
   }
-  if (cf_first) {
-    lam = (long long)g->hst->lambda;
+  if (cf_first && (long long)g->hst->cf_val < lam) {
+    lam = (long long)g->hst->cf_val;
     ProfScope ps(P_WITNESS, g->n0, s);
     CK(side_from_batches(g->side0, g->map0, g->n0, g->fo_tag, g->hst->cf_len, g->sms, s,
                          &g->launches));
     o->src = 3;
     lambda_before = lam;
+  }
+  if (rest_first) {
+    lam = (long long)g->hst->lambda;
+    ProfScope ps(P_WITNESS, g->n0, s);
+    CK(small_side(g->cur_side, g->map0, g->L, g->n0, g->side0, g->sms, g->st, s, &g->launches));
+    o->src = g->hst->small_improved;
+    lambda_before = lam;
+  }
+  if (rest) o->labelled = true;
+  if (rest && g->hst->small_status == 1) {
+    o->solved = true;
+    o->rest_rounds = g->hst->small_rounds;
   }
   o->lambda = lam;
   if (n <= 2 || lam == 0) {
@@ -810,11 +843,10 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     CK(tile_rows(rp, n, M, g->tile_row, s, &g->launches)); }
   if (forest) {
     o->marks_cf = (long long)g->hst->marks_cf;
-    if (o->marks_cf * kForestWeakDiv >= n) {  // enough: the forests are the round's marks
-      o->lambda = lam;
-      return MINCUT_OK;
-    }
+    // solved to the end, or enough: the forests are the round's marks
+    if (o->solved || o->marks_cf * kForestWeakDiv >= n) return MINCUT_OK;
     o->forest_weak = true;
+    o->labelled = false;  // (more marks to come)
   }
   const int* lab_final = nullptr;
   if (c.lp_now && c.lp_iters > 0 && n >= c.lp_min_n) {
@@ -1099,6 +1131,7 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     c.eager_seq = c.skip_concurrent && barely;
     c.cc_skip_pr = cc_low && c.capforest == 1 && op.cf_visit != 2 ? (g->n + 63) / 64 : -1;
     c.forest = forests && g->n < forest_below;
+    c.small_rest = c.forest && small_below == INT_MAX;
     c.lp_now = lp_allowed && (op.lp_every_round || !lp_done);
     c.passes = op.passes > 0 ? op.passes : std::max(32, std::min(g->max_passes, g->n / 4));
     c.seed = op.seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(round + 1);
@@ -1127,7 +1160,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     stl->marks_pr += o.marks_pr;
     stl->marks_cf += o.marks_cf;
     if (o.seq_pass) stl->seq_passes++;
-    if (lambda == 0) break;
+    stl->rounds += o.rest_rounds;
+    if (lambda == 0 || o.solved) break;
     if (o.marks_pr + o.marks_cf == 0) {
       if (!improved) return fail(MINCUT_ERR_INTERNAL, "round made no progress");
       continue;
@@ -1135,7 +1169,7 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     int n2 = 0;
     long long m2 = 0;
     // (the visit-mode choice times each round to its end: no deferral then)
-    rc = contract_current<WT>(g, &n2, &m2, true, op.cf_visit != 2);
+    rc = contract_current<WT>(g, &n2, &m2, true, op.cf_visit != 2, o.labelled);
     if (rc) return rc;
     barely = 2 * (long long)n2 >= (long long)n_before;
     if (op.cf_visit == 2 && rate[mode] < 0) {

@@ -46,10 +46,10 @@
 //
 // Measured against the whole-graph CAPFOREST passes that such rounds needed
 // before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
-// 1,310 ms -> 9.1 ms, 2 x 2^15 81 -> 3.9 ms; against PR tests, label
-// propagation and concurrent passes: R-MAT scale 20 10-core 3.65 -> 1.5 ms,
-// scale 16 1.15 -> 0.66 ms, random weighted n = 150,001 (with its creation)
-// 2.63 -> 1.0 ms.
+// 1,340 ms -> 8.7 ms, 2 x 2^15 83 -> 4.0 ms; against PR tests, label
+// propagation and concurrent passes: R-MAT scale 20 10-core 3.69 -> 0.93 ms
+// (0.75 ms of it here), scale 16 1.15 -> 0.47 ms, random weighted n = 150,001
+// (with its creation) 2.51 -> 0.74 ms.
 #include <algorithm>
 #include <climits>
 
@@ -216,6 +216,11 @@ __device__ __forceinline__ bool fo_join(int* F, int k, int x, int y) {
   return fo_link(F, k, x, vx, y, vy);
 }
 
+// Pieces of a row of `len` entries (at least one: it carries the degree).
+__device__ __forceinline__ int fo_pieces(long long len) {
+  return max(1, (int)((len + kFoChunk - 1) / kFoChunk));
+}
+
 // A vertex about to be scanned takes rank 1 where it is still alone.  Of an
 // edge's two trees the scanned end's has a top of rank 1 and more then, and an
 // unscanned vertex alone is the lesser: it goes under the scanned end's parent
@@ -304,6 +309,8 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int n = a.n;
   const long long lam = (long long)*(volatile unsigned long long*)&a.st->lambda;
+  const int gtid = blockIdx.x * kFoThreads + tid, gsize = gridDim.x * kFoThreads;
+  for (int v = gtid; v < n; v += gsize) a.parent[v] = v;  // nothing joined, however this ends
   if (n <= 2 || lam <= 0 || lam >= kInf) return;  // (the round stops or has no bound)
   const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
   if (kcap < 1) return;
@@ -315,7 +322,6 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   uint8_t* tag = a.tag;
   int* ru = a.r;
   FoCtl* ctl = a.ctl;
-  const int gtid = blockIdx.x * kFoThreads + tid, gsize = gridDim.x * kFoThreads;
   // ---- every vertex a root at every level, nothing scanned; the first batch
   // is vertex 0
   {
@@ -331,8 +337,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     }
     for (int i = tid; i < 256; i += kFoThreads) s_hist[i] = 0;
     if (blockIdx.x == 0) {
-      const long long len = a.rp[1] - a.rp[0];
-      const int chunks = max(1, (int)((len + kFoChunk - 1) / kFoChunk));
+      const int chunks = fo_pieces(a.rp[1] - a.rp[0]);
       for (int c = tid; c < chunks; c += kFoThreads) __stcg(&a.items[c], make_int2(0, c));
       if (tid == 0) {
         atomicExch(&ctl->items, (unsigned)chunks);
@@ -343,6 +348,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   unsigned gen = 0;
   if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
   unsigned start = 0;
+  int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root
   long long best = kInf;
   int best_batch = 0;
   for (int b = 1;; ++b) {
@@ -373,6 +379,8 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
       __syncthreads();
       const int left = s_left, t = s_t;
+      rep = (int)*(volatile unsigned*)&ctl->main - 1;
+      main_root = rep >= 0 ? fo_root(F + (k - 1), k, rep) : -1;
       // the batches before this one are a proper subset while anything is left
       const long long al = *(volatile long long*)&ctl->alpha;
       if (left > 0 && al < best) {
@@ -380,24 +388,32 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
         best_batch = b - 1;
       }
       if (left <= 0) break;
-      for (long long v0 = (long long)blockIdx.x * kFoThreads; v0 < n;
-           v0 += (long long)gridDim.x * kFoThreads) {
-        const int v = (int)v0 + tid;
-        int chunks = 0;
+      // (four vertices a thread: a pass over all of them costs its dependent
+      // loads and block-wide sums once per 2,048)
+      for (long long v0 = (long long)blockIdx.x * (4 * kFoThreads); v0 < n;
+           v0 += (long long)gridDim.x * (4 * kFoThreads)) {
+        const int v = (int)v0 + 4 * tid;
+        int mine = 0;
+        unsigned take = 0;
         if (v < n) {
-          const unsigned tg = tag[v];
-          if ((tg & 127u) == 0) {
-            const int key = min(ru[v], k);
-            if (key >= t) {
-              tag[v] = (uint8_t)(tg | (unsigned)b);
-              atomicSub(&s_hist[key], 1);
-              const long long len = a.rp[v + 1] - a.rp[v];
-              chunks = max(1, (int)((len + kFoChunk - 1) / kFoChunk));
-              fo_scanned(F, k, v, len);
-            }
+          // (the arrays end on 256-byte boundaries; vertices from n on are ignored)
+          const unsigned tg4 = *reinterpret_cast<const unsigned*>(tag + v);
+          const int4 r4 = *reinterpret_cast<const int4*>(ru + v);
+          if ((tg4 & 127u) == 0 && min(r4.x, k) >= t) take |= 1u;
+          if ((tg4 & 0x7f00u) == 0 && min(r4.y, k) >= t) take |= 2u;
+          if ((tg4 & 0x7f0000u) == 0 && min(r4.z, k) >= t) take |= 4u;
+          if ((tg4 & 0x7f000000u) == 0 && min(r4.w, k) >= t) take |= 8u;
+          if (n - v < 4) take &= (1u << (n - v)) - 1u;
+          for (unsigned rest = take; rest; rest &= rest - 1) {
+            const int x = v + __ffs(rest) - 1;
+            const long long len = a.rp[x + 1] - a.rp[x];
+            tag[x] = (uint8_t)(tag[x] | (unsigned)b);
+            atomicSub(&s_hist[min(ru[x], k)], 1);
+            mine += fo_pieces(len);
+            fo_scanned(F, k, x, len);
           }
         }
-        int incl = chunks;
+        int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int u = __shfl_up_sync(FULL, incl, o);
@@ -411,10 +427,16 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
           if (i < wp) before += s_scan[i];
           total += s_scan[i];
         }
-        if (tid == 0 && total) s_base = atomicAdd(&ctl->items, total);
-        __syncthreads();
-        const unsigned at = s_base + before + (unsigned)(incl - chunks);
-        for (int c = 0; c < chunks; ++c) __stcg(&a.items[at + c], make_int2(v, c));
+        if (total) {  // (the same for the whole block)
+          if (tid == 0) s_base = atomicAdd(&ctl->items, total);
+          __syncthreads();
+          unsigned at = s_base + before + (unsigned)(incl - mine);
+          for (; take; take &= take - 1) {
+            const int x = v + __ffs(take) - 1;
+            const int pieces = fo_pieces(a.rp[x + 1] - a.rp[x]);
+            for (int c = 0; c < pieces; ++c) __stcg(&a.items[at++], make_int2(x, c));
+          }
+        }
         __syncthreads();
       }
       if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
@@ -428,8 +450,6 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     const unsigned warps = gridDim.x * (kFoThreads / 32);
     unsigned per = 1;
     while (per < 32 && per * 8 * warps <= nitems) per *= 2;
-    const int rep = (int)*(volatile unsigned*)&ctl->main - 1;
-    const int main_root = rep >= 0 ? fo_root(F + (k - 1), k, rep) : -1;
     if (tid == 0) s_main = rep >= 0;
     long long alpha = 0;
     int qn = 0;  // queued edges of this warp

@@ -384,6 +384,20 @@ cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, 
                         void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side, const int* map0, int n0,
                         uint8_t* side0, int sms, DevState* st, cudaStream_t s, int* launches);
 
+// The same for what the labels L (st->n_next of them) leave of a larger graph,
+// from its rows and without a contracted CSR: st->small_status 1 = solved, 2 =
+// more than kSmMaxN labels or mcap / 2 edges (or as above).  The witness is per
+// label in cur_side; small_side(.., L, ..) carries it to side0 when
+// st->small_improved.  count: three ints; mat: `words` ints of
+// scratch; pieces: n + M / 512 of them.
+template <typename WT>
+cudaError_t small_rest(int n, const int64_t* rp, const int* col, const WT* w, const int* L,
+                       void* ed0, void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side,
+                       int* count, int* mat, long long words, int2* pieces, int sms,
+                       DevState* st, cudaStream_t s, int* launches);
+cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, int n0,
+                       uint8_t* side0, int sms, const DevState* st, cudaStream_t s, int* launches);
+
 // A batch's graphs (at most kSmMaxN vertices each), a block per graph at a
 // time from a work queue: values and sides of those solved, the others'
 // ids in left[0 .. *nleft) for batch_warp_solve.  scratch: `slots` slots of

@@ -218,10 +218,9 @@ __device__ __forceinline__ int sm_level(int* F, int k, int x, int y, int guess) 
 
 // Insert a warp's edges {x, y} from level lo up (units = 0: none), a lane per
 // (edge, level): a lane that walked its own edge's levels would hold the warp
-// up for its longest.  Returns the lane's units inserted.
-__device__ __forceinline__ int sm_insert(int* F, int k, int x, int y, int lo, int units) {
+// up for its longest.
+__device__ __forceinline__ void sm_insert(int* F, int k, int x, int y, int lo, int units) {
   const int lane = threadIdx.x & 31;
-  int gained = 0;
   int want = min(units, k - lo);
   for (;;) {
     int incl = want;
@@ -231,7 +230,7 @@ __device__ __forceinline__ int sm_insert(int* F, int k, int x, int y, int lo, in
       if (lane >= o) incl += u;
     }
     const int total = __shfl_sync(FULL, incl, 31);
-    if (total == 0) return gained;
+    if (total == 0) return;
     const int excl = incl - want;
     int got = 0;
     for (int p0 = 0; p0 < total; p0 += 32) {
@@ -249,7 +248,6 @@ __device__ __forceinline__ int sm_insert(int* F, int k, int x, int y, int lo, in
       const int b0 = max(excl - p0, 0), b1 = min(incl - p0, 32);
       if (b0 < b1) got += __popc(bal & (FULL >> (32 - (b1 - b0)) << b0));
     }
-    gained += got;
     lo += want;  // units whose level was joined meanwhile go on above
     want = max(0, min(want - got, k - lo));
   }
@@ -475,17 +473,15 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
                 if (sm.r[y] < k) atomicAdd(&sm.r[y], units);
                 sm_insert_fast(sm.F, k, x, y, units);
               } else if (units > 0) {
-                lo = sm_level(sm.F, k, x, y, min(*(volatile int*)&sm.r[y], k - 1));
-                if (lo == k) {
-                  units = 0;
-                  if (sm.tag[y] == 0) atomicMax(&sm.r[y], k);
-                }
+                int g = sm.r[y];
+                if (g < k) g = atomicAdd(&sm.r[y], units);
+                lo = sm_level(sm.F, k, x, y, min(g, k - 1));
+                if (lo == k) units = 0;
               }
             }
             if (k <= kSmFast) continue;
             __syncwarp();
-            const int got = sm_insert(sm.F, k, x, y, lo, units);
-            if (got > 0 && sm.tag[y] == 0) atomicAdd(&sm.r[y], got);
+            sm_insert(sm.F, k, x, y, lo, units);
           } while (end && qn > 0);
         }
       }
@@ -612,7 +608,147 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
   return ok;
 }
 
-// The current graph of a single solve (n <= kSmMaxN): its minimum cut below
+// What a round's groups leave of a large graph, when it is small: the edges
+// between different labels (st->n_next of them, at most kSmMaxN).  Up to
+// kSmMatrix labels they are summed in a matrix (zeroed, accumulated, listed), above that listed as they come.  Every edge of the largest
+// group also stands in its other end's row, so that group's rows, most of the
+// graph where the forests join nearly everything, are not read: it is estimated
+// from a sample, and any other choice is as correct.  *count ends above ecap
+// when the edges do not fit.  Measured on the R-MAT scale 20 core (386 labels of
+// 247 K vertices): 57 us for the four launches, against ~450 us of contraction
+// and two host synchronisations; long rows (a first hub stays a vertex of its
+// own) go in pieces: by one warp each they took 346 us.
+constexpr int kSmMatrix = 1024;
+
+__device__ __forceinline__ bool sm_matrix(int n2, long long words) {
+  return n2 <= kSmMatrix && (long long)n2 * n2 <= words;
+}
+
+__global__ void small_zero_kernel(int* mat, long long words, const DevState* st) {
+  const int n2 = st->n_next;
+  if (n2 < 2 || !sm_matrix(n2, words)) return;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n2 * n2; i += gridDim.x * blockDim.x)
+    mat[i] = 0;
+}
+
+constexpr int kSmPiece = 512;  // a longer row is left to small_pieces_kernel, in pieces
+
+// Entries [b, e) of a vertex of label u, by one warp.
+template <typename WT>
+__device__ __forceinline__ void sm_collect(int u, long long b, long long e, int skip, bool matrix,
+                                           int n2, const int* __restrict__ col,
+                                           const WT* __restrict__ w, const int* __restrict__ L,
+                                           SmEdges ed, int ecap, int* count, int* mat) {
+  const int lane = threadIdx.x & 31;
+  for (long long p0 = b; p0 < e; p0 += 32) {
+    int x = u;
+    if (p0 + lane < e) x = L[col[p0 + lane]];
+    const bool keep = x == skip || u < x;  // between two others: from the smaller label
+    if (matrix) {
+      if (keep) atomicAdd(&mat[min(u, x) * n2 + max(u, x)], (int)w[p0 + lane]);
+      continue;
+    }
+    const unsigned bal = __ballot_sync(FULL, keep);
+    if (!bal) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(count, __popc(bal));
+    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
+    if (keep && at < ecap) {
+      ed.ends[at] = (unsigned)u | ((unsigned)x << 16);
+      ed.w[at] = (int)w[p0 + lane];
+    }
+  }
+}
+
+// count[0]: edges listed; [1]: pieces listed; [2]: the label whose rows are
+// skipped.
+template <typename WT>
+__global__ void __launch_bounds__(256)
+    small_collect_kernel(int n, const int64_t* __restrict__ rp, const int* __restrict__ col,
+                         const WT* __restrict__ w, const int* __restrict__ L, SmEdges ed, int ecap,
+                         int* count, int* mat, long long words, int2* pieces, const DevState* st) {
+  __shared__ int s_cnt[kSmMaxN];
+  __shared__ unsigned s_best;
+  const int n2 = st->n_next;
+  if (n2 > kSmMaxN || n2 < 2) return;
+  const bool matrix = sm_matrix(n2, words);
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int i = tid; i < n2; i += 256) s_cnt[i] = 0;
+  if (tid == 0) s_best = 0;
+  __syncthreads();
+  // (the same sample in every block, hence the same choice)
+  atomicAdd(&s_cnt[L[(long long)tid * n / 256]], 1);
+  __syncthreads();
+  for (int i = tid; i < n2; i += 256)
+    if (s_cnt[i]) atomicMax(&s_best, ((unsigned)s_cnt[i] << 16) | (unsigned)i);
+  __syncthreads();
+  const int skip = (int)(s_best & 0xffffu);
+  if (blockIdx.x == 0 && tid == 0) count[2] = skip;
+  const int warp = blockIdx.x * 8 + (tid >> 5), warps = gridDim.x * 8;
+  for (long long v0 = (long long)warp * 32; v0 < n; v0 += (long long)warps * 32) {
+    const int v = (int)v0 + lane;
+    const int lv = v < n ? L[v] : skip;
+    unsigned todo = __ballot_sync(FULL, lv != skip);
+    if (!matrix && __shfl_sync(FULL, todo ? *(volatile int*)count : 0, 0) > ecap) return;
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int u = __shfl_sync(FULL, lv, src);
+      const long long b = rp[v0 + src], e = rp[v0 + src + 1];
+      if (e - b > kSmPiece) {
+        const int k = (int)((e - b + kSmPiece - 1) / kSmPiece);
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&count[1], k);
+        at = __shfl_sync(FULL, at, 0);
+        for (int i = lane; i < k; i += 32) pieces[at + i] = make_int2((int)v0 + src, i);
+      } else {
+        sm_collect<WT>(u, b, e, skip, matrix, n2, col, w, L, ed, ecap, count, mat);
+      }
+    }
+  }
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(256)
+    small_pieces_kernel(const int64_t* __restrict__ rp, const int* __restrict__ col,
+                        const WT* __restrict__ w, const int* __restrict__ L, SmEdges ed, int ecap,
+                        int* count, int* mat, long long words, const int2* __restrict__ pieces,
+                        const DevState* st) {
+  const int n2 = st->n_next;
+  if (n2 > kSmMaxN || n2 < 2) return;
+  const bool matrix = sm_matrix(n2, words);
+  const int k = count[1], skip = count[2];
+  for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < k; i += gridDim.x * 8) {
+    if (!matrix && __shfl_sync(FULL, *(volatile int*)count, 0) > ecap) return;
+    const int2 p = pieces[i];
+    const long long b = rp[p.x] + (long long)p.y * kSmPiece;
+    sm_collect<WT>(L[p.x], b, min(b + kSmPiece, (long long)rp[p.x + 1]), skip, matrix, n2, col, w,
+                   L, ed, ecap, count, mat);
+  }
+}
+
+__global__ void small_list_kernel(const int* __restrict__ mat, long long words, SmEdges ed,
+                                  int ecap, int* count, const DevState* st) {
+  const int n2 = st->n_next, lane = threadIdx.x & 31;
+  if (n2 < 2 || !sm_matrix(n2, words)) return;
+  for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n2 * n2;
+       i0 += gridDim.x * blockDim.x) {
+    const int i = i0 + lane;
+    const int c = i < n2 * n2 ? mat[i] : 0;
+    const unsigned bal = __ballot_sync(FULL, c != 0);
+    if (!bal) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(count, __popc(bal));
+    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
+    if (c != 0 && at < ecap) {
+      ed.ends[at] = (unsigned)(i / n2) | ((unsigned)(i % n2) << 16);
+      ed.w[at] = c;
+    }
+  }
+}
+
+// The current graph of a single solve (n <= kSmMaxN; or, with `count`, the
+// st->n_next vertices and *count edges in ed0): its minimum cut below
 // st->lambda.  st->small_status: 1 solved, 2 bail (too many entries, or a
 // round that could not go on); st->small_improved: what lowered the bound
 // (0: nothing), its witness per vertex of the graph in cur_side.
@@ -620,11 +756,12 @@ template <int T>
 __global__ void __launch_bounds__(T, 1)
     small_solve_kernel(int n, const int64_t* rp, const int* col, const int* w, SmEdges ed0,
                        SmEdges ed1, long long mcap, int fcap, uint32_t pr_mask, uint8_t* cur_side,
-                       DevState* st) {
+                       const int* count, DevState* st) {
   extern __shared__ __align__(16) unsigned char sm_dyn[];
   __shared__ SmShared<T> s;
   const SmMem sm = sm_mem(sm_dyn, kSmMaxN, fcap);
-  if (rp[n] > mcap) {
+  if (count) n = st->n_next;
+  if (count ? n > kSmMaxN || *count > mcap / 2 : rp[n] > mcap) {
     if (threadIdx.x == 0) {
       st->small_status = 2;
       st->small_improved = 0;
@@ -633,7 +770,7 @@ __global__ void __launch_bounds__(T, 1)
   }
   long long lam = (long long)*(volatile unsigned long long*)&st->lambda;
   int source, rounds;
-  const int m = sm_load<T>(sm, s, rp, col, w, 0, n, ed0, (int)(mcap / 2));
+  const int m = count ? *count : sm_load<T>(sm, s, rp, col, w, 0, n, ed0, (int)(mcap / 2));
   source = rounds = 0;
   const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds);
   if (source)
@@ -684,11 +821,12 @@ __global__ void __launch_bounds__(T, 3)
   }
 }
 
-__global__ void side_if_improved_kernel(uint8_t* side0, const int* __restrict__ map0, int n0,
+__global__ void side_if_improved_kernel(uint8_t* side0, const int* __restrict__ map0,
+                                        const int* __restrict__ L, int n0,
                                         const uint8_t* __restrict__ cur, const DevState* st) {
   if (!st->small_improved) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n0; i += gridDim.x * blockDim.x)
-    side0[i] = cur[map0[i]];
+    side0[i] = cur[L ? L[map0[i]] : map0[i]];
 }
 
 }  // namespace
@@ -700,21 +838,60 @@ static SmEdges sm_edges(void* p, long long mcap) {  // mcap / 2 edges
   return SmEdges{static_cast<unsigned*>(p), static_cast<int*>(p) + (mcap / 2 + 1)};
 }
 
-cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,
-                        void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side, const int* map0, int n0,
-                        uint8_t* side0, int sms, DevState* st, cudaStream_t s, int* launches) {
-  if (n < 1 || n > kSmMaxN) return cudaErrorInvalidValue;
+static bool sm_solve_attr() {
   static const bool ok = cudaFuncSetAttribute(small_solve_kernel<kSmThreads>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)sm_bytes(kSmMaxN, kSmFcap)) == cudaSuccess;
-  if (!ok) return cudaErrorInvalidValue;
+  return ok;
+}
+
+cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,
+                        void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side,
+                        const int* map0, int n0, uint8_t* side0, int sms, DevState* st,
+                        cudaStream_t s, int* launches) {
+  if (n < 1 || n > kSmMaxN || !sm_solve_attr()) return cudaErrorInvalidValue;
   small_solve_kernel<kSmThreads><<<1, kSmThreads, sm_bytes(kSmMaxN, kSmFcap), s>>>(
-      n, rp, col, w, sm_edges(ed0, mcap), sm_edges(ed1, mcap), mcap, kSmFcap, pr_mask, cur_side, st);
+      n, rp, col, w, sm_edges(ed0, mcap), sm_edges(ed1, mcap), mcap, kSmFcap, pr_mask, cur_side,
+      nullptr, st);
+  ++*launches;
+  return small_side(cur_side, map0, nullptr, n0, side0, sms, st, s, launches);
+}
+
+cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, int n0,
+                       uint8_t* side0, int sms, const DevState* st, cudaStream_t s,
+                       int* launches) {
   side_if_improved_kernel<<<std::max(1, std::min((n0 + 255) / 256, sms * 8)), 256, 0, s>>>(
-      side0, map0, n0, cur_side, st);
-  *launches += 2;
+      side0, map0, L, n0, cur_side, st);
+  ++*launches;
   return cudaGetLastError();
 }
+
+template <typename WT>
+cudaError_t small_rest(int n, const int64_t* rp, const int* col, const WT* w, const int* L,
+                       void* ed0, void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side,
+                       int* count, int* mat, long long words, int2* pieces, int sms,
+                       DevState* st, cudaStream_t s, int* launches) {
+  if (!sm_solve_attr()) return cudaErrorInvalidValue;
+  cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  const SmEdges ed = sm_edges(ed0, mcap);
+  const int ecap = (int)(mcap / 2);
+  small_zero_kernel<<<sms, 512, 0, s>>>(mat, words, st);
+  small_collect_kernel<WT><<<std::max(1, std::min((n + 255) / 256, sms * 8)), 256, 0, s>>>(
+      n, rp, col, w, L, ed, ecap, count, mat, words, pieces, st);
+  small_pieces_kernel<WT><<<sms * 4, 256, 0, s>>>(rp, col, w, L, ed, ecap, count, mat, words,
+                                                  pieces, st);
+  small_list_kernel<<<sms, 512, 0, s>>>(mat, words, ed, ecap, count, st);
+  small_solve_kernel<kSmThreads><<<1, kSmThreads, sm_bytes(kSmMaxN, kSmFcap), s>>>(
+      0, nullptr, nullptr, nullptr, sm_edges(ed0, mcap), sm_edges(ed1, mcap), mcap, kSmFcap,
+      pr_mask, cur_side, count, st);
+  *launches += 5;
+  return cudaGetLastError();
+}
+template cudaError_t small_rest<int32_t>(int, const int64_t*, const int*, const int32_t*,
+                                         const int*, void*, void*, long long, uint32_t, uint8_t*,
+                                         int*, int*, long long, int2*, int, DevState*,
+                                         cudaStream_t, int*);
 
 // Shared memory of the batch kernel by its largest graph: as many union-find
 // words as let three blocks share an SM (at least 5 levels of the largest).

@@ -64,3 +64,35 @@ def test_random_sparse_20000(seed):
     g = synth.er_connected(20_000, 100_000, 1, 30, 50 + seed)
     c = (g.row_ptr, g.col, g.w.astype(np.int64))
     _check_solve(g.n, c, expect=oracle.noi(g.n, *c)[0])
+
+@pytest.mark.parametrize("clusters,size,hub", [(2, 1200, 0), (300, 8, 0), (300, 8, 700),
+                                               (1023, 4, 0), (1025, 4, 0), (1700, 4, 1500),
+                                               (2040, 3, 0), (2300, 3, 0)])
+def test_what_the_forests_leave(clusters, size, hub):
+    """Heavy clusters joined by light edges: the forests leave one vertex per
+    cluster, summed in a matrix, listed, or too many for either; hubs with rows
+    of several pieces stay vertices of their own."""
+    rng = np.random.default_rng(clusters + size)
+    n = clusters * size
+    first = np.arange(clusters) * size
+    e, w = [], []
+    for i in range(size):  # a heavy cycle within each cluster
+        j = (i + 1) % size
+        if size > 2 or i < j:
+            e += list(zip(first + i, first + j))
+            w += [500] * clusters
+    order = rng.permutation(clusters)  # a light cycle through the clusters, and chords
+    for a, b in [(order, np.roll(order, 1)),
+                 (rng.integers(0, clusters, 3 * clusters), rng.integers(0, clusters, 3 * clusters))]:
+        u = first[a] + rng.integers(0, size, len(a))
+        v = first[b] + rng.integers(0, size, len(b))
+        k = a != b
+        e += list(zip(u[k], v[k]))
+        w += [int(x) for x in rng.integers(1, 9, int(k.sum()))]
+    for h in range(2 if hub else 0):  # hubs: one light edge to each of many vertices
+        e += [(n + h, int(v)) for v in rng.choice(n, hub, replace=False)]
+        w += [1] * hub
+    n += 2 if hub else 0
+    perm = rng.permutation(n)
+    c = canon(n, *G.from_edges(n, [(perm[a], perm[b]) for a, b in e], w))
+    _check_solve(n, c, expect=oracle.noi(n, *c)[0])
