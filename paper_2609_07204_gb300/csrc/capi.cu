@@ -763,35 +763,35 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   const int* col = g->ccol();
   const WT* w = (const WT*)g->cw();
   const WT* deg = (const WT*)g->cdeg();
-  const void* cw32 = g->cw();  // (the 32-bit weights where WT is int32_t)
-  reset_round_kernel<<<1, 1, 0, s>>>(g->st);
-  ++g->launches;
-  if (n >= 2) {
-    ProfScope ps(P_DEGREE, n, s);
-    CK(degrees_min<WT>(deg, n, g->blk, g->st, s, &g->launches));
-  }
   int rc;
   const bool forest = c.forest && n > 2;
+  const bool rest = forest && sizeof(WT) == 4 && c.small_rest;
   if (forest) {
-    // the sort keys are free during the marking: they hold the union-finds
+    // the sort keys and values are free during the marking: they hold the
+    // union-finds, then the list of what is left and the matrix it is summed in
     rc = ensure_forest(g);
     if (rc) return rc;
+    const long long Mb = std::max<long long>(g->Mraw, 1), mcap = std::min(kSmMaxM, Mb);
+    const ForestScratch f{reinterpret_cast<int*>(g->keys[0]), 2 * Mb, g->fo_tag, g->fo_r,
+                          g->fo_items, g->fo_ctl};
+    const SmallList list = small_list(g->keys[0], g->vals[0], Mb, mcap);
     { ProfScope ps(P_FOREST, g->m_pending ? 0 : g->M, s);
-      CK(forest_marks<WT>(n, g->m_pending ? g->m_bound : g->M, rp, col, w, deg,
-                          reinterpret_cast<int*>(g->keys[0]), 2 * std::max<long long>(g->Mraw, 1),
-                          g->fo_tag, g->fo_r, g->fo_items, g->fo_ctl, g->parent, g->fo_qsoft,
-                          g->sms, g->spin_limit, g->st, s, &g->launches)); }
-    if (sizeof(WT) == 4 && c.small_rest) {
-      // the labels, and when few are left the rest of the solve, before the
-      // host has seen anything of the round
-      { ProfScope ps(P_UF, n, s);
-        CK(uf_relabel(g->parent, g->L, g->flags, g->rank, g->part, n, g->st, s, &g->launches)); }
+      CK(forest_marks<WT>(f, n, g->m_pending ? g->m_bound : g->M, rp, col, w, deg, g->parent, g->L,
+                          g->flags, g->rank, g->fo_qsoft, rest ? &list : nullptr, g->sms,
+                          g->spin_limit, g->st, s, &g->launches)); }
+    if (rest) {
+      // and when few are left the rest of the solve, before the host has seen
+      // anything of the round
       ProfScope ps(P_SMALL, n, s);
-      CK(small_rest<int32_t>(n, rp, col, (const int32_t*)cw32, g->L, g->keys[0], g->keys[1],
-                             std::min(kSmMaxM, std::max<long long>(g->Mraw, 1)), c.pr_mask & 3u,
-                             g->cur_side, (int*)g->fo_ctl, (int*)g->vals[0],
-                             std::max<long long>(g->Mraw, 1), g->fo_items, g->sms, g->st, s,
-                             &g->launches));
+      CK(small_rest(g->keys[0], g->keys[1], mcap, forest_count(f), c.pr_mask & 3u, g->cur_side,
+                    g->st, s, &g->launches));
+    }
+  } else {
+    reset_round_kernel<<<1, 1, 0, s>>>(g->st);
+    ++g->launches;
+    if (n >= 2) {
+      ProfScope ps(P_DEGREE, n, s);
+      CK(degrees_min<WT>(deg, n, g->blk, g->st, s, &g->launches));
     }
   }
   rc = sync_state(g);
@@ -803,7 +803,6 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   const long long M = g->M;
   // the degree bound, then what the forests' prefix cuts add to it
   // (and what the one-block solve of the rest lowered it to)
-  const bool rest = forest && sizeof(WT) == 4 && c.small_rest;
   const bool cf_first = forest && g->hst->cf_pass == kForestPass;
   const bool rest_first = rest && g->hst->small_improved != 0;
   long long lam = cf_first || rest_first ? std::min(lambda_before, (long long)g->hst->deg_val)
@@ -829,10 +828,12 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     o->src = g->hst->small_improved;
     lambda_before = lam;
   }
-  if (rest) o->labelled = true;
+  o->labelled = forest;
   if (rest && g->hst->small_status == 1) {
     o->solved = true;
     o->rest_rounds = g->hst->small_rounds;
+  } else if (forest && (long long)g->hst->marks_cf == n - 1) {
+    o->solved = true;  // one component
   }
   o->lambda = lam;
   if (n <= 2 || lam == 0) {

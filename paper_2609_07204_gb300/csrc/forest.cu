@@ -1,5 +1,8 @@
 // forest.cu -- certificate forests: the marking step of a round as one
-// edge-parallel pass over the whole graph (one cooperative kernel).
+// edge-parallel pass over the whole graph, in one cooperative kernel with the
+// rest of the round's head: degree bound before, labels and the list of what is
+// left after (22 launches of 2 to 5 us each otherwise, and as many gaps: R-MAT
+// scale 16 core 473 -> 394 us, 64 served requests 11.9 -> 8.4 ms).
 //
 // Certificate.  Let lam be the round's bound, q a quantum and k = ceil(lam/q).
 // An edge of weight c has floor(c/q) units.  Every edge puts its units into
@@ -46,10 +49,16 @@
 //
 // Measured against the whole-graph CAPFOREST passes that such rounds needed
 // before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
-// 1,340 ms -> 8.7 ms, 2 x 2^15 83 -> 4.0 ms; against PR tests, label
-// propagation and concurrent passes: R-MAT scale 20 10-core 3.69 -> 0.93 ms
-// (0.75 ms of it here), scale 16 1.15 -> 0.47 ms, random weighted n = 150,001
-// (with its creation) 2.51 -> 0.74 ms.
+// 1,340 ms -> 8.8 ms, 2 x 2^15 83 -> 3.7 ms; against PR tests, label
+// propagation and concurrent passes: R-MAT scale 20 10-core 3.69 -> 0.95 ms
+// (0.83 ms of it here), scale 16 1.13 -> 0.39 ms, random weighted n = 150,001
+// (with its creation) 2.25 -> 0.68 ms.
+//
+// What is left: up to kFoMatrix labels it is summed in a matrix, above that
+// listed as it comes.  Measured on the R-MAT scale 20 core (386 labels of 247 K
+// vertices): 57 us as four launches of its own, against ~450 us of contraction
+// and two host synchronisations; long rows (a first hub stays a vertex of its
+// own) go in pieces: by one warp each they took 346 us.
 #include <algorithm>
 #include <climits>
 
@@ -61,6 +70,9 @@ namespace mc {
 namespace {
 
 constexpr int kFoThreads = 512;
+constexpr int kFoPerThread = 32;  // entries per thread that a grid is sized for: more blocks make
+                                  // the barriers dearer (2 x 2^15 cut: 3.7 ms, 4.0 with the
+                                  // whole GPU) and keep other streams' solves waiting
 constexpr int kFoChunk = 64;      // entries of a row handled by one warp at a time
 constexpr int kFoMaxK = 254;      // levels (histogram bins: k + 1)
 constexpr int kFoLevels = 8;      // levels wanted where the weights allow it (qsoft): fewer
@@ -71,6 +83,7 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
 constexpr unsigned kFoAbort = ~0u;
+constexpr int kFoMaxBlocks = 1024;
 
 struct FoCtl {
   unsigned bar;        // grid barrier: arrivals
@@ -79,6 +92,11 @@ struct FoCtl {
   unsigned pad2[31];
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
+  int count;           // edges listed of what is left; INT_MAX: not listed
+  unsigned pieces;     // pieces of long rows listed for that
+  unsigned long long deg_inv;  // ~(minimum degree)
+  int deg_arg_inv;     // INT_MAX - (its smallest vertex)
+  int roots[kFoMaxBlocks];     // components by the block that holds their smallest member
   long long alpha;     // cut of the scanned set
   unsigned next[2];    // items fetched in a batch beyond the first deal (by its parity)
   int hist[256];       // unscanned vertices by min(r, k)
@@ -96,6 +114,15 @@ struct FoArgs {
   int* r;              // per vertex: units that met it while unscanned
   int2* items;         // (vertex, chunk of its row)
   int* parent;
+  int *L, *flags, *rank;  // labels, 1 per root, its exclusive prefix sum
+  // the rest (what the labels leave), when it is asked for: edges listed in
+  // (ends, ew), at most ecap; mat: mat_words ints of scratch
+  int rest;
+  unsigned* ends;
+  int* ew;
+  int ecap;
+  int* mat;
+  long long mat_words;
   FoCtl* ctl;
   DevState* st;
   long long spin;
@@ -107,7 +134,8 @@ struct FoArgs {
 // releases the others through a word of its own line: the arrivals, atomics on
 // one word, do not queue up behind the polls (with both on one word a barrier
 // of 608 blocks took ~10 us).
-__device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spin, int* s_ok) {
+__device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spin, int* s_ok,
+                                           DevState* st) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -123,6 +151,7 @@ __device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spi
         if (++it > spin) {  // (the value ends the wait of the others, too)
           asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->release), "r"(kFoAbort)
                        : "memory");
+          set_error(st, ERR_TIMEOUT);
           v = kFoAbort;
           break;
         }
@@ -296,6 +325,98 @@ __device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units,
   return asked - units;
 }
 
+// Batch b: the unscanned vertices with min(r, k) >= t are tagged, take their
+// ranks and are listed.  (A function of its own: inlined, its loads push the
+// scan's registers out.)
+__device__ __noinline__ void fo_select(const FoArgs& a, int k, int b, int t, int* s_hist,
+                                       unsigned* s_scan, unsigned* s_base) {
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int n = a.n;
+  int* F = a.F;
+  uint8_t* tag = a.tag;
+  const int* ru = a.r;
+  FoCtl* ctl = a.ctl;
+        // (four vertices a thread: a pass over all of them costs its dependent
+        // loads and block-wide sums once per 2,048)
+        for (long long v0 = (long long)blockIdx.x * (4 * kFoThreads); v0 < n;
+             v0 += (long long)gridDim.x * (4 * kFoThreads)) {
+          const int v = (int)v0 + 4 * tid;
+          int mine = 0;
+          unsigned take = 0;
+          if (v < n) {
+            // (the arrays end on 256-byte boundaries; vertices from n on are ignored)
+            const unsigned tg4 = *reinterpret_cast<const unsigned*>(tag + v);
+            const int4 r4 = *reinterpret_cast<const int4*>(ru + v);
+            if ((tg4 & 127u) == 0 && min(r4.x, k) >= t) take |= 1u;
+            if ((tg4 & 0x7f00u) == 0 && min(r4.y, k) >= t) take |= 2u;
+            if ((tg4 & 0x7f0000u) == 0 && min(r4.z, k) >= t) take |= 4u;
+            if ((tg4 & 0x7f000000u) == 0 && min(r4.w, k) >= t) take |= 8u;
+            if (n - v < 4) take &= (1u << (n - v)) - 1u;
+            for (unsigned rest = take; rest; rest &= rest - 1) {
+              const int x = v + __ffs(rest) - 1;
+              const long long len = a.rp[x + 1] - a.rp[x];
+              tag[x] = (uint8_t)(tag[x] | (unsigned)b);
+              atomicSub(&s_hist[min(ru[x], k)], 1);
+              mine += fo_pieces(len);
+              fo_scanned(F, k, x, len);
+            }
+          }
+          int incl = mine;
+  #pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += u;
+          }
+          if (lane == 31) s_scan[wp] = incl;
+          __syncthreads();
+          unsigned before = 0, total = 0;
+  #pragma unroll
+          for (int i = 0; i < kFoThreads / 32; ++i) {
+            if (i < wp) before += s_scan[i];
+            total += s_scan[i];
+          }
+          if (total) {  // (the same for the whole block)
+            if (tid == 0) *s_base = atomicAdd(&ctl->items, total);
+            __syncthreads();
+            unsigned at = *s_base + before + (unsigned)(incl - mine);
+            for (; take; take &= take - 1) {
+              const int x = v + __ffs(take) - 1;
+              const int pieces = fo_pieces(a.rp[x + 1] - a.rp[x]);
+              for (int c = 0; c < pieces; ++c) __stcg(&a.items[at++], make_int2(x, c));
+            }
+          }
+          __syncthreads();
+        }
+}
+
+constexpr int kFoMatrix = 1024;  // labels that are summed in a matrix
+constexpr int kFoPiece = 512;    // entries of a long row that one warp lists
+
+// Entries [b, e) of a vertex of label u, by one warp.
+template <typename WT>
+__device__ __noinline__ void fo_collect(const FoArgs& a, int u, long long b, long long e, int skip,
+                                        bool matrix, int n2, const WT* w) {
+  const int lane = threadIdx.x & 31;
+  for (long long p0 = b; p0 < e; p0 += 32) {
+    int x = u;
+    if (p0 + lane < e) x = a.L[a.col[p0 + lane]];
+    const bool keep = x == skip || u < x;  // between two others: from the smaller label
+    if (matrix) {
+      if (keep) atomicAdd(&a.mat[min(u, x) * n2 + max(u, x)], (int)w[p0 + lane]);
+      continue;
+    }
+    const unsigned bal = __ballot_sync(FULL, keep);
+    if (!bal) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&a.ctl->count, __popc(bal));
+    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
+    if (keep && at < a.ecap) {
+      a.ends[at] = (unsigned)u | ((unsigned)x << 16);
+      a.ew[at] = (int)w[p0 + lane];
+    }
+  }
+}
+
 template <typename WT>
 __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   __shared__ int s_hist[256];   // this block's changes since the last flush
@@ -306,22 +427,85 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   __shared__ int2 s_q[kFoThreads / 32][64];      // queued edges of each warp
   __shared__ uint8_t s_qu[kFoThreads / 32][64];  // and their units
   __shared__ long long s_alpha[kFoThreads / 32];
+  // the block's view of the round (the same in all of them): bound, minimum
+  // degree, smallest prefix cut and the batch it ends with
+  __shared__ long long s_lam, s_best;
+  __shared__ unsigned long long s_dmin;
+  __shared__ int s_best_batch;
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int n = a.n;
-  const long long lam = (long long)*(volatile unsigned long long*)&a.st->lambda;
   const int gtid = blockIdx.x * kFoThreads + tid, gsize = gridDim.x * kFoThreads;
-  for (int v = gtid; v < n; v += gsize) a.parent[v] = v;  // nothing joined, however this ends
-  if (n <= 2 || lam <= 0 || lam >= kInf) return;  // (the round stops or has no bound)
-  const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
-  if (kcap < 1) return;
-  const long long q = max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + kFoLevels - 1) / kFoLevels));
-  const int k = (int)((lam + q - 1) / q);
   const WT* __restrict__ w = reinterpret_cast<const WT*>(a.w);
   const WT* __restrict__ deg = reinterpret_cast<const WT*>(a.deg);
+  FoCtl* ctl = a.ctl;
+  unsigned gen = 0;
+  // ---- degree bound (Sec. 2.1), and a clean round state
+  const long long lam_in = (long long)*(volatile unsigned long long*)&a.st->lambda;
+  unsigned long long dmin = ~0ull;
+  for (int v = gtid; v < n; v += gsize) {
+    a.parent[v] = v;  // nothing joined, however this ends
+    dmin = min(dmin, (unsigned long long)(long long)deg[v]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dmin = min(dmin, __shfl_xor_sync(FULL, dmin, o));
+  if (lane == 0) s_alpha[wp] = (long long)dmin;
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < kFoThreads / 32; ++i) dmin = min(dmin, (unsigned long long)s_alpha[i]);
+    atomicMax(&ctl->deg_inv, ~dmin);
+    if (blockIdx.x == 0) {
+      DevState* st = a.st;
+      st->marks_pr = 0;
+      st->marks_cf = 0;
+      st->emit_count = 0;
+      st->lp_val = ~0ull;
+      st->lp_label = -1;
+      st->cf_val = ~0ull;
+      st->cf_pass = -1;
+      st->cf_len = 0;
+      st->cf_nscanned = 0;
+      st->cf_nmarks = 0;
+      st->claimed = 0;
+      ctl->count = INT_MAX;
+    }
+  }
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  dmin = ~__ldcg(&ctl->deg_inv);
+  const long long lam = min(lam_in, (long long)dmin);
+  {
+    int arg = INT_MAX;
+    for (int v = gtid; v < n && arg == INT_MAX; v += gsize)
+      if ((unsigned long long)(long long)deg[v] == dmin) arg = v;
+    arg = __reduce_min_sync(FULL, arg);
+    if (lane == 0) s_scan[wp] = (unsigned)arg;
+    __syncthreads();
+    if (tid == 0) {
+      for (int i = 1; i < kFoThreads / 32; ++i) arg = min(arg, (int)s_scan[i]);
+      if (arg != INT_MAX) atomicMax(&ctl->deg_arg_inv, INT_MAX - arg);
+    }
+  }
+  if (tid == 0) {
+    s_lam = lam;
+    s_dmin = dmin;
+    s_best = kInf;
+    s_best_batch = 0;
+  }
+  const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
+  if (n <= 2 || lam <= 0 || kcap < 1) {  // (the round stops)
+    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+    if (gtid == 0) {
+      a.st->deg_val = dmin;
+      a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
+      a.st->lambda = (unsigned long long)lam;
+    }
+    return;
+  }
+  // (the quantum, like the bound, fits the weight type)
+  const WT q = (WT)max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + kFoLevels - 1) / kFoLevels));
+  const int k = (int)((lam + q - 1) / q);
   int* F = a.F;
   uint8_t* tag = a.tag;
   int* ru = a.r;
-  FoCtl* ctl = a.ctl;
   // ---- every vertex a root at every level, nothing scanned; the first batch
   // is vertex 0
   {
@@ -345,12 +529,9 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
   }
-  unsigned gen = 0;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
   unsigned start = 0;
   int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root
-  long long best = kInf;
-  int best_batch = 0;
   for (int b = 1;; ++b) {
     if (b > 1) {
       // ---- the batch: the highest r until 1 / kFoFrac of the vertices left
@@ -383,63 +564,13 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       main_root = rep >= 0 ? fo_root(F + (k - 1), k, rep) : -1;
       // the batches before this one are a proper subset while anything is left
       const long long al = *(volatile long long*)&ctl->alpha;
-      if (left > 0 && al < best) {
-        best = al;
-        best_batch = b - 1;
+      if (tid == 0 && left > 0 && al < s_best) {
+        s_best = al;
+        s_best_batch = b - 1;
       }
       if (left <= 0) break;
-      // (four vertices a thread: a pass over all of them costs its dependent
-      // loads and block-wide sums once per 2,048)
-      for (long long v0 = (long long)blockIdx.x * (4 * kFoThreads); v0 < n;
-           v0 += (long long)gridDim.x * (4 * kFoThreads)) {
-        const int v = (int)v0 + 4 * tid;
-        int mine = 0;
-        unsigned take = 0;
-        if (v < n) {
-          // (the arrays end on 256-byte boundaries; vertices from n on are ignored)
-          const unsigned tg4 = *reinterpret_cast<const unsigned*>(tag + v);
-          const int4 r4 = *reinterpret_cast<const int4*>(ru + v);
-          if ((tg4 & 127u) == 0 && min(r4.x, k) >= t) take |= 1u;
-          if ((tg4 & 0x7f00u) == 0 && min(r4.y, k) >= t) take |= 2u;
-          if ((tg4 & 0x7f0000u) == 0 && min(r4.z, k) >= t) take |= 4u;
-          if ((tg4 & 0x7f000000u) == 0 && min(r4.w, k) >= t) take |= 8u;
-          if (n - v < 4) take &= (1u << (n - v)) - 1u;
-          for (unsigned rest = take; rest; rest &= rest - 1) {
-            const int x = v + __ffs(rest) - 1;
-            const long long len = a.rp[x + 1] - a.rp[x];
-            tag[x] = (uint8_t)(tag[x] | (unsigned)b);
-            atomicSub(&s_hist[min(ru[x], k)], 1);
-            mine += fo_pieces(len);
-            fo_scanned(F, k, x, len);
-          }
-        }
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(FULL, incl, o);
-          if (lane >= o) incl += u;
-        }
-        if (lane == 31) s_scan[wp] = incl;
-        __syncthreads();
-        unsigned before = 0, total = 0;
-#pragma unroll
-        for (int i = 0; i < kFoThreads / 32; ++i) {
-          if (i < wp) before += s_scan[i];
-          total += s_scan[i];
-        }
-        if (total) {  // (the same for the whole block)
-          if (tid == 0) s_base = atomicAdd(&ctl->items, total);
-          __syncthreads();
-          unsigned at = s_base + before + (unsigned)(incl - mine);
-          for (; take; take &= take - 1) {
-            const int x = v + __ffs(take) - 1;
-            const int pieces = fo_pieces(a.rp[x + 1] - a.rp[x]);
-            for (int c = 0; c < pieces; ++c) __stcg(&a.items[at++], make_int2(x, c));
-          }
-        }
-        __syncthreads();
-      }
-      if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+      fo_select(a, k, b, t, s_hist, s_scan, &s_base);
+      if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
     }
     // ---- scan the batch: a warp walks the entries of a few items (short rows,
     // pieces of long ones) as one list, fetched as warps get free (dealt in
@@ -492,12 +623,12 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
           int y = 0, u = 0;
           if (p < total) {
             y = a.col[e];
-            const long long c = (long long)w[e];
+            const WT c = w[e];
             const unsigned ty = tag[y], tx = tag[xx];
             const int by = (int)(ty & 127u);
-            u = (int)min((long long)k, q == 1 ? c : c / q);
+            u = (int)min((WT)k, q == 1 ? c : c / q);
             if (by != 0 && by < b) {  // inserted when y was scanned
-              alpha -= 2 * c;
+              alpha -= 2 * (long long)c;
             } else {
               // both ends in this batch: the smaller id inserts
               if (by == b) alpha -= c;
@@ -574,16 +705,16 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
     start = end;
-    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
   }
   // ---- the round's marks: the components of the last level (the last that
   // the bound still asks for: a prefix cut may have lowered it), each under its
   // smallest member (r, done with, holds it per root; a warp's vertices of one
   // root send one atomic)
-  const long long lam_end = min(lam, best);
+  const long long best = s_best, lam_end = min(s_lam, best);
   int* Fe = F + (lam_end > 0 ? (int)((lam_end + q - 1) / q) - 1 : 0);
   for (int v = gtid; v < n; v += gsize) ru[v] = INT_MAX;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
   unsigned joined = 0;
   for (int v0 = gtid - lane; v0 < n; v0 += gsize) {
     const int v = v0 + lane;
@@ -592,22 +723,154 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     if (r >= 0 && (same & lanemask_lt()) == 0) atomicMin(&ru[r], v);
     joined += r >= 0 && r != v;
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok)) return;
-  for (int v = gtid; v < n; v += gsize) a.parent[v] = ru[fo_root(Fe, k, v)];
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  // ---- labels: the components by smallest member; a block counts those of its
+  // own run of vertices, then numbers them
+  const int per = (int)(((long long)n + gridDim.x - 1) / gridDim.x);
+  const int vb = (int)min((long long)n, (long long)blockIdx.x * per), ve = min(n, vb + per);
+  int mine = 0;
+  for (int v = vb + tid; v < ve; v += kFoThreads) {
+    const int p = ru[fo_root(Fe, k, v)];
+    a.parent[v] = p;
+    mine += p == v;
+  }
+  mine = __reduce_add_sync(FULL, mine);
+  if (lane == 0) s_scan[wp] = (unsigned)mine;
   joined = warp_sum(joined);
-  if (lane == 0 && joined) atomicAdd(&a.st->marks_cf, (unsigned long long)joined);
-  if (blockIdx.x == 0 && tid == 0) {
-    if (best < lam) {
-      atomicMin(&a.st->lambda, (unsigned long long)best);
-      a.st->cf_val = (unsigned long long)best;
-      a.st->cf_pass = kForestPass;
-      a.st->cf_len = best_batch;
+  if (lane == 0) s_alpha[wp] = joined;
+  __syncthreads();
+  if (tid == 0) {
+    int sum = 0;
+    long long j = 0;
+    for (int i = 0; i < kFoThreads / 32; ++i) {
+      sum += (int)s_scan[i];
+      j += s_alpha[i];
+    }
+    __stcg(&ctl->roots[blockIdx.x], sum);
+    if (j) atomicAdd(&a.st->marks_cf, (unsigned long long)j);
+    if (blockIdx.x == 0) {
+      a.st->deg_val = s_dmin;
+      a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
+      a.st->lambda = (unsigned long long)lam_end;
+      if (best < s_lam) {
+        a.st->cf_val = (unsigned long long)best;
+        a.st->cf_pass = kForestPass;
+        a.st->cf_len = s_best_batch;
+      }
     }
   }
-}
-
-__global__ void fo_timeout_kernel(const FoCtl* c, DevState* st) {
-  if (c->release == kFoAbort) set_error(st, ERR_TIMEOUT);
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  int n2 = 0, base = 0;
+  for (int i = tid; i < (int)gridDim.x; i += kFoThreads) {
+    const int c = __ldcg(&ctl->roots[i]);
+    n2 += c;
+    if (i < (int)blockIdx.x) base += c;
+  }
+  n2 = __reduce_add_sync(FULL, n2);
+  base = __reduce_add_sync(FULL, base);
+  __syncthreads();
+  if (lane == 0) {
+    s_all[wp] = n2;
+    s_hist[wp] = base;
+  }
+  __syncthreads();
+  n2 = base = 0;
+  for (int i = 0; i < kFoThreads / 32; ++i) {
+    n2 += s_all[i];
+    base += s_hist[i];
+  }
+  if (gtid == 0) a.st->n_next = n2;
+  for (int v0 = vb; v0 < ve; v0 += kFoThreads) {
+    const int v = v0 + tid;
+    const bool root = v < ve && a.parent[v] == v;
+    const unsigned bal = __ballot_sync(FULL, root);
+    __syncthreads();
+    if (lane == 0) s_scan[wp] = (unsigned)__popc(bal);
+    __syncthreads();
+    int before = base, total = 0;
+    for (int i = 0; i < kFoThreads / 32; ++i) {
+      if (i < wp) before += (int)s_scan[i];
+      total += (int)s_scan[i];
+    }
+    if (v < ve) {
+      a.flags[v] = root;
+      a.rank[v] = before + __popc(bal & lanemask_lt());
+    }
+    base += total;
+  }
+  const bool rest = a.rest && n2 >= 2 && n2 <= kSmMaxN;
+  const bool matrix = n2 <= kFoMatrix && (long long)n2 * n2 <= a.mat_words;
+  if (rest && matrix)
+    for (int i = gtid; i < n2 * n2; i += gsize) a.mat[i] = 0;
+  if (rest && gtid == 0) ctl->count = 0;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  for (int v = gtid; v < n; v += gsize) a.L[v] = a.rank[a.parent[v]];
+  if (!rest) return;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  // ---- what is left: the edges between different labels.  Up to kFoMatrix
+  // labels they are summed in a matrix, above that listed as they come (count
+  // ends above ecap when they do not fit).  Every edge of the largest group also
+  // stands in its other end's row, so that group's rows, most of the graph where
+  // the forests join nearly everything, are not read: it is estimated from a
+  // sample, and any other choice is as correct.
+  int* s_cnt = reinterpret_cast<int*>(s_q);
+  static_assert(sizeof(s_q) >= kSmMaxN * sizeof(int), "label counts");
+  for (int i = tid; i < n2; i += kFoThreads) s_cnt[i] = 0;
+  if (tid == 0) s_base = 0;
+  __syncthreads();
+  // (the same sample in every block, hence the same choice)
+  atomicAdd(&s_cnt[a.L[(long long)tid * n / kFoThreads]], 1);
+  __syncthreads();
+  for (int i = tid; i < n2; i += kFoThreads)
+    if (s_cnt[i]) atomicMax(&s_base, ((unsigned)s_cnt[i] << 16) | (unsigned)i);
+  __syncthreads();
+  const int skip = (int)(s_base & 0xffffu);
+  const int gwarp = gtid >> 5, nwarps = gsize >> 5;
+  for (long long v0 = (long long)gwarp * 32; v0 < n; v0 += (long long)nwarps * 32) {
+    const int v = (int)v0 + lane;
+    const int lv = v < n ? a.L[v] : skip;
+    unsigned todo = __ballot_sync(FULL, lv != skip);
+    if (!matrix && __shfl_sync(FULL, todo ? *(volatile int*)&ctl->count : 0, 0) > a.ecap) break;
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int u = __shfl_sync(FULL, lv, src);
+      const long long rb = a.rp[v0 + src], re = a.rp[v0 + src + 1];
+      if (re - rb > kFoPiece) {  // a long row goes in pieces, below
+        const int np = (int)((re - rb + kFoPiece - 1) / kFoPiece);
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&ctl->pieces, (unsigned)np);
+        at = __shfl_sync(FULL, at, 0);
+        for (int i = lane; i < np; i += 32) __stcg(&a.items[at + i], make_int2((int)v0 + src, i));
+      } else {
+        fo_collect<WT>(a, u, rb, re, skip, matrix, n2, w);
+      }
+    }
+  }
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  const int np = (int)__ldcg(&ctl->pieces);
+  for (int i = gwarp; i < np; i += nwarps) {
+    if (!matrix && __shfl_sync(FULL, *(volatile int*)&ctl->count, 0) > a.ecap) break;
+    const int2 p = __ldcg(&a.items[i]);
+    const long long rb = a.rp[p.x] + (long long)p.y * kFoPiece;
+    fo_collect<WT>(a, a.L[p.x], rb, min(rb + kFoPiece, (long long)a.rp[p.x + 1]), skip, matrix, n2,
+                   w);
+  }
+  if (!matrix) return;
+  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  for (int i0 = gtid - lane; i0 < n2 * n2; i0 += gsize) {
+    const int i = i0 + lane;
+    const int c = i < n2 * n2 ? __ldcg(&a.mat[i]) : 0;
+    const unsigned bal = __ballot_sync(FULL, c != 0);
+    if (!bal) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&ctl->count, __popc(bal));
+    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
+    if (c != 0 && at < a.ecap) {
+      a.ends[at] = (unsigned)(i / n2) | ((unsigned)(i % n2) << 16);
+      a.ew[at] = c;
+    }
+  }
 }
 
 __global__ void side_batch_kernel(uint8_t* side0, const int* __restrict__ map0, int n0,
@@ -624,10 +887,10 @@ long long forest_item_cap(long long n, long long M) { return n + M / kFoChunk + 
 size_t forest_ctl_bytes() { return sizeof(FoCtl); }
 
 template <typename WT>
-cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, const WT* w,
-                         const WT* deg, int* F, long long fcap, uint8_t* tag, int* r,
-                         int2* items, void* ctl, int* parent, long long qsoft, int sms, long long spin, DevState* st,
-                         cudaStream_t s, int* launches) {
+cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64_t* rp,
+                         const int* col, const WT* w, const WT* deg, int* parent, int* L,
+                         int* flags, int* rank, long long qsoft, const SmallList* rest, int sms,
+                         long long spin, DevState* st, cudaStream_t s, int* launches) {
   static int per_sm[2] = {0, 0};
   const int wi = sizeof(WT) == 8 ? 1 : 0;
   if (!per_sm[wi]) {
@@ -637,7 +900,7 @@ cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, 
     if (e != cudaSuccess) return e;
     per_sm[wi] = std::max(1, p);
   }
-  cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(FoCtl), s);
+  cudaError_t e = cudaMemsetAsync(f.ctl, 0, sizeof(FoCtl), s);
   if (e != cudaSuccess) return e;
   FoArgs a{};
   a.n = n;
@@ -645,26 +908,40 @@ cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, 
   a.col = col;
   a.w = w;
   a.deg = deg;
-  a.F = F;
-  a.fcap = fcap;
-  a.tag = tag;
-  a.r = r;
+  a.F = f.F;
+  a.fcap = f.fcap;
+  a.tag = f.tag;
+  a.r = f.r;
   a.qsoft = qsoft;
-  a.items = items;
+  a.items = f.items;
   a.parent = parent;
-  a.ctl = static_cast<FoCtl*>(ctl);
+  a.L = L;
+  a.flags = flags;
+  a.rank = rank;
+  if (rest) {
+    a.rest = 1;
+    a.ends = rest->ends;
+    a.ew = rest->w;
+    a.ecap = rest->cap;
+    a.mat = rest->mat;
+    a.mat_words = rest->mat_words;
+  }
+  a.ctl = static_cast<FoCtl*>(f.ctl);
   a.st = st;
   a.spin = spin;
-  const long long want = (std::max<long long>(M, n) + 2 * kFoThreads - 1) / (2 * kFoThreads);
-  const int blocks = (int)std::max<long long>(1, std::min<long long>(want, (long long)sms * per_sm[wi]));
+  const long long want =
+      (std::max<long long>(M, n) + kFoPerThread * kFoThreads - 1) / (kFoPerThread * kFoThreads);
+  const int blocks = (int)std::max<long long>(
+      1, std::min<long long>({want, (long long)sms * per_sm[wi], (long long)kFoMaxBlocks}));
   void* params[] = {&a};
   e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
                                   params, 0, s);
   if (e != cudaSuccess) return e;
-  fo_timeout_kernel<<<1, 1, 0, s>>>(a.ctl, st);
-  *launches += 2;
+  ++*launches;
   return cudaGetLastError();
 }
+
+const int* forest_count(const ForestScratch& f) { return &static_cast<const FoCtl*>(f.ctl)->count; }
 
 cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uint8_t* tag, int last,
                               int sms, cudaStream_t s, int* launches) {
@@ -675,9 +952,10 @@ cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uin
 }
 
 #define MC_FO_INST(WT)                                                                           \
-  template cudaError_t forest_marks<WT>(int, long long, const int64_t*, const int*, const WT*,   \
-                                        const WT*, int*, long long, uint8_t*, int*, int2*,       \
-                                        void*, int*, long long, int, long long, DevState*, cudaStream_t, int*);
+  template cudaError_t forest_marks<WT>(const ForestScratch&, int, long long, const int64_t*,    \
+                                        const int*, const WT*, const WT*, int*, int*, int*,      \
+                                        int*, long long, const SmallList*, int, long long,       \
+                                        DevState*, cudaStream_t, int*);
 MC_FO_INST(int32_t)
 MC_FO_INST(int64_t)
 

@@ -351,23 +351,43 @@ cudaError_t capforest_warp_passes(int n, long long M, const int64_t* rp, const i
                                   int* launches);
 
 // --------------------------------------------------------------- forest.cu
-// Certificate forests of the current graph: parent[v] = the smallest vertex
-// of v's component of the last forest (vertices of one component have
-// connectivity at least st->lambda at launch), the number of joined vertices
-// added to st->marks_cf; prefix cuts below the bound lower st->lambda and
-// name their witness in cf_val, cf_pass = kForestPass, cf_len = last batch
-// (side_from_batches over `state`).  Does nothing when n <= 2 or the bound is
-// 0.  F: fcap ints of scratch, at least 2 per vertex; state: n; items:
-// forest_item_cap(n, M); ctl: forest_ctl_bytes().  One cooperative kernel;
-// its grid barriers wait at most `spin` reads (ERR_TIMEOUT).
+// The head of a round led by certificate forests, one cooperative kernel:
+// resets the round state; the degree bound (deg_val, deg_arg, st->lambda);
+// the forests of the current graph: parent[v] = the smallest vertex of v's
+// component of the last forest (vertices of one component have connectivity
+// at least the bound), the number of joined vertices in st->marks_cf; prefix
+// cuts below the bound lower st->lambda and name their witness in cf_val,
+// cf_pass = kForestPass, cf_len = last batch (side_from_batches over tag);
+// the labels L with st->n_next, flags and rank as uf_relabel gives them; and,
+// with `rest`, when 2 to kSmMaxN labels are left, the list of the edges
+// between them (*forest_count edges, above rest->cap when they do not fit,
+// INT_MAX when there is no list).  Without joins and labels when n <= 2 or the
+// bound is 0.  Its grid barriers wait at most `spin` reads (ERR_TIMEOUT).
+struct ForestScratch {
+  int* F;          // fcap ints, at least 2 per vertex
+  long long fcap;
+  uint8_t* tag;    // n
+  int* r;          // n
+  int2* items;     // forest_item_cap(n, M)
+  void* ctl;       // forest_ctl_bytes()
+};
+struct SmallList {  // undirected edges: ends u | v << 16, weights
+  unsigned* ends;
+  int* w;
+  int cap;
+  int* mat;             // scratch
+  long long mat_words;
+};
 constexpr int kForestPass = -0x7fffffff;
+constexpr int kSmMaxN = 2048;  // vertices of the one-block solver (small.cu)
 long long forest_item_cap(long long n, long long M);
 size_t forest_ctl_bytes();
 template <typename WT>
-cudaError_t forest_marks(int n, long long M, const int64_t* rp, const int* col, const WT* w,
-                         const WT* deg, int* F, long long fcap, uint8_t* tag, int* r,
-                         int2* items, void* ctl, int* parent, long long qsoft, int sms, long long spin, DevState* st,
-                         cudaStream_t s, int* launches);
+cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64_t* rp,
+                         const int* col, const WT* w, const WT* deg, int* parent, int* L,
+                         int* flags, int* rank, long long qsoft, const SmallList* rest, int sms,
+                         long long spin, DevState* st, cudaStream_t s, int* launches);
+const int* forest_count(const ForestScratch& f);  // (on the device)
 cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uint8_t* tag, int last,
                               int sms, cudaStream_t s, int* launches);
 
@@ -378,23 +398,19 @@ cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uin
 // st->small_status says 1 = solved, 2 = left to the other rounds (more than
 // mcap entries, or a round that joined nothing).  ed0, ed1: mcap words
 // and 2 more each; cur_side: n bytes.
-constexpr int kSmMaxN = 2048;
 constexpr long long kSmMaxM = 1ll << 17;
 cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,
                         void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side, const int* map0, int n0,
                         uint8_t* side0, int sms, DevState* st, cudaStream_t s, int* launches);
 
-// The same for what the labels L (st->n_next of them) leave of a larger graph,
-// from its rows and without a contracted CSR: st->small_status 1 = solved, 2 =
-// more than kSmMaxN labels or mcap / 2 edges (or as above).  The witness is per
-// label in cur_side; small_side(.., L, ..) carries it to side0 when
-// st->small_improved.  count: three ints; mat: `words` ints of
-// scratch; pieces: n + M / 512 of them.
-template <typename WT>
-cudaError_t small_rest(int n, const int64_t* rp, const int* col, const WT* w, const int* L,
-                       void* ed0, void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side,
-                       int* count, int* mat, long long words, int2* pieces, int sms,
-                       DevState* st, cudaStream_t s, int* launches);
+// The same for what a round's labels (st->n_next of them) leave of a larger
+// graph, the *count edges listed in ed0 (small_list) by forest_marks:
+// st->small_status 2 also when there is no list or it did not fit.  The witness
+// is per label in cur_side; small_side(.., L, ..) carries it to side0 when
+// st->small_improved.
+SmallList small_list(void* ed0, void* mat, long long mat_words, long long mcap);
+cudaError_t small_rest(void* ed0, void* ed1, long long mcap, const int* count, uint32_t pr_mask,
+                       uint8_t* cur_side, DevState* st, cudaStream_t s, int* launches);
 cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, int n0,
                        uint8_t* side0, int sms, const DevState* st, cudaStream_t s, int* launches);
 

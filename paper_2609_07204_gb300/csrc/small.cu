@@ -608,145 +608,6 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
   return ok;
 }
 
-// What a round's groups leave of a large graph, when it is small: the edges
-// between different labels (st->n_next of them, at most kSmMaxN).  Up to
-// kSmMatrix labels they are summed in a matrix (zeroed, accumulated, listed), above that listed as they come.  Every edge of the largest
-// group also stands in its other end's row, so that group's rows, most of the
-// graph where the forests join nearly everything, are not read: it is estimated
-// from a sample, and any other choice is as correct.  *count ends above ecap
-// when the edges do not fit.  Measured on the R-MAT scale 20 core (386 labels of
-// 247 K vertices): 57 us for the four launches, against ~450 us of contraction
-// and two host synchronisations; long rows (a first hub stays a vertex of its
-// own) go in pieces: by one warp each they took 346 us.
-constexpr int kSmMatrix = 1024;
-
-__device__ __forceinline__ bool sm_matrix(int n2, long long words) {
-  return n2 <= kSmMatrix && (long long)n2 * n2 <= words;
-}
-
-__global__ void small_zero_kernel(int* mat, long long words, const DevState* st) {
-  const int n2 = st->n_next;
-  if (n2 < 2 || !sm_matrix(n2, words)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n2 * n2; i += gridDim.x * blockDim.x)
-    mat[i] = 0;
-}
-
-constexpr int kSmPiece = 512;  // a longer row is left to small_pieces_kernel, in pieces
-
-// Entries [b, e) of a vertex of label u, by one warp.
-template <typename WT>
-__device__ __forceinline__ void sm_collect(int u, long long b, long long e, int skip, bool matrix,
-                                           int n2, const int* __restrict__ col,
-                                           const WT* __restrict__ w, const int* __restrict__ L,
-                                           SmEdges ed, int ecap, int* count, int* mat) {
-  const int lane = threadIdx.x & 31;
-  for (long long p0 = b; p0 < e; p0 += 32) {
-    int x = u;
-    if (p0 + lane < e) x = L[col[p0 + lane]];
-    const bool keep = x == skip || u < x;  // between two others: from the smaller label
-    if (matrix) {
-      if (keep) atomicAdd(&mat[min(u, x) * n2 + max(u, x)], (int)w[p0 + lane]);
-      continue;
-    }
-    const unsigned bal = __ballot_sync(FULL, keep);
-    if (!bal) continue;
-    int at = 0;
-    if (lane == 0) at = atomicAdd(count, __popc(bal));
-    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
-    if (keep && at < ecap) {
-      ed.ends[at] = (unsigned)u | ((unsigned)x << 16);
-      ed.w[at] = (int)w[p0 + lane];
-    }
-  }
-}
-
-// count[0]: edges listed; [1]: pieces listed; [2]: the label whose rows are
-// skipped.
-template <typename WT>
-__global__ void __launch_bounds__(256)
-    small_collect_kernel(int n, const int64_t* __restrict__ rp, const int* __restrict__ col,
-                         const WT* __restrict__ w, const int* __restrict__ L, SmEdges ed, int ecap,
-                         int* count, int* mat, long long words, int2* pieces, const DevState* st) {
-  __shared__ int s_cnt[kSmMaxN];
-  __shared__ unsigned s_best;
-  const int n2 = st->n_next;
-  if (n2 > kSmMaxN || n2 < 2) return;
-  const bool matrix = sm_matrix(n2, words);
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (int i = tid; i < n2; i += 256) s_cnt[i] = 0;
-  if (tid == 0) s_best = 0;
-  __syncthreads();
-  // (the same sample in every block, hence the same choice)
-  atomicAdd(&s_cnt[L[(long long)tid * n / 256]], 1);
-  __syncthreads();
-  for (int i = tid; i < n2; i += 256)
-    if (s_cnt[i]) atomicMax(&s_best, ((unsigned)s_cnt[i] << 16) | (unsigned)i);
-  __syncthreads();
-  const int skip = (int)(s_best & 0xffffu);
-  if (blockIdx.x == 0 && tid == 0) count[2] = skip;
-  const int warp = blockIdx.x * 8 + (tid >> 5), warps = gridDim.x * 8;
-  for (long long v0 = (long long)warp * 32; v0 < n; v0 += (long long)warps * 32) {
-    const int v = (int)v0 + lane;
-    const int lv = v < n ? L[v] : skip;
-    unsigned todo = __ballot_sync(FULL, lv != skip);
-    if (!matrix && __shfl_sync(FULL, todo ? *(volatile int*)count : 0, 0) > ecap) return;
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int u = __shfl_sync(FULL, lv, src);
-      const long long b = rp[v0 + src], e = rp[v0 + src + 1];
-      if (e - b > kSmPiece) {
-        const int k = (int)((e - b + kSmPiece - 1) / kSmPiece);
-        int at = 0;
-        if (lane == 0) at = atomicAdd(&count[1], k);
-        at = __shfl_sync(FULL, at, 0);
-        for (int i = lane; i < k; i += 32) pieces[at + i] = make_int2((int)v0 + src, i);
-      } else {
-        sm_collect<WT>(u, b, e, skip, matrix, n2, col, w, L, ed, ecap, count, mat);
-      }
-    }
-  }
-}
-
-template <typename WT>
-__global__ void __launch_bounds__(256)
-    small_pieces_kernel(const int64_t* __restrict__ rp, const int* __restrict__ col,
-                        const WT* __restrict__ w, const int* __restrict__ L, SmEdges ed, int ecap,
-                        int* count, int* mat, long long words, const int2* __restrict__ pieces,
-                        const DevState* st) {
-  const int n2 = st->n_next;
-  if (n2 > kSmMaxN || n2 < 2) return;
-  const bool matrix = sm_matrix(n2, words);
-  const int k = count[1], skip = count[2];
-  for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < k; i += gridDim.x * 8) {
-    if (!matrix && __shfl_sync(FULL, *(volatile int*)count, 0) > ecap) return;
-    const int2 p = pieces[i];
-    const long long b = rp[p.x] + (long long)p.y * kSmPiece;
-    sm_collect<WT>(L[p.x], b, min(b + kSmPiece, (long long)rp[p.x + 1]), skip, matrix, n2, col, w,
-                   L, ed, ecap, count, mat);
-  }
-}
-
-__global__ void small_list_kernel(const int* __restrict__ mat, long long words, SmEdges ed,
-                                  int ecap, int* count, const DevState* st) {
-  const int n2 = st->n_next, lane = threadIdx.x & 31;
-  if (n2 < 2 || !sm_matrix(n2, words)) return;
-  for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n2 * n2;
-       i0 += gridDim.x * blockDim.x) {
-    const int i = i0 + lane;
-    const int c = i < n2 * n2 ? mat[i] : 0;
-    const unsigned bal = __ballot_sync(FULL, c != 0);
-    if (!bal) continue;
-    int at = 0;
-    if (lane == 0) at = atomicAdd(count, __popc(bal));
-    at = __shfl_sync(FULL, at, 0) + __popc(bal & lanemask_lt());
-    if (c != 0 && at < ecap) {
-      ed.ends[at] = (unsigned)(i / n2) | ((unsigned)(i % n2) << 16);
-      ed.w[at] = c;
-    }
-  }
-}
-
 // The current graph of a single solve (n <= kSmMaxN; or, with `count`, the
 // st->n_next vertices and *count edges in ed0): its minimum cut below
 // st->lambda.  st->small_status: 1 solved, 2 bail (too many entries, or a
@@ -761,7 +622,7 @@ __global__ void __launch_bounds__(T, 1)
   __shared__ SmShared<T> s;
   const SmMem sm = sm_mem(sm_dyn, kSmMaxN, fcap);
   if (count) n = st->n_next;
-  if (count ? n > kSmMaxN || *count > mcap / 2 : rp[n] > mcap) {
+  if (count ? *count > mcap / 2 || n > kSmMaxN : rp[n] > mcap) {
     if (threadIdx.x == 0) {
       st->small_status = 2;
       st->small_improved = 0;
@@ -866,32 +727,20 @@ cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, i
   return cudaGetLastError();
 }
 
-template <typename WT>
-cudaError_t small_rest(int n, const int64_t* rp, const int* col, const WT* w, const int* L,
-                       void* ed0, void* ed1, long long mcap, uint32_t pr_mask, uint8_t* cur_side,
-                       int* count, int* mat, long long words, int2* pieces, int sms,
-                       DevState* st, cudaStream_t s, int* launches) {
+SmallList small_list(void* ed0, void* mat, long long mat_words, long long mcap) {
+  const SmEdges e = sm_edges(ed0, mcap);
+  return SmallList{e.ends, e.w, (int)(mcap / 2), static_cast<int*>(mat), mat_words};
+}
+
+cudaError_t small_rest(void* ed0, void* ed1, long long mcap, const int* count, uint32_t pr_mask,
+                       uint8_t* cur_side, DevState* st, cudaStream_t s, int* launches) {
   if (!sm_solve_attr()) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  const SmEdges ed = sm_edges(ed0, mcap);
-  const int ecap = (int)(mcap / 2);
-  small_zero_kernel<<<sms, 512, 0, s>>>(mat, words, st);
-  small_collect_kernel<WT><<<std::max(1, std::min((n + 255) / 256, sms * 8)), 256, 0, s>>>(
-      n, rp, col, w, L, ed, ecap, count, mat, words, pieces, st);
-  small_pieces_kernel<WT><<<sms * 4, 256, 0, s>>>(rp, col, w, L, ed, ecap, count, mat, words,
-                                                  pieces, st);
-  small_list_kernel<<<sms, 512, 0, s>>>(mat, words, ed, ecap, count, st);
   small_solve_kernel<kSmThreads><<<1, kSmThreads, sm_bytes(kSmMaxN, kSmFcap), s>>>(
       0, nullptr, nullptr, nullptr, sm_edges(ed0, mcap), sm_edges(ed1, mcap), mcap, kSmFcap,
       pr_mask, cur_side, count, st);
-  *launches += 5;
+  ++*launches;
   return cudaGetLastError();
 }
-template cudaError_t small_rest<int32_t>(int, const int64_t*, const int*, const int32_t*,
-                                         const int*, void*, void*, long long, uint32_t, uint8_t*,
-                                         int*, int*, long long, int2*, int, DevState*,
-                                         cudaStream_t, int*);
 
 // Shared memory of the batch kernel by its largest graph: as many union-find
 // words as let three blocks share an SM (at least 5 levels of the largest).
