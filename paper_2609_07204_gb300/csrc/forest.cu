@@ -63,6 +63,7 @@
 #include <climits>
 
 #include "common.cuh"
+#include "grid_barrier.cuh"
 #include "kernels.h"
 
 namespace mc {
@@ -82,14 +83,10 @@ constexpr int kFoFrac = 12;       // a batch takes at least 1 / kFoFrac of the v
 constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
-constexpr unsigned kFoAbort = ~0u;
 constexpr int kFoMaxBlocks = 1024;
 
 struct FoCtl {
-  unsigned bar;        // grid barrier: arrivals
-  unsigned pad[31];
-  unsigned release;    // grid barrier: the last one complete, or kFoAbort
-  unsigned pad2[31];
+  GridBar bar;
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
   int count;           // edges listed of what is left; INT_MAX: not listed
@@ -128,43 +125,6 @@ struct FoArgs {
   long long spin;
   long long qsoft;     // quantum that loses little of the weights
 };
-
-// Grid barrier number `gen` (1, 2, ...): false when the wait ran out (here or
-// in another block), after which every block leaves.  The last block to arrive
-// releases the others through a word of its own line: the arrivals, atomics on
-// one word, do not queue up behind the polls (with both on one word a barrier
-// of 608 blocks took ~10 us).
-__device__ __forceinline__ bool fo_barrier(FoCtl* c, unsigned gen, long long spin, int* s_ok,
-                                           DevState* st) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    bool ok = true;
-    if (atomicAdd(&c->bar, 1u) + 1u == gen * gridDim.x) {
-      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->release), "r"(gen) : "memory");
-    } else {
-      unsigned v = 0;
-      long long it = 0;
-      for (;;) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->release) : "memory");
-        if (v >= gen) break;
-        if (++it > spin) {  // (the value ends the wait of the others, too)
-          asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->release), "r"(kFoAbort)
-                       : "memory");
-          set_error(st, ERR_TIMEOUT);
-          v = kFoAbort;
-          break;
-        }
-        __nanosleep(20);
-      }
-      ok = v != kFoAbort;
-    }
-    __threadfence();
-    *s_ok = ok ? 1 : 0;
-  }
-  __syncthreads();
-  return *s_ok != 0;
-}
 
 // A level's union-find, linked by rank: a root's word is -1 - rank, another's
 // its parent, and (rank, id) grows from child to parent, so concurrent links
@@ -469,7 +429,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       ctl->count = INT_MAX;
     }
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   dmin = ~__ldcg(&ctl->deg_inv);
   const long long lam = min(lam_in, (long long)dmin);
   {
@@ -492,7 +452,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   }
   const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
   if (n <= 2 || lam <= 0 || kcap < 1) {  // (the round stops)
-    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+    if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
     if (gtid == 0) {
       a.st->deg_val = dmin;
       a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
@@ -529,7 +489,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   unsigned start = 0;
   int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root
   for (int b = 1;; ++b) {
@@ -570,7 +530,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
       if (left <= 0) break;
       fo_select(a, k, b, t, s_hist, s_scan, &s_base);
-      if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+      if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
     }
     // ---- scan the batch: a warp walks the entries of a few items (short rows,
     // pieces of long ones) as one list, fetched as warps get free (dealt in
@@ -705,7 +665,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
     start = end;
-    if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+    if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   }
   // ---- the round's marks: the components of the last level (the last that
   // the bound still asks for: a prefix cut may have lowered it), each under its
@@ -714,7 +674,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   const long long best = s_best, lam_end = min(s_lam, best);
   int* Fe = F + (lam_end > 0 ? (int)((lam_end + q - 1) / q) - 1 : 0);
   for (int v = gtid; v < n; v += gsize) ru[v] = INT_MAX;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   unsigned joined = 0;
   for (int v0 = gtid - lane; v0 < n; v0 += gsize) {
     const int v = v0 + lane;
@@ -723,7 +683,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     if (r >= 0 && (same & lanemask_lt()) == 0) atomicMin(&ru[r], v);
     joined += r >= 0 && r != v;
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   // ---- labels: the components by smallest member; a block counts those of its
   // own run of vertices, then numbers them
   const int per = (int)(((long long)n + gridDim.x - 1) / gridDim.x);
@@ -759,7 +719,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   int n2 = 0, base = 0;
   for (int i = tid; i < (int)gridDim.x; i += kFoThreads) {
     const int c = __ldcg(&ctl->roots[i]);
@@ -803,10 +763,10 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
   if (rest && matrix)
     for (int i = gtid; i < n2 * n2; i += gsize) a.mat[i] = 0;
   if (rest && gtid == 0) ctl->count = 0;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   for (int v = gtid; v < n; v += gsize) a.L[v] = a.rank[a.parent[v]];
   if (!rest) return;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   // ---- what is left: the edges between different labels.  Up to kFoMatrix
   // labels they are summed in a matrix, above that listed as they come (count
   // ends above ecap when they do not fit).  Every edge of the largest group also
@@ -847,7 +807,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
       }
     }
   }
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   const int np = (int)__ldcg(&ctl->pieces);
   for (int i = gwarp; i < np; i += nwarps) {
     if (!matrix && __shfl_sync(FULL, *(volatile int*)&ctl->count, 0) > a.ecap) break;
@@ -857,7 +817,7 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
                    w);
   }
   if (!matrix) return;
-  if (!fo_barrier(ctl, ++gen, a.spin, &s_ok, a.st)) return;
+  if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   for (int i0 = gtid - lane; i0 < n2 * n2; i0 += gsize) {
     const int i = i0 + lane;
     const int c = i < n2 * n2 ? __ldcg(&a.mat[i]) : 0;

@@ -159,3 +159,37 @@ def test_noalloc_rejects_oversized_graph():
         mc.mincut_contract_csr_noalloc(n, rp, z, z, lab, 1, rp_out, z, z)
     assert e.value.status == mc.MINCUT_ERR_OVERFLOW
     assert "262144" in mc.mincut_last_error()
+
+
+@pytest.mark.parametrize("n,n2,skew", [(2, 1, 0), (300, 300, 0), (5000, 3, 0), (5000, 40, 0),
+                                       (5000, 900, 0), (9000, 2000, 1), (9000, 60, 2),
+                                       (16000, 5, 0), (262144, 262144, 0), (262144, 7, 0)])
+def test_noalloc_row_lengths(n, n2, skew):
+    """Labels whose rows a warp sorts, a block sorts, or neither; one label with
+    most of the entries; the largest vertex count; hubs of long rows."""
+    rng = np.random.default_rng(n + n2)
+    m = min(130_000, 4 * n)
+    u, v = rng.integers(0, n, m), rng.integers(0, n, m)
+    if skew == 2:
+        u[: m // 4] = 0
+    k = u != v
+    pair = np.unique(np.minimum(u, v)[k] * n + np.maximum(u, v)[k])
+    u, v = pair // n, pair % n
+    w = rng.integers(1, 40, len(u))
+    src, dst, ww = np.concatenate([u, v]), np.concatenate([v, u]), np.concatenate([w, w])
+    order = np.argsort(src * n + dst, kind="stable")
+    src, dst, ww = src[order], dst[order], ww[order]
+    rp = np.zeros(n + 1, np.int64)
+    rp[1:] = np.cumsum(np.bincount(src, minlength=n))
+    g = synth.Graph(n, rp, dst.astype(np.int32), ww.astype(np.int32), {})
+    labels = rng.integers(0, n2, n).astype(np.int32) if not skew else \
+        np.where(rng.random(n) < 0.6, 0, rng.integers(0, n2, n)).astype(np.int32)
+    key = labels[src].astype(np.int64) * n2 + labels[dst]
+    keep = labels[src] != labels[dst]
+    uniq, inv = np.unique(key[keep], return_inverse=True)
+    sums = np.zeros(len(uniq), np.int64)
+    np.add.at(sums, inv, ww[keep])
+    m2, rp_out, col_out, w_out = _call(g, labels, n2)
+    assert m2 == len(uniq)
+    assert np.array_equal(rp_out[1:], np.cumsum(np.bincount(uniq // n2, minlength=n2)))
+    assert np.array_equal(col_out, uniq % n2) and np.array_equal(w_out, sums)
