@@ -629,15 +629,17 @@ int contract_current(mincut_graph* g, int* n2_out, long long* m2_out, bool compo
     int rc = ensure_rows(g);
     if (rc) return rc;
     ProfScope ps(P_UF, n, s);
-    CK(rows_classify(n, n, g->crp(), g->L, g->rows, s, &g->launches));
-    CK(rows_dense_mark(n, &g->st->n_next, g->rows, s, &g->launches));
+    CK(rows_classify(n, n, &g->st->n_next, matrix_limit(M), g->crp(), g->L, g->rows, s,
+                     &g->launches));
+    CK(rows_dense_mark(n, &g->st->n_next, matrix_limit(M), g->rows, s, &g->launches));
   }
   int rc = sync_state(g);
   if (rc) return rc;
   const int n2 = g->hst->n_next;
   const int nxt = g->cur == 0 ? 1 : 0;
+  const bool matrix = try_rows && (long long)n2 * n2 <= matrix_limit(M);
   bool rowwise = false;
-  if (try_rows && n2 > 1) {
+  if (try_rows && n2 > 1 && !matrix) {
     rowwise = 4 * (long long)(g->hst->single_entries + g->hst->dense_entries) >= M;
     if (rowwise) {
       // the dense accumulators this round uses must be zero: slots below
@@ -653,7 +655,18 @@ int contract_current(mincut_graph* g, int* n2_out, long long* m2_out, bool compo
     }
   }
   long long m2 = 0;
-  if (rowwise) {
+  if (matrix) {
+    { ProfScope ps(P_EMIT, M, s);
+      CK(matrix_contract<WT>(n, M, n2, g->crp(), g->ccol(), (const WT*)g->cw(), g->L, g->tile_row,
+                             g->keys[0], g->rp[nxt], g->col[nxt], (WT*)g->w[nxt],
+                             (WT*)g->degb[nxt], &g->st->m_rows, s, &g->launches)); }
+    m2 = -1;
+    if (!defer_m) {
+      rc = sync_state(g);
+      if (rc) return rc;
+      m2 = g->hst->m_rows;
+    }
+  } else if (rowwise) {
     rc = contract_rows<WT>(g, n2, nxt, &m2, defer_m);
     if (rc) return rc;
   } else {
@@ -1321,7 +1334,6 @@ int contract_round_impl(mincut_graph* g, const mincut_round_options* ro,
   if (rc) return rc;
   const int n = g->n;
   if (ro->groups || ro->pair_u) {
-    CK(uf_init(g->parent, n, s, &g->launches));
     CK(tile_rows(g->crp(), n, g->M, g->tile_row, s, &g->launches));
     if (ro->groups) {
       int* gd = g->flags;  // n ints; consumed before uf_relabel reuses them
@@ -1329,6 +1341,7 @@ int contract_round_impl(mincut_graph* g, const mincut_round_options* ro,
       CK(uf_from_groups(g->parent, gd, g->gmin, n, g->st, s, &g->launches));
     } else {
       if (ro->npairs < 0 || ro->npairs > g->Mraw) return fail(MINCUT_ERR_INVALID, "npairs");
+      CK(uf_init(g->parent, n, s, &g->launches));
       int* pu = reinterpret_cast<int*>(g->keys[1]);
       int* pv = pu + ro->npairs;
       if (ro->npairs > 0) {
@@ -1337,8 +1350,8 @@ int contract_round_impl(mincut_graph* g, const mincut_round_options* ro,
       }
       CK(uf_hook_pairs(g->parent, pu, pv, ro->npairs, n, g->st, s, &g->launches));
     }
-    rc = sync_state(g);
-    if (rc) return rc;
+    // (a group or pair out of range is skipped there, and refused at the
+    // contraction's first synchronisation, before anything of the graph changes)
     int n2;
     long long m2;
     rc = contract_current<WT>(g, &n2, &m2, false);

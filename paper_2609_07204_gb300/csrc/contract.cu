@@ -41,7 +41,27 @@ constexpr int kMovedBit = (int)0x80000000u;  // vinfo: neighbour's group has sev
 __device__ __forceinline__ unsigned sr_hash(int l) { return (unsigned)l * 0x9E3779B1u; }
 
 // cnt[L[x]] += 1 for every vertex (one atomic per distinct label of a warp).
-__global__ void group_count_kernel(const int* __restrict__ L, int n, int* __restrict__ cnt) {
+// The row classification's counters, in one launch.
+__global__ void rows_clear_kernel(int n, const int* __restrict__ n2p, long long mat_limit,
+                                  int* __restrict__ cnt, int* __restrict__ gen,
+                                  int* __restrict__ dsum, unsigned long long* single_entries,
+                                  unsigned long long* dense_entries, int* ndense) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *single_entries = 0;
+    *dense_entries = 0;
+    *ndense = 0;
+  }
+  if ((long long)*n2p * *n2p <= mat_limit) return;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    cnt[i] = 0;
+    gen[i] = 0;
+    dsum[i] = 0;
+  }
+}
+
+__global__ void group_count_kernel(const int* __restrict__ L, int n, const int* __restrict__ n2p,
+                                   long long mat_limit, int* __restrict__ cnt) {
+  if ((long long)*n2p * *n2p <= mat_limit) return;
   const int lane = threadIdx.x & 31;
   for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
     const int x = base + threadIdx.x;
@@ -57,7 +77,9 @@ __global__ void group_count_kernel(const int* __restrict__ L, int n, int* __rest
 __global__ void single_entries_kernel(const int64_t* __restrict__ rp, const int* __restrict__ L,
                                       int n, const int* __restrict__ cnt, int* __restrict__ gen,
                                       int* __restrict__ vinfo, int* __restrict__ rep,
-                                      int* __restrict__ dsum, unsigned long long* single_entries) {
+                                      int* __restrict__ dsum, unsigned long long* single_entries,
+                                      const int* __restrict__ n2p, long long mat_limit) {
+  if ((long long)*n2p * *n2p <= mat_limit) return;
   unsigned long long s = 0;
   const int lane = threadIdx.x & 31;
   for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
@@ -92,12 +114,13 @@ __global__ void single_entries_kernel(const int64_t* __restrict__ rp, const int*
 // n2 is read on the device (the union-find relabel's vertex count), so the
 // decision needs no synchronisation of its own; the capacity is
 // dense_capacity(n2): min(n2, dense_slots / n2).
-__global__ void dense_mark_kernel(const int* __restrict__ n2p, long long dense_slots,
+__global__ void dense_mark_kernel(const int* __restrict__ n2p, long long mat_limit,
+                                  long long dense_slots,
                                   const int* __restrict__ dsum, int* __restrict__ gen,
                                   int* __restrict__ did, int* ndense,
                                   unsigned long long* dense_entries) {
   const int n2 = *n2p;
-  if (n2 <= 1) return;
+  if (n2 <= 1 || (long long)n2 * n2 <= mat_limit) return;
   const int max_dense = (int)min((long long)n2, dense_slots / n2);
   if (max_dense <= 0) return;
   const int thr = max(n2 / 16, 256);
@@ -1197,16 +1220,16 @@ __global__ void fr_moved_kernel(int n, const int64_t* __restrict__ rp,
 
 }  // namespace
 
-cudaError_t rows_classify(int n, int n2, const int64_t* rp, const int* L, const RowScratch& rs,
-                          cudaStream_t s, int* launches) {
-  cudaMemsetAsync(rs.cnt, 0, (size_t)n2 * sizeof(int), s);
-  cudaMemsetAsync(rs.gen, 0, (size_t)n2 * sizeof(int), s);
-  cudaMemsetAsync(rs.single_entries, 0, sizeof(unsigned long long), s);
-  cudaMemsetAsync(rs.dsum, 0, (size_t)n2 * sizeof(int), s);
-  group_count_kernel<<<grid_blocks(n, 256), 256, 0, s>>>(L, n, rs.cnt);
+cudaError_t rows_classify(int n, int n2, const int* n2_dev, long long mat_limit, const int64_t* rp,
+                          const int* L, const RowScratch& rs, cudaStream_t s, int* launches) {
+  rows_clear_kernel<<<grid_blocks(n2, 256), 256, 0, s>>>(n2, n2_dev, mat_limit, rs.cnt, rs.gen,
+                                                         rs.dsum, rs.single_entries,
+                                                         rs.dense_entries, rs.ndense);
+  group_count_kernel<<<grid_blocks(n, 256), 256, 0, s>>>(L, n, n2_dev, mat_limit, rs.cnt);
   single_entries_kernel<<<grid_blocks(n, 256), 256, 0, s>>>(rp, L, n, rs.cnt, rs.gen, rs.vinfo,
-                                                            rs.rep, rs.dsum, rs.single_entries);
-  *launches += 2;
+                                                            rs.rep, rs.dsum, rs.single_entries, n2_dev,
+                                                            mat_limit);
+  *launches += 3;
   return cudaGetLastError();
 }
 
@@ -1214,12 +1237,10 @@ int dense_capacity(int n2, const RowScratch& rs) {
   return (int)std::min<long long>(n2, rs.dense_slots / std::max(n2, 1));
 }
 
-cudaError_t rows_dense_mark(int n_bound, const int* n2_dev, const RowScratch& rs, cudaStream_t s,
-                            int* launches) {
-  cudaMemsetAsync(rs.ndense, 0, sizeof(int), s);
-  cudaMemsetAsync(rs.dense_entries, 0, sizeof(unsigned long long), s);
+cudaError_t rows_dense_mark(int n_bound, const int* n2_dev, long long mat_limit,
+                            const RowScratch& rs, cudaStream_t s, int* launches) {
   dense_mark_kernel<<<grid_blocks(n_bound, 256), 256, 0, s>>>(
-      n2_dev, rs.dense_slots, rs.dsum, rs.gen, rs.did, rs.ndense, rs.dense_entries);
+      n2_dev, mat_limit, rs.dense_slots, rs.dsum, rs.gen, rs.did, rs.ndense, rs.dense_entries);
   ++*launches;
   return cudaGetLastError();
 }
