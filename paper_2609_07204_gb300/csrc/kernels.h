@@ -490,7 +490,7 @@ cudaError_t rows_dense_mark(int n_bound, const int* n2_dev, long long mat_limit,
 // groups, this form and the row-wise or sorted one (us): 3 K entries to 52
 // 91 / 191; 320 K to 563 123 / 247; 4.8 M to 2,188 206 / 431; 24 M to 4,896
 // 487 / 1,088; with few or uneven groups the gap is wider (24 M to 2: 576 /
-// 7,515).  Beyond it the triangle would not fit the scratch of 64-bit weights.
+// 7,515).
 long long matrix_limit(long long M);
 template <typename WT>
 cudaError_t matrix_contract(int n, long long M, int n2, const int64_t* rp, const int* col,

@@ -4,12 +4,13 @@
 // left of a large graph after its first rounds).
 //
 // A round is the degree bound, the certificate forests of forest.cu (same
-// certificate, same batches of highest r; the union-finds are in shared memory) and the contraction.  The graph is a list of undirected
-// edges (both ends in one word, and the weight): a round relabels the ends and
-// drops the loops, and that is all of the contraction -- the forests take
-// parallel edges as they come, so nothing is sorted or summed.  Every pass of
-// a round is a stream over that list; an edge is inserted in the batch that
-// scans its first end.
+// certificate, same batches of highest r; the union-finds are in shared
+// memory) and the contraction.  The graph is a list of undirected edges (both
+// ends in one word, and the weight): a round relabels the ends and drops the
+// loops, and that is all of the contraction -- the forests take parallel edges
+// as they come, so nothing is sorted or summed.  Every pass of a round is a
+// stream over that list; an edge is inserted in the batch that scans its first
+// end.
 //
 // A round that joins nothing and lowers nothing first drops the soft quantum
 // (weights in units of up to half their mean, for few levels), then leaves the
@@ -24,8 +25,8 @@
 // n x levels of them per round) and by block barriers (7-10 batches per round),
 // against one dependent visit per vertex (~0.8 us) of the one-warp solver and
 // the whole-graph passes.  Measured (whole calls, one GB300): G(2000, 16000)
-// 2.16 -> 0.51 ms, a 256-vertex graph created and solved 0.84 -> 0.29 ms,
-// 4,096 graphs (6.3 M edges) 5.44 -> 2.32 ms, 64 served requests 125 -> 75 ms.
+// 2.16 -> 0.42 ms, a 256-vertex graph created and solved 0.90 -> 0.21 ms,
+// 4,096 graphs (6.3 M edges) 5.44 -> 1.64 ms.
 #include <algorithm>
 #include <climits>
 
@@ -39,7 +40,7 @@ namespace {
 constexpr int kSmMaxK = 254;
 constexpr int kSmUnroll = 4;    // edges per lane loaded ahead
 constexpr int kSmLevels = 6;    // levels wanted (soft quantum)
-constexpr int kSmFast = 8;      // levels of the register path
+constexpr int kSmFast = 8;      // levels inserted at once
 constexpr int kSmFrac = 4;      // a batch takes at least 1 / kSmFrac of the vertices left
 constexpr int kSmBatches = 32;  // from this batch on, everything left is one batch
 
@@ -78,9 +79,10 @@ template <int T>
 struct SmShared {
   unsigned long long red[T / 32];
   int warp_cnt[T / 32];
-  long long alpha;
+  long long part[T / 32];  // sum: the scanned set's cut weight (see sm_total)
   unsigned long long key;
   int cnt, item;
+  unsigned hist[T / 32][5];
   uint2 q[T / 32][64];
 };
 
@@ -139,6 +141,41 @@ __device__ __forceinline__ bool sm_join(int* F, int k, int x, int y) {
     }
     if (p < 0) vx = p;
     else x = sm_root(F, k, p, vx);
+  }
+}
+
+// At most kSmFast levels: a lane per (edge, level), 32 / k of the queued edges
+// {x, y | units} at a time.  Each lane compares the words of its level (paths
+// are short, so most joined levels show), then the lanes of an edge's first
+// `units` levels above the last one so joined link them: where y is alone
+// (fo_scanned), which is most, by one CAS, else by sm_join.  A lane per edge
+// that walked its levels in turn (sm_insert_fast) took ~8 K cycles a call at any
+// fill; 4,096 graphs took 2.15 ms with it and take 1.80 with this (1.64 with the
+// rest of the change), a G(2000, 16000) round of 32 warps, which is bound by
+// issue rather than by that latency, 200 and 255 us: so blocks of few warps and
+// rounds of few edges.
+__device__ __forceinline__ void sm_insert_wide(int* F, int k, int take, const uint2* q) {
+  const int lane = threadIdx.x & 31;
+  const int g = lane / k, i = lane - g * k;
+  const bool act = g < take;
+  const uint2 it = q[act ? g : 0];
+  const int x = it.x & 0xffff, y = it.x >> 16, units = (int)it.y;
+  const int a = *(volatile int*)&F[x * k + i], b = *(volatile int*)&F[y * k + i];
+  const int px = a < 0 ? x : a;
+  const unsigned field = ((1u << k) - 1u);
+  const int at = act ? g * k : 0;
+  const unsigned closed = __ballot_sync(FULL, act && px == (b < 0 ? y : b)) >> at & field;
+  int lo = 32 - __clz(closed), want = act ? min(units, k - lo) : 0;
+  bool alone = b == -1;
+  for (;;) {
+    bool ok = false;
+    if (i >= lo && i < lo + want)
+      ok = (alone && atomicCAS(&F[y * k + i], -1, px) == -1) || sm_join(F + i, k, x, y);
+    const int got = __popc(__ballot_sync(FULL, ok) >> at & field);
+    lo += want;  // units whose level was joined meanwhile go on above
+    want = max(0, min(want - got, k - lo));
+    if (!__any_sync(FULL, want > 0)) return;
+    alone = false;
   }
 }
 
@@ -269,6 +306,14 @@ __device__ __forceinline__ unsigned long long sm_min(unsigned long long v, SmSha
   return s.key;
 }
 
+// Sum of the warps' parts (each warp adds to its own: 64-bit atomics on one
+// shared word spin, ~2 K cycles a batch with 32 warps).
+template <int T>
+__device__ __forceinline__ long long sm_total(const SmShared<T>& s) {
+  const int lane = threadIdx.x & 31;
+  return warp_sum(lane < T / 32 ? s.part[lane] : 0ll);
+}
+
 // Unscanned vertices with at least t units.
 template <int T>
 __device__ __forceinline__ int sm_count(const SmMem& sm, int n, int t) {
@@ -278,6 +323,56 @@ __device__ __forceinline__ int sm_count(const SmMem& sm, int n, int t) {
     c += __syncthreads_count(v < n && sm.tag[v] == 0 && sm.r[v] >= t);
   }
   return c;
+}
+
+// The batch threshold at most kSmFast levels: the largest t that `need` of the
+// vertices left have (1 if none), 0 where no vertex left has a unit or `all`.
+// Returns the vertices left.  One pass and one barrier: each warp's counts per
+// key, 16 bits each (a graph has at most kSmMaxN vertices), added up by every
+// warp for itself.  The bisection over block-wide counts that more levels take
+// took 12 K cycles of each batch of a
+// G(2000, 16000) round, this 9 K (most of it the new tags); with the loads of
+// the edge list four at a time that solve went from 455 to 418 us.
+template <int T>
+__device__ __forceinline__ int sm_select(const SmMem& sm, SmShared<T>& s, int n, int k, bool all,
+                                         int& t) {
+  static_assert(kSmFast <= 9 && kSmMaxN < 65536, "counts per key");
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  unsigned long long h[3] = {0, 0, 0};
+  for (int v = threadIdx.x; v < n; v += T)
+    if (sm.tag[v] == 0) {
+      const int key = min(sm.r[v], k);
+      const unsigned long long one = 1ull << (16 * (key & 3));
+      if (key < 4) h[0] += one;
+      else if (key < 8) h[1] += one;
+      else h[2] += one;
+    }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const unsigned x = __reduce_add_sync(FULL, (unsigned)(h[i / 2] >> (32 * (i & 1))));
+    if (lane == 0) s.hist[wp][i] = x;
+  }
+  __syncthreads();
+  unsigned c[5];
+  int left = 0;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    c[i] = __reduce_add_sync(FULL, lane < T / 32 ? s.hist[lane][i] : 0u);
+    left += (int)(c[i] & 0xffff) + (int)(c[i] >> 16);
+  }
+  t = 0;
+  const int units = left - (int)(c[0] & 0xffff);  // vertices with any
+  if (units > 0 && !all) {
+    const int need = max(1, left / kSmFrac);
+    int have = 0;
+    t = 1;
+#pragma unroll
+    for (int key = 9; key >= 1; --key) {
+      have += (int)(c[key / 2] >> (16 * (key & 1)) & 0xffff);
+      if (have >= need) t = max(t, key);
+    }
+  }
+  return left;
 }
 
 // Lists the undirected edges of rows [v0, v0 + n) in `ed` (ends relative to
@@ -293,32 +388,48 @@ __device__ int sm_load(const SmMem& sm, SmShared<T>& s, const int64_t* rp, const
   if (tid == 0) s.cnt = 0;
   __syncthreads();
   const int M = srp[n];
-  for (int e0 = tid - lane; e0 < M; e0 += T) {
-    const int e = e0 + lane;
-    bool keep = false;
-    int u = 0, v = 0, c = 0;
-    if (e < M) {
-      v = col[base + e] - v0;
-      c = w[base + e];
-      int lo = 0, hi = n;  // u: the row with srp[u] <= e < srp[u + 1]
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (srp[mid] <= e) lo = mid;
-        else hi = mid;
-      }
-      u = lo;
-      keep = u < v;
+  // (kSmUnroll entries per lane at a time: their loads and row searches overlap)
+  for (int e0 = tid; e0 - lane < M; e0 += T * kSmUnroll) {
+    int u[kSmUnroll], v[kSmUnroll], c[kSmUnroll];
+    int lo[kSmUnroll], hi[kSmUnroll];
+#pragma unroll
+    for (int j = 0; j < kSmUnroll; ++j) {
+      const int e = e0 + j * T;
+      v[j] = e < M ? col[base + e] - v0 : -1;
+      c[j] = e < M ? w[base + e] : 0;
+      lo[j] = 0;
+      hi[j] = n;
     }
-    const unsigned bal = __ballot_sync(FULL, keep);
-    int at = 0;
-    if (lane == 0 && bal) at = atomicAdd(&s.cnt, __popc(bal));
-    at = __shfl_sync(FULL, at, 0);
-    if (keep) {
-      at += __popc(bal & lanemask_lt());
-      if (at < ecap) {
-        ed.ends[at] = (unsigned)u | ((unsigned)v << 16);
-        ed.w[at] = c;
+    // the row with srp[row] <= e < srp[row + 1]
+    for (int half = n; half > 1; half = (half + 1) >> 1) {
+#pragma unroll
+      for (int j = 0; j < kSmUnroll; ++j) {
+        const int mid = (lo[j] + hi[j]) >> 1;
+        if (hi[j] - lo[j] > 1) {
+          if (srp[mid] <= e0 + j * T) lo[j] = mid;
+          else hi[j] = mid;
+        }
       }
+    }
+    unsigned bal[kSmUnroll];
+    int cnt = 0;
+#pragma unroll
+    for (int j = 0; j < kSmUnroll; ++j) {
+      u[j] = lo[j];
+      bal[j] = __ballot_sync(FULL, u[j] < v[j]);
+      cnt += __popc(bal[j]);
+    }
+    int at = 0;
+    if (lane == 0 && cnt) at = atomicAdd(&s.cnt, cnt);
+    at = __shfl_sync(FULL, at, 0);
+#pragma unroll
+    for (int j = 0; j < kSmUnroll; ++j) {
+      const int o = at + __popc(bal[j] & lanemask_lt());
+      if (u[j] < v[j] && o < ecap) {
+        ed.ends[o] = (unsigned)u[j] | ((unsigned)v[j] << 16);
+        ed.w[o] = c[j];
+      }
+      at += __popc(bal[j]);
     }
   }
   __syncthreads();
@@ -343,7 +454,6 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     const SmEdges ed = cur ? ed1 : ed0;
     // ---- degree bound
     for (int v = tid; v < n; v += T) sm.deg[v] = 0;
-    if (tid == 0) s.alpha = 0;
     __syncthreads();
     long long wsum = 0;
     for (int e = tid; e < m; e += T) {
@@ -354,8 +464,9 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
       wsum += c;
     }
     wsum = warp_sum(wsum);
-    if (lane == 0 && wsum) atomicAdd(reinterpret_cast<unsigned long long*>(&s.alpha), (unsigned long long)wsum);
+    if (lane == 0) s.part[wp] = wsum;
     __syncthreads();
+    wsum = sm_total<T>(s);
     unsigned long long best = ~0ull;
     for (int v = tid; v < n; v += T)
       best = min(best, ((unsigned long long)(unsigned)sm.deg[v] << 32) | (unsigned)v);
@@ -371,7 +482,7 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
       break;
     }
     ++rounds;
-    const long long mean = s.alpha / max(m, 1);
+    const long long mean = wsum / max(m, 1);
     const int kcap = min(kSmMaxK, sm.fcap / n);
     if (kcap < 1) break;
     const long long qmin = (lam + kcap - 1) / kcap;
@@ -380,14 +491,17 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     const long long qw = max(qmin, soft ? min((mean + 1) / 2, (lam + kSmLevels - 1) / kSmLevels) : 1ll);
     const int q = (int)qw;  // (at most the bound, a degree)
     const int k = (int)((lam + qw - 1) / qw);
-    __syncthreads();  // (s.alpha is read above)
+    __syncthreads();  // (the parts are read above)
+    const bool fast = k <= kSmFast;
+    const bool wide = fast && (T <= 256 || m <= T);
+    const int group = wide ? 32 / k : 32;  // edges inserted together
     // ---- all roots, nothing scanned, the first batch is vertex 0
     for (int i = tid; i < n * k; i += T) sm.F[i] = i < k ? -2 : -1;
     for (int v = tid; v < n; v += T) {
       sm.r[v] = 0;
       sm.tag[v] = v == 0 ? 1 : 0;
     }
-    if (tid == 0) s.alpha = sm.deg[0];
+    if (lane == 0) s.part[wp] = wp == 0 ? sm.deg[0] : 0;
     __syncthreads();
     long long best_alpha = kInf;
     int best_batch = 0;
@@ -396,19 +510,23 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
         // the largest t that takes 1 / kSmFrac of the vertices left, by
         // bisection over block-wide counts (a shared histogram would serialise
         // its few hot words); t = 1 where the queue is smaller than that
-        const int left = sm_count<T>(sm, n, 0);
-        int t = 0;
-        if (left > 0 && b < kSmBatches && sm_count<T>(sm, n, 1) > 0) {
-          const int need = max(1, left / kSmFrac);
-          int lo = 1, hi = k;
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (sm_count<T>(sm, n, mid) >= need) lo = mid;
-            else hi = mid - 1;
+        int t = 0, left;
+        if (fast) {
+          left = sm_select<T>(sm, s, n, k, b >= kSmBatches, t);
+        } else {
+          left = sm_count<T>(sm, n, 0);
+          if (left > 0 && b < kSmBatches && sm_count<T>(sm, n, 1) > 0) {
+            const int need = max(1, left / kSmFrac);
+            int lo = 1, hi = k;
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (sm_count<T>(sm, n, mid) >= need) lo = mid;
+              else hi = mid - 1;
+            }
+            t = lo;
           }
-          t = lo;
         }
-        const long long al = s.alpha;
+        const long long al = sm_total<T>(s);
         if (left > 0 && al < best_alpha) {
           best_alpha = al;
           best_batch = b - 1;
@@ -427,66 +545,75 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
             }
           }
         add = warp_sum(add);
-        if (lane == 0 && add) atomicAdd(reinterpret_cast<unsigned long long*>(&s.alpha), (unsigned long long)add);
+        if (lane == 0) s.part[wp] += add;
         __syncthreads();
       }
       // ---- the edges whose first end is in this batch
       long long sub = 0;
       int qn = 0;
-      for (int e0 = wp * (32 * kSmUnroll); e0 < m || qn > 0; e0 += T * kSmUnroll) {
+      // few edges are dealt out one by one, so that every warp has some
+      const bool spread = m <= 2 * T;
+      for (int i0 = 0; i0 < m; i0 += T * kSmUnroll) {
+        const int e0 = i0 + (spread ? lane * (T / 32) + wp : wp * (32 * kSmUnroll) + lane);
+        const int stp = spread ? T : 32;
+        const bool last = i0 + T * kSmUnroll >= m;
         unsigned d[kSmUnroll];
+        int c[kSmUnroll];
+        bool keep[kSmUnroll];
+#pragma unroll
+        for (int j = 0; j < kSmUnroll; ++j) d[j] = e0 + j * stp < m ? ed.ends[e0 + j * stp] : 0u;
 #pragma unroll
         for (int j = 0; j < kSmUnroll; ++j) {
-          const int e = e0 + j * 32 + lane;
-          d[j] = e < m ? ed.ends[e] : 0u;
+          const int e = e0 + j * stp;
+          const int tu = sm.tag[d[j] & 0xffff], tv = sm.tag[d[j] >> 16];
+          const bool now = e < m && (tu == b || tv == b);
+          c[j] = now ? ed.w[e] : 0;
+          keep[j] = now && (tu == b || tu == 0) && (tv == b || tv == 0);
+          if (now && tu != 0 && tv != 0) sub += c[j];  // now inside the scanned set
+          if (tu != b) d[j] = d[j] >> 16 | d[j] << 16;  // x scanned, y the far end
         }
 #pragma unroll
         for (int j = 0; j < kSmUnroll; ++j) {
-          const int e = e0 + j * 32 + lane;
-          const int u = d[j] & 0xffff, v = d[j] >> 16;
-          const int tu = sm.tag[u], tv = sm.tag[v];
-          bool keep = false;
-          if (e < m && (tu == b || tv == b)) {
-            if (tu != 0 && tv != 0) sub += ed.w[e];  // now inside the scanned set
-            keep = (tu == b || tu == 0) && (tv == b || tv == 0);
+          const int units = !keep[j] ? 0 : min(k, q == 1 ? c[j] : c[j] / q);
+          const unsigned bal = __ballot_sync(FULL, units > 0);
+          if (units > 0) {
+            if (fast && sm.r[d[j] >> 16] < k) atomicAdd(&sm.r[d[j] >> 16], units);
+            s.q[wp][qn + __popc(bal & lanemask_lt())] = make_uint2(d[j], (unsigned)units);
           }
-          const unsigned bal = __ballot_sync(FULL, keep);
-          // x scanned, y the far end
-          if (keep)
-            s.q[wp][qn + __popc(bal & lanemask_lt())] =
-                make_uint2(tu == b ? d[j] : (unsigned)v | ((unsigned)u << 16), (unsigned)e);
           qn += __popc(bal);
-          const bool end = j == kSmUnroll - 1 && e0 + T * kSmUnroll >= m;  // the warp's last edges
-          if (qn < 32 && !(end && qn > 0)) continue;
-          do {
+          const bool end = j == kSmUnroll - 1 && last;  // the warp's last edges
+          while (qn >= group || (end && qn > 0)) {
             __syncwarp();
-            const int take = min(qn, 32);
+            const int take = min(qn, group);
             qn -= take;
-            int x = 0, y = 0, units = 0, lo = 0;
-            if (lane < take) {
-              const uint2 it = s.q[wp][qn + lane];
-              x = it.x & 0xffff;
-              y = it.x >> 16;
-              const int c = ed.w[it.y];
-              units = min(k, q == 1 ? c : c / q);
-              if (units > 0 && k <= kSmFast) {
-                if (sm.r[y] < k) atomicAdd(&sm.r[y], units);
-                sm_insert_fast(sm.F, k, x, y, units);
-              } else if (units > 0) {
-                int g = sm.r[y];
-                if (g < k) g = atomicAdd(&sm.r[y], units);
-                lo = sm_level(sm.F, k, x, y, min(g, k - 1));
-                if (lo == k) units = 0;
+            if (wide) {
+              sm_insert_wide(sm.F, k, take, &s.q[wp][qn]);
+            } else if (fast) {
+              if (lane < take) {
+                const uint2 it = s.q[wp][qn + lane];
+                sm_insert_fast(sm.F, k, it.x & 0xffff, it.x >> 16, (int)it.y);
               }
+            } else {
+              int x = 0, y = 0, u = 0, lo = 0;
+              if (lane < take) {
+                const uint2 it = s.q[wp][qn + lane];
+                x = it.x & 0xffff;
+                y = it.x >> 16;
+                u = (int)it.y;
+                int g = sm.r[y];
+                if (g < k) g = atomicAdd(&sm.r[y], u);
+                lo = sm_level(sm.F, k, x, y, min(g, k - 1));
+                if (lo == k) u = 0;
+              }
+              __syncwarp();
+              sm_insert(sm.F, k, x, y, lo, u);
             }
-            if (k <= kSmFast) continue;
             __syncwarp();
-            sm_insert(sm.F, k, x, y, lo, units);
-          } while (end && qn > 0);
+          }
         }
       }
       sub = warp_sum(sub);
-      if (lane == 0 && sub) atomicAdd(reinterpret_cast<unsigned long long*>(&s.alpha), (unsigned long long)(-2 * sub));
+      if (lane == 0) s.part[wp] -= 2 * sub;
       __syncthreads();
     }
     __syncthreads();

@@ -55,3 +55,28 @@ def test_heavy_and_light_weights():
         heavy = ((src + c[1]) % 7 == 0)
         w[heavy] *= 900_000  # by the sum of the ends: symmetric
         _check_solve(n, (c[0], c[1], w))
+
+
+@pytest.mark.parametrize("whi", [1, 3, 40])
+@pytest.mark.parametrize("n", [17, 200, 1023, 1500])
+def test_level_counts(n, whi):
+    """Least degrees from 2 to 12 (as many levels under unit weights, one lane
+    per edge and level up to 8, the general insertion beyond), with fewer edges
+    than a block's threads and with more; alone and as a batch."""
+    rng = np.random.default_rng(n + whi)
+    graphs = []
+    for k in range(1, 12):
+        d = k if n * k % 2 == 0 else k + 1
+        u = np.repeat(np.arange(n), (d + 1) // 2)
+        v = (u + np.tile(np.arange(1, (d + 1) // 2 + 1), n)) % n
+        x = rng.integers(0, n, 2 * n if k % 3 == 0 else 3)
+        y = rng.integers(0, n, len(x))
+        u, v = np.concatenate([u, x]), np.concatenate([v, y])
+        keep = u != v
+        pair = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
+        w = rng.integers(1, whi + 1, len(pair))
+        graphs.append((n, *canon(n, *G.from_edges(n, np.stack([pair // n, pair % n], 1), w))))
+    expect = [oracle.noi(*g)[0] for g in graphs]
+    for g, e in zip(graphs, expect):
+        _check_solve(g[0], g[1:], expect=e)
+    _check_batch(graphs, expect)
