@@ -75,6 +75,7 @@ constexpr int kFoPerThread = 32;  // entries per thread that a grid is sized for
                                   // the barriers dearer (2 x 2^15 cut: 3.7 ms, 4.0 with the
                                   // whole GPU) and keep other streams' solves waiting
 constexpr int kFoChunk = 64;      // entries of a row handled by one warp at a time
+constexpr int kFoOwnPieces = 4;  // pieces of a row that its own thread lists
 constexpr int kFoMaxK = 254;      // levels (histogram bins: k + 1)
 constexpr int kFoLevels = 8;      // levels wanted where the weights allow it (qsoft): fewer
                                   // unions, and on random weights 1..100 all of the joins
@@ -229,6 +230,20 @@ __device__ __forceinline__ void fo_scanned(int* F, int k, int v, long long len) 
   }
 }
 
+// atomicCAS where `on` (0 elsewhere), predicated: under a branch of its own each
+// of several waits for the one before (a batch of 2,392 edges of 25 units, 57 us
+// with branches, takes 30; one of 293,570 such edges 102 and 64).
+__device__ __forceinline__ int fo_cas_if(bool on, int* p, int old, int to) {
+  int r = 0;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %4, 0;\n\t"
+      "@q atom.relaxed.gpu.global.cas.b32 %0, [%1], %2, %3;\n\t}"
+      : "+r"(r)
+      : "l"(p), "r"(old), "r"(to), "r"((int)on)
+      : "memory");
+  return r;
+}
+
 // Insert `units` units of the edge {x, y}, level `guess` tried first; returns
 // the units inserted, or -1 if the last level joins x and y already.
 __device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units, int guess) {
@@ -268,15 +283,15 @@ __device__ __forceinline__ int fo_insert(int* F, int k, int x, int y, int units,
   int* py = F + (long long)y * k;
   while (lo < k && units > 0) {
     const int cnt = min(min(units, k - lo), 4);
-    int p[4];
+    int a[4], b[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      p[j] = 0;  // not -1: this level is left to fo_join
-      if (j < cnt) {
-        const int a = px[lo + j], b = py[lo + j];
-        if (b == -1) p[j] = atomicCAS(&py[lo + j], -1, a < 0 ? x : a);
-      }
+      a[j] = j < cnt ? px[lo + j] : 0;
+      b[j] = j < cnt ? py[lo + j] : 0;
     }
+    int p[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) p[j] = fo_cas_if(b[j] == -1, &py[lo + j], -1, a[j] < 0 ? x : a[j]);
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (j < cnt && (p[j] == -1 || fo_join(F + lo + j, k, x, y))) --units;
@@ -339,10 +354,22 @@ __device__ __noinline__ void fo_select(const FoArgs& a, int k, int b, int t, int
             if (tid == 0) *s_base = atomicAdd(&ctl->items, total);
             __syncthreads();
             unsigned at = *s_base + before + (unsigned)(incl - mine);
-            for (; take; take &= take - 1) {
+            // (a warp writes a long row's pieces together: by the row's own thread the
+            // 4,600 of a contracted vertex took 320 us, and the grid waited)
+            for (unsigned any = __ballot_sync(FULL, take != 0); any;
+                 any = __ballot_sync(FULL, take != 0)) {
               const int x = v + __ffs(take) - 1;
-              const int pieces = fo_pieces(a.rp[x + 1] - a.rp[x]);
-              for (int c = 0; c < pieces; ++c) __stcg(&a.items[at++], make_int2(x, c));
+              const int pieces = take ? fo_pieces(a.rp[x + 1] - a.rp[x]) : 0;
+              if (pieces <= kFoOwnPieces)
+                for (int c = 0; c < pieces; ++c) __stcg(&a.items[at + c], make_int2(x, c));
+              for (unsigned big = __ballot_sync(FULL, pieces > kFoOwnPieces); big; big &= big - 1) {
+                const int src = __ffs(big) - 1;
+                const int bx = __shfl_sync(FULL, x, src), bp = __shfl_sync(FULL, pieces, src);
+                const unsigned ba = __shfl_sync(FULL, at, src);
+                for (int c = lane; c < bp; c += 32) __stcg(&a.items[ba + c], make_int2(bx, c));
+              }
+              at += pieces;
+              take &= take - 1;
             }
           }
           __syncthreads();
@@ -377,8 +404,10 @@ __device__ __noinline__ void fo_collect(const FoArgs& a, int u, long long b, lon
   }
 }
 
+// (two blocks per SM, stated: without the 2 the compiler takes the same 64
+// registers and spills 664 bytes, with it 52)
 template <typename WT>
-__global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
+__global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   __shared__ int s_hist[256];   // this block's changes since the last flush
   __shared__ int s_all[256];
   __shared__ unsigned s_scan[kFoThreads / 32];
@@ -545,7 +574,9 @@ __global__ void __launch_bounds__(kFoThreads) forest_kernel(FoArgs a) {
     long long alpha = 0;
     int qn = 0;  // queued edges of this warp
     __syncthreads();
-    unsigned i0 = (unsigned)(blockIdx.x * (kFoThreads / 32) + wp) * per;
+    // (the first ones dealt over the blocks before the warps of a block: the few
+    // items of a small batch spread over the SMs, 39 of them 57 -> 53 us)
+    unsigned i0 = ((unsigned)wp * gridDim.x + blockIdx.x) * per;
     while (i0 < nitems || qn > 0) {
       int x = -1, len = 0;
       unsigned eb = 0;

@@ -96,3 +96,21 @@ def test_what_the_forests_leave(clusters, size, hub):
     perm = rng.permutation(n)
     c = canon(n, *G.from_edges(n, [(perm[a], perm[b]) for a, b in e], w))
     _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+
+
+@pytest.mark.parametrize("deg", [255, 256, 257, 1000, 2900])
+@pytest.mark.parametrize("w", [1, 300])
+def test_hub_in_a_batch(deg, w):
+    """A vertex whose row is listed by its own thread (up to four pieces of 64)
+    or by its warp, met inside the graph and not only as the first vertex; light
+    edges, and edges of many units at once."""
+    n = 3000
+    rng = np.random.default_rng(deg + w)
+    hub = 1234
+    spokes = rng.choice(np.setdiff1d(np.arange(n), [hub]), deg, replace=False)
+    e = [(i, (i + d) % n) for i in range(n) for d in (1, 2, 7)]
+    ww = [int(x) for x in rng.integers(1, 4, len(e))]
+    e += [(hub, int(v)) for v in spokes]
+    ww += [w] * deg
+    c = canon(n, *G.from_edges(n, e, ww))
+    _check_solve(n, c, expect=oracle.noi(n, *c)[0])
