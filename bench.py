@@ -57,6 +57,7 @@ METRIC = "exact min-cut edges/s & contraction HBM GB/s; batched solves/s, p50/p9
 ALG_BYTES = {
     "degree": 4,            # read w
     "pr_marks": 8,          # read col + w (PR1/PR2; PR3/PR4 row reads are extra)
+    "forest": 8,            # read col + w once
     "lp_sweep": 12,         # read col + w, gather one label
     "lp_bound": 12,         # read col + w, gather one label
     "capforest_passes": 8,  # read col + w once
@@ -88,6 +89,8 @@ LATENCY_BOUND = {
                      "load and a gather of its neighbours' keys); the HBM fraction is tiny by "
                      "construction",
     "capforest_passes": "latency-bound: one chain of dependent pops per warp",
+    "forest": "latency-bound: per edge a chain of dependent union-find reads and "
+              "compare-and-swaps, in 7 to 40 grid-wide batches",
 }
 
 # Timed steps and end-to-end steps of each main-line workload by default

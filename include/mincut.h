@@ -180,8 +180,8 @@ void mincut_default_round_options(mincut_round_options* ro);
  * triples (an asymmetric input passes only on a collision); other inputs are
  * checked exactly after canonicalisation.  Sizes: n <= 2^31 - 2 and
  * M = row_ptr[n] <= 2^31 - 1 (MINCUT_ERR_OVERFLOW beyond, before any device
- * work); in practice device memory bounds them first (about 208 bytes per
- * vertex and 126 per entry, mincut_graph_footprint). */
+ * work); in practice device memory bounds them first (about 221 bytes per
+ * vertex and 127 per entry, mincut_graph_footprint). */
 int mincut_graph_from_csr(int64_t n, const int64_t* row_ptr, const int32_t* col,
                           const int32_t* w, uint32_t flags, void* cuda_stream,
                           const mincut_allocator* alloc, mincut_graph** out);
@@ -191,7 +191,15 @@ int mincut_graph_from_csr(int64_t n, const int64_t* row_ptr, const int32_t* col,
  * words): bit v (word v/64, bit v%64) is 1 iff vertex v is on the side of a
  * minimum cut that does not contain vertex 0; both sides are non-empty.
  * stats is nullable.  Starts from the input graph (solve does not consume
- * the rounds run by mincut_contract_round). */
+ * the rounds run by mincut_contract_round).
+ * A round's marks come from certificate forests of the whole graph (edges of a
+ * Nagamochi-Ibaraki decomposition; their prefix cuts lower the bound, too:
+ * lambda_source 3, joins counted in marks_cf) and, where those join few
+ * vertices, from label propagation, PR1..PR4 and CAPFOREST; graphs of at most
+ * 2048 vertices and 2^17 entries (total weight below 2^31), the input or what
+ * is left of it, are solved by one thread block.  Any of deterministic,
+ * seq_kernel, seq_passes, cf_visit, max_rounds and lp_every_round other than 0
+ * asks for the rounds without either. */
 int mincut_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut_value,
                  uint64_t* side_bitmap, mincut_stats* stats);
 
@@ -296,8 +304,9 @@ int mincut_contract_csr_noalloc(int64_t n, const int64_t* row_ptr, const int32_t
                                 int32_t* w_out, int64_t* m_out, void* cuda_stream);
 
 /* Estimated peak device bytes of one graph with n vertices and m_directed
- * CSR entries (creation, a solve with label propagation, total weight below
- * 2^31); used by the server's admission control. */
+ * CSR entries (creation, a solve with certificate forests and label
+ * propagation, total weight below 2^31); used by the server's admission
+ * control. */
 int64_t mincut_graph_footprint(int64_t n, int64_t m_directed);
 
 /* Graphs created without a user allocator take device memory from a pool per

@@ -398,7 +398,8 @@ bool galloc(mincut_graph* g, T** out, long long count) {
 // The buffers that `allocate` asks for (galloc / dev_alloc calls, the same on
 // every run) as one allocation: a stream-ordered allocation and its release
 // cost ~2 us, and a graph has some 80 buffers.  dev_free does nothing for a
-// buffer of a slab but its first, which is the slab.
+// buffer of a slab but its first, which is the slab.  Where no single block of
+// the whole size is to be had they are allocated one by one.
 template <typename F>
 bool in_slab(mincut_graph* g, F allocate) {
   g->counting = true;
@@ -407,7 +408,7 @@ bool in_slab(mincut_graph* g, F allocate) {
   g->counting = false;
   const size_t total = g->counted;
   void* p = dev_alloc(g, total);
-  if (!p) return false;
+  if (!p) return allocate();
   g->slab = static_cast<unsigned char*>(p);
   g->slab_left = total;
   const bool ok = allocate();
@@ -532,6 +533,9 @@ int ensure_forest(mincut_graph* g) {
                galloc(g, &g->fo_items, forest_item_cap(g->n0, g->M0)) &&
                galloc(g, &g->fo_ctl, (long long)forest_ctl_bytes());
       })) {
+    if (g->fo_tag) dev_free(g, g->fo_tag);
+    if (g->fo_r) dev_free(g, g->fo_r);
+    if (g->fo_items) dev_free(g, g->fo_items);
     g->fo_ctl = nullptr;
     return fail(MINCUT_ERR_OOM, "forest buffers");
   }
@@ -1144,7 +1148,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     c.skip_concurrent = skip_cc && g->n <= kSkipConcurrentMaxN;
     c.eager_seq = c.skip_concurrent && barely;
     c.cc_skip_pr = cc_low && c.capforest == 1 && op.cf_visit != 2 ? (g->n + 63) / 64 : -1;
-    c.forest = forests && g->n < forest_below;
+    // (without room for their buffers the round does without them)
+    c.forest = forests && g->n < forest_below && ensure_forest(g) == MINCUT_OK;
     c.small_rest = c.forest && small_below == INT_MAX;
     c.lp_now = lp_allowed && (op.lp_every_round || !lp_done);
     c.passes = op.passes > 0 ? op.passes : std::max(32, std::min(g->max_passes, g->n / 4));
@@ -1627,7 +1632,8 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
     }
   }
   cudaStreamSynchronize(s);
-  dev_free(g, rp_raw);  // (and col_raw with it)
+  dev_free(g, rp_raw);  // (and col_raw with it, where they are one block)
+  dev_free(g, col_raw);
   dev_free(g, w_raw);
   int rc = g->wt64 ? canonicalize_input<int64_t>(g, n, Mraw, validate)
                    : canonicalize_input<int32_t>(g, n, Mraw, validate);
@@ -2046,9 +2052,9 @@ int64_t mincut_graph_footprint(int64_t n, int64_t m_directed) {
   cudaGetLastError();
   const long long P = graph_max_passes(n, sms);
   // 8-byte weights and sums double the weight terms; this bound assumes
-  // 4-byte ones (total weight < 2^31) plus the label-propagation and the
-  // row-wise contraction buffers
-  return (int64_t)(208 * n + 126 * m_directed + 4096 * P + (1 << 20));
+  // 4-byte ones (total weight < 2^31) plus the label-propagation, the row-wise
+  // contraction and the certificate forests' buffers
+  return (int64_t)(221 * n + 127 * m_directed + 4096 * P + (1 << 20));
 }
 
 int mincut_batch_from_csr(int64_t num_graphs, const int64_t* vertex_offsets,

@@ -114,3 +114,46 @@ def test_hub_in_a_batch(deg, w):
     ww += [w] * deg
     c = canon(n, *G.from_edges(n, e, ww))
     _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+
+
+@pytest.mark.parametrize("refused", [1, 2, 3])
+def test_allocations_refused(refused, monkeypatch):
+    """The first requests of a solve refused by the caller's allocator: buffers
+    that come as one block are asked for one by one, and a round without room
+    for the forests does without them."""
+    class Refusing(mc._TorchAllocator):
+        def __init__(self, device):
+            super().__init__(device)
+            self.refuse = 0
+            give = self._alloc
+
+            def _alloc(nbytes, stream, ctx):
+                if self.refuse > 0:
+                    self.refuse -= 1
+                    return None
+                return give(nbytes, stream, ctx)
+
+            self._give, self._alloc = give, type(give)(_alloc)
+            self.struct = mc.MincutAllocator(self._alloc, self._free, None)
+
+    monkeypatch.setattr(mc, "_TorchAllocator", Refusing)
+    n = 3000
+    rng = np.random.default_rng(refused)
+    g = G.random_graph(n, 10.0 / n, rng, 1, 20, connected=True)
+    c = canon(n, *g)
+    dev = [mc_dev(x) for x in (np.asarray(c[0], np.int64), np.asarray(c[1], np.int32),
+                               np.asarray(c[2], np.int32))]
+    h = mc.mincut_graph_from_csr(n, *dev, use_torch_allocator=True)
+    expect = oracle.noi(n, *c)[0]
+    for _ in range(2):
+        h._allocator.refuse = refused
+        value, bitmap, _ = mc.mincut_solve(h)
+        h._allocator.refuse = 0
+        side = mc.bitmap_to_side(bitmap, n)
+        assert value == expect and oracle.cut_weight(n, *c, side) == expect
+    h.destroy()
+
+
+def mc_dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
