@@ -17,7 +17,11 @@ namespace mc {
 namespace {
 
 constexpr int kMatThreads = 256;
-constexpr int kMatShared = 32768;  // bytes of a block's own triangles
+// Bytes of a block's own triangles: what the default 48 KB leave beside the
+// tile's rows (16,416 bytes), in whole 256.
+constexpr int kMatShared = (48 * 1024 - (int)sizeof(TileRowsSmem)) / 256 * 256;
+static_assert(kMatShared >= 32000 && kMatShared + sizeof(TileRowsSmem) <= 48 * 1024,
+              "own triangles and tile rows share a block's default shared memory");
 constexpr size_t kMatHead = 256;   // the ticket, then the row counts
 
 __device__ __forceinline__ int tri(int i, int j) {  // i < j
@@ -233,6 +237,7 @@ cudaError_t matrix_contract(int n, long long M, int n2, const int64_t* rp, const
     mat_acc_kernel<WT><<<grid, kETThreads, (size_t)cells * copies * sizeof(WT), s>>>(
         n, M, rp, col, w, L, tile_row, ntiles, cells, copies, mat);
     ++*launches;
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
   mat_count_kernel<WT><<<n2, kMatThreads, 0, s>>>(n2, mat, ticket, cnt, rp2, deg2, total);
   mat_write_kernel<WT><<<n2, kMatThreads, 0, s>>>(n2, mat, rp2, col2, w2);

@@ -49,6 +49,27 @@ def test_contract_to_few_vertices(n, m, whi, n2, skew):
     g.destroy()
 
 
+@pytest.mark.parametrize("whi", [1, 4000])
+def test_own_triangles_of_many_tiles(whi):
+    """Enough entries that a block sums several tiles in triangles of its own:
+    the vertex counts around which the copies that fit beside the tile's rows
+    change (91: one copy fewer, or none), 32-bit and 64-bit totals."""
+    n, m = 200_000, 5_100_000
+    g0 = synth.er(n, m, 1, whi, 5)
+    g = make(n, g0.row_ptr, g0.col, g0.w)
+    rng = np.random.default_rng(whi)
+    for n2 in (90, 91, 92, 128, 129):
+        groups = rng.integers(0, n2, n).astype(np.int32)
+        groups[:n2] = np.arange(n2)
+        ro = mc.default_round_options()
+        ro.groups = groups.ctypes.data
+        mc.mincut_graph_reset(g)
+        assert mc.mincut_contract_round(g, ro)["n_out"] == n2
+        exp = oracle.contract(n, g0.row_ptr, g0.col, g0.w, oracle.labels_from_groups(groups)[1], n2)
+        assert_csr_equal(mc.mincut_graph_export_csr(g), exp)
+    g.destroy()
+
+
 def test_refused_groups_leave_the_graph():
     g0 = synth.er(5000, 60_000, 1, 9, 5)
     g = make(5000, g0.row_ptr, g0.col, g0.w)
