@@ -124,7 +124,7 @@ struct FoArgs {
   FoCtl* ctl;
   DevState* st;
   long long spin;
-  long long qsoft;     // quantum that loses little of the weights
+  long long qsoft;     // half the mean weight of the input
 };
 
 // A level's union-find, linked by rank: a root's word is -1 - rank, another's
@@ -376,6 +376,33 @@ __device__ __noinline__ void fo_select(const FoArgs& a, int k, int b, int t, int
         }
 }
 
+// The quantum that loses little of the weights: half the mean (`half`), and
+// where a typical weight (the median of a sample, the same in every block) is
+// larger, at most the part that divides it evenly.  Just above half of weights
+// that are nearly all alike, as half their mean is with a few heavier ones
+// among them, it drops half of each and the last level joins nothing: planted
+// cut 2 x 2^13 with weights of 10^5 (64-bit) 24.8 -> 2.4 ms.  Half the median
+// itself, smaller on weights with a long tail, is slower there (Pareto 1.2 on
+// that cut 1.5 -> 2.6 ms: more units to insert, the same joins).
+template <typename WT>
+__device__ __forceinline__ long long fo_quantum(const WT* __restrict__ w, long long M,
+                                                long long half, unsigned* s_scan) {
+  if (M <= 0) return half;
+  const int tid = threadIdx.x;
+  const unsigned long long x = (unsigned long long)w[tid * M / kFoThreads];
+  int bits = __reduce_max_sync(FULL, 64 - __clzll((long long)x));
+  if ((tid & 31) == 0) s_scan[tid >> 5] = (unsigned)bits;
+  __syncthreads();
+  for (int i = 0; i < kFoThreads / 32; ++i) bits = max(bits, (int)s_scan[i]);
+  // the largest value that half of the sample reaches, bit by bit
+  unsigned long long v = 0;
+  for (int b = bits - 1; b >= 0; --b)
+    if (__syncthreads_count(x >= (v | 1ull << b)) * 2 >= kFoThreads) v |= 1ull << b;
+  __syncthreads();
+  const long long typical = (long long)v;
+  return typical > half ? typical / ((typical + half - 1) / half) : half;
+}
+
 constexpr int kFoMatrix = 1024;  // labels that are summed in a matrix
 constexpr int kFoPiece = 512;    // entries of a long row that one warp lists
 
@@ -428,6 +455,7 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   const WT* __restrict__ deg = reinterpret_cast<const WT*>(a.deg);
   FoCtl* ctl = a.ctl;
   unsigned gen = 0;
+  const long long qsoft = fo_quantum<WT>(w, a.rp[n], a.qsoft, s_scan);
   // ---- degree bound (Sec. 2.1), and a clean round state
   const long long lam_in = (long long)*(volatile unsigned long long*)&a.st->lambda;
   unsigned long long dmin = ~0ull;
@@ -490,7 +518,7 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     return;
   }
   // (the quantum, like the bound, fits the weight type)
-  const WT q = (WT)max((lam + kcap - 1) / kcap, min(a.qsoft, (lam + kFoLevels - 1) / kFoLevels));
+  const WT q = (WT)max((lam + kcap - 1) / kcap, min(qsoft, (lam + kFoLevels - 1) / kFoLevels));
   const int k = (int)((lam + q - 1) / q);
   int* F = a.F;
   uint8_t* tag = a.tag;

@@ -59,6 +59,18 @@ def test_planted_cut_64bit_weights():
     big = (s.row_ptr, s.col, s.w.astype(np.int64) * 60_000)
     _check_solve(s.n, big, expect=lam * 60_000)
 
+@pytest.mark.parametrize("w", [3, 1000, 60_000])
+def test_weights_nearly_alike(w):
+    """Equal weights with a few heavier ones among them: half their mean lies
+    above half of most, which must not cost the forests half of each edge
+    (64-bit sums with the largest)."""
+    s = synth.planted(1 << 13, 21 << 13, 20, 25, 1, 3)
+    src = np.repeat(np.arange(s.n), np.diff(s.row_ptr))
+    ww = np.where((src + s.col) % 97 == 0, w + w // 2, w)  # by the sum of the ends: symmetric
+    c = (s.row_ptr, s.col, ww.astype(np.int64))
+    assert _check_solve(s.n, c, expect=oracle.noi(s.n, *c)[0])["seq_passes"] == 0
+
+
 @pytest.mark.parametrize("seed", range(3))
 def test_random_sparse_20000(seed):
     g = synth.er_connected(20_000, 100_000, 1, 30, 50 + seed)
