@@ -128,6 +128,51 @@ def test_hub_in_a_batch(deg, w):
     _check_solve(n, c, expect=oracle.noi(n, *c)[0])
 
 
+def _torus(a, b, w, rng):
+    i = np.arange(a * b).reshape(a, b)
+    e = np.concatenate([np.stack([i.ravel(), np.roll(i, -1, k).ravel()], 1) for k in (0, 1)])
+    return a * b, G.from_edges(a * b, e, [int(x) for x in rng.integers(1, w + 1, len(e))])
+
+
+def _ladder(n, w, rng):
+    i = np.arange(n)
+    j = (i + 1) % n
+    e = np.concatenate([np.stack([i, j], 1), np.stack([n + i, n + j], 1), np.stack([i, n + i], 1)])
+    return 2 * n, G.from_edges(2 * n, e, [int(x) for x in rng.integers(1, w + 1, len(e))])
+
+
+def _forest_ms(n, c, expect):
+    """Device time of the forest kernel in a default solve."""
+    _check_solve(n, c, expect=expect)
+    g = mc.mincut_graph_from_csr(n, *c)
+    mc.mincut_solve(g)
+    mc.mincut_solve(g, mc.default_options(profile=1))
+    prof = mc.mincut_profile_read(g)
+    g.destroy()
+    return prof["forest"]["ms"]
+
+
+@pytest.mark.parametrize("name,limit", [("torus", 1.0), ("ladder", 1.0), ("wheel", 0.7),
+                                        ("tree", 0.5)])
+def test_thin_frontiers(name, limit):
+    """Graphs on which a batch is a handful of vertices: the forests do not
+    take a hundred batches for them (1.6 ms and more; the tree 0.8)."""
+    rng = np.random.default_rng(5)
+    if name == "wheel":
+        s = synth.wheel(4097, seed=1)
+        n, g, expect = s.n, (s.row_ptr, s.col, s.w.astype(np.int64)), 8192
+    elif name == "tree":
+        n = 50_000
+        w = rng.integers(1, 51, n - 1)
+        p = rng.permutation(n)
+        e = np.stack([p[1:], p[(rng.random(n - 1) * np.arange(1, n)).astype(np.int64)]], 1)
+        g, expect = G.from_edges(n, e, [int(x) for x in w]), int(w.min())
+    else:
+        n, g = _torus(60, 60, 50, rng) if name == "torus" else _ladder(3000, 20, rng)
+        expect = oracle.noi(n, *canon(n, *g))[0]
+    assert _forest_ms(n, canon(n, *g), expect) < limit
+
+
 @pytest.mark.parametrize("refused", [1, 2, 3])
 def test_allocations_refused(refused, monkeypatch):
     """The first requests of a solve refused by the caller's allocator: buffers
