@@ -92,6 +92,16 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 // many places, is slower (that grid 1.41, 1.29 and 1.13).  With one level
 // there is no order to keep: a tree of 50,000 0.89 -> 0.29.
 constexpr int kFoThin = 512;
+// Vertices sampled, and entries of each; fewer than 1 / kFoAble of them with a
+// unit for every level: no batch is scanned (a wheel, whose spokes have no units
+// and whose rim edges have three for eight levels: 4,097 vertices 0.65 -> 0.36
+// ms, 40,001 0.91 -> 0.61; elsewhere no change, the sample is taken beside the clearing).
+// Not "more than a unit for every level", which would also spare a wheel of unit
+// weights: that gives up R-MAT graphs whose many leaves have just enough (scale
+// 18 with a cycle through all 2.4 -> 4.3 ms).
+constexpr int kFoSample = 512;
+constexpr int kFoSampleRow = 256;
+constexpr int kFoAble = 16;
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
 constexpr int kFoMaxBlocks = 1024;
@@ -101,6 +111,7 @@ struct FoCtl {
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
   int count;           // edges listed of what is left; INT_MAX: not listed
+  int able;            // sampled vertices that the last level can join
   unsigned pieces;     // pieces of long rows listed for that
   unsigned long long deg_inv;  // ~(minimum degree)
   int deg_arg_inv;     // INT_MAX - (its smallest vertex)
@@ -533,6 +544,18 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   int* F = a.F;
   uint8_t* tag = a.tag;
   int* ru = a.r;
+  // ---- a vertex that the last level joins has a unit in every level: where
+  // hardly any of a sample has as many, the forests would join next to nothing
+  for (int i = gtid >> 5; i < kFoSample; i += gsize >> 5) {
+    const int v = (int)((long long)i * n / kFoSample);
+    const long long rb = a.rp[v], re = min((long long)a.rp[v + 1], rb + kFoSampleRow);
+    int units = 0;
+    for (long long e0 = rb; e0 < re && units < k; e0 += 32) {
+      const WT c = e0 + lane < re ? w[e0 + lane] : WT(0);
+      units += __reduce_add_sync(FULL, (int)min((WT)k, q == 1 ? c : c / q));
+    }
+    if (lane == 0 && units >= k) atomicAdd(&ctl->able, 1);
+  }
   // ---- every vertex a root at every level, nothing scanned; the first batch
   // is vertex 0
   {
@@ -557,6 +580,14 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     }
   }
   if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
+  if (__ldcg(&ctl->able) * kFoAble < kFoSample) {
+    if (gtid == 0) {
+      a.st->deg_val = dmin;
+      a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
+      a.st->lambda = (unsigned long long)lam;
+    }
+    return;
+  }
   unsigned start = 0;
   int thin = 0, queued_before = 1;  // (of the thread that chooses the batch)
   int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root

@@ -173,6 +173,15 @@ def test_thin_frontiers(name, limit):
     assert _forest_ms(n, canon(n, *g), expect) < limit
 
 
+@pytest.mark.parametrize("n", [2050, 4097, 40_001])
+def test_nothing_to_join(n):
+    """A wheel's spokes have no units and its rim too few for the last level:
+    no batch is scanned (0.3 ms with)."""
+    s = synth.wheel(n, seed=1)
+    c = (s.row_ptr, s.col, s.w.astype(np.int64))
+    assert _forest_ms(n, c, 2 * (n - 2) + 2) < 0.15
+
+
 @pytest.mark.parametrize("refused", [1, 2, 3])
 def test_allocations_refused(refused, monkeypatch):
     """The first requests of a solve refused by the caller's allocator: buffers
