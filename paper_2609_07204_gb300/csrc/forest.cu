@@ -74,6 +74,15 @@ constexpr int kFoThreads = 512;
 constexpr int kFoPerThread = 32;  // entries per thread that a grid is sized for: more blocks make
                                   // the barriers dearer (2 x 2^15 cut: 3.7 ms, 4.0 with the
                                   // whole GPU) and keep other streams' solves waiting
+// Up to kFoFew blocks, whose barriers are cheap, are sized for kFoFewPerThread
+// entries a thread on graphs of at most kFoSparse entries per vertex, else one
+// block's while they are small: wheel of 4,097 and unit weights 523 -> 415 us
+// whole, torus of 60 x 60 656 -> 335, random n = 20,000 of degree 3 553 -> 390;
+// 16 blocks or 8 entries 0-10% slower.  Not on denser ones: more warps insert
+// more out of order, and a small planted cut (2 x 2^10) loses its joins (2.5 -> 3.1 ms).
+constexpr int kFoFewPerThread = 4;
+constexpr int kFoFew = 32;
+constexpr int kFoSparse = 8;
 constexpr int kFoChunk = 64;      // entries of a row handled by one warp at a time
 constexpr int kFoOwnPieces = 4;  // pieces of a row that its own thread lists
 constexpr int kFoMaxK = 254;      // levels (histogram bins: k + 1)
@@ -996,8 +1005,14 @@ cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64
   a.spin = spin;
   const long long want =
       (std::max<long long>(M, n) + kFoPerThread * kFoThreads - 1) / (kFoPerThread * kFoThreads);
+  const long long few =
+      M > (long long)kFoSparse * n
+          ? 1
+          : std::min<long long>(kFoFew,
+                                (std::max<long long>(M, n) + kFoFewPerThread * kFoThreads - 1) /
+                                    (kFoFewPerThread * kFoThreads));
   const int blocks = (int)std::max<long long>(
-      1, std::min<long long>({want, (long long)sms * per_sm[wi], (long long)kFoMaxBlocks}));
+      1, std::min<long long>({std::max(want, few), (long long)sms * per_sm[wi], (long long)kFoMaxBlocks}));
   void* params[] = {&a};
   e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
                                   params, 0, s);

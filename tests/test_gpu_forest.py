@@ -182,6 +182,30 @@ def test_nothing_to_join(n):
     assert _forest_ms(n, c, 2 * (n - 2) + 2) < 0.15
 
 
+def test_small_graphs_use_several_blocks():
+    """A wheel of unit weights, which the forests do not help: they stay cheap
+    (0.2 ms by one block)."""
+    s = synth.wheel(4097, seed=1)
+    c = (s.row_ptr, s.col, np.ones_like(s.w, dtype=np.int64))
+    assert _forest_ms(s.n, c, 3) < 0.15
+
+
+@pytest.mark.parametrize("m", [3071, 3072, 3073, 9999, 10_000, 10_001, 57_343, 57_344, 57_345])
+def test_block_counts(m):
+    """Entries around the numbers at which the kernel's grid changes (10,000
+    edges: eight entries per vertex)."""
+    n = 2500
+    rng = np.random.default_rng(m)
+    p = rng.permutation(n)  # a random cycle, then other pairs up to m
+    pair = np.minimum(p, np.roll(p, 1)) * n + np.maximum(p, np.roll(p, 1))
+    u, v = rng.integers(0, n, (2, 3 * m))
+    extra = np.setdiff1d((np.minimum(u, v) * n + np.maximum(u, v))[u != v], pair)
+    pair = np.concatenate([pair, rng.choice(extra, m - n, replace=False)])
+    c = canon(n, *G.from_edges(n, np.stack([pair // n, pair % n], 1), rng.integers(1, 10, m)))
+    assert c[0][-1] == 2 * m
+    _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+
+
 @pytest.mark.parametrize("refused", [1, 2, 3])
 def test_allocations_refused(refused, monkeypatch):
     """The first requests of a solve refused by the caller's allocator: buffers
