@@ -99,8 +99,12 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 // without forests), grid of 300 x 300 2.37 -> 0.86, wheel of 4,097 1.84 -> 0.65.
 // Scanning a 64th, a 16th or a quarter of the vertices first, to go on from
 // many places, is slower (that grid 1.41, 1.29 and 1.13).  With one level
-// there is no order to keep: a tree of 50,000 0.89 -> 0.29.
-constexpr int kFoThin = 512;
+// there is no order to keep: a tree of 50,000 0.89 -> 0.29.  A larger limit does
+// no more for these, whose frontiers are far below it, and ends the batching of
+// small planted cuts too early: of 2 x 2^12 vertices and minimum degree 30 the forests
+// join 0.09 instead of 0.2 with 512, and the whole-graph pass it then takes makes
+// the solve 7.4 ms instead of 2.9 (2 x 2^11 4.3 and 0.9, 256 the same).
+constexpr int kFoThin = 64;
 // Vertices sampled, and entries of each; fewer than 1 / kFoAble of them with a
 // unit for every level: no batch is scanned (a wheel, whose spokes have no units
 // and whose rim edges have three for eight levels: 4,097 vertices 0.65 -> 0.36

@@ -59,6 +59,18 @@ def test_planted_cut_64bit_weights():
     big = (s.row_ptr, s.col, s.w.astype(np.int64) * 60_000)
     _check_solve(s.n, big, expect=lam * 60_000)
 
+@pytest.mark.parametrize("log_nb,cross,seed", [(10, 9, 11), (11, 9, 5), (12, 25, 3)])
+def test_small_planted_cuts(log_nb, cross, seed):
+    """The forests join enough of them, in every round, that no whole-graph
+    pass runs."""
+    nb = 1 << log_nb
+    s = synth.planted(nb, 21 * nb, 30, cross, 1, seed)
+    c = (s.row_ptr, s.col, s.w.astype(np.int64))
+    lam = oracle.noi(s.n, *c)[0]
+    for _ in range(5):
+        assert _check_solve(s.n, c, expect=lam)["seq_passes"] == 0
+
+
 @pytest.mark.parametrize("w", [3, 1000, 60_000])
 def test_weights_nearly_alike(w):
     """Equal weights with a few heavier ones among them: half their mean lies
