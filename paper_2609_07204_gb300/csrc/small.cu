@@ -12,9 +12,9 @@
 // stream over that list; an edge is inserted in the batch that scans its first
 // end.
 //
-// A round that joins nothing and lowers nothing first drops the soft quantum
-// (weights in units of up to half their mean, for few levels), then leaves the
-// graph to the caller's other rounds (bail): Algorithm 2's progress guarantee
+// A round that joins next to nothing (kSmSlow) and lowers nothing first drops the
+// soft quantum (weights in units of up to half their mean, for few levels), then
+// leaves the graph to the caller's other rounds (bail): Algorithm 2's progress guarantee
 // needs an exact maximum-adjacency order.  Counted on the CPU on the batched
 // workload (n 20 to 2,000, average degree 3 to 12, weights 1 to 100): 6 levels
 // with PR1 / PR2 take 2.85 rounds per graph and no graph is left, 16 levels
@@ -42,6 +42,16 @@ constexpr int kSmUnroll = 4;    // edges per lane loaded ahead
 constexpr int kSmLevels = 6;    // levels wanted (soft quantum)
 constexpr int kSmFast = 8;      // levels inserted at once
 constexpr int kSmFrac = 4;      // a batch takes at least 1 / kSmFrac of the vertices left
+// Joining less than this a round is left to the other rounds, whose many
+// whole-graph passes join up to one vertex each: cycles whose weights are all
+// equal by now lose one vertex a round here (a cycle of 50,000 vertices with
+// weights of 1 to 100 57.4 -> 3.2 ms, a ring of 3,000 cliques of 8 141 -> 22; with
+// 1 / 32 a cycle of 5,000 4.3 instead of 2.8).
+constexpr int kSmSlow = 8;      // a round joins at least 1 / kSmSlow of the vertices,
+constexpr int kSmSlowMin = 64;  // of fewer than kSmSlowMin any
+constexpr int kSmThin = 32;     // twice in a row fewer vertices queued, and less than half as many
+                                // again as before: everything left is one batch (see kFoThin;
+                                // wheel of 1,025 766 -> 429 us, with both 380)
 constexpr int kSmBatches = 32;  // from this batch on, everything left is one batch
 
 // Shared memory of a block, for graphs of up to `cap` vertices.
@@ -327,7 +337,7 @@ __device__ __forceinline__ int sm_count(const SmMem& sm, int n, int t) {
 
 // The batch threshold at most kSmFast levels: the largest t that `need` of the
 // vertices left have (1 if none), 0 where no vertex left has a unit or `all`.
-// Returns the vertices left.  One pass and one barrier: each warp's counts per
+// Returns the vertices left; queued: those of them with any unit.  One pass and one barrier: each warp's counts per
 // key, 16 bits each (a graph has at most kSmMaxN vertices), added up by every
 // warp for itself.  The bisection over block-wide counts that more levels take
 // took 12 K cycles of each batch of a
@@ -335,7 +345,7 @@ __device__ __forceinline__ int sm_count(const SmMem& sm, int n, int t) {
 // the edge list four at a time that solve went from 455 to 418 us.
 template <int T>
 __device__ __forceinline__ int sm_select(const SmMem& sm, SmShared<T>& s, int n, int k, bool all,
-                                         int& t) {
+                                         int& t, int& queued) {
   static_assert(kSmFast <= 9 && kSmMaxN < 65536, "counts per key");
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   unsigned long long h[3] = {0, 0, 0};
@@ -361,8 +371,8 @@ __device__ __forceinline__ int sm_select(const SmMem& sm, SmShared<T>& s, int n,
     left += (int)(c[i] & 0xffff) + (int)(c[i] >> 16);
   }
   t = 0;
-  const int units = left - (int)(c[0] & 0xffff);  // vertices with any
-  if (units > 0 && !all) {
+  queued = left - (int)(c[0] & 0xffff);
+  if (queued > 0 && !all) {
     const int need = max(1, left / kSmFrac);
     int have = 0;
     t = 1;
@@ -504,6 +514,7 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     if (lane == 0) s.part[wp] = wp == 0 ? sm.deg[0] : 0;
     __syncthreads();
     long long best_alpha = kInf;
+    int thin = 0, queued_before = 1;
     int best_batch = 0;
     for (int b = 1;; ++b) {
       if (b > 1) {
@@ -511,11 +522,19 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
         // bisection over block-wide counts (a shared histogram would serialise
         // its few hot words); t = 1 where the queue is smaller than that
         int t = 0, left;
+        int queued;
         if (fast) {
-          left = sm_select<T>(sm, s, n, k, b >= kSmBatches, t);
+          left = sm_select<T>(sm, s, n, k, b >= kSmBatches, t, queued);
         } else {
           left = sm_count<T>(sm, n, 0);
-          if (left > 0 && b < kSmBatches && sm_count<T>(sm, n, 1) > 0) {
+          queued = sm_count<T>(sm, n, 1);
+        }
+        thin = queued < kSmThin && 2 * queued < 3 * queued_before ? thin + 1 : 0;
+        queued_before = queued;
+        if (thin >= 2) {
+          t = 0;
+        } else if (!fast) {
+          if (left > 0 && b < kSmBatches && queued > 0) {
             const int need = max(1, left / kSmFrac);
             int lo = 1, hi = k;
             while (lo < hi) {
@@ -661,14 +680,12 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
       n2 += total;
       __syncthreads();
     }
-    if (n2 == n) {
-      if (lowered) continue;  // again, from the lower bound
-      if (q > qmin) {
-        soft = false;
-        continue;
-      }
-      break;  // bail
+    if (!lowered && n - n2 < (n < kSmSlowMin ? 1 : n / kSmSlow)) {
+      // (a finer quantum does not help where a thin frontier and PR joined nothing)
+      if (!soft || q == qmin || (thin >= 2 && pr_mask && n2 == n)) break;  // bail
+      soft = false;
     }
+    if (n2 == n) continue;  // again, from the lower bound or with the finer quantum
     for (int v = tid; v < n; v += T) {
       int x = v;
       while (top[x * k] >= 0) x = top[x * k];

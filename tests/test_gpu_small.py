@@ -80,3 +80,36 @@ def test_level_counts(n, whi):
     for g, e in zip(graphs, expect):
         _check_solve(g[0], g[1:], expect=e)
     _check_batch(graphs, expect)
+
+
+@pytest.mark.parametrize("n,whi", [(50_000, 100), (1500, 2)])
+def test_rounds_that_join_next_to_nothing(n, whi):
+    """Cycles whose minimum weights repeat: once only those are left (500 and
+    more), a round here joins a single vertex, and the others take over, until 63
+    vertices are left: at most 61 such rounds, and those before them, which join
+    an eighth or a vertex per whole-graph pass."""
+    rng = np.random.default_rng(n)
+    w = rng.integers(1, whi + 1, n)
+    st = _check_solve(n, canon(n, *G.cycle(n, [int(x) for x in w])), expect=int(np.sort(w)[:2].sum()))
+    assert st["rounds"] <= 61 + 40
+
+
+@pytest.mark.parametrize("kind", ["wheel", "unit cycle", "ladder"])
+def test_thin_and_slow_in_a_batch(kind):
+    """The same graphs in a batch, where what the block solver gives up goes to
+    the one-warp solver."""
+    graphs, expect = [], []
+    for i, n in enumerate((20, 63, 64, 65, 200, 600)):
+        if kind == "wheel":
+            s = synth.wheel(n, seed=i)
+            graphs.append((s.n, *canon(s.n, *_graph(s))))
+        elif kind == "unit cycle":
+            graphs.append((n, *canon(n, *G.cycle(n))))
+        else:
+            e = [(j, (j + 1) % n) for j in range(n)]
+            e += [(n + a, n + b) for a, b in e] + [(j, n + j) for j in range(n)]
+            w = np.random.default_rng(i).integers(1, 20, len(e))
+            graphs.append((2 * n, *canon(2 * n, *G.from_edges(2 * n, e, [int(x) for x in w]))))
+        expect.append(oracle.noi(*graphs[-1])[0])
+    for kw in (dict(), dict(pr_mask=0)):
+        _check_batch(graphs, expect, mc.default_options(**kw))
