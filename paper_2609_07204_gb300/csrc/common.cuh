@@ -56,7 +56,8 @@ struct DevState {
   int ndense;                         // contraction: dense groups asked for this round
   int m_rows;                         // contraction: entries of the row-wise contracted graph
   int internal_code;                  // which internal check failed (0: none), for the message
-  int small_status;                   // one-block solve: 1 solved, 2 left to the other rounds
+  int small_status;                   // one-block solve: 1 solved, 2 left to the other rounds,
+                                      // 3 left to those without certificate forests
   int small_improved;                 // one-block solve: what lowered the bound (as lambda_src)
   int small_rounds;                   // one-block solve: rounds it ran
   unsigned long long wsum;            // input check: sum of the directed entries' weights

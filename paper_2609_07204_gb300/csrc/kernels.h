@@ -396,7 +396,8 @@ cudaError_t side_from_batches(uint8_t* side0, const int* map0, int n0, const uin
 // total below 2^31) in one block, from the bound st->lambda: lowers
 // st->lambda, side0 (through map0) gets the witness when it did, and
 // st->small_status says 1 = solved, 2 = left to the other rounds (more than
-// mcap entries, or a round that joined nothing).  ed0, ed1: mcap words
+// mcap entries, or a round that joined next to nothing for want of levels), 3 = left to
+// the rounds without certificate forests (they would join no more).  ed0, ed1: mcap words
 // and 2 more each; cur_side: n bytes.
 constexpr long long kSmMaxM = 1ll << 17;
 cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,

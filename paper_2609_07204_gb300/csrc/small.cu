@@ -448,16 +448,19 @@ __device__ int sm_load(const SmMem& sm, SmShared<T>& s, const int64_t* rp, const
 
 // All rounds on the n0-vertex graph of the m edges in ed[0].  lam_io: the
 // bound so far, lowered to the smallest cut found (its witness then in
-// sm.side and source 1: a degree, 3: a prefix cut; else 0).  False: some round could not go on (bail).
+// sm.side and source 1: a degree, 3: a prefix cut; else 0).  False: some round could
+// not go on (bail); limited: with more levels, which the grid-wide forests have, it might.
 template <int T>
 __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges ed1, int m, int n0,
-                         uint32_t pr_mask, long long& lam_io, int& source, int& rounds) {
+                         uint32_t pr_mask, long long& lam_io, int& source, int& rounds,
+                         bool& limited) {
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   long long lam = lam_io;
   int n = n0, cur = 0;
   bool soft = true;
   source = 0;
   rounds = 0;
+  limited = false;
   for (int i = tid; i < n0; i += T) sm.map[i] = (unsigned short)i;
   bool ok = false;
   for (int round = 0; round < 2 * n0 + 8; ++round) {
@@ -682,7 +685,10 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     }
     if (!lowered && n - n2 < (n < kSmSlowMin ? 1 : n / kSmSlow)) {
       // (a finer quantum does not help where a thin frontier and PR joined nothing)
-      if (!soft || q == qmin || (thin >= 2 && pr_mask && n2 == n)) break;  // bail
+      if (!soft || q == qmin || (thin >= 2 && pr_mask && n2 == n)) {
+        limited = qmin > (mean + 1) / 2;
+        break;  // bail
+      }
       soft = false;
     }
     if (n2 == n) continue;  // again, from the lower bound or with the finer quantum
@@ -754,8 +760,8 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
 
 // The current graph of a single solve (n <= kSmMaxN; or, with `count`, the
 // st->n_next vertices and *count edges in ed0): its minimum cut below
-// st->lambda.  st->small_status: 1 solved, 2 bail (too many entries, or a
-// round that could not go on); st->small_improved: what lowered the bound
+// st->lambda.  st->small_status: 1 solved, 2 bail (too many entries, or too few
+// levels for a round), 3 bail and no use for the grid-wide forests; st->small_improved: what lowered the bound
 // (0: nothing), its witness per vertex of the graph in cur_side.
 template <int T>
 __global__ void __launch_bounds__(T, 1)
@@ -775,14 +781,15 @@ __global__ void __launch_bounds__(T, 1)
   }
   long long lam = (long long)*(volatile unsigned long long*)&st->lambda;
   int source, rounds;
+  bool limited = true;
   const int m = count ? *count : sm_load<T>(sm, s, rp, col, w, 0, n, ed0, (int)(mcap / 2));
   source = rounds = 0;
-  const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds);
+  const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds, limited);
   if (source)
     for (int i = threadIdx.x; i < n; i += T) cur_side[i] = sm.side[i];
   if (threadIdx.x == 0) {
     st->lambda = (unsigned long long)lam;
-    st->small_status = ok ? 1 : 2;
+    st->small_status = ok ? 1 : limited ? 2 : 3;
     st->small_improved = source;
     st->small_rounds = rounds;
   }
@@ -814,8 +821,9 @@ __global__ void __launch_bounds__(T, 3)
     const int v0 = voff0[gi], n = voff0[gi + 1] - v0;
     long long lam = kInf;
     int source, rounds;
+    bool limited;
     const int m = sm_load<T>(sm, s, rp0, col0, w0, v0, n, ed0, half);
-    const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds);
+    const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds, limited);
     if (ok)
       for (int i = threadIdx.x; i < n; i += T) side0[v0 + i] = sm.side[i];
     if (threadIdx.x == 0) {

@@ -94,6 +94,32 @@ def test_rounds_that_join_next_to_nothing(n, whi):
     assert st["rounds"] <= 61 + 40
 
 
+@pytest.mark.parametrize("n", [1025, 2048])
+def test_given_up_once(n):
+    """A wheel that the block solver gives up: the grid-wide forests, whose
+    certificate is the same, do not try it again; and a clique ring whose rest
+    it gives up is not taken again at once."""
+    s = synth.wheel(n, seed=1)
+    c = _graph(s)
+    _check_solve(n, c, expect=2 * (n - 2) + 2)
+    g = mc.mincut_graph_from_csr(n, *c)
+    mc.mincut_solve(g, mc.default_options(profile=1))
+    assert "forest" not in mc.mincut_profile_read(g)
+    g.destroy()
+    k = 100  # cliques of 25 in a ring of light edges: a unit cycle of 100 is left
+    e = [(25 * i + a, 25 * i + b) for i in range(k) for a in range(25) for b in range(a)]
+    w = [10] * len(e) + [2] * k
+    e += [(25 * i, (25 * i + 26) % (25 * k)) for i in range(k)]
+    c = canon(25 * k, *G.from_edges(25 * k, e, w))
+    _check_solve(25 * k, c, expect=4)
+    g = mc.mincut_graph_from_csr(25 * k, *c)
+    mc.mincut_solve(g, mc.default_options(profile=1))
+    prof = mc.mincut_profile_read(g)
+    # once led by the forests with the rest behind them, and once when a quarter is left
+    assert prof["forest"]["launches"] == 1 and prof["small_solve"]["launches"] <= 2
+    g.destroy()
+
+
 @pytest.mark.parametrize("kind", ["wheel", "unit cycle", "ladder"])
 def test_thin_and_slow_in_a_batch(kind):
     """The same graphs in a batch, where what the block solver gives up goes to
