@@ -939,9 +939,11 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     if (rc) return rc;
     if (flags_dev && M > 0)
       CK(cudaMemcpyAsync(c.pr_flags_host, flags_dev, (size_t)M, cudaMemcpyDeviceToHost, s));
-    const long long marks = (long long)(g->hst->marks_pr + g->hst->marks_cf);
+    // (without what weak forests joined before: a few joins are no reason to do
+    // without the whole passes, nor marks of the concurrent ones)
     o->marks_pr = (long long)g->hst->marks_pr;
-    o->marks_cc = (long long)g->hst->marks_cf;
+    o->marks_cc = (long long)g->hst->marks_cf - o->marks_cf;
+    const long long marks = o->marks_pr + o->marks_cc;
     o->cc_ran = c.capforest == 1 && n > 2 && !c.skip_concurrent &&
                 !(c.cc_skip_pr >= 0 && o->marks_pr >= c.cc_skip_pr);
     // the sequential pass when the round marked nothing (Algorithm 2), and on

@@ -71,6 +71,20 @@ def test_small_planted_cuts(log_nb, cross, seed):
         assert _check_solve(s.n, c, expect=lam)["seq_passes"] == 0
 
 
+def test_weak_forests_on_a_large_graph():
+    """A unit cycle, of which the forests join one vertex and the other marks
+    none: every round runs the whole-graph passes, the first one too."""
+    n = 12_000
+    p = np.random.default_rng(1).permutation(n)
+    c = canon(n, *G.from_edges(n, np.stack([p, np.roll(p, -1)], 1)))
+    _check_solve(n, c, expect=2)
+    g = mc.mincut_graph_from_csr(n, *c)
+    mc.mincut_solve(g, mc.default_options(profile=1))
+    prof = mc.mincut_profile_read(g)
+    g.destroy()
+    assert prof["capforest_seq"]["launches"] == prof["pr_marks"]["launches"]
+
+
 @pytest.mark.parametrize("w", [3, 1000, 60_000])
 def test_weights_nearly_alike(w):
     """Equal weights with a few heavier ones among them: half their mean lies
