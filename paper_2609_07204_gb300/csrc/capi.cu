@@ -526,20 +526,23 @@ int ensure_seq_multi(mincut_graph* g, int want) {
   return k;
 }
 
-int ensure_forest(mincut_graph* g) {
-  if (g->fo_ctl) return MINCUT_OK;
-  if (!in_slab(g, [&] {
+// False: no room, which is no error (a solve does without the forests then).
+bool ensure_forest(mincut_graph* g) {
+  if (g->fo_ctl) return true;
+  g->fo_tag = nullptr;
+  g->fo_r = nullptr;
+  g->fo_items = nullptr;
+  if (in_slab(g, [&] {
         return galloc(g, &g->fo_tag, g->n0) && galloc(g, &g->fo_r, g->n0) &&
                galloc(g, &g->fo_items, forest_item_cap(g->n0, g->M0)) &&
                galloc(g, &g->fo_ctl, (long long)forest_ctl_bytes());
-      })) {
-    if (g->fo_tag) dev_free(g, g->fo_tag);
-    if (g->fo_r) dev_free(g, g->fo_r);
-    if (g->fo_items) dev_free(g, g->fo_items);
-    g->fo_ctl = nullptr;
-    return fail(MINCUT_ERR_OOM, "forest buffers");
-  }
-  return MINCUT_OK;
+      }))
+    return true;
+  if (g->fo_tag) dev_free(g, g->fo_tag);
+  if (g->fo_r) dev_free(g, g->fo_r);
+  if (g->fo_items) dev_free(g, g->fo_items);
+  g->fo_ctl = nullptr;
+  return false;
 }
 
 int ensure_lp(mincut_graph* g) {
@@ -792,8 +795,6 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
   if (forest) {
     // the sort keys and values are free during the marking: they hold the
     // union-finds, then the list of what is left and the matrix it is summed in
-    rc = ensure_forest(g);
-    if (rc) return rc;
     const long long Mb = std::max<long long>(g->Mraw, 1), mcap = std::min(kSmMaxM, Mb);
     const ForestScratch f{reinterpret_cast<int*>(g->keys[0]), 2 * Mb, g->fo_tag, g->fo_r,
                           g->fo_items, g->fo_ctl};
@@ -1159,8 +1160,12 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     c.skip_concurrent = skip_cc && g->n <= kSkipConcurrentMaxN;
     c.eager_seq = c.skip_concurrent && barely;
     c.cc_skip_pr = cc_low && c.capforest == 1 && op.cf_visit != 2 ? (g->n + 63) / 64 : -1;
-    // (without room for their buffers the round does without them)
-    c.forest = forests && g->n < forest_below && ensure_forest(g) == MINCUT_OK;
+    // (without room for their buffers the solve does without them)
+    c.forest = forests && g->n < forest_below;
+    if (c.forest && !ensure_forest(g)) {
+      c.forest = false;
+      forest_below = 0;
+    }
     c.small_rest = c.forest && small_below == INT_MAX;
     c.lp_now = lp_allowed && (op.lp_every_round || !lp_done);
     c.passes = op.passes > 0 ? op.passes : std::max(32, std::min(g->max_passes, g->n / 4));

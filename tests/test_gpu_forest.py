@@ -270,6 +270,38 @@ def test_allocations_refused(refused, monkeypatch):
     h.destroy()
 
 
+def test_refusal_is_no_error(monkeypatch):
+    """Both requests for the forests' buffers refused: the solve does without
+    them to its end, asks no more for them, and leaves no message."""
+    class Refusing(mc._TorchAllocator):
+        def __init__(self, device):
+            super().__init__(device)
+            self.refuse = 0
+            give = self._alloc
+
+            def _alloc(nbytes, stream, ctx):
+                if self.refuse > 0:
+                    self.refuse -= 1
+                    return None
+                return give(nbytes, stream, ctx)
+
+            self._give, self._alloc = give, type(give)(_alloc)
+            self.struct = mc.MincutAllocator(self._alloc, self._free, None)
+
+    monkeypatch.setattr(mc, "_TorchAllocator", Refusing)
+    nb = 1 << 11
+    s = synth.planted(nb, 21 * nb, 30, 9, 1, 5)
+    h = mc.mincut_graph_from_csr(s.n, mc_dev(s.row_ptr.astype(np.int64)),
+                                 mc_dev(s.col.astype(np.int32)), mc_dev(s.w.astype(np.int32)),
+                                 use_torch_allocator=True)
+    h._allocator.refuse = 2
+    value, _, st = mc.mincut_solve(h, mc.default_options(profile=1))
+    assert value == oracle.noi(s.n, s.row_ptr, s.col, s.w.astype(np.int64))[0]
+    assert st["rounds"] > 1 and mc.mincut_last_error() == ""
+    assert "forest" not in mc.mincut_profile_read(h)
+    h.destroy()
+
+
 def mc_dev(a):
     import torch
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
