@@ -79,8 +79,8 @@ __device__ BwSlot bw_slot(int* base, long long slot_words, int slot, int nmax, i
 }
 
 __global__ void __launch_bounds__(kBwWarps * 32)
-    batch_warp_kernel(const int* __restrict__ list, int nlist_max,
-                      const int* __restrict__ nlist_dev, int* cursor,
+    batch_warp_kernel(const int* __restrict__ list, int nlist, const int* __restrict__ more,
+                      const int* __restrict__ nmore_dev, int* cursor,
                       const int* __restrict__ voff0, const int64_t* __restrict__ rp0,
                       const int* __restrict__ col0, const int* __restrict__ w0, int* scratch,
                       long long slot_words, int nmax, int mmax, uint32_t pr_mask,
@@ -103,14 +103,14 @@ __global__ void __launch_bounds__(kBwWarps * 32)
   unsigned* l2 = l1 + kBwMaxN / 32;                            // kBwMaxN / 1024
   int* tl = reinterpret_cast<int*>(l2 + kBwMaxN / 1024);       // 32
   int* tcount = tl + 32;                                       // 1
-  const int nlist = nlist_dev ? min(*nlist_dev, nlist_max) : nlist_max;
+  const int nitems = nlist + (nmore_dev ? *nmore_dev : 0);
   int fail = 0;  // the first failed check: 1 rounds, 2 union-find, 3 / 4 tree descent
   for (;;) {
     int item = 0;
     if (lane == 0) item = atomicAdd(cursor, 1);
     item = __shfl_sync(FULL, item, 0);
-    if (item >= nlist) break;
-    const int gi = list[item];
+    if (item >= nitems) break;
+    const int gi = item < nlist ? list[item] : more[item - nlist];
     const int v0 = voff0[gi], n0 = voff0[gi + 1] - v0;
     const long long e0 = rp0[v0];
     // the graph in local ids, buffer 0
@@ -405,21 +405,21 @@ cudaError_t batch_warp_mark(const int* list, int nlist, int* done_g, DevState* s
   return cudaGetLastError();
 }
 
-cudaError_t batch_warp_solve(const int* list, int nlist, const int* nlist_dev, int* cursor,
-                             const int* voff0,
+cudaError_t batch_warp_solve(const int* list, int nlist, const int* more, const int* nmore_dev,
+                             int* cursor, const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
                              unsigned long long* lam_g, uint8_t* side0, DevState* st,
                              cudaStream_t s, int* launches) {
-  if (nlist <= 0) return cudaSuccess;
+  if (nlist <= 0 && !nmore_dev) return cudaSuccess;
   if (nmax > kBwMaxN) return cudaErrorInvalidValue;
   cudaMemsetAsync(cursor, 0, sizeof(int), s);
   if (slots < kBwWarps || slots % kBwWarps) return cudaErrorInvalidValue;
   const int blocks = slots / kBwWarps;
   if (!bw_set_smem()) return cudaErrorInvalidValue;
   batch_warp_kernel<<<blocks, kBwWarps * 32, kBwSmemBytes, s>>>(
-      list, nlist, nlist_dev, cursor, voff0, rp0, col0, w0, scratch, batch_warp_slot_words(nmax, mmax), nmax,
-      mmax, pr_mask, lam_g, side0, st);
+      list, nlist, more, nmore_dev, cursor, voff0, rp0, col0, w0, scratch,
+      batch_warp_slot_words(nmax, mmax), nmax, mmax, pr_mask, lam_g, side0, st);
   ++*launches;
   return cudaGetLastError();
 }

@@ -70,10 +70,10 @@ cudaError_t batch_warp_mark(const int* list, int nlist, int* done_g, DevState* s
 // weights, total below 2^31) into lam_g and side0.  scratch: slots slots (a
 // multiple of batch_warp_block_warps()) of
 // batch_warp_slot_words(nmax, mmax) ints; every listed graph has at most nmax
-// vertices and mmax entries.  cursor: one int of work-queue state.  nlist_dev
-// (nullable): the number of listed graphs, at most nlist, on the device.
-cudaError_t batch_warp_solve(const int* list, int nlist, const int* nlist_dev, int* cursor,
-                             const int* voff0,
+// vertices and mmax entries.  cursor: one int of work-queue state.  more,
+// nmore_dev (nullable): *nmore_dev further graphs, the number on the device.
+cudaError_t batch_warp_solve(const int* list, int nlist, const int* more, const int* nmore_dev,
+                             int* cursor, const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
                              unsigned long long* lam_g, uint8_t* side0, DevState* st,

@@ -136,6 +136,40 @@ def test_batch_repeated_solves_replay_captured_launches(own_stream):
     B.destroy()
 
 
+@pytest.mark.parametrize("det", [0, 1])
+def test_batch_tiny_graphs(det):
+    """Around the sizes at which a graph goes to a warp instead of a block
+    (32 vertices; 64 with six entries per vertex), alone and mixed."""
+    rng = np.random.default_rng(5)
+    graphs = []
+    for n in (3, 4, 31, 32, 33, 63, 64, 65):
+        for deg in (2.2, 5.8, 6.2, 12):
+            s = synth.cycle_plus(n, min(deg, n - 1), 1, 50, int(rng.integers(1 << 30)))
+            graphs.append((s.n, *oracle.canonicalize(s.n, s.row_ptr, s.col, s.w.astype(np.int64))))
+    expect = [oracle.stoer_wagner(*g)[0] for g in graphs]
+    opts = mc.default_options(deterministic=det)
+    _check_batch(graphs, expect, opts)
+    tiny = [i for i, g in enumerate(graphs) if g[0] <= 32]
+    big = [i for i, g in enumerate(graphs) if g[0] > 64]
+    for part in (tiny, big):
+        _check_batch([graphs[i] for i in part], [expect[i] for i in part], opts)
+
+
+def test_batch_tiny_graphs_are_no_slower_than_warps():
+    """4,096 dense graphs of 8 vertices: the default batch takes the time of
+    the one-warp solver (2.8 times that by a block each)."""
+    rng = np.random.default_rng(7)
+    g = [(8, *G.complete(8, int(w))) for w in rng.integers(1, 100, 4096)]
+    B = mc.mincut_batch_from_csr(*mc.pack_graphs(g))
+    ms = []
+    for det in (0, 1):
+        opts = mc.default_options(deterministic=det)
+        times = [mc.mincut_batch_solve(B, opts)[2]["ms_total"] for _ in range(9)]
+        ms.append(sorted(times)[4])
+    B.destroy()
+    assert ms[0] < 1.5 * ms[1], ms
+
+
 def test_batch_rejects_cross_graph_edge_and_tiny_graph():
     c1 = oracle.canonicalize(3, *G.cycle(3))
     c2 = oracle.canonicalize(3, *G.cycle(3))
