@@ -223,6 +223,7 @@ struct mincut_graph {
   int max_graph_n = 0;
   // graphs solved one per warp (batch_warp.cu)
   int bw_threshold = -1;      // the list below holds the graphs with n <= this
+  bool bw_dense_out = false;  // but the dense ones (bw_dense)
   int* bw_list = nullptr;     // graph ids, most entries first, the tiny ones (bw_tiny) behind
   int bw_count = 0, bw_big = 0, bw_nmax = 0, bw_mmax = 0;
   int* bw_cursor = nullptr;    // work queues of the block and the warp solver, then the
@@ -1670,18 +1671,26 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
 // 319 / 182 and 110 / 145, of 96 185 / 209 and 127 / 171.
 bool bw_tiny(int n, int m) { return n <= 32 || (n <= 64 && m >= 6 * n); }
 
+// Graphs that the round kernels solve faster than one warp, and that the block
+// solver has too few levels for: entries enough to keep a block per graph
+// busy.  One graph, warp against round kernels: 600 vertices of degree 40
+// 2.6 / 1.7 ms, of degree 120 8.1 / 2.7; 2,000 of degree 40 8.4 / 4.6, of degree
+// 120 29.2 / 7.0; 160 of 600 and degree 40 2.8 / 2.3, 40 of 1,000 and degree 120
+// 17.4 / 5.3.  Below (300 of degree 40, 2,000 of degree 12) about equal or slower.
+bool bw_dense(int n, int m) { return m >= 20000 && m >= 24 * n; }
+
 // The graphs of a batch with at most `threshold` vertices (and at most
-// kBwMaxN), most entries first and the tiny ones last, for the block and the
+// kBwMaxN; not the dense ones where dense_out), most entries first and the tiny ones last, for the block and the
 // warp solver; the scratch (at most ~2 GB of slots).
-int bw_prepare(mincut_graph* g, int threshold) {
+int bw_prepare(mincut_graph* g, int threshold, bool dense_out) {
   threshold = std::min(threshold, kBwMaxN);
-  if (threshold == g->bw_threshold) return MINCUT_OK;
+  if (threshold == g->bw_threshold && dense_out == g->bw_dense_out) return MINCUT_OK;
   const int G = g->batch.G;
   std::vector<int> ids;
   int nmax = 0, mmax = 0;
   for (int i = 0; i < G; ++i) {
     const int ng = (int)(g->voff0_h[i + 1] - g->voff0_h[i]);
-    if (ng > threshold) continue;
+    if (ng > threshold || (dense_out && bw_dense(ng, g->batch_m[i]))) continue;
     ids.push_back(i);
     nmax = std::max(nmax, ng);
     mmax = std::max(mmax, g->batch_m[i]);
@@ -1692,6 +1701,7 @@ int bw_prepare(mincut_graph* g, int threshold) {
                       return !bw_tiny((int)(g->voff0_h[i + 1] - g->voff0_h[i]), g->batch_m[i]);
                     }) - ids.begin());
   g->bw_threshold = threshold;
+  g->bw_dense_out = dense_out;
   g->bw_count = (int)ids.size();
   g->bw_nmax = nmax;
   g->bw_mmax = std::max(mmax, 1);
@@ -1788,7 +1798,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
   if (op.spin_limit > 0) g->spin_limit = op.spin_limit;
   // the small graphs are the warp solver's: the round kernels treat them as done
   {
-    const int rc0 = bw_prepare(g, small_n);
+    const int rc0 = bw_prepare(g, small_n, op.batch_small_n == 0);
     if (rc0) return rc0;
   }
   mincut_stats stl{};
@@ -1846,6 +1856,10 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
     CK(cudaMemsetAsync(g->side0, 0, (size_t)g->n0, s));
     if (g->bw_count > 0)
       CK(batch_warp_mark(g->bw_list, g->bw_count, b.done_g, g->st, s, &g->launches));
+    // whole passes for every graph, and no concurrent ones, also where all these
+    // graphs are small (dense ones, see bw_dense: 20 of 600 vertices and degree 120 9.4
+    // -> 3.7 ms)
+    const bool whole = op.deterministic || (op.batch_small_n == 0 && g->max_graph_n <= kBwMaxN);
     const int table = op.pass_table > 0 ? std::min(op.pass_table, g->max_table) : g->max_table;
     for (int round = 0; g->bw_count < G && round < max_rounds; ++round) {
       const int n = g->n;
@@ -1869,7 +1883,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
         CK(pr_marks<WT>(n, M, rp, col, w, deg, g->tile_row, op.pr_mask, op.pr_budget, g->parent,
                         nullptr, g->short_bits, g->st, s, &g->launches, &v));
       }
-      if (!op.deterministic) {
+      if (!whole) {
         ProfScope ps(P_CF_PASSES, M, s);
         CK(cudaMemsetAsync(g->owner, 0, (size_t)n * sizeof(int), s));
         PassConfig pc;
@@ -1885,7 +1899,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
       { ProfScope ps(P_CF_SEQ, M, s);
         CK(capforest_sequential_batch<WT>(G, rp, col, w, deg, g->parent, (WT*)g->seq_r,
                                           g->batch_levels, b.level_off, g->seq_order,
-                                          g->max_graph_n, op.deterministic ? 1 : 0, v, g->st, s,
+                                          g->max_graph_n, whole ? 1 : 0, v, g->st, s,
                                           &g->launches)); }
       { ProfScope ps(P_WITNESS, g->n0, s);
         CK(batch_witness(G, g->n0, b, g->visit_log, table, g->pass_len, g->seq_order, g->cur_side,
@@ -2176,7 +2190,7 @@ int mincut_batch_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut
   if (op.pass_table != 0 && (op.pass_table < 256 || op.pass_table > 2048 ||
                              (op.pass_table & (op.pass_table - 1))))
     return fail(MINCUT_ERR_INVALID, "pass_table must be a power of two in [256, 2048]");
-  // 0: every graph the small solvers can take.  (On 4,096 graphs of 20 to 2,000
+  // 0: every graph the small solvers can take, but the dense ones.  (On 4,096 graphs of 20 to 2,000
   // vertices a block per graph takes 2.3 ms, one warp per graph 5.4, the round
   // kernels 13.3; lower thresholds lie between, and timing them on the first
   // solve cost a new batch 50 ms.)

@@ -170,6 +170,33 @@ def test_batch_tiny_graphs_are_no_slower_than_warps():
     assert ms[0] < 1.5 * ms[1], ms
 
 
+@pytest.mark.parametrize("det", [0, 1])
+def test_batch_dense_graphs(det):
+    """Graphs of 20,000 entries and 24 per vertex, and just below either: the
+    former take the round kernels, alone and among others, and a batch of them
+    no longer than by warps."""
+    rng = np.random.default_rng(3)
+    dense, other = [], []
+    for n, m, part in ((600, 24_000, dense), (300, 10_000, dense), (800, 10_000, dense),
+                       (833, 9_999, other), (860, 10_100, other), (100, 4_950, other)):
+        u, v = np.triu_indices(n, 1)
+        pick = rng.choice(len(u), m, replace=False)
+        w = rng.integers(1, 21, m)
+        c = oracle.canonicalize(n, *G.from_edges(n, np.stack([u[pick], v[pick]], 1), w))
+        part.append((n, *c))
+    for graphs, rounds in ((dense, True), (other, False), (other + dense, True)):
+        expect = [oracle.noi(*g)[0] for g in graphs]
+        st = _check_batch(graphs, expect, mc.default_options(deterministic=det))
+        assert (st["rounds"] > 0) == rounds
+    B = mc.mincut_batch_from_csr(*mc.pack_graphs(dense))
+    ms = []
+    for small in (0, 2048):
+        opts = mc.default_options(deterministic=det, batch_small_n=small)
+        ms.append(min(mc.mincut_batch_solve(B, opts)[2]["ms_total"] for _ in range(5)))
+    B.destroy()
+    assert ms[0] < ms[1], ms
+
+
 def test_batch_rejects_cross_graph_edge_and_tiny_graph():
     c1 = oracle.canonicalize(3, *G.cycle(3))
     c2 = oracle.canonicalize(3, *G.cycle(3))
