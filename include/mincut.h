@@ -97,8 +97,9 @@ typedef struct mincut_options {
     int32_t batch_small_n;   /* mincut_batch_solve: graphs of at most this many vertices (and at
                                 most 2048) are solved each on its own, a thread block per graph
                                 (deterministic = 1: a warp, one CAPFOREST pass per round; of
-                                pr_mask only PR1/PR2 either way); the others share the batch's
-                                round kernels.  0 = auto (2048, but graphs of at least 20,000
+                                pr_mask only PR1/PR2 either way; graphs that join next to
+                                nothing so then share rounds with all of pr_mask); the others
+                                share the batch's round kernels.  0 = auto (2048, but graphs of at least 20,000
                                 entries and 24 per vertex share the round kernels); < 0 = every
                                 graph in the round kernels */
     int32_t seq_kernel;      /* kernel of the whole-graph CAPFOREST passes: 0 (default) one

@@ -56,6 +56,27 @@ __global__ void batch_start_kernel(int G, unsigned long long* lam_g, int* done_g
   }
 }
 
+__global__ void batch_reopen_kernel(const int* __restrict__ left, int nleft, int G,
+                                    unsigned long long* lam_g, int* done_g, DevState* st) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nleft; i += gridDim.x * blockDim.x) {
+    lam_g[left[i]] = (unsigned long long)kInf;
+    done_g[left[i]] = 0;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->batch_done = G - nleft;
+    st->batch_left = 0;
+  }
+}
+
+__global__ void batch_unfinished_kernel(int G, int* done_g, int* left, DevState* st) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
+    if (done_g[g]) continue;
+    done_g[g] = 1;
+    left[atomicAdd(&st->batch_left, 1)] = g;
+    atomicAdd(&st->batch_done, 1);
+  }
+}
+
 __global__ void batch_round_reset_kernel(int G, const unsigned long long* lam_g,
                                          unsigned long long* lam_before,
                                          unsigned long long* deg_best,
@@ -226,6 +247,20 @@ cudaError_t batch_gid(const int* voff, int G, int n, int* gid, cudaStream_t s, i
 cudaError_t batch_start(int G, unsigned long long* lam_g, int* done_g, cudaStream_t s,
                         int* launches) {
   batch_start_kernel<<<gridb(G, 256), 256, 0, s>>>(G, lam_g, done_g);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t batch_reopen(const int* left, int nleft, int G, unsigned long long* lam_g, int* done_g,
+                         DevState* st, cudaStream_t s, int* launches) {
+  batch_reopen_kernel<<<gridb(nleft, 256), 256, 0, s>>>(left, nleft, G, lam_g, done_g, st);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t batch_unfinished(int G, int* done_g, int* left, DevState* st, cudaStream_t s,
+                             int* launches) {
+  batch_unfinished_kernel<<<gridb(G, 256), 256, 0, s>>>(G, done_g, left, st);
   ++*launches;
   return cudaGetLastError();
 }

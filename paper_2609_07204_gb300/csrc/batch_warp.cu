@@ -34,6 +34,10 @@ namespace mc {
 
 namespace {
 
+// A first round that joins fewer than 1 / kBwLeftDiv of at least kBwLeftMin vertices
+// (a wheel's, one of n): the graph is left to the rounds with PR3 / PR4.
+constexpr int kBwLeftMin = 64;
+constexpr int kBwLeftDiv = 32;
 constexpr int kBwWarps = 1;  // warps per block (each warp has its own graphs)
 constexpr int kBwWarpSmemWords = kBwMaxN + (kBwMaxN + 1) + kBwMaxN + (kBwMaxN + 1) + kBwMaxN +
                                  kBwMaxN + kBwMaxN / 32 + kBwMaxN / 1024 + 32 + 1;
@@ -84,7 +88,7 @@ __global__ void __launch_bounds__(kBwWarps * 32)
                       const int* __restrict__ voff0, const int64_t* __restrict__ rp0,
                       const int* __restrict__ col0, const int* __restrict__ w0, int* scratch,
                       long long slot_words, int nmax, int mmax, uint32_t pr_mask,
-                      unsigned long long* lam_g, uint8_t* side0, DevState* st) {
+                      unsigned long long* lam_g, uint8_t* side0, int* left, DevState* st) {
   // per warp, in dynamic shared memory (kBwWarpSmemWords ints each): the
   // keys (r values in a pass, then the accumulator), the current graph's row
   // offsets, its degrees (then the labels), the group counts and members,
@@ -127,6 +131,7 @@ __global__ void __launch_bounds__(kBwWarps * 32)
     __syncwarp();
     long long lam = kInf;
     int n = n0, cur = 0;
+    bool given_up = false;
     for (int round = 0;; ++round) {
       if (round > 2 * n0 + 8) {  // cannot happen (see the header); reported, not looped on
         fail = fail ? fail : 1;
@@ -265,6 +270,10 @@ __global__ void __launch_bounds__(kBwWarps * 32)
         if (r != v) lab[v] = lab[r];
       }
       __syncwarp();
+      if (left && round == 0 && n >= kBwLeftMin && (n - n2) * kBwLeftDiv < n) {
+        given_up = true;
+        break;
+      }
       if (n2 == n) continue;  // no marks (the pass lowered the bound): again, lower bound
       // ---- members of each group (counting sort by label)
       for (int g = lane; g <= n2; g += 32) scnt[g] = 0;
@@ -354,7 +363,10 @@ __global__ void __launch_bounds__(kBwWarps * 32)
       n = n2;
       if (n2 <= 1) break;
     }
-    if (lane == 0) lam_g[gi] = (unsigned long long)lam;
+    if (lane == 0) {
+      if (given_up) left[atomicAdd(&st->batch_left, 1)] = gi;
+      else lam_g[gi] = (unsigned long long)lam;
+    }
     __syncwarp();
   }
   if (fail) {
@@ -409,7 +421,7 @@ cudaError_t batch_warp_solve(const int* list, int nlist, const int* more, const 
                              int* cursor, const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
-                             unsigned long long* lam_g, uint8_t* side0, DevState* st,
+                             unsigned long long* lam_g, uint8_t* side0, int* left, DevState* st,
                              cudaStream_t s, int* launches) {
   if (nlist <= 0 && !nmore_dev) return cudaSuccess;
   if (nmax > kBwMaxN) return cudaErrorInvalidValue;
@@ -419,7 +431,7 @@ cudaError_t batch_warp_solve(const int* list, int nlist, const int* more, const 
   if (!bw_set_smem()) return cudaErrorInvalidValue;
   batch_warp_kernel<<<blocks, kBwWarps * 32, kBwSmemBytes, s>>>(
       list, nlist, more, nmore_dev, cursor, voff0, rp0, col0, w0, scratch,
-      batch_warp_slot_words(nmax, mmax), nmax, mmax, pr_mask, lam_g, side0, st);
+      batch_warp_slot_words(nmax, mmax), nmax, mmax, pr_mask, lam_g, side0, left, st);
   ++*launches;
   return cudaGetLastError();
 }

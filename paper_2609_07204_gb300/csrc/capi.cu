@@ -226,9 +226,9 @@ struct mincut_graph {
   bool bw_dense_out = false;  // but the dense ones (bw_dense)
   int* bw_list = nullptr;     // graph ids, most entries first, the tiny ones (bw_tiny) behind
   int bw_count = 0, bw_big = 0, bw_nmax = 0, bw_mmax = 0;
-  int* bw_cursor = nullptr;    // work queues of the block and the warp solver, then the
-                               // number of graphs the block solver left
-  int* bw_left = nullptr;      // and their ids
+  int* bw_cursor = nullptr;    // work queues of the block and the warp solver, then the number
+                               // of graphs with too few levels for the block solver
+  int* bw_left = nullptr;      // graphs given up (st->batch_left), then, from G on, the latter
   int* bw_scratch = nullptr;
   long long bw_scratch_words = 0;
   int bw_slots = 0;
@@ -1668,8 +1668,11 @@ int create_impl(int64_t n64, const int64_t* row_ptr, const int32_t* col, const i
 // has little to do on them.  Batches of equal graphs, block against warp: 4,096
 // of 8 vertices 598 / 212 us, of 32 with degree 8 846 / 408 and degree 3 371 /
 // 336, of 48 784 / 596 and 388 / 497, of 64 790 / 770 and 401 / 594; 256 of 64
-// 319 / 182 and 110 / 145, of 96 185 / 209 and 127 / 171.
-bool bw_tiny(int n, int m) { return n <= 32 || (n <= 64 && m >= 6 * n); }
+// 319 / 182 and 110 / 145, of 96 185 / 209 and 127 / 171.  And those with too
+// many edges per vertex for the block's levels: 640 of 100 vertices and degree 30
+// 2,321 / 611, of 300 and degree 30 3,757 / 2,022 (one of each 449 / 302 and 1,187 /
+// 949); of 600 and degree 20 1,579 / 2,613.
+bool bw_tiny(int n, int m) { return n <= 32 || (n <= 64 && m >= 6 * n) || m >= 24 * n; }
 
 // Graphs that the round kernels solve faster than one warp, and that the block
 // solver has too few levels for: entries enough to keep a block per graph
@@ -1708,7 +1711,7 @@ int bw_prepare(mincut_graph* g, int threshold, bool dense_out) {
   if (ids.empty()) return MINCUT_OK;
   if (!g->bw_list) {
     if (!galloc(g, &g->bw_list, G) || !galloc(g, &g->bw_cursor, 4) ||
-        !galloc(g, &g->bw_left, G))
+        !galloc(g, &g->bw_left, 2ll * G))
       return fail(MINCUT_ERR_OOM, "batch warp list");
   }
   CK(cudaMemcpyAsync(g->bw_list, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice,
@@ -1732,28 +1735,31 @@ int bw_prepare(mincut_graph* g, int threshold, bool dense_out) {
   return MINCUT_OK;
 }
 
-// The listed small graphs: a block per graph (small.cu), then one warp for
-// each of the tiny ones and of those it left; in the deterministic mode all of
-// them one warp each.
+// The listed small graphs: a block per graph (small.cu), then a warp for each of
+// the tiny ones and of those with too few levels for a block; in the deterministic
+// mode all of them one warp each.  Those given up are left to batch_left_over
+// (st->batch_left) where pr has PR3 or PR4, else a warp solves them too.
 cudaError_t bw_solve_list(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s,
                           int* launches) {
   BatchState& b = g->batch;
   if (!blocks)
     return batch_warp_solve(g->bw_list, g->bw_count, nullptr, nullptr, g->bw_cursor, b.voff0,
                             g->rp0, g->col0, (const int*)g->w0, g->bw_scratch, g->bw_slots,
-                            g->bw_nmax, g->bw_mmax, pr, b.lam_g, g->side0, g->st, s, launches);
+                            g->bw_nmax, g->bw_mmax, pr & 3u, b.lam_g, g->side0,
+                            pr > 3u ? g->bw_left : nullptr, g->st, s, launches);
   const int tiny = g->bw_count - g->bw_big;
+  int* few = g->bw_left + b.G;
   cudaError_t e = small_batch(g->bw_list, g->bw_big, g->bw_cursor, b.voff0, g->rp0, g->col0,
                               (const int*)g->w0, g->bw_scratch,
                               batch_warp_slot_words(g->bw_nmax, g->bw_mmax), g->bw_slots,
-                              g->bw_nmax, g->bw_mmax, pr, b.lam_g, g->side0, g->bw_left,
-                              g->bw_cursor + 2, g->sms, s, launches);
+                              g->bw_nmax, g->bw_mmax, pr & 3u, b.lam_g, g->side0, few,
+                              g->bw_cursor + 2, pr > 3u ? g->bw_left : few,
+                              pr > 3u ? &g->st->batch_left : g->bw_cursor + 2, g->sms, s, launches);
   if (e == cudaSuccess)
-    e = batch_warp_solve(g->bw_list + g->bw_big, tiny, g->bw_left,
+    e = batch_warp_solve(g->bw_list + g->bw_big, tiny, few,
                          g->bw_big ? g->bw_cursor + 2 : nullptr, g->bw_cursor + 1, b.voff0, g->rp0,
-                         g->col0, (const int*)g->w0, g->bw_scratch,
-                         std::min(g->bw_slots, std::max(g->sms, tiny)), g->bw_nmax, g->bw_mmax,
-                         pr, b.lam_g, g->side0, g->st, s, launches);
+                         g->col0, (const int*)g->w0, g->bw_scratch, g->bw_slots, g->bw_nmax,
+                         g->bw_mmax, pr & 3u, b.lam_g, g->side0, nullptr, g->st, s, launches);
   return e;
 }
 
@@ -1781,6 +1787,118 @@ cudaError_t bw_enqueue(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s
   if (e == cudaSuccess) e = batch_warp_mark(g->bw_list, g->bw_count, b.done_g, g->st, s, launches);
   if (e == cudaSuccess) e = bw_solve_list(g, pr, blocks, s, launches);
   return e;
+}
+
+// Rounds that all open graphs of a batch share, until they are done; with `live`,
+// the number of their vertices, until a round does not halve it.  whole: whole
+// passes for every graph and no concurrent ones.
+template <typename WT>
+int batch_rounds(mincut_graph* g, const mincut_options& op, bool whole, int max_rounds,
+                 long long live, mincut_stats* stl) {
+  cudaStream_t s = g->stream;
+  BatchState& b = g->batch;
+  const int G = b.G;
+  const int table = op.pass_table > 0 ? std::min(op.pass_table, g->max_table) : g->max_table;
+  for (int round = 0; round < max_rounds; ++round) {
+    const int n = g->n;
+    const long long M = g->M;
+    const int64_t* rp = g->crp();
+    const int* col = g->ccol();
+    const WT* w = (const WT*)g->cw();
+    const WT* deg = (const WT*)g->cdeg();
+    reset_round_kernel<<<1, 1, 0, s>>>(g->st);
+    ++g->launches;
+    CK(batch_round_reset(G, b, s, &g->launches));
+    { ProfScope ps(P_DEGREE, n, s);
+      CK(batch_degree_bound<WT>(n, G, deg, b, &g->st->batch_done, s, &g->launches)); }
+    { ProfScope ps(P_TILES, n, s);
+      CK(tile_rows(rp, n, M, g->tile_row, s, &g->launches)); }
+    { ProfScope ps(P_UF, n, s);
+      CK(uf_init(g->parent, n, s, &g->launches)); }
+    const BatchView v = b.view();
+    if (op.pr_mask) {
+      ProfScope ps(P_PR, M, s);
+      CK(pr_marks<WT>(n, M, rp, col, w, deg, g->tile_row, op.pr_mask, op.pr_budget, g->parent,
+                      nullptr, g->short_bits, g->st, s, &g->launches, &v));
+    }
+    if (!whole) {
+      ProfScope ps(P_CF_PASSES, M, s);
+      CK(cudaMemsetAsync(g->owner, 0, (size_t)n * sizeof(int), s));
+      PassConfig pc;
+      pc.table = table;
+      pc.warps_per_block = 4;
+      pc.passes = op.passes > 0 ? std::min(op.passes, g->max_passes)
+                                : std::max(32, std::min(g->max_passes, n / 4));
+      pc.seed = op.seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(round + 1);
+      pc.private_visit = op.cf_visit == 1 ? 1 : 0;
+      CK(capforest_passes<WT>(n, rp, col, w, deg, g->owner, g->parent, g->visit_log, g->pass_best,
+                              g->pass_len, g->pass_counter, pc, g->st, s, &g->launches, &v));
+    }
+    { ProfScope ps(P_CF_SEQ, M, s);
+      CK(capforest_sequential_batch<WT>(G, rp, col, w, deg, g->parent, (WT*)g->seq_r,
+                                        g->batch_levels, b.level_off, g->seq_order,
+                                        g->max_graph_n, whole ? 1 : 0, v, g->st, s,
+                                        &g->launches)); }
+    { ProfScope ps(P_WITNESS, g->n0, s);
+      CK(batch_witness(G, g->n0, b, g->visit_log, table, g->pass_len, g->seq_order, g->cur_side,
+                       g->map0, g->side0, g->st, s, &g->launches)); }
+    CK(batch_collapse(n, b, g->parent, s, &g->launches));
+    stl->rounds++;
+    stl->entries_processed += M;
+    int n2 = 0;
+    long long m2 = 0;
+    int rc = contract_current<WT>(g, &n2, &m2, true);
+    if (rc) return rc;
+    CK(batch_new_offsets(G, b, g->rank, g->st, s, &g->launches));
+    std::swap(b.voff, b.voff_next);
+    CK(batch_gid(b.voff, G, n2, b.gid, s, &g->launches));
+    const int done = g->hst->batch_done;
+    if (done >= G) break;
+    if (live > 0) {  // (each finished graph is one vertex)
+      const long long now = n2 - done;
+      if (2 * now > live) break;
+      live = now;
+    }
+  }
+  return MINCUT_OK;
+}
+
+// The graphs that the block or the warp solver gave up (g->hst->batch_left of
+// them, in g->bw_left): PR1 / PR2 and one pass join next to nothing in them, so
+// they share rounds with all the PR tests while those halve them, then take a warp
+// each to the end (100 wheels of 200 to 300 vertices: 54.8 ms by warps alone, 0.84 like this; 40 pairs of interleaved cycles, which it does not
+// help, 37.3 and 37.5).
+template <typename WT>
+int batch_left_over(mincut_graph* g, const mincut_options& op, int max_rounds, mincut_stats* stl) {
+  cudaStream_t s = g->stream;
+  BatchState& b = g->batch;
+  const int G = b.G, L = g->hst->batch_left;
+  std::vector<int> ids((size_t)L);
+  CK(cudaMemcpyAsync(ids.data(), g->bw_left, (size_t)L * sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  long long live = 0;
+  for (int i : ids) live += g->voff0_h[i + 1] - g->voff0_h[i];
+  const int* voff = b.voff;
+  CK(cudaMemcpyAsync(b.voff, b.voff0, (size_t)(G + 1) * sizeof(int), cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemcpyAsync(b.gid, b.gid0, (size_t)g->n0 * sizeof(int), cudaMemcpyDeviceToDevice, s));
+  iota_kernel<<<std::min((g->n0 + 255) / 256, g->sms * 8), 256, 0, s>>>(g->map0, g->n0);
+  ++g->launches;
+  CK(batch_reopen(g->bw_left, L, G, b.lam_g, b.done_g, g->st, s, &g->launches));
+  g->cur = -1;
+  g->n = g->n0;
+  g->M = g->M0;
+  int rc = batch_rounds<WT>(g, op, op.deterministic != 0, max_rounds, live, stl);
+  if (rc) return rc;
+  if (b.voff != voff) std::swap(b.voff, b.voff_next);  // (captured launches name it)
+  if (g->hst->batch_done < G) {
+    ProfScope ps(P_BATCH_WARP, G - g->hst->batch_done, s);
+    CK(batch_unfinished(G, b.done_g, g->bw_left, g->st, s, &g->launches));
+    CK(batch_warp_solve(nullptr, 0, g->bw_left, &g->st->batch_left, g->bw_cursor + 1, b.voff0,
+                        g->rp0, g->col0, (const int*)g->w0, g->bw_scratch,
+                        std::min(g->bw_slots, std::max(g->sms, L)), g->bw_nmax, g->bw_mmax,
+                        op.pr_mask & 3u, b.lam_g, g->side0, nullptr, g->st, s, &g->launches));
+  }
+  return sync_state(g);
 }
 
 template <typename WT>
@@ -1814,7 +1932,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
     key.threshold = g->bw_threshold;
     key.scratch = g->bw_scratch;
     key.voff = b.voff;
-    key.pr = op.pr_mask & 3u;
+    key.pr = op.pr_mask;
     key.blocks = !op.deterministic;
     g->bw_key_runs = key == g->bw_key ? g->bw_key_runs + 1 : 1;
     g->bw_key = key;
@@ -1860,71 +1978,23 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
     // graphs are small (dense ones, see bw_dense: 20 of 600 vertices and degree 120 9.4
     // -> 3.7 ms)
     const bool whole = op.deterministic || (op.batch_small_n == 0 && g->max_graph_n <= kBwMaxN);
-    const int table = op.pass_table > 0 ? std::min(op.pass_table, g->max_table) : g->max_table;
-    for (int round = 0; g->bw_count < G && round < max_rounds; ++round) {
-      const int n = g->n;
-      const long long M = g->M;
-      const int64_t* rp = g->crp();
-      const int* col = g->ccol();
-      const WT* w = (const WT*)g->cw();
-      const WT* deg = (const WT*)g->cdeg();
-      reset_round_kernel<<<1, 1, 0, s>>>(g->st);
-      ++g->launches;
-      CK(batch_round_reset(G, b, s, &g->launches));
-      { ProfScope ps(P_DEGREE, n, s);
-        CK(batch_degree_bound<WT>(n, G, deg, b, &g->st->batch_done, s, &g->launches)); }
-      { ProfScope ps(P_TILES, n, s);
-        CK(tile_rows(rp, n, M, g->tile_row, s, &g->launches)); }
-      { ProfScope ps(P_UF, n, s);
-        CK(uf_init(g->parent, n, s, &g->launches)); }
-      const BatchView v = b.view();
-      if (op.pr_mask) {
-        ProfScope ps(P_PR, M, s);
-        CK(pr_marks<WT>(n, M, rp, col, w, deg, g->tile_row, op.pr_mask, op.pr_budget, g->parent,
-                        nullptr, g->short_bits, g->st, s, &g->launches, &v));
-      }
-      if (!whole) {
-        ProfScope ps(P_CF_PASSES, M, s);
-        CK(cudaMemsetAsync(g->owner, 0, (size_t)n * sizeof(int), s));
-        PassConfig pc;
-        pc.table = table;
-        pc.warps_per_block = 4;
-        pc.passes = op.passes > 0 ? std::min(op.passes, g->max_passes)
-                                  : std::max(32, std::min(g->max_passes, n / 4));
-        pc.seed = op.seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(round + 1);
-        pc.private_visit = op.cf_visit == 1 ? 1 : 0;
-        CK(capforest_passes<WT>(n, rp, col, w, deg, g->owner, g->parent, g->visit_log, g->pass_best,
-                                g->pass_len, g->pass_counter, pc, g->st, s, &g->launches, &v));
-      }
-      { ProfScope ps(P_CF_SEQ, M, s);
-        CK(capforest_sequential_batch<WT>(G, rp, col, w, deg, g->parent, (WT*)g->seq_r,
-                                          g->batch_levels, b.level_off, g->seq_order,
-                                          g->max_graph_n, whole ? 1 : 0, v, g->st, s,
-                                          &g->launches)); }
-      { ProfScope ps(P_WITNESS, g->n0, s);
-        CK(batch_witness(G, g->n0, b, g->visit_log, table, g->pass_len, g->seq_order, g->cur_side,
-                         g->map0, g->side0, g->st, s, &g->launches)); }
-      CK(batch_collapse(n, b, g->parent, s, &g->launches));
-      stl.rounds++;
-      stl.entries_processed += M;
-      int n2 = 0;
-      long long m2 = 0;
-      int rc = contract_current<WT>(g, &n2, &m2, true);
-      if (rc) return rc;
-      CK(batch_new_offsets(G, b, g->rank, g->st, s, &g->launches));
-      std::swap(b.voff, b.voff_next);
-      CK(batch_gid(b.voff, G, n2, b.gid, s, &g->launches));
-      if (g->hst->batch_done >= G) break;
+    if (g->bw_count < G) {
+      const int rc1 = batch_rounds<WT>(g, op, whole, max_rounds, 0, &stl);
+      if (rc1) return rc1;
     }
     if (g->bw_count > 0) {
       ProfScope ps(P_BATCH_WARP, g->bw_count, s);
       // PR1 / PR2 only: on one warp the PR3 / PR4 intersections cost several
       // times the rest of a graph's solve (the pass of each round marks anyway)
-      CK(bw_solve_list(g, op.pr_mask & 3u, !op.deterministic, s, &g->launches));
+      CK(bw_solve_list(g, op.pr_mask, !op.deterministic, s, &g->launches));
     }
   }
   int rc = sync_state(g);
   if (rc) return rc;
+  if (g->hst->batch_left > 0 && op.pr_mask > 3u) {
+    rc = batch_left_over<WT>(g, op, max_rounds, &stl);
+    if (rc) return rc;
+  }
   if (g->hst->batch_done < G) return fail(MINCUT_ERR_INTERNAL, "batch did not finish in %d rounds", max_rounds);
   CK(batch_values(b.lam_g, G, g->batch_vals, s, &g->launches));
   CK(cudaMemcpyAsync(cut_values, g->batch_vals, (size_t)G * sizeof(long long), cudaMemcpyDeviceToHost, s));

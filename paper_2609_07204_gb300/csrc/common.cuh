@@ -50,6 +50,7 @@ struct DevState {
   long long tile_counter[8];   // per-pass tile counters of the radix sort
   int lambda_src;              // 1 degree, 2 LP, 3 CAPFOREST (set by the witness step)
   int batch_done;              // graphs of a batch that finished
+  int batch_left;              // graphs of a batch that the small-graph solvers gave up
   long long sym_balance;       // symmetry check: entries u < v minus entries u > v
   unsigned long long single_entries;  // contraction: entries of single-vertex groups' rows
   unsigned long long dense_entries;   // contraction: entries of dense groups' rows

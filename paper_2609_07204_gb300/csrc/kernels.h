@@ -72,12 +72,20 @@ cudaError_t batch_warp_mark(const int* list, int nlist, int* done_g, DevState* s
 // batch_warp_slot_words(nmax, mmax) ints; every listed graph has at most nmax
 // vertices and mmax entries.  cursor: one int of work-queue state.  more,
 // nmore_dev (nullable): *nmore_dev further graphs, the number on the device.
+// left (nullable): takes the graphs whose first round joins next to nothing,
+// st->batch_left of them, instead.
 cudaError_t batch_warp_solve(const int* list, int nlist, const int* more, const int* nmore_dev,
                              int* cursor, const int* voff0,
                              const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                              int slots, int nmax, int mmax, uint32_t pr_mask,
-                             unsigned long long* lam_g, uint8_t* side0, DevState* st,
+                             unsigned long long* lam_g, uint8_t* side0, int* left, DevState* st,
                              cudaStream_t s, int* launches);
+// Graphs left[0 .. nleft) open again (no bound, not done); and the other way
+// round: those not done listed in left[0 .. st->batch_left), then done.
+cudaError_t batch_reopen(const int* left, int nleft, int G, unsigned long long* lam_g, int* done_g,
+                         DevState* st, cudaStream_t s, int* launches);
+cudaError_t batch_unfinished(int G, int* done_g, int* left, DevState* st, cudaStream_t s,
+                             int* launches);
 cudaError_t batch_bitmap(const uint8_t* side0, int n0, const BatchState& b, u64* bitmap,
                          cudaStream_t s, int* launches);
 cudaError_t batch_check_edges(int n, const int64_t* rp, const int* col, const int* gid,
@@ -417,13 +425,14 @@ cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, i
 
 // A batch's graphs (at most kSmMaxN vertices each), a block per graph at a
 // time from a work queue: values and sides of those solved, the others'
-// ids in left[0 .. *nleft) for batch_warp_solve.  scratch: `slots` slots of
+// ids in few[0 .. *nfew) (too few levels for them; set to 0 here) and
+// left[0 .. *nleft) (added to).  scratch: `slots` slots of
 // slot_words >= 2 mmax + 8 words.
 cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff0,
                         const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                         long long slot_words, int slots, int nmax, int mmax, uint32_t pr_mask,
-                        unsigned long long* lam_g, uint8_t* side0, int* left, int* nleft, int sms,
-                        cudaStream_t s, int* launches);
+                        unsigned long long* lam_g, uint8_t* side0, int* few, int* nfew, int* left,
+                        int* nleft, int sms, cudaStream_t s, int* launches);
 
 // ------------------------------------------------------------- contract.cu
 // Row-wise contraction when most groups are single vertices: singleton rows

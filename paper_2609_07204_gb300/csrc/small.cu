@@ -499,6 +499,11 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     const int kcap = min(kSmMaxK, sm.fcap / n);
     if (kcap < 1) break;
     const long long qmin = (lam + kcap - 1) / kcap;
+    // too few levels for the weights: hardly an edge has a unit
+    if (qmin >= 2 * max(mean, 1ll)) {
+      limited = true;
+      break;  // bail
+    }
     // soft quantum: as few levels as the size asks for, at most half the mean
     // weight
     const long long qw = max(qmin, soft ? min((mean + 1) / 2, (lam + kSmLevels - 1) / kSmLevels) : 1ll);
@@ -796,15 +801,16 @@ __global__ void __launch_bounds__(T, 1)
 }
 
 // A batch's graphs list[0 .. nlist) (largest first), a block per graph at a
-// time: lam_g and side0 of each; those that bail go to left[0 .. *nleft).
+// time: lam_g and side0 of each; those that bail go to few[0 .. *nfew) when
+// it was for want of levels, else to left[0 .. *nleft).
 // Block b's edges: `words` words at scratch + b * slot_words.
 template <int T>
 __global__ void __launch_bounds__(T, 3)
     small_batch_kernel(const int* __restrict__ list, int nlist, int* cursor,
                        const int* __restrict__ voff0, const int64_t* rp0, const int* col0,
                        const int* w0, int* scratch, long long slot_words, int mmax, int cap,
-                       int fcap, uint32_t pr_mask, unsigned long long* lam_g, uint8_t* side0, int* left,
-                       int* nleft) {
+                       int fcap, uint32_t pr_mask, unsigned long long* lam_g, uint8_t* side0,
+                       int* few, int* nfew, int* left, int* nleft) {
   extern __shared__ __align__(16) unsigned char sm_dyn[];
   __shared__ SmShared<T> s;
   const SmMem sm = sm_mem(sm_dyn, cap, fcap);
@@ -821,13 +827,14 @@ __global__ void __launch_bounds__(T, 3)
     const int v0 = voff0[gi], n = voff0[gi + 1] - v0;
     long long lam = kInf;
     int source, rounds;
-    bool limited;
+    bool limited = true;
     const int m = sm_load<T>(sm, s, rp0, col0, w0, v0, n, ed0, half);
     const bool ok = m >= 0 && sm_solve<T>(sm, s, ed0, ed1, m, n, pr_mask, lam, source, rounds, limited);
     if (ok)
       for (int i = threadIdx.x; i < n; i += T) side0[v0 + i] = sm.side[i];
     if (threadIdx.x == 0) {
       if (ok) lam_g[gi] = (unsigned long long)lam;
+      else if (limited) few[atomicAdd(nfew, 1)] = gi;
       else left[atomicAdd(nleft, 1)] = gi;
     }
     __syncthreads();  // (the next graph reuses the block's shared memory)
@@ -903,8 +910,8 @@ static int sm_batch_fcap(int nmax) { return std::max(4096, std::min(10240, 16 * 
 cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff0,
                         const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                         long long slot_words, int slots, int nmax, int mmax, uint32_t pr_mask,
-                        unsigned long long* lam_g, uint8_t* side0, int* left, int* nleft, int sms,
-                        cudaStream_t s, int* launches) {
+                        unsigned long long* lam_g, uint8_t* side0, int* few, int* nfew, int* left,
+                        int* nleft, int sms, cudaStream_t s, int* launches) {
   if (nlist <= 0) return cudaSuccess;
   if (nmax > kSmMaxN || slots < 1) return cudaErrorInvalidValue;
   const int cap = sm_batch_cap(nmax), fcap = sm_batch_fcap(nmax);
@@ -921,11 +928,11 @@ cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff
   if (e != cudaSuccess) return e;
   const int blocks = std::min({nlist, slots, sms * std::max(1, per_sm)});
   e = cudaMemsetAsync(cursor, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(nleft, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(nfew, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   small_batch_kernel<kSmBatchThreads><<<blocks, kSmBatchThreads, bytes, s>>>(
       list, nlist, cursor, voff0, rp0, col0, w0, scratch, slot_words, mmax, cap, fcap, pr_mask, lam_g,
-      side0, left, nleft);
+      side0, few, nfew, left, nleft);
   ++*launches;
   return cudaGetLastError();
 }

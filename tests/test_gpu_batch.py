@@ -184,10 +184,10 @@ def test_batch_dense_graphs(det):
         w = rng.integers(1, 21, m)
         c = oracle.canonicalize(n, *G.from_edges(n, np.stack([u[pick], v[pick]], 1), w))
         part.append((n, *c))
-    for graphs, rounds in ((dense, True), (other, False), (other + dense, True)):
+    for graphs in (dense, other, other + dense):
         expect = [oracle.noi(*g)[0] for g in graphs]
         st = _check_batch(graphs, expect, mc.default_options(deterministic=det))
-        assert (st["rounds"] > 0) == rounds
+        assert st["rounds"] > 0 or graphs is other
     B = mc.mincut_batch_from_csr(*mc.pack_graphs(dense))
     ms = []
     for small in (0, 2048):
@@ -195,6 +195,50 @@ def test_batch_dense_graphs(det):
         ms.append(min(mc.mincut_batch_solve(B, opts)[2]["ms_total"] for _ in range(5)))
     B.destroy()
     assert ms[0] < ms[1], ms
+
+
+@pytest.mark.parametrize("det", [0, 1])
+@pytest.mark.parametrize("kind", ["wheels", "interleaved cycles", "unit cycles", "mixed"])
+def test_batch_graphs_given_up(kind, det):
+    """Graphs that the block and the warp solver give up share rounds with all
+    the PR tests, then take a warp each where those do not help; alone, among
+    ordinary ones, repeatedly (captured launches) and with fewer PR tests."""
+    graphs = []
+    if kind in ("wheels", "mixed"):
+        graphs += [synth.wheel(n, seed=n) for n in (40, 63, 64, 65, 66, 200, 301, 600)]
+    if kind in ("interleaved cycles", "mixed"):
+        graphs += [synth.dblcyc(n, seed=n) for n in (34, 66, 130)]
+    if kind == "mixed":
+        graphs += [synth.batch_graph(4, i) for i in range(40)]
+    graphs = [(s.n, s.row_ptr, s.col, s.w.astype(np.int64)) for s in graphs]
+    if kind in ("unit cycles", "mixed"):
+        graphs += [(n, *oracle.canonicalize(n, *G.cycle(n))) for n in (64, 65, 300)]
+    expect = [oracle.noi(*g)[0] for g in graphs]
+    vo, rp, col, w = mc.pack_graphs(graphs)
+    B = mc.mincut_batch_from_csr(vo, rp, col, w)
+    opts = mc.default_options(deterministic=det)
+    for _ in range(4):
+        st = _solve_and_check(B, vo, graphs, expect, opts)
+        assert st["rounds"] > 0
+    _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=1 - det))
+    for mask in (0x7, 0x3, 0):
+        _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=det, pr_mask=mask))
+    _solve_and_check(B, vo, graphs, expect, opts)
+    B.destroy()
+
+
+@pytest.mark.parametrize("det", [0, 1])
+def test_batch_of_wheels_is_no_slower_than_rounds(det):
+    """40 wheels of about 250 vertices: no more than twice the time of the
+    round kernels, which solve them in one round (60 times by warps)."""
+    graphs = [synth.wheel(230 + i, seed=i) for i in range(40)]
+    B = mc.mincut_batch_from_csr(*mc.pack_graphs([(s.n, s.row_ptr, s.col, s.w) for s in graphs]))
+    ms = []
+    for small in (0, -1):
+        opts = mc.default_options(deterministic=det, batch_small_n=small)
+        ms.append(sorted(mc.mincut_batch_solve(B, opts)[2]["ms_total"] for _ in range(7))[3])
+    B.destroy()
+    assert ms[0] < 2 * ms[1], ms
 
 
 def test_batch_rejects_cross_graph_edge_and_tiny_graph():
