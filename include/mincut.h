@@ -326,8 +326,9 @@ int mincut_release_cached(int device);
  * admitted requests stay under hbm_cap_bytes (a request alone is always
  * admitted).  A worker that takes a request with n <= pack_max_n also takes
  * the small requests queued right behind it (up to pack_max_requests and
- * pack_max_vertices; of at most 2,048 vertices, whatever pack_max_n says) and
- * solves them as one packed batch; larger requests are solved alone.  Values are exact, so a request's value does not depend
+ * pack_max_vertices) and solves them as one packed batch.  Requests of 2,049 to
+ * pack_max_n vertices are packed, apart from smaller ones, only where at least 32
+ * per worker queue in a row; other larger requests are solved alone.  Values are exact, so a request's value does not depend
  * on what it was solved with. */
 typedef struct mincut_server mincut_server;
 typedef struct mincut_server_options {

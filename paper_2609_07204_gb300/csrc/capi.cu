@@ -1866,8 +1866,8 @@ int batch_rounds(mincut_graph* g, const mincut_options& op, bool whole, int max_
 // The graphs that the block or the warp solver gave up (g->hst->batch_left of
 // them, in g->bw_left): PR1 / PR2 and one pass join next to nothing in them, so
 // they share rounds with all the PR tests while those halve them, then take a warp
-// each to the end (100 wheels of 200 to 300 vertices: 54.8 ms by warps alone, 0.84 like this; 40 pairs of interleaved cycles, which it does not
-// help, 37.3 and 37.5).
+// each to the end (100 wheels of 200 to 300 vertices: 54.8 ms by warps alone, 0.84
+// like this; 40 pairs of interleaved cycles, which it does not help, 37.3 and 37.5).
 template <typename WT>
 int batch_left_over(mincut_graph* g, const mincut_options& op, int max_rounds, mincut_stats* stl) {
   cudaStream_t s = g->stream;

@@ -149,6 +149,8 @@ void solve_packed(const mincut_server_options& o, cudaStream_t s, std::vector<Re
   }
 }
 
+constexpr int kPackRun = 32;
+
 void worker_loop(mincut_server* S, int wid) {
   (void)wid;
   cudaSetDevice(S->opt.device);
@@ -175,15 +177,28 @@ void worker_loop(mincut_server* S, int wid) {
       take.push_back(h);
       S->inflight_bytes += h->footprint;
       S->inflight += 1;
-      // packed together: what a batch solves a block per graph; beyond that a
-      // request alone (0.3 ms) is faster than its share of the round kernels
-      // (10 ms and more a batch)
-      const int64_t pack_n = std::min<int64_t>(o.pack_max_n, mc::kBwMaxN);
+      // packed together: what a batch solves a block per graph.  Larger requests
+      // share the round kernels of a batch (10 ms for 60 of 2,049 to 4,096 vertices),
+      // alone they take 0.45 ms of one worker: they are packed where each worker would
+      // have kPackRun of them to do (one worker, those 60: 27.4 -> 10.3 ms; four
+      // workers take 8 ms alone and 10 packed)
+      int64_t lo = 0, pack_n = std::min<int64_t>(o.pack_max_n, mc::kBwMaxN);
+      if (h->n > pack_n && h->n <= o.pack_max_n) {
+        size_t run = 0;
+        const size_t want = (size_t)kPackRun * o.workers - 1;
+        while (run < S->queue.size() && run < want && S->queue[run]->n > pack_n &&
+               S->queue[run]->n <= o.pack_max_n)
+          ++run;
+        if (run == want) {
+          lo = pack_n;
+          pack_n = o.pack_max_n;
+        }
+      }
       if (h->n <= pack_n && o.pack_max_requests > 1) {
         int64_t verts = h->n;
         while (!S->queue.empty() && (int)take.size() < o.pack_max_requests) {
           const ReqPtr& q = S->queue.front();
-          if (q->n > pack_n || verts + q->n > o.pack_max_vertices ||
+          if (q->n <= lo || q->n > pack_n || verts + q->n > o.pack_max_vertices ||
               S->inflight_bytes + q->footprint > o.hbm_cap_bytes)
             break;
           verts += q->n;

@@ -93,3 +93,21 @@ def test_server_borrowed_pinned_requests_equal_oracle(requests_small, oracle_val
     vals = [S.wait(i)[0] for i in ids]
     S.close()
     assert vals == oracle_values[:40]
+
+
+def test_server_packs_larger_requests_for_few_workers():
+    """Requests above the small-graph solvers' size, at most pack_max_n: packed
+    when one worker has a long run of them, not when they are few, and not
+    together with small ones."""
+    big = [synth.cycle_plus(2049 + 3 * i, 6, 1, 30, i) for i in range(120)]
+    small = [synth.cycle_plus(40 + i, 5, 1, 30, i) for i in range(8)]
+    want = [oracle.noi(g.n, g.row_ptr, g.col, g.w)[0] for g in big + small]
+    for count, packed in ((120, True), (20, False)):
+        S = mc.Server(workers=1, want_bitmap=0)
+        sub = big[:count] + small
+        ids = [S.submit(g.n, g.row_ptr, g.col, g.w) for g in sub]
+        vals = [S.wait(i, bitmap=False)[0] for i in ids]
+        st = S.stats()
+        S.close()
+        assert vals == want[:count] + want[120:]
+        assert (st["packed_requests"] > len(small)) == packed
