@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mc {
 
@@ -392,10 +393,11 @@ long long batch_warp_slot_words(int nmax, int mmax) {
 int batch_warp_block_warps() { return kBwWarps; }
 
 bool bw_set_smem() {
-  static const bool ok = cudaFuncSetAttribute(batch_warp_kernel,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kBwSmemBytes) == cudaSuccess;
-  return ok;
+  static OncePerDevice once;
+  return once([] {
+    return cudaFuncSetAttribute(batch_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kBwSmemBytes) == cudaSuccess;
+  });
 }
 
 int batch_warp_slots(int sms) {

@@ -60,6 +60,7 @@
 // and two host synchronisations; long rows (a first hub stays a vertex of its
 // own) go in pieces: by one warp each they took 346 us.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 
 #include "common.cuh"
@@ -969,14 +970,14 @@ cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64
                          const int* col, const WT* w, const WT* deg, int* parent, int* L,
                          int* flags, int* rank, long long qsoft, const SmallList* rest, int sms,
                          long long spin, DevState* st, cudaStream_t s, int* launches) {
-  static int per_sm[2] = {0, 0};
-  const int wi = sizeof(WT) == 8 ? 1 : 0;
-  if (!per_sm[wi]) {
-    int p = 0;
+  static std::atomic<int> known{0};  // (the kernel's, on any sm_103a device)
+  int per_sm = known.load(std::memory_order_relaxed);
+  if (!per_sm) {
     const cudaError_t e =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, forest_kernel<WT>, kFoThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, forest_kernel<WT>, kFoThreads, 0);
     if (e != cudaSuccess) return e;
-    per_sm[wi] = std::max(1, p);
+    per_sm = std::max(1, per_sm);
+    known.store(per_sm, std::memory_order_relaxed);
   }
   cudaError_t e = cudaMemsetAsync(f.ctl, 0, sizeof(FoCtl), s);
   if (e != cudaSuccess) return e;
@@ -1016,7 +1017,7 @@ cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64
                                 (std::max<long long>(M, n) + kFoFewPerThread * kFoThreads - 1) /
                                     (kFoFewPerThread * kFoThreads));
   const int blocks = (int)std::max<long long>(
-      1, std::min<long long>({std::max(want, few), (long long)sms * per_sm[wi], (long long)kFoMaxBlocks}));
+      1, std::min<long long>({std::max(want, few), (long long)sms * per_sm, (long long)kFoMaxBlocks}));
   void* params[] = {&a};
   e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
                                   params, 0, s);

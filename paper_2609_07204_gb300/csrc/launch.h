@@ -1,0 +1,32 @@
+// launch.h -- host helpers for launches that depend on the device or context.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <atomic>
+
+namespace mc {
+
+// What a kernel needs set up on each device before its first launch there (an
+// attribute of a function belongs to the device that is current): run at the
+// first call on a device and at any later one until it succeeds.  Threads may
+// run it side by side.
+class OncePerDevice {
+ public:
+  template <typename F>
+  bool operator()(F set_up) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
+    if (dev >= kDevices) return set_up();
+    if (done_[dev].load(std::memory_order_acquire)) return true;
+    if (!set_up()) return false;
+    done_[dev].store(true, std::memory_order_release);
+    return true;
+  }
+
+ private:
+  static constexpr int kDevices = 128;
+  std::atomic<bool> done_[kDevices] = {};
+};
+
+}  // namespace mc

@@ -32,6 +32,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mc {
 
@@ -859,10 +860,12 @@ static SmEdges sm_edges(void* p, long long mcap) {  // mcap / 2 edges
 }
 
 static bool sm_solve_attr() {
-  static const bool ok = cudaFuncSetAttribute(small_solve_kernel<kSmThreads>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)sm_bytes(kSmMaxN, kSmFcap)) == cudaSuccess;
-  return ok;
+  static OncePerDevice once;
+  return once([] {
+    return cudaFuncSetAttribute(small_solve_kernel<kSmThreads>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sm_bytes(kSmMaxN, kSmFcap)) == cudaSuccess;
+  });
 }
 
 cudaError_t small_solve(int n, const int64_t* rp, const int* col, const int* w, void* ed0,
@@ -916,12 +919,14 @@ cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff
   if (nmax > kSmMaxN || slots < 1) return cudaErrorInvalidValue;
   const int cap = sm_batch_cap(nmax), fcap = sm_batch_fcap(nmax);
   const size_t bytes = sm_bytes(cap, fcap);
-  static const bool ok = cudaFuncSetAttribute(
-                             small_batch_kernel<kSmBatchThreads>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sm_bytes(sm_batch_cap(kSmMaxN), sm_batch_fcap(kSmMaxN))) ==
-                         cudaSuccess;
-  if (!ok) return cudaErrorInvalidValue;
+  static OncePerDevice once;
+  const auto set_up = [] {
+    return cudaFuncSetAttribute(small_batch_kernel<kSmBatchThreads>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sm_bytes(sm_batch_cap(kSmMaxN), sm_batch_fcap(kSmMaxN))) ==
+           cudaSuccess;
+  };
+  if (!once(set_up)) return cudaErrorInvalidValue;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm, small_batch_kernel<kSmBatchThreads>, kSmBatchThreads, bytes);
