@@ -66,6 +66,7 @@
 #include "common.cuh"
 #include "grid_barrier.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mc {
 
@@ -1019,8 +1020,10 @@ cudaError_t forest_marks(const ForestScratch& f, int n, long long M, const int64
   const int blocks = (int)std::max<long long>(
       1, std::min<long long>({std::max(want, few), (long long)sms * per_sm, (long long)kFoMaxBlocks}));
   void* params[] = {&a};
-  e = cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(blocks), dim3(kFoThreads),
-                                  params, 0, s);
+  e = launch_fitting(blocks, [&](int fitting) {
+    return cudaLaunchCooperativeKernel((const void*)forest_kernel<WT>, dim3(fitting),
+                                       dim3(kFoThreads), params, 0, s);
+  });
   if (e != cudaSuccess) return e;
   ++*launches;
   return cudaGetLastError();

@@ -29,4 +29,16 @@ class OncePerDevice {
   std::atomic<bool> done_[kDevices] = {};
 };
 
+// A cooperative launch of at most `blocks` blocks, for a kernel that any grid
+// will do for: where the stream's context holds fewer at once than the device
+// (a partition of its SMs), the refused launch is repeated with half of them.
+template <typename F>
+cudaError_t launch_fitting(int blocks, F launch) {
+  for (;; blocks /= 2) {
+    const cudaError_t e = launch(blocks);
+    if (e != cudaErrorCooperativeLaunchTooLarge || blocks <= 1) return e;
+    cudaGetLastError();  // (the refusal is answered)
+  }
+}
+
 }  // namespace mc

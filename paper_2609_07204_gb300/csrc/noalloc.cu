@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "grid_barrier.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 using namespace mc;
 
@@ -497,8 +498,10 @@ int mincut_contract_csr_noalloc(int64_t n, const int64_t* row_ptr, const int32_t
     unsigned char bytes[kOffCtl - kOffState + sizeof(NaHead)];
   } back;
   if (cudaMemsetAsync(st, 0, kOffCtl - kOffState + sizeof(NaHead), s) != cudaSuccess ||
-      cudaLaunchCooperativeKernel((const void*)noalloc_kernel, dim3(blocks), dim3(kNaThreads),
-                                  params, 0, s) != cudaSuccess ||
+      launch_fitting(blocks, [&](int fitting) {
+        return cudaLaunchCooperativeKernel((const void*)noalloc_kernel, dim3(fitting),
+                                           dim3(kNaThreads), params, 0, s);
+      }) != cudaSuccess ||
       cudaMemcpyAsync(&back, st, sizeof(back), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return na_fail(MINCUT_ERR_CUDA, "contraction failed");

@@ -50,3 +50,25 @@ def test_set_up_runs_once_on_each_device(tmp_path):
   fake_device = 0;
   if (!once(good) || runs != 6) return 6;
 """) == 0
+
+
+def test_refused_cooperative_launches_shrink(tmp_path):
+    assert _run(tmp_path, """
+  int tried = 0, last = 0, room = 0;
+  auto launch = [&](int blocks) {
+    ++tried;
+    last = blocks;
+    return blocks <= room ? cudaSuccess : cudaErrorCooperativeLaunchTooLarge;
+  };
+  for (room = 1; room <= 400; ++room) {
+    tried = fake_cleared = 0;
+    if (mc::launch_fitting(304, launch) != cudaSuccess || last > room || last < 1) return 1;
+    if (last != 304 && 2 * last + 1 <= room) return 2;  // (halved no further than needed)
+    if (fake_cleared != tried - 1) return 3;            // (each refusal is cleared)
+  }
+  room = 0;  // not even one block
+  if (mc::launch_fitting(304, launch) != cudaErrorCooperativeLaunchTooLarge || last != 1) return 4;
+  tried = 0;  // other errors are the caller's
+  auto broken = [&](int) { ++tried; return cudaErrorInvalidValue; };
+  if (mc::launch_fitting(304, broken) != cudaErrorInvalidValue || tried != 1) return 5;
+""") == 0
