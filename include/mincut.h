@@ -81,7 +81,8 @@ typedef struct mincut_options {
     uint64_t seed;           /* start-vertex seed of the concurrent passes */
     int32_t deterministic;   /* 1: one sequential CAPFOREST pass from vertex 0 per round */
     int32_t max_rounds;      /* 0 = unlimited */
-    int64_t spin_limit;      /* iteration limit of bounded device waits (0 = default) */
+    int64_t spin_limit;      /* iteration limit of bounded device waits (0 = default); a solve
+                                whose certificate forests run into it goes on without them */
     int32_t profile;         /* 1: time every kernel with CUDA events (mincut_profile_read) */
     int32_t init_bound;      /* 0: bounds inside the rounds only (default); 1: first run the
                                 coarsening heuristic of Sec. 2.1 "Lowering the upper bound"

@@ -773,6 +773,7 @@ struct RoundOut {
   bool solved = false;     // the rest of the solve ran behind the round's forests
   int rest_rounds = 0;     // and its rounds
   int rest_left = 0;       // vertices of a rest that the one-block solver gave up (status 3)
+  bool forest_timeout = false;  // a wait of the forests ran out: the other marks ran instead
   bool forest_weak = false;  // the forests joined too little: the other marks ran too
   bool cc_ran = false;     // the concurrent passes ran (were not skipped)
   long long cf_nscanned = 0, cf_nmarks = 0;
@@ -820,6 +821,18 @@ int mark_round(mincut_graph* g, const RoundCfg& c, long long lambda_before, Roun
     }
   }
   rc = sync_state(g);
+  if (rc == MINCUT_ERR_DEVICE_TIMEOUT && forest) {
+    // spin_limit is too short for the forests' grid barriers, which wait for a
+    // whole batch (up to milliseconds): the round's other kernels do without them
+    set_last_error("");
+    CK(cudaMemsetAsync(&g->st->error, 0, sizeof(g->st->error), s));
+    rc = set_lambda(g, lambda_before);
+    if (rc) return rc;
+    RoundCfg without = c;
+    without.forest = without.small_rest = false;
+    o->forest_timeout = true;
+    return mark_round<WT>(g, without, lambda_before, o);
+  }
   if (rc) return rc;
   if (g->m_pending) {  // the previous contraction's entry count came with this sync
     g->M = g->hst->m_rows;
@@ -1178,7 +1191,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
     if (rc) return rc;
     if (o.src) stl->lambda_source = o.src;
     if (o.forest_weak) forest_below = n_before / 2;
-    if (!c.forest || o.forest_weak) lp_done = true;
+    if (o.forest_timeout) forest_below = 0;
+    if (!c.forest || o.forest_weak || o.forest_timeout) lp_done = true;
     // concurrent passes that marked almost nothing before the whole-graph
     // passes had to run: small graphs skip them in the next round
     // (and keep skipping them while those passes keep running)

@@ -232,6 +232,33 @@ def test_block_counts(m):
     _check_solve(n, c, expect=oracle.noi(n, *c)[0])
 
 
+@pytest.mark.parametrize("kind", ["cliques", "random"])
+def test_wait_that_runs_out(kind):
+    """A limit of one poll, which the grid barriers run into at once: the kernel
+    returns an error status, the solve goes on without the forests, and the
+    graph and the context stay usable."""
+    if kind == "cliques":
+        k = 100  # a ring of cliques of 25
+        n = 25 * k
+        e = [(25 * i + a, 25 * i + b) for i in range(k) for a in range(25) for b in range(a)]
+        w = [10] * len(e) + [2] * k
+        e += [(25 * i, (25 * i + 26) % n) for i in range(k)]
+        c = canon(n, *G.from_edges(n, e, w))
+    else:
+        s = synth.cycle_plus(2600, 40, 1, 1, 3)
+        n, c = s.n, (s.row_ptr, s.col, s.w.astype(np.int64))
+    expect = oracle.noi(n, *c)[0]
+    g = mc.mincut_graph_from_csr(n, *c)
+    for opts in (mc.default_options(spin_limit=1, profile=1), mc.default_options(spin_limit=1 << 22)):
+        value, bitmap, _ = mc.mincut_solve(g, opts)
+        side = mc.bitmap_to_side(bitmap, n)
+        assert value == expect and oracle.cut_weight(n, *c, side) == expect
+        assert mc.mincut_last_error() == ""
+        if opts.profile:  # tried once, and not again in the solve
+            assert mc.mincut_profile_read(g)["forest"]["launches"] == 1
+    g.destroy()
+
+
 @pytest.mark.parametrize("refused", [1, 2, 3])
 def test_allocations_refused(refused, monkeypatch):
     """The first requests of a solve refused by the caller's allocator: buffers
