@@ -283,10 +283,10 @@ def measure_batched(mc, n_graphs: int = 4096, alone: int = 256, reps: int = 3):
         graphs.append((s.n, s.row_ptr, s.col, s.w))
     vo, rp, col, w = mc.pack_graphs(graphs)
     B = mc.mincut_batch_from_csr(vo, rp, col, w)
-    mc.mincut_batch_solve(B, bitmap=False)  # first solve: times the warp-solver thresholds
+    mc.mincut_batch_solve(B, bitmap=False)
     small_n, small_graphs = mc.mincut_batch_info(B)
     paths = {}
-    for name, t in (("round_kernels_only", -1), ("one_warp_per_graph_only", 2048)):
+    for name, t in (("round_kernels_only", -1), ("small_graph_solvers_only", 2048)):
         o = mc.default_options(batch_small_n=t)
         mc.mincut_batch_solve(B, o, bitmap=False)
         tp = []

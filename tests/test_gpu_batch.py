@@ -95,6 +95,44 @@ def test_batch_warp_path_weighted_and_pr_variants():
         _check_batch(graphs, expect, mc.default_options(batch_small_n=2048, pr_mask=mask))
 
 
+def test_warp_solver_weighted_and_pr_variants():
+    """The one-warp solver itself (deterministic mode) on weighted graphs up to
+    its size limit, with and without the PR tests, against NOI; twice each, so
+    that its launches are also captured."""
+    rng = np.random.default_rng(18)
+    graphs, expect = [], []
+    for i in range(24):
+        n = int(rng.integers(100, 700)) if i % 4 else 2048
+        s = synth.cycle_plus(n, rng.uniform(4.0, 14.0), 1, 100, 300 + i)
+        graphs.append((n, s.row_ptr, s.col, s.w.astype(np.int64)))
+        expect.append(oracle.noi(*graphs[-1])[0])
+    vo, rp, col, w = mc.pack_graphs(graphs)
+    B = mc.mincut_batch_from_csr(vo, rp, col, w)
+    for mask in (0xF, 0x3, 0x1, 0x0):
+        for _ in range(2):
+            _solve_and_check(B, vo, graphs, expect, mc.default_options(
+                deterministic=1, batch_small_n=2048, pr_mask=mask))
+    B.destroy()
+
+
+def test_replay_follows_the_mode():
+    """Captured launches of the block and of the warp solver on one batch: a
+    change of mode takes the other's launches, not the captured ones."""
+    graphs, expect = [], []
+    for i in range(60):
+        s = synth.batch_graph(4, 2000 + i)
+        graphs.append((s.n, s.row_ptr, s.col, s.w.astype(np.int64)))
+        expect.append(oracle.noi(s.n, s.row_ptr, s.col, s.w)[0])
+    vo, rp, col, w = mc.pack_graphs(graphs)
+    B = mc.mincut_batch_from_csr(vo, rp, col, w)
+    launches = {0: set(), 1: set()}
+    for det in (0, 0, 0, 1, 1, 1, 0, 1, 0, 0, 0):
+        st = _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=det))
+        launches[det].add(st["kernel_launches"])
+    assert len(launches[0]) == len(launches[1]) == 1 and launches[0] != launches[1]
+    B.destroy()
+
+
 def _solve_and_check(B, vo, graphs, expect, opts):
     vals, bm, st = mc.mincut_batch_solve(B, opts)
     side_all = mc.bitmap_to_side(bm, int(vo[-1]))

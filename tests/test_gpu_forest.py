@@ -259,6 +259,24 @@ def test_wait_that_runs_out(kind):
     g.destroy()
 
 
+@pytest.mark.parametrize("kw", [dict(max_rounds=1 << 30), dict(lp_every_round=1),
+                                dict(seq_passes=2, seed=7), dict(lp_min_n=2, max_rounds=1 << 30)])
+def test_solves_without_forests(kw):
+    """Whole solves by label propagation, PR tests and the passes, which the
+    options that ask for them still reach."""
+    for s in (synth.workload_rmat_core(14, 5, 2), synth.planted(1 << 10, 21 << 10, 30, 9, 1, 11),
+              synth.cycle_plus(12_000, 7, 1, 40, 3)):
+        c = (s.row_ptr, s.col, s.w.astype(np.int64))
+        expect = oracle.noi(s.n, *c)[0]
+        _check_solve(s.n, c, mc.default_options(**kw), expect=expect)
+        g = mc.mincut_graph_from_csr(s.n, *c)
+        mc.mincut_solve(g, mc.default_options(profile=1, **kw))
+        prof = mc.mincut_profile_read(g)
+        assert "forest" not in prof and "small_solve" not in prof and "capforest_passes" in prof
+        assert "lp_sweep" in prof or s.n < 10_000 and kw.get("lp_min_n") != 2
+        g.destroy()
+
+
 @pytest.mark.parametrize("refused", [1, 2, 3])
 def test_allocations_refused(refused, monkeypatch):
     """The first requests of a solve refused by the caller's allocator: buffers
