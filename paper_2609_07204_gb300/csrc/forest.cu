@@ -107,16 +107,14 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 // join 0.09 instead of 0.2 with 512, and the whole-graph pass it then takes makes
 // the solve 7.4 ms instead of 2.9 (2 x 2^11 4.3 and 0.9, 256 the same).
 constexpr int kFoThin = 64;
-// Vertices sampled, and entries of each; fewer than 1 / kFoAble of them with a
-// unit for every level: no batch is scanned (a wheel, whose spokes have no units
-// and whose rim edges have three for eight levels: 4,097 vertices 0.65 -> 0.36
-// ms, 40,001 0.91 -> 0.61; elsewhere no change, the sample is taken beside the clearing).
-// Not "more than a unit for every level", which would also spare a wheel of unit
-// weights: that gives up R-MAT graphs whose many leaves have just enough (scale
-// 18 with a cycle through all 2.4 -> 4.3 ms).
-constexpr int kFoSample = 512;
-constexpr int kFoSampleRow = 256;
-constexpr int kFoAble = 16;
+// Units per vertex (of the sampled weights) below kFoUnits / 10 of the levels: no
+// batch is scanned, since every level takes nearly one per vertex before the next
+// gets any, and the last would join next to nothing.  0.5 on regular graphs (unit
+// cycles, tori, hypercubes) and on wheels, whose spokes have no units (4,097
+// vertices 0.65 -> 0.33 ms, 40,001 0.91 -> 0.60); below it too where many levels round much
+// away (5,000 vertices of degree 200 and weights 1 to 100 16.4 -> 13.6 ms); 0.69 on planted
+// cuts of minimum degree 30, whose first round joins a tenth to a fifth.
+constexpr int kFoUnits = 6;
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
 constexpr int kFoMaxBlocks = 1024;
@@ -126,7 +124,6 @@ struct FoCtl {
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
   int count;           // edges listed of what is left; INT_MAX: not listed
-  int able;            // sampled vertices that the last level can join
   unsigned pieces;     // pieces of long rows listed for that
   unsigned long long deg_inv;  // ~(minimum degree)
   int deg_arg_inv;     // INT_MAX - (its smallest vertex)
@@ -420,12 +417,9 @@ __device__ __noinline__ void fo_select(const FoArgs& a, int k, int b, int t, int
 // cut 2 x 2^13 with weights of 10^5 (64-bit) 24.8 -> 2.4 ms.  Half the median
 // itself, smaller on weights with a long tail, is slower there (Pareto 1.2 on
 // that cut 1.5 -> 2.6 ms: more units to insert, the same joins).
-template <typename WT>
-__device__ __forceinline__ long long fo_quantum(const WT* __restrict__ w, long long M,
-                                                long long half, unsigned* s_scan) {
-  if (M <= 0) return half;
+__device__ __forceinline__ long long fo_quantum(unsigned long long x, long long half,
+                                                unsigned* s_scan) {
   const int tid = threadIdx.x;
-  const unsigned long long x = (unsigned long long)w[tid * M / kFoThreads];
   int bits = __reduce_max_sync(FULL, 64 - __clzll((long long)x));
   if ((tid & 31) == 0) s_scan[tid >> 5] = (unsigned)bits;
   __syncthreads();
@@ -491,7 +485,9 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   const WT* __restrict__ deg = reinterpret_cast<const WT*>(a.deg);
   FoCtl* ctl = a.ctl;
   unsigned gen = 0;
-  const long long qsoft = fo_quantum<WT>(w, a.rp[n], a.qsoft, s_scan);
+  const long long M = a.rp[n];
+  const unsigned long long sample = M > 0 ? (unsigned long long)w[tid * M / kFoThreads] : 0;
+  const long long qsoft = fo_quantum(sample, a.qsoft, s_scan);
   // ---- degree bound (Sec. 2.1), and a clean round state
   const long long lam_in = (long long)*(volatile unsigned long long*)&a.st->lambda;
   unsigned long long dmin = ~0ull;
@@ -544,7 +540,22 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     s_best_batch = 0;
   }
   const int kcap = (int)min((long long)kFoMaxK, a.fcap / n);
-  if (n <= 2 || lam <= 0 || kcap < 1) {  // (the round stops)
+  bool scan = n > 2 && lam > 0 && kcap >= 1;  // (else the round stops)
+  // (the quantum, like the bound, fits the weight type)
+  const WT q = scan ? (WT)max((lam + kcap - 1) / kcap,
+                              min(qsoft, (lam + kFoLevels - 1) / kFoLevels))
+                    : (WT)1;
+  const int k = scan ? (int)((lam + q - 1) / q) : 1;
+  if (scan) {
+    // units per vertex: M / 2 edges of the sample's mean
+    const int units = __reduce_add_sync(FULL, (int)min((unsigned long long)k, sample / (unsigned long long)q));
+    if (lane == 0) s_all[wp] = units;  // (s_scan is still read)
+    __syncthreads();
+    long long sum = 0;
+    for (int i = 0; i < kFoThreads / 32; ++i) sum += s_all[i];
+    scan = 10 * sum * M >= 2ll * kFoThreads * kFoUnits * k * n;
+  }
+  if (!scan) {
     if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
     if (gtid == 0) {
       a.st->deg_val = dmin;
@@ -553,24 +564,9 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     }
     return;
   }
-  // (the quantum, like the bound, fits the weight type)
-  const WT q = (WT)max((lam + kcap - 1) / kcap, min(qsoft, (lam + kFoLevels - 1) / kFoLevels));
-  const int k = (int)((lam + q - 1) / q);
   int* F = a.F;
   uint8_t* tag = a.tag;
   int* ru = a.r;
-  // ---- a vertex that the last level joins has a unit in every level: where
-  // hardly any of a sample has as many, the forests would join next to nothing
-  for (int i = gtid >> 5; i < kFoSample; i += gsize >> 5) {
-    const int v = (int)((long long)i * n / kFoSample);
-    const long long rb = a.rp[v], re = min((long long)a.rp[v + 1], rb + kFoSampleRow);
-    int units = 0;
-    for (long long e0 = rb; e0 < re && units < k; e0 += 32) {
-      const WT c = e0 + lane < re ? w[e0 + lane] : WT(0);
-      units += __reduce_add_sync(FULL, (int)min((WT)k, q == 1 ? c : c / q));
-    }
-    if (lane == 0 && units >= k) atomicAdd(&ctl->able, 1);
-  }
   // ---- every vertex a root at every level, nothing scanned; the first batch
   // is vertex 0
   {
@@ -595,14 +591,6 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     }
   }
   if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
-  if (__ldcg(&ctl->able) * kFoAble < kFoSample) {
-    if (gtid == 0) {
-      a.st->deg_val = dmin;
-      a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
-      a.st->lambda = (unsigned long long)lam;
-    }
-    return;
-  }
   unsigned start = 0;
   int thin = 0, queued_before = 1;  // (of the thread that chooses the batch)
   int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root

@@ -208,6 +208,22 @@ def test_nothing_to_join(n):
     assert _forest_ms(n, c, 2 * (n - 2) + 2) < 0.15
 
 
+@pytest.mark.parametrize("n,deg,whi", [(2500, 150, 100), (2500, 200, 20)])
+def test_too_few_units_for_the_levels(n, deg, whi):
+    """Degrees close to the bound once the units are rounded: the last level
+    cannot join much, and no batch of the first round is scanned (2 ms and more
+    with)."""
+    s = synth.cycle_plus(n, deg, 1, whi, 3)
+    c = (s.row_ptr, s.col, s.w.astype(np.int64))
+    _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+    g = mc.mincut_graph_from_csr(n, *c)
+    ro = mc.default_options(profile=1)
+    mc.mincut_solve(g, ro)
+    prof = mc.mincut_profile_read(g)["forest"]
+    assert prof["ms"] < 0.25 * prof["launches"], prof
+    g.destroy()
+
+
 def test_small_graphs_use_several_blocks():
     """A wheel of unit weights, which the forests do not help: they stay cheap
     (0.2 ms by one block)."""
