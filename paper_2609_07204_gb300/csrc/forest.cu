@@ -106,7 +106,14 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 // small planted cuts too early: of 2 x 2^12 vertices and minimum degree 30 the forests
 // join 0.09 instead of 0.2 with 512, and the whole-graph pass it then takes makes
 // the solve 7.4 ms instead of 2.9 (2 x 2^11 4.3 and 0.9, 256 the same).
+// Until a frontier has once been wide (a kFoWideDiv-th of the vertices, at most
+// kFoWide), that is the limit: discs in the plane and balls in a 3-d grid grow by less than
+// half beyond a few dozen vertices (50,000 points of degree 12 and weights 1 to 30, whole solve,
+// 2.4 -> 0.65 ms; grid of 40^3 and weights 1 to 20 1.8 -> 0.73; 3,000 points 0.84 -> 0.32,
+// with a 16th as the limit 0.84).
 constexpr int kFoThin = 64;
+constexpr int kFoWideDiv = 8;
+constexpr int kFoWide = 2048;
 // Units per vertex (of the sampled weights) below kFoUnits / 10 of the levels: no
 // batch is scanned, since every level takes nearly one per vertex before the next
 // gets any, and the last would join next to nothing.  0.5 on regular graphs (unit
@@ -592,7 +599,9 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   }
   if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
   unsigned start = 0;
-  int thin = 0, queued_before = 1;  // (of the thread that chooses the batch)
+  // (of the thread that chooses the batch)
+  int thin = 0, queued_before = 1, wide = 0;
+  const int wide_from = min(max(n / kFoWideDiv, kFoThin), kFoWide);
   int rep = -1, main_root = -1;  // a vertex of the main component of the last level, its root
   for (int b = 1;; ++b) {
     if (b > 1) {
@@ -617,7 +626,9 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
           }
           // a frontier that stays thin never fills a batch: everything left
           const int queued = left - s_all[0];
-          thin = queued < kFoThin && 2 * queued < 3 * queued_before ? thin + 1 : 0;
+          wide = max(wide, queued);
+          const int limit = wide < wide_from ? wide_from : kFoThin;
+          thin = queued < limit && 2 * queued < 3 * queued_before ? thin + 1 : 0;
           queued_before = queued;
           if (acc == 0 || thin >= 2 || k == 1 || b >= kFoBatches) t = 0;
           s_t = t;

@@ -199,6 +199,23 @@ def test_thin_frontiers(name, limit):
     assert _forest_ms(n, canon(n, *g), expect) < limit
 
 
+def _cube(a, rng):
+    """Periodic a x a x a grid, weights 1 to 20."""
+    i = np.arange(a ** 3).reshape(a, a, a)
+    e = np.concatenate([np.stack([i.ravel(), np.roll(i, -1, d).ravel()], 1) for d in range(3)])
+    p = rng.permutation(a ** 3)
+    return a ** 3, G.from_edges(a ** 3, p[e], [int(x) for x in rng.integers(1, 21, len(e))])
+
+
+@pytest.mark.parametrize("a,limit", [(15, 0.6), (40, 0.9)])
+def test_frontiers_that_grow_slowly(a, limit):
+    """Balls in a 3-d grid: frontiers of hundreds that grow by less than half
+    (0.8 and 1.5 ms by batches)."""
+    n, g = _cube(a, np.random.default_rng(6))
+    c = canon(n, *g)
+    assert _forest_ms(n, c, oracle.noi(n, *c)[0]) < limit
+
+
 @pytest.mark.parametrize("n", [2050, 4097, 40_001])
 def test_nothing_to_join(n):
     """A wheel's spokes have no units and its rim too few for the last level:
