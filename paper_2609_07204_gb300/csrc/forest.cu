@@ -114,13 +114,25 @@ constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
 constexpr int kFoThin = 64;
 constexpr int kFoWideDiv = 8;
 constexpr int kFoWide = 2048;
-// Units per vertex (of the sampled weights) below kFoUnits / 10 of the levels: no
-// batch is scanned, since every level takes nearly one per vertex before the next
-// gets any, and the last would join next to nothing.  0.5 on regular graphs (unit
-// cycles, tori, hypercubes) and on wheels, whose spokes have no units (4,097
-// vertices 0.65 -> 0.33 ms, 40,001 0.91 -> 0.60); below it too where many levels round much
-// away (5,000 vertices of degree 200 and weights 1 to 100 16.4 -> 13.6 ms); 0.69 on planted
-// cuts of minimum degree 30, whose first round joins a tenth to a fifth.
+// Vertices sampled, and entries of each; fewer than 1 / kFoAble of them with a
+// unit for every level, which a vertex that the last level joins has: no batch is
+// scanned (a wheel, whose spokes have no units and whose rim edges have three for
+// eight levels: 4,097 vertices 0.65 -> 0.36 ms, 40,001 0.91 -> 0.61; elsewhere no
+// change, the sample is taken beside the clearing).  Not "more than a unit for
+// every level", which would also spare a wheel of unit weights: that gives up
+// R-MAT graphs whose many leaves have just enough (scale 18 with a cycle through
+// all 2.4 -> 4.3 ms).
+constexpr int kFoSample = 512;
+constexpr int kFoSampleRow = 256;
+constexpr int kFoAble = 16;
+// None either where at least kFoManyLevels levels are asked for and there are
+// (by the sampled weights) units per vertex for fewer than kFoUnits / 10 of them: every level
+// takes nearly one per vertex before the next gets any, the last joins next to nothing,
+// and many levels cost milliseconds (5,000 vertices of degree 200 and weights 1
+// to 100 16.4 -> 13.6 ms).  Not with few levels: on graphs as near to regular whose
+// minimum cut is a prefix cut, that lowers the bound and the forests join nearly all
+// (two random 30-regular graphs of 50,000 vertices joined by 9 edges: 2.5 ms, 108 without).
+constexpr int kFoManyLevels = 128;
 constexpr int kFoUnits = 6;
 constexpr unsigned kFoMain = 128; // tag bit: known to be in the main component of F_{k-1}
 
@@ -131,6 +143,7 @@ struct FoCtl {
   unsigned items;      // work items listed so far
   unsigned main;       // 1 + a vertex of the main component of F_{k-1} (0: none yet)
   int count;           // edges listed of what is left; INT_MAX: not listed
+  int able;            // sampled vertices that the last level can join
   unsigned pieces;     // pieces of long rows listed for that
   unsigned long long deg_inv;  // ~(minimum degree)
   int deg_arg_inv;     // INT_MAX - (its smallest vertex)
@@ -553,7 +566,7 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
                               min(qsoft, (lam + kFoLevels - 1) / kFoLevels))
                     : (WT)1;
   const int k = scan ? (int)((lam + q - 1) / q) : 1;
-  if (scan) {
+  if (scan && k >= kFoManyLevels) {
     // units per vertex: M / 2 edges of the sample's mean
     const int units = __reduce_add_sync(FULL, (int)min((unsigned long long)k, sample / (unsigned long long)q));
     if (lane == 0) s_all[wp] = units;  // (s_scan is still read)
@@ -574,6 +587,17 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   int* F = a.F;
   uint8_t* tag = a.tag;
   int* ru = a.r;
+  // ---- vertices with a unit for every level, of a sample
+  for (int i = gtid >> 5; i < kFoSample; i += gsize >> 5) {
+    const int v = (int)((long long)i * n / kFoSample);
+    const long long rb = a.rp[v], re = min((long long)a.rp[v + 1], rb + kFoSampleRow);
+    int units = 0;
+    for (long long e0 = rb; e0 < re && units < k; e0 += 32) {
+      const WT c = e0 + lane < re ? w[e0 + lane] : WT(0);
+      units += __reduce_add_sync(FULL, (int)min((WT)k, q == 1 ? c : c / q));
+    }
+    if (lane == 0 && units >= k) atomicAdd(&ctl->able, 1);
+  }
   // ---- every vertex a root at every level, nothing scanned; the first batch
   // is vertex 0
   {
@@ -598,6 +622,14 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
     }
   }
   if (!grid_barrier(&ctl->bar, ++gen, a.spin, &s_ok, a.st)) return;
+  if (__ldcg(&ctl->able) * kFoAble < kFoSample) {
+    if (gtid == 0) {
+      a.st->deg_val = dmin;
+      a.st->deg_arg = INT_MAX - ctl->deg_arg_inv;
+      a.st->lambda = (unsigned long long)lam;
+    }
+    return;
+  }
   unsigned start = 0;
   // (of the thread that chooses the batch)
   int thin = 0, queued_before = 1, wide = 0;

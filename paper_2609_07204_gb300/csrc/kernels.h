@@ -370,7 +370,7 @@ cudaError_t capforest_warp_passes(int n, long long M, const int64_t* rp, const i
 // with `rest`, when 2 to kSmMaxN labels are left, the list of the edges
 // between them (*forest_count edges, above rest->cap when they do not fit,
 // INT_MAX when there is no list).  Without joins and labels when n <= 2, the
-// bound is 0 or there are too few units per vertex for the levels.  Its grid barriers wait at most `spin` reads (ERR_TIMEOUT).
+// bound is 0 or the last level could join next to nothing.  Its grid barriers wait at most `spin` reads (ERR_TIMEOUT).
 struct ForestScratch {
   int* F;          // fcap ints, at least 2 per vertex
   long long fcap;

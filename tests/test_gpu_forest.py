@@ -225,6 +225,22 @@ def test_nothing_to_join(n):
     assert _forest_ms(n, c, 2 * (n - 2) + 2) < 0.15
 
 
+@pytest.mark.parametrize("d,n,cross", [(4, 8000, 1), (10, 5000, 5), (30, 3000, 9)])
+def test_cut_between_regular_graphs(d, n, cross):
+    """Two random regular graphs, degrees at the bound: a prefix cut is the
+    minimum cut, and the forests need no whole-graph pass after it."""
+    rng = np.random.default_rng(d)
+    e = []
+    for half in (0, n):
+        for _ in range(d // 2):
+            p = half + rng.permutation(n)
+            e.append(np.stack([p, np.roll(p, 1)], 1))
+    e.append(np.stack([rng.integers(0, n, cross), n + rng.integers(0, n, cross)], 1))
+    c = canon(2 * n, *G.from_edges(2 * n, np.concatenate(e)))
+    st = _check_solve(2 * n, c, expect=oracle.noi(2 * n, *c)[0])
+    assert st["seq_passes"] == 0
+
+
 @pytest.mark.parametrize("n,deg,whi", [(2500, 150, 100), (2500, 200, 20)])
 def test_too_few_units_for_the_levels(n, deg, whi):
     """Degrees close to the bound once the units are rounded: the last level
