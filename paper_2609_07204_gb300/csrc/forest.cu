@@ -429,17 +429,20 @@ __device__ __noinline__ void fo_select(const FoArgs& a, int k, int b, int t, int
         }
 }
 
-// The quantum that loses little of the weights: half the mean (`half`), and
-// where a typical weight (the median of a sample, the same in every block) is
-// larger, at most the part that divides it evenly.  Just above half of weights
-// that are nearly all alike, as half their mean is with a few heavier ones
-// among them, it drops half of each and the last level joins nothing: planted
-// cut 2 x 2^13 with weights of 10^5 (64-bit) 24.8 -> 2.4 ms.  Half the median
-// itself, smaller on weights with a long tail, is slower there (Pareto 1.2 on
-// that cut 1.5 -> 2.6 ms: more units to insert, the same joins).
+// The quantum that loses little of the weights: half the mean (`half`).  Just
+// above half of weights that are nearly all alike, as half their mean is with a few
+// heavier ones among them, that drops half of each and the last level joins
+// nothing; so where most of a sample (the same in every block) lose 3 tenths and more
+// of themselves, the quantum divides the median of it evenly instead, if that is
+// larger: planted cut 2 x 2^13 with weights of 10^5 (64-bit) 24.8 -> 2.4 ms.  Not
+// always: finer quanta mean more units to insert for the same joins (two 10-regular
+// graphs of 20,000 with weights 1 to 5 0.97 -> 1.34 ms so; Pareto 1.2 weights on the
+// planted cut 1.5 -> 2.6 ms by half the median).
 __device__ __forceinline__ long long fo_quantum(unsigned long long x, long long half,
                                                 unsigned* s_scan) {
   const int tid = threadIdx.x;
+  if (__syncthreads_count((x % (unsigned long long)half) * 10 >= 3 * x) * 10 < 6 * kFoThreads)
+    return half;
   int bits = __reduce_max_sync(FULL, 64 - __clzll((long long)x));
   if ((tid & 31) == 0) s_scan[tid >> 5] = (unsigned)bits;
   __syncthreads();
