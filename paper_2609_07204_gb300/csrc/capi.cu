@@ -227,8 +227,8 @@ struct mincut_graph {
   int* bw_list = nullptr;     // graph ids, most entries first, the tiny ones (bw_tiny) behind
   int bw_count = 0, bw_big = 0, bw_nmax = 0, bw_mmax = 0;
   int* bw_cursor = nullptr;    // work queues of the block and the warp solver, then the number
-                               // of graphs with too few levels for the block solver
-  int* bw_left = nullptr;      // graphs given up (st->batch_left), then, from G on, the latter
+                               // of graphs that the former left
+  int* bw_left = nullptr;      // graphs given up (st->batch_left), then, from G on, those
   int* bw_scratch = nullptr;
   long long bw_scratch_words = 0;
   int bw_slots = 0;
@@ -1750,9 +1750,11 @@ int bw_prepare(mincut_graph* g, int threshold, bool dense_out) {
 }
 
 // The listed small graphs: a block per graph (small.cu), then a warp for each of
-// the tiny ones and of those with too few levels for a block; in the deterministic
-// mode all of them one warp each.  Those given up are left to batch_left_over
-// (st->batch_left) where pr has PR3 or PR4, else a warp solves them too.
+// the tiny ones and of those the blocks left; in the deterministic mode all of them
+// one warp each.  Those whose first round there joins next to nothing, too, are
+// left to batch_left_over (st->batch_left) where pr has PR3 or PR4.  (Not those
+// the blocks left at once: its rounds read the whole batch, 1 ms for 4,096 graphs,
+// of which now and then one is left.)
 cudaError_t bw_solve_list(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s,
                           int* launches) {
   BatchState& b = g->batch;
@@ -1762,18 +1764,18 @@ cudaError_t bw_solve_list(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_
                             g->bw_nmax, g->bw_mmax, pr & 3u, b.lam_g, g->side0,
                             pr > 3u ? g->bw_left : nullptr, g->st, s, launches);
   const int tiny = g->bw_count - g->bw_big;
-  int* few = g->bw_left + b.G;
+  int* more = g->bw_left + b.G;
   cudaError_t e = small_batch(g->bw_list, g->bw_big, g->bw_cursor, b.voff0, g->rp0, g->col0,
                               (const int*)g->w0, g->bw_scratch,
                               batch_warp_slot_words(g->bw_nmax, g->bw_mmax), g->bw_slots,
-                              g->bw_nmax, g->bw_mmax, pr & 3u, b.lam_g, g->side0, few,
-                              g->bw_cursor + 2, pr > 3u ? g->bw_left : few,
-                              pr > 3u ? &g->st->batch_left : g->bw_cursor + 2, g->sms, s, launches);
+                              g->bw_nmax, g->bw_mmax, pr & 3u, b.lam_g, g->side0, more,
+                              g->bw_cursor + 2, g->sms, s, launches);
   if (e == cudaSuccess)
-    e = batch_warp_solve(g->bw_list + g->bw_big, tiny, few,
+    e = batch_warp_solve(g->bw_list + g->bw_big, tiny, more,
                          g->bw_big ? g->bw_cursor + 2 : nullptr, g->bw_cursor + 1, b.voff0, g->rp0,
                          g->col0, (const int*)g->w0, g->bw_scratch, g->bw_slots, g->bw_nmax,
-                         g->bw_mmax, pr & 3u, b.lam_g, g->side0, nullptr, g->st, s, launches);
+                         g->bw_mmax, pr & 3u, b.lam_g, g->side0,
+                         pr > 3u ? g->bw_left : nullptr, g->st, s, launches);
   return e;
 }
 
@@ -1877,11 +1879,11 @@ int batch_rounds(mincut_graph* g, const mincut_options& op, bool whole, int max_
   return MINCUT_OK;
 }
 
-// The graphs that the block or the warp solver gave up (g->hst->batch_left of
-// them, in g->bw_left): PR1 / PR2 and one pass join next to nothing in them, so
+// The graphs that the warp solver gave up (g->hst->batch_left of them, in
+// g->bw_left): PR1 / PR2 and one pass join next to nothing in them, so
 // they share rounds with all the PR tests while those halve them, then take a warp
-// each to the end (100 wheels of 200 to 300 vertices: 54.8 ms by warps alone, 0.84
-// like this; 40 pairs of interleaved cycles, which it does not help, 37.3 and 37.5).
+// each to the end (100 wheels of 200 to 300 vertices: 54.8 ms by warps alone, 1.08
+// like this; 40 pairs of interleaved cycles, which it does not help, 37.3 and 38.2).
 template <typename WT>
 int batch_left_over(mincut_graph* g, const mincut_options& op, int max_rounds, mincut_stats* stl) {
   cudaStream_t s = g->stream;

@@ -425,14 +425,13 @@ cudaError_t small_side(const uint8_t* cur_side, const int* map0, const int* L, i
 
 // A batch's graphs (at most kSmMaxN vertices each), a block per graph at a
 // time from a work queue: values and sides of those solved, the others'
-// ids in few[0 .. *nfew) (too few levels for them; set to 0 here) and
-// left[0 .. *nleft) (added to).  scratch: `slots` slots of
+// ids in left[0 .. *nleft).  scratch: `slots` slots of
 // slot_words >= 2 mmax + 8 words.
 cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff0,
                         const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                         long long slot_words, int slots, int nmax, int mmax, uint32_t pr_mask,
-                        unsigned long long* lam_g, uint8_t* side0, int* few, int* nfew, int* left,
-                        int* nleft, int sms, cudaStream_t s, int* launches);
+                        unsigned long long* lam_g, uint8_t* side0, int* left, int* nleft, int sms,
+                        cudaStream_t s, int* launches);
 
 // ------------------------------------------------------------- contract.cu
 // Row-wise contraction when most groups are single vertices: singleton rows

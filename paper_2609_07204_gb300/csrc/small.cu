@@ -49,6 +49,7 @@ constexpr int kSmFrac = 4;      // a batch takes at least 1 / kSmFrac of the ver
 // weights of 1 to 100 57.4 -> 3.2 ms, a ring of 3,000 cliques of 8 141 -> 22; with
 // 1 / 32 a cycle of 5,000 4.3 instead of 2.8).
 constexpr int kSmSlow = 8;      // a round joins at least 1 / kSmSlow of the vertices,
+constexpr int kSmSlowBatch = 32;  // in a batch, where the warp solver comes after, of them,
 constexpr int kSmSlowMin = 64;  // of fewer than kSmSlowMin any
 constexpr int kSmThin = 32;     // twice in a row fewer vertices queued, and less than half as many
                                 // again as before: everything left is one batch (see kFoThin;
@@ -689,7 +690,7 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
       n2 += total;
       __syncthreads();
     }
-    if (!lowered && n - n2 < (n < kSmSlowMin ? 1 : n / kSmSlow)) {
+    if (!lowered && n - n2 < (n < kSmSlowMin ? 1 : n / (T > 256 ? kSmSlow : kSmSlowBatch))) {
       // (a finer quantum does not help where a thin frontier and PR joined nothing)
       if (!soft || q == qmin || (thin >= 2 && pr_mask && n2 == n)) {
         limited = qmin > (mean + 1) / 2;
@@ -802,8 +803,7 @@ __global__ void __launch_bounds__(T, 1)
 }
 
 // A batch's graphs list[0 .. nlist) (largest first), a block per graph at a
-// time: lam_g and side0 of each; those that bail go to few[0 .. *nfew) when
-// it was for want of levels, else to left[0 .. *nleft).
+// time: lam_g and side0 of each; those that bail go to left[0 .. *nleft).
 // Block b's edges: `words` words at scratch + b * slot_words.
 template <int T>
 __global__ void __launch_bounds__(T, 3)
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(T, 3)
                        const int* __restrict__ voff0, const int64_t* rp0, const int* col0,
                        const int* w0, int* scratch, long long slot_words, int mmax, int cap,
                        int fcap, uint32_t pr_mask, unsigned long long* lam_g, uint8_t* side0,
-                       int* few, int* nfew, int* left, int* nleft) {
+                       int* left, int* nleft) {
   extern __shared__ __align__(16) unsigned char sm_dyn[];
   __shared__ SmShared<T> s;
   const SmMem sm = sm_mem(sm_dyn, cap, fcap);
@@ -835,7 +835,6 @@ __global__ void __launch_bounds__(T, 3)
       for (int i = threadIdx.x; i < n; i += T) side0[v0 + i] = sm.side[i];
     if (threadIdx.x == 0) {
       if (ok) lam_g[gi] = (unsigned long long)lam;
-      else if (limited) few[atomicAdd(nfew, 1)] = gi;
       else left[atomicAdd(nleft, 1)] = gi;
     }
     __syncthreads();  // (the next graph reuses the block's shared memory)
@@ -913,8 +912,8 @@ static int sm_batch_fcap(int nmax) { return std::max(4096, std::min(10240, 16 * 
 cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff0,
                         const int64_t* rp0, const int* col0, const int* w0, int* scratch,
                         long long slot_words, int slots, int nmax, int mmax, uint32_t pr_mask,
-                        unsigned long long* lam_g, uint8_t* side0, int* few, int* nfew, int* left,
-                        int* nleft, int sms, cudaStream_t s, int* launches) {
+                        unsigned long long* lam_g, uint8_t* side0, int* left, int* nleft, int sms,
+                        cudaStream_t s, int* launches) {
   if (nlist <= 0) return cudaSuccess;
   if (nmax > kSmMaxN || slots < 1) return cudaErrorInvalidValue;
   const int cap = sm_batch_cap(nmax), fcap = sm_batch_fcap(nmax);
@@ -933,11 +932,11 @@ cudaError_t small_batch(const int* list, int nlist, int* cursor, const int* voff
   if (e != cudaSuccess) return e;
   const int blocks = std::min({nlist, slots, sms * std::max(1, per_sm)});
   e = cudaMemsetAsync(cursor, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(nfew, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(nleft, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   small_batch_kernel<kSmBatchThreads><<<blocks, kSmBatchThreads, bytes, s>>>(
       list, nlist, cursor, voff0, rp0, col0, w0, scratch, slot_words, mmax, cap, fcap, pr_mask, lam_g,
-      side0, few, nfew, left, nleft);
+      side0, left, nleft);
   ++*launches;
   return cudaGetLastError();
 }

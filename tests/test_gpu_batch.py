@@ -265,6 +265,16 @@ def test_batch_graphs_given_up(kind, det):
     B.destroy()
 
 
+def test_ordinary_graphs_take_no_shared_rounds():
+    """What the blocks leave of an ordinary batch a warp each finishes: rounds
+    over the whole batch would cost more than all the rest."""
+    graphs = [synth.batch_graph(4, 5000 + i) for i in range(1200)]
+    B = mc.mincut_batch_from_csr(*mc.pack_graphs([(s.n, s.row_ptr, s.col, s.w) for s in graphs]))
+    for _ in range(8):
+        assert mc.mincut_batch_solve(B, bitmap=False)[2]["rounds"] == 0
+    B.destroy()
+
+
 @pytest.mark.parametrize("det", [0, 1])
 def test_batch_of_wheels_is_no_slower_than_rounds(det):
     """40 wheels of about 250 vertices: no more than twice the time of the
