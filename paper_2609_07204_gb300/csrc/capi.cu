@@ -1162,7 +1162,8 @@ int exact_rounds(mincut_graph* g, const mincut_options& op, RoundCfg c, bool lp_
         stl->entries_processed += g->m_pending ? g->hst->m_rows : g->M;
         break;
       }
-      small_below = g->n / kSmallRetryDiv;
+      // (with half the vertices there are twice the levels)
+      small_below = g->n / (g->hst->small_status == 3 ? kSmallRetryDiv : 2);
       if (g->hst->small_status == 3) forest_below = small_below;
     }
     if (op.cf_visit == 2) {

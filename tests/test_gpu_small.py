@@ -120,6 +120,22 @@ def test_given_up_once(n):
     g.destroy()
 
 
+def test_too_few_levels():
+    """A dense small graph: the block solver has too few levels for it and the
+    forests too few units per level, both see so at once, and the block solver
+    takes over when half the vertices are left."""
+    s = synth.cycle_plus(500, 200, 1, 20, 5)
+    c = _graph(s)
+    _check_solve(s.n, c, expect=oracle.noi(s.n, *c)[0])
+    g = mc.mincut_graph_from_csr(s.n, *c)
+    mc.mincut_solve(g)
+    mc.mincut_solve(g, mc.default_options(profile=1))
+    prof = mc.mincut_profile_read(g)
+    g.destroy()
+    assert prof["forest"]["launches"] == 1 and prof["forest"]["ms"] < 0.25, prof
+    assert prof["small_solve"]["launches"] == 2, prof
+
+
 @pytest.mark.parametrize("kind", ["wheel", "unit cycle", "ladder"])
 def test_thin_and_slow_in_a_batch(kind):
     """The same graphs in a batch, where what the block solver gives up goes to
