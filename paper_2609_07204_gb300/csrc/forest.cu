@@ -93,25 +93,25 @@ constexpr int kFoLevels = 8;      // levels wanted where the weights allow it (q
 constexpr int kFoBatches = 100;   // from this batch on, everything left is one batch
 constexpr int kFoFrac = 12;       // a batch takes at least 1 / kFoFrac of the vertices left,
 constexpr int kFoTail = 64;       // and at least 1 / kFoTail of all
-// Twice in a row fewer than kFoThin vertices queued and less than half as many
-// again as before: a frontier that does not grow like this one (a cycle's, a
-// wheel's rim, a grid's) pays 12 to 20 us a batch for a few vertices until
-// kFoBatches; all at once, the forests of such sparse graphs join as much.
-// Whole solves: torus of 300 x 300 and weights 1 to 50, 2.64 -> 0.79 ms (0.86
-// without forests), grid of 300 x 300 2.37 -> 0.86, wheel of 4,097 1.84 -> 0.65.
-// Scanning a 64th, a 16th or a quarter of the vertices first, to go on from
-// many places, is slower (that grid 1.41, 1.29 and 1.13).  With one level
-// there is no order to keep: a tree of 50,000 0.89 -> 0.29.  A larger limit does
-// no more for these, whose frontiers are far below it, and ends the batching of
-// small planted cuts too early: of 2 x 2^12 vertices and minimum degree 30 the forests
-// join 0.09 instead of 0.2 with 512, and the whole-graph pass it then takes makes
-// the solve 7.4 ms instead of 2.9 (2 x 2^11 4.3 and 0.9, 256 the same).
-// Until a frontier has once been wide (a kFoWideDiv-th of the vertices, at most
-// kFoWide), that is the limit: discs in the plane and balls in a 3-d grid grow by less than
-// half beyond a few dozen vertices (50,000 points of degree 12 and weights 1 to 30, whole solve,
-// 2.4 -> 0.65 ms; grid of 40^3 and weights 1 to 20 1.8 -> 0.73; 3,000 points 0.84 -> 0.32,
-// with a 16th as the limit 0.84).
+// A frontier that hardly grows (a cycle's, a wheel's rim, a grid's, a ball's in the
+// plane or in space) pays 12 to 20 us a batch for a few vertices until kFoBatches;
+// all at once, the forests of such graphs join as much.  So everything left is one batch
+// after two in a row that queue less than half as many again as the one before,
+// until the queue has once held a kFoWideDiv-th of the vertices (at least kFoThin,
+// at most kFoWide).  Whole solves: torus of 300 x 300 and weights 1 to 50 2.64 -> 0.79 ms
+// (0.86 without forests), grid of 300 x 300 2.37 -> 0.86 (1.77), grid of 40^3 and
+// weights 1 to 20 1.8 -> 0.73 (1.07), 50,000 points of degree 12 2.4 -> 0.65 (0.82),
+// 3,000 points 0.84 -> 0.32 (0.43; with a 16th for the 8th 0.84).  Scanning a 64th, a
+// 16th or a quarter of the vertices first, to go on from many places, is slower
+// (that 300 x 300 grid 1.41, 1.29 and 1.13).  With one level there is no order to
+// keep: a tree of 50,000 0.89 -> 0.29.
+// Once the queue has been wide it takes kFoThinLate in a row below kFoThin: a scanned
+// region's last vertices come in small batches, too, and their prefix cuts lower
+// the bound (planted cut 2 x 5,000 with Pareto 1.5 weights 0.80 ms, 1.54 when two were
+// enough).  Nor is a larger kFoThin of use: with 256 and 512 the forests of small planted
+// cuts (2 x 2^11, 2 x 2^12) join 0.09 instead of 0.2 and need whole-graph passes.
 constexpr int kFoThin = 64;
+constexpr int kFoThinLate = 6;
 constexpr int kFoWideDiv = 8;
 constexpr int kFoWide = 2048;
 // Vertices sampled, and entries of each; fewer than 1 / kFoAble of them with a
@@ -662,10 +662,10 @@ __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
           // a frontier that stays thin never fills a batch: everything left
           const int queued = left - s_all[0];
           wide = max(wide, queued);
-          const int limit = wide < wide_from ? wide_from : kFoThin;
-          thin = queued < limit && 2 * queued < 3 * queued_before ? thin + 1 : 0;
+          const bool narrow = wide < wide_from;
+          thin = queued < (narrow ? wide_from : kFoThin) && 2 * queued < 3 * queued_before ? thin + 1 : 0;
           queued_before = queued;
-          if (acc == 0 || thin >= 2 || k == 1 || b >= kFoBatches) t = 0;
+          if (acc == 0 || thin >= (narrow ? 2 : kFoThinLate) || k == 1 || b >= kFoBatches) t = 0;
           s_t = t;
           s_left = left;
         }

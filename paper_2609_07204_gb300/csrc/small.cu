@@ -47,13 +47,16 @@ constexpr int kSmFrac = 4;      // a batch takes at least 1 / kSmFrac of the ver
 // whole-graph passes join up to one vertex each: cycles whose weights are all
 // equal by now lose one vertex a round here (a cycle of 50,000 vertices with
 // weights of 1 to 100 57.4 -> 3.2 ms, a ring of 3,000 cliques of 8 141 -> 22; with
-// 1 / 32 a cycle of 5,000 4.3 instead of 2.8).
-constexpr int kSmSlow = 8;      // a round joins at least 1 / kSmSlow of the vertices,
+// 1 / 32 a cycle of 5,000 4.3 instead of 2.8).  Two such rounds in a row: what
+// little the first joins may lower the next degree bound (a random 3-regular graph of
+// 1,500 with a few doubled edges 0.47 ms, 2.6 when one was enough).
+constexpr int kSmSlow = 8;      // one of two rounds joins at least 1 / kSmSlow of the vertices,
 constexpr int kSmSlowBatch = 32;  // in a batch, where the warp solver comes after, of them,
 constexpr int kSmSlowMin = 64;  // of fewer than kSmSlowMin any
 constexpr int kSmThin = 32;     // twice in a row fewer vertices queued, and less than half as many
                                 // again as before: everything left is one batch (see kFoThin;
                                 // wheel of 1,025 766 -> 429 us, with both 380)
+constexpr int kSmThinLate = 6;  // (six times once it has been wider)
 constexpr int kSmBatches = 32;  // from this batch on, everything left is one batch
 
 // Shared memory of a block, for graphs of up to `cap` vertices.
@@ -459,7 +462,7 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   long long lam = lam_io;
   int n = n0, cur = 0;
-  bool soft = true;
+  bool soft = true, slow = false;
   source = 0;
   rounds = 0;
   limited = false;
@@ -526,7 +529,7 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
     if (lane == 0) s.part[wp] = wp == 0 ? sm.deg[0] : 0;
     __syncthreads();
     long long best_alpha = kInf;
-    int thin = 0, queued_before = 1;
+    int thin = 0, queued_before = 1, widest = 0;
     int best_batch = 0;
     for (int b = 1;; ++b) {
       if (b > 1) {
@@ -541,9 +544,10 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
           left = sm_count<T>(sm, n, 0);
           queued = sm_count<T>(sm, n, 1);
         }
+        widest = max(widest, queued);
         thin = queued < kSmThin && 2 * queued < 3 * queued_before ? thin + 1 : 0;
         queued_before = queued;
-        if (thin >= 2) {
+        if (thin >= (widest < kSmThin ? 2 : kSmThinLate)) {
           t = 0;
         } else if (!fast) {
           if (left > 0 && b < kSmBatches && queued > 0) {
@@ -692,9 +696,14 @@ __device__ bool sm_solve(const SmMem& sm, SmShared<T>& s, SmEdges ed0, SmEdges e
       n2 += total;
       __syncthreads();
     }
-    if (!lowered && n - n2 < (n < kSmSlowMin ? 1 : n / (T > 256 ? kSmSlow : kSmSlowBatch))) {
+    const int least = n < kSmSlowMin ? 1 : n / (T > 256 ? kSmSlow : kSmSlowBatch);
+    if (lowered || n - n2 >= least) {
+      slow = false;
+    } else if (n2 < n && !slow) {
+      slow = true;  // (what little it joined may lower the next degree bound)
+    } else {
       // (a finer quantum does not help where a thin frontier and PR joined nothing)
-      if (!soft || q == qmin || (thin >= 2 && pr_mask && n2 == n)) {
+      if (!soft || q == qmin || (widest < kSmThin && thin >= 2 && pr_mask && n2 == n)) {
         limited = qmin > (mean + 1) / 2;
         break;  // bail
       }

@@ -120,6 +120,20 @@ def test_given_up_once(n):
     g.destroy()
 
 
+def test_one_slow_round():
+    """A 3-regular graph with a few doubled edges: PR2 joins only their ends,
+    and the next degree bound is the minimum cut; no whole-graph pass is needed."""
+    n = 1500
+    rng = np.random.default_rng(5)
+    p, q = rng.permutation(n), rng.permutation(n)
+    pair = np.sort(np.concatenate([np.stack([p, np.roll(p, 1)], 1), q.reshape(-1, 2)]), 1)
+    pair, w = np.unique(np.concatenate([pair, np.sort(np.stack([p[:9], np.roll(p, 1)[:9]], 1), 1)]),
+                        axis=0, return_counts=True)
+    c = canon(n, *G.from_edges(n, pair, [int(x) for x in w]))
+    st = _check_solve(n, c, expect=oracle.noi(n, *c)[0])
+    assert st["seq_passes"] == 0
+
+
 def test_too_few_levels():
     """A dense small graph: the block solver has too few levels for it and the
     forests too few units per level, both see so at once, and the block solver
