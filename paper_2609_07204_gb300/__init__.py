@@ -376,7 +376,7 @@ def mincut_batch_solve(g: Graph, opts: Optional[MincutOptions] = None, *, bitmap
 
 
 def mincut_batch_info(g: Graph) -> tuple[int, int]:
-    """(vertex threshold of the one-warp-per-graph solver used by the last
+    """(vertex threshold of the small-graph solvers used by the last
     batch solve, number of graphs it solved)."""
     t = ctypes.c_int32(0)
     k = ctypes.c_int64(0)

@@ -232,7 +232,7 @@ struct mincut_graph {
   int* bw_scratch = nullptr;
   long long bw_scratch_words = 0;
   int bw_slots = 0;
-  // the launches of a solve whose graphs all take the one-warp solver,
+  // the launches of a solve whose graphs all take the small-graph solvers,
   // captured as a CUDA graph at the second solve with the same split
   cudaGraphExec_t bw_exec = nullptr;
   cudaStream_t bw_capture = nullptr;  // private stream the launches are captured on
@@ -1781,8 +1781,8 @@ cudaError_t bw_solve_list(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_
 }
 
 // A solve whose graphs all take the small solvers: state reset, then the
-// warp solver over the whole list (no round kernels, no host decisions
-// before the completion check).  Only stream-ordered calls, so that it can
+// solvers over the whole list (no round kernels, no host decisions before the
+// completion check).  Only stream-ordered calls, so that it can
 // be captured.
 cudaError_t bw_enqueue(mincut_graph* g, uint32_t pr, bool blocks, cudaStream_t s,
                        int* launches) {
@@ -1931,7 +1931,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
   g->M = g->M0;
   g->m_pending = false;
   if (op.spin_limit > 0) g->spin_limit = op.spin_limit;
-  // the small graphs are the warp solver's: the round kernels treat them as done
+  // the small graphs have their own solvers: the round kernels treat them as done
   {
     const int rc0 = bw_prepare(g, small_n, op.batch_small_n == 0);
     if (rc0) return rc0;
@@ -1941,7 +1941,7 @@ int batch_solve_impl(mincut_graph* g, const mincut_options& op, int64_t* cut_val
   stl.m_input = g->M0 / 2;
   const int max_rounds = op.max_rounds > 0 ? op.max_rounds : g->max_graph_n + 8;
   if (G > 0 && g->bw_count == G && !tl_prof) {
-    // every graph on the one-warp solver (no profiling): the same launches
+    // every graph on the small-graph solvers (no profiling): the same launches
     // on every solve of this batch, replayed from a CUDA graph once the
     // same split comes a second time (a batch solved once pays no capture);
     // captured on a private stream, since the caller's may be the legacy one
@@ -2278,7 +2278,7 @@ int mincut_batch_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut
                              (op.pass_table & (op.pass_table - 1))))
     return fail(MINCUT_ERR_INVALID, "pass_table must be a power of two in [256, 2048]");
   // 0: every graph the small solvers can take, but the dense ones.  (On 4,096 graphs of 20 to 2,000
-  // vertices a block per graph takes 2.3 ms, one warp per graph 5.4, the round
+  // vertices a block per graph takes 1.4 ms, one warp per graph 5.4, the round
   // kernels 13.3; lower thresholds lie between, and timing them on the first
   // solve cost a new batch 50 ms.)
   const int small_n = op.batch_small_n > 0  ? std::min(op.batch_small_n, kBwMaxN)

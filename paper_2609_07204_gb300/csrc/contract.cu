@@ -40,7 +40,6 @@ constexpr int kMovedBit = (int)0x80000000u;  // vinfo: neighbour's group has sev
 
 __device__ __forceinline__ unsigned sr_hash(int l) { return (unsigned)l * 0x9E3779B1u; }
 
-// cnt[L[x]] += 1 for every vertex (one atomic per distinct label of a warp).
 // The row classification's counters, in one launch.
 __global__ void rows_clear_kernel(int n, const int* __restrict__ n2p, long long mat_limit,
                                   int* __restrict__ cnt, int* __restrict__ gen,
@@ -59,6 +58,7 @@ __global__ void rows_clear_kernel(int n, const int* __restrict__ n2p, long long 
   }
 }
 
+// cnt[L[x]] += 1 for every vertex (one atomic per distinct label of a warp).
 __global__ void group_count_kernel(const int* __restrict__ L, int n, const int* __restrict__ n2p,
                                    long long mat_limit, int* __restrict__ cnt) {
   if ((long long)*n2p * *n2p <= mat_limit) return;

@@ -49,9 +49,9 @@
 //
 // Measured against the whole-graph CAPFOREST passes that such rounds needed
 // before (whole solves, one GB300): planted cut 2 x 2^19 (n = 1.02 M, m = 21 M)
-// 1,340 ms -> 8.8 ms, 2 x 2^15 83 -> 3.7 ms; against PR tests, label
-// propagation and concurrent passes: R-MAT scale 20 10-core 3.69 -> 0.95 ms
-// (0.83 ms of it here), scale 16 1.13 -> 0.39 ms, random weighted n = 150,001
+// 1,340 ms -> 8.8 ms, 2 x 2^15 83 -> 3.3 ms; against PR tests, label
+// propagation and concurrent passes: R-MAT scale 20 10-core 3.69 -> 0.87 ms
+// (0.73 ms of it here), scale 16 1.13 -> 0.39 ms, random weighted n = 150,001
 // (with its creation) 2.25 -> 0.68 ms.
 //
 // What is left: up to kFoMatrix labels it is summed in a matrix, above that
@@ -485,7 +485,7 @@ __device__ __noinline__ void fo_collect(const FoArgs& a, int u, long long b, lon
 }
 
 // (two blocks per SM, stated: without the 2 the compiler takes the same 64
-// registers and spills 664 bytes, with it 52)
+// registers and spills 664 bytes, with it 8, or 12 for 64-bit weights)
 template <typename WT>
 __global__ void __launch_bounds__(kFoThreads, 2) forest_kernel(FoArgs a) {
   __shared__ int s_hist[256];   // this block's changes since the last flush

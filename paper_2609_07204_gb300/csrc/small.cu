@@ -26,7 +26,7 @@
 // against one dependent visit per vertex (~0.8 us) of the one-warp solver and
 // the whole-graph passes.  Measured (whole calls, one GB300): G(2000, 16000)
 // 2.16 -> 0.42 ms, a 256-vertex graph created and solved 0.90 -> 0.21 ms,
-// 4,096 graphs (6.3 M edges) 5.44 -> 1.64 ms.
+// 4,096 graphs (6.3 M edges) 5.44 -> 1.45 ms.
 #include <algorithm>
 #include <climits>
 
