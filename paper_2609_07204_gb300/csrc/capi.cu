@@ -1905,6 +1905,10 @@ int batch_left_over(mincut_graph* g, const mincut_options& op, int max_rounds, m
   g->n = g->n0;
   g->M = g->M0;
   int rc = batch_rounds<WT>(g, op, op.deterministic != 0, max_rounds, live, stl);
+  if (rc == MINCUT_ERR_OOM) {  // (no room for a contraction's buffers: warps need none)
+    set_last_error("");
+    rc = sync_state(g);
+  }
   if (rc) return rc;
   if (b.voff != voff) std::swap(b.voff, b.voff_next);  // (captured launches name it)
   if (g->hst->batch_done < G) {

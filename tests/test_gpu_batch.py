@@ -276,6 +276,49 @@ def test_ordinary_graphs_take_no_shared_rounds():
 
 
 @pytest.mark.parametrize("det", [0, 1])
+def test_given_up_graphs_without_room_for_rounds(det):
+    """No memory for the contractions of shared rounds: a warp each finishes
+    the graphs that were given up, as it needs none."""
+    import ctypes
+
+    class Limited(mc._TorchAllocator):
+        def __init__(self, device):
+            super().__init__(device)
+            self.left = 1 << 30
+            give = self._alloc
+
+            def _alloc(nbytes, stream, ctx):
+                if self.left <= 0:
+                    return None
+                self.left -= 1
+                return give(nbytes, stream, ctx)
+
+            self._give, self._alloc = give, type(give)(_alloc)
+            self.struct = mc.MincutAllocator(self._alloc, self._free, None)
+
+    graphs = [synth.wheel(n, seed=n) for n in (70, 90, 130)]
+    graphs = [(s.n, s.row_ptr, s.col, s.w.astype(np.int64)) for s in graphs]
+    expect = [oracle.noi(*g)[0] for g in graphs]
+    vo, rp, col, w = mc.pack_graphs(graphs)
+    keep = [np.ascontiguousarray(vo, np.int64), np.ascontiguousarray(rp, np.int64),
+            np.ascontiguousarray(col, np.int32), np.ascontiguousarray(w, np.int32)]
+    alloc, out = Limited(0), ctypes.c_void_p(0)
+    rc = mc.load_library().mincut_batch_from_csr(
+        len(vo) - 1, *(a.ctypes.data for a in keep), mc.MINCUT_HOST_PTRS, ctypes.c_void_p(0),
+        ctypes.byref(alloc.struct), ctypes.byref(out))
+    assert rc == 0
+    B = mc.Graph(out.value, int(vo[-1]), keep, alloc)
+    B.G, B.vertex_offsets = len(vo) - 1, keep[0]
+    alloc.left = 4  # the small-graph solvers' lists and scratch
+    for _ in range(3):
+        _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=det))
+        assert mc.mincut_last_error() == ""
+    alloc.left = 1 << 30
+    _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=det))
+    B.destroy()
+
+
+@pytest.mark.parametrize("det", [0, 1])
 def test_batch_of_wheels_is_no_slower_than_rounds(det):
     """40 wheels of about 250 vertices: no more than twice the time of the
     round kernels, which solve them in one round (60 times by warps)."""
