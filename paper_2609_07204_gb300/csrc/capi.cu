@@ -2292,6 +2292,13 @@ int mincut_batch_solve(mincut_graph* g, const mincut_options* opts, int64_t* cut
   {
     ProfGuard pg(g, op.profile != 0);
     rc = batch_solve_impl<int32_t>(g, op, cut_values, side_bitmap, stats, small_n);
+    if (rc == MINCUT_ERR_OOM && op.batch_small_n == 0 && g->bw_count < g->batch.G &&
+        g->max_graph_n <= kBwMaxN) {
+      // no room for the round kernels' buffers: the dense graphs do without
+      set_last_error("");
+      op.batch_small_n = kBwMaxN;
+      rc = batch_solve_impl<int32_t>(g, op, cut_values, side_bitmap, stats, small_n);
+    }
   }
   g->cur = -1;
   g->n = g->n0;

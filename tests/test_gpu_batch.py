@@ -276,27 +276,28 @@ def test_ordinary_graphs_take_no_shared_rounds():
 
 
 @pytest.mark.parametrize("det", [0, 1])
-def test_given_up_graphs_without_room_for_rounds(det):
+@pytest.mark.parametrize("kind", ["given up", "dense"])
+def test_no_room_for_rounds(kind, det):
     """No memory for the contractions of shared rounds: a warp each finishes
-    the graphs that were given up, as it needs none."""
+    the graphs that were given up, and the dense ones, as it needs none."""
     import ctypes
 
     class Limited(mc._TorchAllocator):
         def __init__(self, device):
             super().__init__(device)
-            self.left = 1 << 30
+            self.left, self.refuse = 1 << 30, 0
             give = self._alloc
 
             def _alloc(nbytes, stream, ctx):
-                if self.left <= 0:
-                    return None
                 self.left -= 1
-                return give(nbytes, stream, ctx)
+                self.refuse -= 1
+                return None if self.left < 0 or self.refuse >= 0 else give(nbytes, stream, ctx)
 
             self._give, self._alloc = give, type(give)(_alloc)
             self.struct = mc.MincutAllocator(self._alloc, self._free, None)
 
-    graphs = [synth.wheel(n, seed=n) for n in (70, 90, 130)]
+    graphs = ([synth.wheel(n, seed=n) for n in (70, 90, 130)] if kind == "given up" else
+              [synth.cycle_plus(500, 50, 1, 20, i) for i in range(3)])
     graphs = [(s.n, s.row_ptr, s.col, s.w.astype(np.int64)) for s in graphs]
     expect = [oracle.noi(*g)[0] for g in graphs]
     vo, rp, col, w = mc.pack_graphs(graphs)
@@ -309,8 +310,9 @@ def test_given_up_graphs_without_room_for_rounds(det):
     assert rc == 0
     B = mc.Graph(out.value, int(vo[-1]), keep, alloc)
     B.G, B.vertex_offsets = len(vo) - 1, keep[0]
-    alloc.left = 4  # the small-graph solvers' lists and scratch
+    alloc.left = 4 if kind == "given up" else 1 << 30  # the small-graph solvers' lists and scratch
     for _ in range(3):
+        alloc.refuse = 2 if kind == "dense" else 0  # the buffers as one block, then the first
         _solve_and_check(B, vo, graphs, expect, mc.default_options(deterministic=det))
         assert mc.mincut_last_error() == ""
     alloc.left = 1 << 30
